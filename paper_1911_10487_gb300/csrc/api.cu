@@ -945,7 +945,8 @@ TapeLayout tape_layout(const fs_diff_plan* p) {
   size_t off = 0;
   T.L = off; off = align_up(off + 16 * F * N2 * p->P1);
   T.y = off; off = align_up(off + 16 * F * N2 * P.m1);
-  T.Vx = off; off = align_up(off + cxs * F * P.m * N2);
+  // V and u without a gap: one inverse transform writes both
+  T.Vx = off; off += cxs * F * P.m * N2;
   T.ux = off; off = align_up(off + cxs * F * P.m * N2);
   T.xi = off; off = align_up(off + rs * P.m * N2);
   T.la = off; off = align_up(off + 8 * F);
