@@ -19,11 +19,11 @@
  * the convention of PyTorch's complex autograd.
  *
  * Precision.  FS_FP64: everything in FP64.  FS_MIXED: W, xi, c, the FFTs and the
- * pointwise step 3 in FP32 (complex64 / float32 arrays); the per-mode normal
- * matrices, their Cholesky factors and the solves stay in FP64.
+ * pointwise step 3 in FP32 (complex64 / float32 arrays); the per-mode solves (the
+ * rank-one closed form) in two-float arithmetic (about 48 bits) and FP64.
  *
- * Memory.  A plan owns the per-mode normal matrices A_nu A_nu^H (they depend on
- * the geometry and frequencies only; 16 n_omega N^2 M1 (M1+1)/2 bytes).  Every
+ * Memory.  A plan owns per-mode tables of the kernel's factors (they depend on the
+ * geometry and frequencies only; about 16 n_omega N^2 (M1 + M/4 + 4) bytes).  Every
  * other buffer is caller-owned device memory: a tape (written by the forward,
  * read by VJP and JVP) and a scratch buffer, both 256-byte aligned, of the sizes
  * the *_bytes functions return.  A tape stays valid until the next forward into
@@ -45,7 +45,7 @@ extern "C" {
 typedef struct fs_diff_plan fs_diff_plan;
 
 /* Plan for one geometry, precision and frequency list (omega: host, n_omega
-   entries).  Allocates the normal matrices and enqueues their computation.
+   entries).  Allocates the mode tables and enqueues their computation.
    FS_EINVAL / FS_EUNSUPPORTED as fs_reconstruct; FS_ENOMEM if the allocation
    fails.  The plan keeps `ctx` (not owned) and must be destroyed before it. */
 fs_status fs_diff_plan_create(fs_ctx* ctx, const fs_geometry* geom, fs_precision prec, const double* omega,

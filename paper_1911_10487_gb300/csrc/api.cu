@@ -921,16 +921,19 @@ struct fs_diff_plan {
   Problem P;
   bool fp64 = true;
   int gb = 1;              // blocks per frequency of the per-mode kernels
-  size_t P1 = 0;           // packed lower-triangle entries per mode
-  void* buf = nullptr;     // normal matrices, then the twiddle table
-  double2* gram = nullptr;
+  void* buf = nullptr;     // the mode tables, then the twiddle table
+  DiffTables<double> t64;
+  DiffTables<float> t32;
   void* tw = nullptr;
+  template <typename R> const DiffTables<R>& tables() const;
 };
+template <> const DiffTables<double>& fs_diff_plan::tables<double>() const { return t64; }
+template <> const DiffTables<float>& fs_diff_plan::tables<float>() const { return t32; }
 
 namespace {
 
 struct TapeLayout {
-  size_t L, y, Vx, ux, xi, la, total;
+  size_t c, g, Vx, ux, xi, la, total;
 };
 struct ScratchLayout {
   size_t min, mout, xsp, partial, total;
@@ -943,13 +946,13 @@ TapeLayout tape_layout(const fs_diff_plan* p) {
   const size_t N2 = (size_t)P.n * P.n, F = P.n_omega;
   TapeLayout T;
   size_t off = 0;
-  T.L = off; off = align_up(off + 16 * F * N2 * p->P1);
-  T.y = off; off = align_up(off + 16 * F * N2 * P.m1);
+  T.c = off; off = align_up(off + 16 * F * N2);
+  T.g = off; off = align_up(off + 16 * F * N2 * P.m1);
   // V and u without a gap: one inverse transform writes both
   T.Vx = off; off += cxs * F * P.m * N2;
   T.ux = off; off = align_up(off + cxs * F * P.m * N2);
   T.xi = off; off = align_up(off + rs * P.m * N2);
-  T.la = off; off = align_up(off + 8 * F);
+  T.la = off; off = align_up(off + 16 * F);  // log alpha, alpha
   T.total = off;
   return T;
 }
@@ -988,12 +991,11 @@ fs_status diff_forward(fs_diff_plan* p, char* tape, char* scr, const void* W, co
   double* part = (double*)(scr + S.partial);
   double* la = (double*)(tape + T.la);
   cudaError_t e;
-  if ((e = cudaMemcpyAsync(la, log_alpha, 8 * F, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
-    return cuda_fail(ctx, e, "log_alpha copy");
+  if ((e = launch_diff_alpha(log_alpha, (int)F, la, s)) != cudaSuccess) return cuda_fail(ctx, e, "alpha");
   if ((e = launch_fft2_dense<R>((cx<R>*)W, wt, P.n, F * P.m1, false, tw, s)) != cudaSuccess)
     return cuda_fail(ctx, e, "fft2 W");
-  if ((e = launch_diff_forward<R>(P, p->gb, p->gram, wt, la, (double2*)(tape + T.L), (double2*)(tape + T.y), vt, ut,
-                                  part, ctx->ctr, s)) != cudaSuccess)
+  if ((e = launch_diff_forward<R>(P, p->tables<R>(), wt, la + F, (double2*)(tape + T.c), tape + T.g, vt, ut, part,
+                                  ctx->ctr, s)) != cudaSuccess)
     return cuda_fail(ctx, e, "diff forward");
   // V~ and U~ are adjacent, as are V and u in the tape: one inverse transform
   if ((e = launch_fft2_dense<R>(vt, (cx<R>*)(tape + T.Vx), P.n, 2 * F * P.m, true, tw, s)) != cudaSuccess)
@@ -1030,9 +1032,8 @@ fs_status diff_vjp(fs_diff_plan* p, const char* tape, char* scr, const void* gxi
     if ((e = launch_fft2_dense<R>(Vb, vbt, P.n, 2 * F * P.m, false, tw, s)) != cudaSuccess)
       return cuda_fail(ctx, e, "fft2 V-bar, u-bar");
   }
-  if ((e = launch_diff_vjp<R>(P, p->gb, (const double2*)(tape + T.L), (const double2*)(tape + T.y),
-                              gxi ? vbt : nullptr, gxi ? ubt : nullptr, la, gphi, gW ? wbt : nullptr, part, s)) !=
-      cudaSuccess)
+  if ((e = launch_diff_vjp<R>(P, p->tables<R>(), (const double2*)(tape + T.c), tape + T.g, gxi ? vbt : nullptr,
+                              gxi ? ubt : nullptr, la + F, gphi, gW ? wbt : nullptr, part, s)) != cudaSuccess)
     return cuda_fail(ctx, e, "diff vjp");
   if (gW && (e = launch_fft2_dense<R>(wbt, (cx<R>*)gW, P.n, F * P.m1, true, tw, s)) != cudaSuccess)
     return cuda_fail(ctx, e, "ifft2 W-bar");
@@ -1064,7 +1065,7 @@ fs_status diff_jvp(fs_diff_plan* p, const char* tape, char* scr, int n_dir, cons
     cx<R>* dux = dVx + (long long)nd * F * MN2;
     if ((e = launch_fft2_dense<R>((cx<R>*)dWc, dwt, P.n, (long long)nd * F * P.m1, false, tw, s)) != cudaSuccess)
       return cuda_fail(ctx, e, "fft2 dW");
-    if ((e = launch_diff_jvp<R>(P, p->gb, nd, (const double2*)(tape + T.L), (const double2*)(tape + T.y), dwt, la,
+    if ((e = launch_diff_jvp<R>(P, p->tables<R>(), nd, (const double2*)(tape + T.c), tape + T.g, dwt, la + F,
                                 dla ? dla + (long long)d0 * F : nullptr, dvt, dut, part, s)) != cudaSuccess)
       return cuda_fail(ctx, e, "diff jvp");
     if ((e = launch_fft2_dense<R>(dvt, dVx, P.n, 2LL * nd * F * P.m, true, tw, s)) != cudaSuccess)
@@ -1100,19 +1101,26 @@ fs_status fs_diff_plan_create(fs_ctx* ctx, const fs_geometry* g, fs_precision pr
   p->ctx = ctx;
   p->P = make_problem(g, n_omega, omega, 0.0, c0, o);
   p->fp64 = prec == FS_FP64;
-  p->gb = diff_blocks_per_omega(g->n, n_omega);
-  p->P1 = (size_t)g->m1 * (g->m1 + 1) / 2;
-  const size_t gbytes = align_up(16 * (size_t)n_omega * g->n * g->n * p->P1);
+  p->gb = diff_blocks_per_omega(g->n);
+  const size_t tbytes = align_up(p->fp64 ? diff_tables<double>(p->P, nullptr, nullptr, nullptr)
+                                         : diff_tables<float>(p->P, nullptr, nullptr, nullptr));
   const size_t twb = (p->fp64 ? 16 : 8) * (size_t)g->n;
-  if (cudaMalloc(&p->buf, gbytes + twb) != cudaSuccess) {
+  if (cudaMalloc(&p->buf, tbytes + twb) != cudaSuccess) {
     delete p;
-    return fail(ctx, FS_ENOMEM, "normal matrices (%lld bytes)", (long long)(gbytes + twb));
+    return fail(ctx, FS_ENOMEM, "mode tables (%lld bytes)", (long long)(tbytes + twb));
   }
-  p->gram = (double2*)p->buf;
-  p->tw = (char*)p->buf + gbytes;
-  e = p->fp64 ? launch_twiddles<double>((double2*)p->tw, g->n, ctx->stream)
-              : launch_twiddles<float>((float2*)p->tw, g->n, ctx->stream);
-  if (e == cudaSuccess) e = launch_diff_gram(p->P, p->gram, ctx->stream);
+  p->tw = (char*)p->buf + tbytes;
+  if (p->fp64) {
+    DiffTablesOut<double> to;
+    diff_tables<double>(p->P, p->buf, &p->t64, &to);
+    e = launch_twiddles<double>((double2*)p->tw, g->n, ctx->stream);
+    if (e == cudaSuccess) e = launch_diff_tables<double>(p->P, p->t64, to, ctx->stream);
+  } else {
+    DiffTablesOut<float> to;
+    diff_tables<float>(p->P, p->buf, &p->t32, &to);
+    e = launch_twiddles<float>((float2*)p->tw, g->n, ctx->stream);
+    if (e == cudaSuccess) e = launch_diff_tables<float>(p->P, p->t32, to, ctx->stream);
+  }
   if (e != cudaSuccess) {
     cudaFree(p->buf);
     delete p;

@@ -3,223 +3,359 @@
 //
 //   (W, log alpha) -> (xi, Phi),   Phi_omega = sum_nu ||A_nu V~_nu - W~_nu||^2.
 //
-// Per mode nu of frequency omega the matrix of eq. (8) is assembled as
-// A_kl = E_k P_l (E_k = gamma e^{i k_z (z_k - z_top)}, P_l = e^{i k_z (z_top - z'_l)})
-// and scaled to unit Frobenius norm, A^ = A / sqrt(tr), tr = ||A||_F^2:
+// Every data plane lies above X, so the matrix of eq. (8) is exactly rank one,
+// A_kl = E_k P_l with E_k = gamma e^{i k_z (z_k - z_top)}, P_l = e^{i k_z (z_top - z'_l)}
+// (solve_rank1.cu), and (A A^H + alpha I)^-1 needs no matrix at all.  With e = E / ||E||,
+// tr = ||E||^2 ||P||^2, mu = tr / (tr + alpha), kappa = alpha / (tr + alpha),
+// eta = ||E|| / (tr + alpha) and c = e^H b:
 //
-//   G^ = A^ A^^H                      dense, FP64; depends on geometry and omega only,
-//                                     computed once per plan (k_diff_gram)
-//   H^ = G^ + alpha' I = L L^H        alpha' = alpha / tr; Cholesky per alpha (saved)
-//   y' = H^^-1 b,  V~ = A^^H y' / sqrt(tr)     (= A^H (A A^H + alpha I)^-1 b, the
-//                                     normal solution of Sec. 4 comment b, dual form)
-//   U~ = U~0 + omega^2 T V~           eq. (9), two affine scans over the planes
-//   Phi_nu = alpha'^2 ||y'||^2        (dual residual identity b - A V~ = alpha y)
-//
+//   V~_l = conj(P_l) eta c                    (= A^H (A A^H + alpha I)^-1 b)
+//   U~_l = U~0_l + T_l V~_l                   eq. (9): V~ is a power of q = e^{i k_z h_z}
+//                                             along the planes, so its two recurrences sum
+//                                             to the factor T_l of the geometry,
+//       evanescent (q real):  T_l = gamma (sum_{j <= l} q^2j + (M - 1 - l))
+//       propagating (|q| = 1): T_l = gamma ((l + 1) + sum_{1 <= j <= M-1-l} q^2j)
+//   Phi  = ||g||^2 + kappa^2 mu (1 + kappa) |c|^2,  g = b - mu (1 + kappa) c e
 // then V = F^-1[V~], u = F^-1[U~] and xi = Re(sum conj(u) V) / sum |u|^2 (step 3).
-// The VJP and JVP reuse the saved factor L and y'; in scaled form
-//   b-bar   = H^^-1 (A^ t / sqrt(tr) + 2 alpha'^2 Phi-bar y'),
-//             t = V~-bar + (omega^2 T)^H U~-bar
-//   lnalpha-bar = -alpha' Re(b-bar^H y') + 2 Phi-bar alpha'^2 ||y'||^2
-//   y-dot'  = H^^-1 (b-dot - lnalpha-dot alpha' y'),  V~-dot = A^^H y-dot' / sqrt(tr)
-//   Phi-dot = 2 alpha'^2 (lnalpha-dot ||y'||^2 + Re y'^H y-dot').
-// Modes with no solution (grazing, or a matrix that underflowed, or alpha' beyond
-// AP_MAX where V~ is zero in FP64) keep V~ = 0; their tape slot holds b, their
-// residual.  Gradients use grad z = dL/dRe z + i dL/dIm z.
+//   VJP:  tau = sum_l P_l (V~-bar_l + conj(T_l) U~-bar_l)
+//         b-bar = eta tau e + 2 Phi-bar g       (g is half the gradient of Phi in b)
+//         lnalpha-bar = -kappa Re(conj(tau) eta c) + 2 Phi-bar kappa^2 mu |c|^2
+//   JVP:  c-dot = e^H b-dot,  V~-dot_l = conj(P_l) eta (c-dot - kappa lnalpha-dot c),
+//         U~-dot_l = T_l V~-dot_l,
+//         Phi-dot = 2 Re g^H b-dot + 2 kappa^2 mu lnalpha-dot |c|^2
+// The tape keeps c and g per mode.  Modes with no solution (grazing, a matrix that
+// underflowed, or alpha / tr beyond AP_MAX where V~ is zero in FP64) are mu = eta = 0,
+// kappa = 1: V~ = 0 and g = b, their residual.  Gradients use grad z = dL/dRe z + i dL/dIm z.
 //
-// The per-mode kernels run one warp per mode: lane k owns row k of H (and of L),
-// the triangular solves broadcast the pivot value with a shuffle, and the
-// Toeplitz kernel of eq. (9) is the warp scan of modes.cuh.  Per-frequency sums
-// (Phi, lnalpha-bar, Phi-dot) go to per-block partials reduced in a fixed order,
-// so results do not depend on scheduling.
+// What bounds it.  A dense factorisation costs ~(4/3) M1^3 FP64 operations per mode, and
+// all N^2 modes are solved at a fixed alpha; the closed form is O(M1 + M) per mode, and the
+// kernels stream their fields (128^2 x 64, 32 data planes, 4 frequencies, mixed precision;
+// Cholesky factors before, this form now): forward 16.6 ms -> 58 us for 150 MB, VJP 8.6 ms ->
+// 95 us for 170 MB, 16 JVP directions 107.8 ms -> 557 us for 1.4 GB.  A block holds 32 consecutive modes (lanes: every
+// access to a plane is one 256-byte row) and splits the data planes and blocks of PB X planes
+// over its DG warps, so that a small grid still fills the SMs.  The geometry (e, q, gamma, and
+// P and T at one plane of each block of PB) is tabulated once per plan in FP64; inside a block
+// of planes P and T follow by at most PB - 1 products, whose rounding is that of the
+// exponentials themselves.  FS_FP64 computes in FP64, FS_MIXED in two-float arithmetic
+// (~48 bits, twofloat.cuh) on the FP32 pipe from tables split into two floats: on this GPU
+// FP64 instructions and conversions run at 1/64 of the FP32 rate, and the fields in and out
+// are FP32.
+// Per-frequency sums (Phi, lnalpha-bar, Phi-dot) go to per-block partials reduced in a fixed
+// order, so results do not depend on scheduling.
 #include <math.h>
 
 #include "diff.cuh"
 #include "modes.cuh"
+#include "twofloat.cuh"
 
 namespace fl {
 
 namespace {
 
-constexpr int DW = 4;             // warps (modes in flight) per block
-constexpr int GT = 128;           // threads of the normal-matrix kernel
-constexpr double AP_MAX = 1e290;  // alpha' above this: H^ = alpha' I to FP64, V~ = 0
+constexpr int PB = DIFF_PB;       // X planes per block of planes
+constexpr int DG = 8;             // warps per block
+constexpr int DT = 32 * DG;       // threads per block of the per-mode kernels
+constexpr int KC = DENSE_M1 / DG; // data planes per warp
+constexpr int JG = 4;             // JVP directions per pass over the planes
+constexpr double AP_MAX = 1e290;  // alpha / tr above this: V~ = 0 in FP64
+static_assert(DENSE_M <= PB * DG, "one block of planes per warp");
+static_assert(DENSE_M1 == KC * DG, "data planes dealt over the warps");
 
-struct WarpMem {
-  double2 H[DENSE_M1][DENSE_M1 + 1];  // H^ (lower triangle) -> Cholesky factor L
-  double2 E[DENSE_M1];              // E_k / sqrt(sum |E|^2)
-  double2 Pz[DENSE_M];              // P_l / sqrt(sum |P|^2)
-  double2 v[DENSE_M], t[DENSE_M], F[DENSE_M], B[DENSE_M];
-  double dinv[DENSE_M1];            // 1 / L_jj
+// The arithmetic of the per-mode kernels: FP64, or two-float in the mixed precision.
+template <typename R> struct Wide;
+template <> struct Wide<double> {
+  using T = double;   // value
+  using S = double;   // one component in a table
+  using SC = double2; // a complex value on the tape
+  __device__ __forceinline__ static T ld(const S* p) { return *p; }
+  __device__ __forceinline__ static S st(double x) { return x; }
+  __device__ __forceinline__ static T from(double x) { return x; }
+  __device__ __forceinline__ static T from_r(double x) { return x; }
+  __device__ __forceinline__ static double d(T x) { return x; }
+  __device__ __forceinline__ static double r(T x) { return x; }
+  __device__ __forceinline__ static T neg(T a) { return -a; }
+  __device__ __forceinline__ static T add(T a, T b) { return a + b; }
+  __device__ __forceinline__ static T mul(T a, T b) { return a * b; }
+  __device__ __forceinline__ static T mulr(T a, double x) { return a * x; }
+  __device__ __forceinline__ static T fma(T a, T b, T c) { return a * b + c; }
+  __device__ __forceinline__ static T fmar(T a, double x, T c) { return a * x + c; }
+  __device__ __forceinline__ static T wsum(T a) { return warp_sum(a); }
+  __device__ __forceinline__ static SC pack(T re, T im) { return make_double2(re, im); }
+  __device__ __forceinline__ static void unpack(SC v, T& re, T& im) { re = v.x; im = v.y; }
+};
+template <> struct Wide<float> {
+  using T = ff;
+  using S = float2;
+  using SC = float4;
+  __device__ __forceinline__ static T ld(const S* p) { const float2 v = *p; return ff{v.x, v.y}; }
+  __device__ __forceinline__ static S st(double x) { const ff v = ff_from(x); return make_float2(v.hi, v.lo); }
+  __device__ __forceinline__ static T from(double x) { return ff_from(x); }
+  __device__ __forceinline__ static T from_r(float x) { return ff{x, 0.f}; }
+  __device__ __forceinline__ static double d(T x) { return ff_to(x); }
+  __device__ __forceinline__ static float r(T x) { return x.hi + x.lo; }
+  __device__ __forceinline__ static T neg(T a) { return ff_neg(a); }
+  __device__ __forceinline__ static T add(T a, T b) { return ff_add(a, b); }
+  __device__ __forceinline__ static T mul(T a, T b) { return ff_mul(a, b); }
+  __device__ __forceinline__ static T mulr(T a, float x) { return ff_mul_f(a, x); }
+  __device__ __forceinline__ static T fma(T a, T b, T c) { return ff_add(ff_mul(a, b), c); }
+  __device__ __forceinline__ static T fmar(T a, float x, T c) { return ff_add(ff_mul_f(a, x), c); }
+  __device__ __forceinline__ static T wsum(T a) { return ff_warp_sum(a); }
+  __device__ __forceinline__ static SC pack(T re, T im) { return make_float4(re.hi, re.lo, im.hi, im.lo); }
+  __device__ __forceinline__ static void unpack(SC v, T& re, T& im) { re = ff{v.x, v.y}; im = ff{v.z, v.w}; }
 };
 
-struct ModeGeo {
-  double2 gamma, q;  // omega^2 h_z (-i / 2 k_z);  e^{i k_z h_z}
-  double tr, rs;     // ||A||_F^2, 1 / sqrt(tr)
-  bool usable;
+template <typename T> struct WC { T re, im; };  // complex value
+
+// 2^e for -252 <= e <= 252 as a product of two floats (both finite and normal)
+__device__ __forceinline__ float2 pow2_pair(int e) {
+  e = e < -252 ? -252 : (e > 252 ? 252 : e);
+  const int a = e / 2, b = e - a;
+  return make_float2(__int_as_float((a + 127) << 23), __int_as_float((b + 127) << 23));
+}
+__device__ __forceinline__ int exponent_of(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff) - 1023; }
+__device__ __forceinline__ int exponent_of(float x) { return (int)((__float_as_int(x) >> 23) & 0xff) - 127; }
+
+// A complex factor that multiplies wide values into outputs.  Two-float holds it as a
+// mantissa and a power of two: FP64 reaches factors (eta c, 2 Phi-bar N^2) outside the FP32
+// range whose products with the fields are inside it.
+template <typename R> struct Factor;
+template <> struct Factor<double> {
+  double re, im;
+  __device__ __forceinline__ static Factor make(double2 v) { return Factor{v.x, v.y}; }
+  __device__ __forceinline__ double out(double x) const { return x; }
+};
+template <> struct Factor<float> {
+  ff re, im;
+  float2 s;
+  __device__ __forceinline__ static Factor make(double2 v) {
+    const double a = fmax(fabs(v.x), fabs(v.y));
+    int e = 0;
+    if (a > 0.0 && isfinite(a)) e = exponent_of(a);
+    e = e < -252 ? -252 : (e > 252 ? 252 : e);
+    const double sc = __longlong_as_double((long long)(1023 - e) << 52);
+    Factor f;
+    f.re = ff_from(v.x * sc);
+    f.im = ff_from(v.y * sc);
+    f.s = pow2_pair(e);
+    return f;
+  }
+  __device__ __forceinline__ float out(ff x) const { return ((x.hi + x.lo) * s.x) * s.y; }
 };
 
-// Wavenumber, kernel factors and the scaled E, P of mode nu (one full warp).
-__device__ ModeGeo mode_setup(const Problem& P, int om, long long nu, double2* E, double2* Pz) {
-  const int lane = threadIdx.x & 31;
-  const int N = P.n, n = P.m1, m = P.m;
+// exponent of the largest of the warp's values (uniform; 0 for all zero): sums of squares
+// and products are taken of values scaled by its power of two, which keeps them in the
+// FP32 range of the two-float form.  FP64 needs none.
+__device__ __forceinline__ int warp_exponent(float a) {
+  for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
+  const int e = exponent_of(a);
+  return a > 0.f ? (e < -120 ? -120 : (e > 120 ? 120 : e)) : 0;
+}
+__device__ __forceinline__ int warp_exponent(double) { return 0; }
+__device__ __forceinline__ double scale_by(double x, int) { return x; }
+__device__ __forceinline__ ff scale_by(ff x, int e) {
+  const float s = __int_as_float((e + 127) << 23);
+  return ff{x.hi * s, x.lo * s};
+}
+__device__ __forceinline__ float scale_by(float x, int e) { return x * __int_as_float((e + 127) << 23); }
+__device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
+
+// ---------------------------------------------------------------------------
+// tables of the geometry, one block per 32 modes (k_diff_tables, once per plan), FP64
+// ---------------------------------------------------------------------------
+struct ModeK {
+  double2 kz, gamma;
+  bool prop, grazing;
+};
+__device__ __forceinline__ ModeK mode_k(const Problem& P, int om, long long nu) {
+  const int N = P.n;
   const int i2 = (int)(nu / N), i1 = (int)(nu - (long long)i2 * N);
   const int m1 = i1 < N / 2 ? i1 : i1 - N, m2 = i2 < N / 2 ? i2 : i2 - N;
   const int msq = m1 * m1 + m2 * m2;
-  ModeGeo g;
-  const bool grazing = msq >= P.graz_lo[om] && msq <= P.graz_hi[om];
-  const double k0 = P.omega[om] / P.c0;
-  const double kn = 2.0 * M_PI / P.period;
-  const double qq = k0 * k0 - kn * kn * (double)msq;
-  double2 kz = qq >= 0.0 ? make_double2(sqrt(qq), 0.0) : make_double2(0.0, sqrt(-qq));
-  const double g0 = 0.5 * P.omega[om] * P.omega[om] * P.hz;
-  if (grazing) {
-    kz = make_double2(1.0, 0.0);  // k_z = 0: excluded; placeholder keeps the arithmetic finite
-    g.gamma = make_double2(0.0, 0.0);
-  } else {
-    g.gamma = qq >= 0.0 ? make_double2(0.0, -g0 / kz.x) : make_double2(-g0 / kz.y, 0.0);
-  }
-  const double ztop = P.z1 + (m - 0.5) * P.hz;
-  const double2 e = lane < n ? g.gamma * exp_ikz(kz, P.zy[lane] - ztop) : make_double2(0, 0);
-  const int l0 = lane, l1 = lane + 32;
-  const double2 p0 = l0 < m ? exp_ikz(kz, ztop - (P.z1 + (l0 + 0.5) * P.hz)) : make_double2(0, 0);
-  const double2 p1 = l1 < m ? exp_ikz(kz, ztop - (P.z1 + (l1 + 0.5) * P.hz)) : make_double2(0, 0);
-  const double sE = warp_sum(abs2(e));
-  const double sP = warp_sum(abs2(p0) + abs2(p1));
-  g.tr = sE * sP;
-  g.usable = !grazing && g.tr > 0.0;
-  g.rs = g.usable ? 1.0 / sqrt(g.tr) : 0.0;
-  if (g.usable) {
-    const double re = 1.0 / sqrt(sE), rp = 1.0 / sqrt(sP);
-    if (lane < n) E[lane] = re * e;
-    if (l0 < m) Pz[l0] = rp * p0;
-    if (l1 < m) Pz[l1] = rp * p1;
-  }
-  g.q = exp_ikz(kz, P.hz);
-  __syncwarp();
+  ModeK g;
+  g.grazing = msq >= P.graz_lo[om] && msq <= P.graz_hi[om];
+  const double qq = P.k0[om] * P.k0[om] - P.kn * P.kn * (double)msq;
+  g.prop = qq >= 0.0;
+  const double kz = g.grazing ? 1.0 : sqrt(fabs(qq));  // k_z = 0 is excluded: a placeholder
+  g.kz = g.prop ? make_double2(kz, 0.0) : make_double2(0.0, kz);
+  const double gm = g.grazing ? 0.0 : -P.g0[om] / kz;
+  g.gamma = g.prop ? make_double2(0.0, gm) : make_double2(gm, 0.0);
   return g;
 }
 
-__device__ __forceinline__ long long col_off(int j, int n) { return (long long)j * n - (long long)j * (j - 1) / 2; }
-
-// packed lower triangle (column-major: column j holds rows j..n-1) <-> S.H
-__device__ __forceinline__ void load_lower(WarpMem& S, const double2* __restrict__ src, int n, int lane) {
-  for (int j = 0; j < n; ++j)
-    if (lane < n - j) S.H[j + lane][j] = src[col_off(j, n) + lane];
-  __syncwarp();
-}
-__device__ __forceinline__ void store_lower(double2* __restrict__ dst, const WarpMem& S, int n, int lane) {
-  for (int j = 0; j < n; ++j)
-    if (lane < n - j) dst[col_off(j, n) + lane] = S.H[j + lane][j];
-}
-
-// (row, column) of the packed lower triangle in column-major order (column j holds
-// rows j..n-1), one entry per element, for the trailing updates of the Cholesky
-// factorisation; built once per block for the problem's M1.
-constexpr int MAX_P1 = DENSE_M1 * (DENSE_M1 + 1) / 2;
-__device__ void build_rc(unsigned short* rc, int n) {
-  const int P1 = n * (n + 1) / 2;
-  for (int e = threadIdx.x; e < P1; e += blockDim.x) {
-    int j = 0;
-    while (col_off(j + 1, n) <= e) ++j;
-    const int r = j + (int)(e - col_off(j, n));
-    rc[e] = (unsigned short)(r << 8 | j);
+template <typename R>
+__global__ void __launch_bounds__(DT) k_diff_tables(Problem P, DiffTables<R> tab, DiffTablesOut<R> out) {
+  using W = Wide<R>;
+  __shared__ double2 p2[DENSE_M][32];  // |P_l|^2 (evanescent) or P_l^2 (propagating)
+  __shared__ double es[DG][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int om = blockIdx.y, n = P.m1, m = P.m;
+  const long long N2 = (long long)P.n * P.n;
+  const long long nu = (long long)blockIdx.x * 32 + lane;
+  const bool valid = nu < N2;
+  const ModeK g = mode_k(P, om, valid ? nu : 0);
+  const double ztop = P.z1 + (m - 0.5) * P.hz;
+  // E_k: an evanescent E is scaled by e^{k_z (z_min - z_top)}, so that its direction e keeps
+  // full precision where ||E|| underflows
+  const double base = g.prop ? ztop : P.zy_min;
+  double2 e[KC];
+  double se = 0.0;
+#pragma unroll
+  for (int i = 0; i < KC; ++i) {
+    const int k = w + DG * i;
+    e[i] = k < n ? g.gamma * exp_ikz(g.kz, P.zy[k] - base) : make_double2(0.0, 0.0);
+    se += abs2(e[i]);
   }
-}
-
-// In-place Cholesky H = L L^H of the lower triangle (right-looking).  The pivot
-// column is scaled by lane (lane k, row k); the trailing update of step j -- the
-// entries (r, c), j < c <= r, a contiguous suffix of the packed order -- is dealt
-// evenly over the 32 lanes, so the FP64 pipe is not spent on idle lanes.  A pivot
-// that is not positive (H not positive definite to rounding) is replaced by the
-// smallest positive double and reported through `bad`.
-__device__ void cholesky(WarpMem& S, int n, int lane, const unsigned short* rc, bool& bad) {
-  const int P1 = n * (n + 1) / 2;
-  for (int j = 0; j < n; ++j) {
-    double d = S.H[j][j].x;
-    if (!(d > 0.0)) { bad = true; d = 2.2250738585072014e-308; }
-    const double ljj = sqrt(d), inv = rcp64(ljj);
-    __syncwarp();
-    if (lane == j) { S.H[j][j] = make_double2(ljj, 0.0); S.dinv[j] = inv; }
-    if (lane > j && lane < n) S.H[lane][j] = inv * S.H[lane][j];
-    __syncwarp();
-    for (int e = (int)col_off(j + 1, n) + lane; e < P1; e += 32) {
-      const int r = rc[e] >> 8, c = rc[e] & 255;
-      S.H[r][c] = S.H[r][c] - mulc(S.H[r][j], S.H[c][j]);
+  es[w][lane] = se;
+  for (int l = w; l < m; l += DG) {
+    const double2 p = exp_ikz(g.kz, ztop - (P.z1 + (l + 0.5) * P.hz));
+    p2[l][lane] = g.prop ? p * p : make_double2(abs2(p), 0.0);
+    const int a = l / PB, top = min(PB * a + PB, m) - 1;
+    if (l == top && valid) {
+      const long long at = ((long long)om * tab.nb + a) * N2 + nu;
+      out.pr[at] = W::st(p.x);
+      out.pi[at] = W::st(p.y);
     }
-    __syncwarp();
   }
-}
-
-__device__ void set_dinv(WarpMem& S, int n, int lane) {
-  if (lane < n) S.dinv[lane] = rcp64(S.H[lane][lane].x);
-  __syncwarp();
-}
-
-// x = (L L^H)^-1 r, lane k holding r_k (zero for lanes >= n) and returning x_k
-__device__ double2 chol_solve(const WarpMem& S, int n, int lane, double2 r) {
-  for (int j = 0; j < n; ++j) {
-    double2 zj = make_double2(__shfl_sync(0xffffffffu, r.x, j), __shfl_sync(0xffffffffu, r.y, j));
-    zj = S.dinv[j] * zj;
-    if (lane == j) r = zj;
-    if (lane > j && lane < n) r = r - S.H[lane][j] * zj;
+  __syncthreads();
+  double nn = 0.0;
+  for (int i = 0; i < DG; ++i) nn += es[i][lane];  // ||E||^2, scaled
+  const double rn = nn > 0.0 ? 1.0 / sqrt(nn) : 0.0;
+  if (valid)
+#pragma unroll
+    for (int i = 0; i < KC; ++i) {
+      const int k = w + DG * i;
+      if (k < n) {
+        const long long at = ((long long)om * n + k) * N2 + nu;
+        out.er[at] = W::st(rn * e[i].x);
+        out.ei[at] = W::st(rn * e[i].y);
+      }
+    }
+  if (w == 0 && valid) {
+    const long long at = (long long)om * N2 + nu;
+    const double sc = g.prop ? 1.0 : exp(-g.kz.y * (P.zy_min - ztop));
+    const double ne = sqrt(nn) * sc;
+    const double2 q = exp_ikz(g.kz, P.hz);
+    out.q[at] = typename DiffTables<R>::S2{W::st(q.x), W::st(q.y)};
+    out.g[at] = W::st(g.prop ? g.gamma.y : g.gamma.x);
+    // sums from the top plane down: sum_{j <= l} q^2j = sum |P_{M-1-j}|^2 (evanescent),
+    // sum_{1 <= j <= n} q^2j = sum P_{M-1-j}^2 (propagating)
+    double2 acc = make_double2(0.0, 0.0);
+    for (int j = 0; j < m; ++j) {
+      // evanescent: acc = sum_{i <= j} q^2i belongs to plane j, stored at block starts
+      // propagating: acc = sum_{1 <= i <= j} q^2i belongs to plane M-1-j, stored at block tops
+      if (!g.prop || j > 0) acc = acc + p2[m - 1 - j][lane];
+      const int l = g.prop ? m - 1 - j : j, a = l / PB;
+      if (g.prop ? l == min(PB * a + PB, m) - 1 : l == PB * a) {
+        const double2 s = g.gamma * acc;
+        const long long ab = ((long long)om * tab.nb + a) * N2 + nu;
+        out.sr[ab] = W::st(s.x);
+        out.si[ab] = W::st(s.y);
+      }
+    }
+    const double sp = g.prop ? (double)m : acc.x;  // ||P||^2
+    const double tr = g.grazing ? 0.0 : ne * ne * sp;
+    out.tr[at] = tr;
+    out.ne[at] = tr > 0.0 ? (g.prop ? -ne : ne) : (g.prop ? -0.0 : 0.0);  // the sign marks propagating modes
   }
-  for (int j = n - 1; j >= 0; --j) {
-    double2 xj = make_double2(__shfl_sync(0xffffffffu, r.x, j), __shfl_sync(0xffffffffu, r.y, j));
-    xj = S.dinv[j] * xj;
-    if (lane == j) r = xj;
-    if (lane < j) r = r - cmul_conj_a(S.H[j][lane], xj);
-  }
-  return r;
-}
-
-// v_l = rs sum_k conj(A^_kl) y_k for l = lane, lane + 32 (A^_kl = E_k P_l)
-__device__ void apply_AH(const WarpMem& S, int n, int m, int lane, double2 y, double rs, double2& v0, double2& v1) {
-  const double2 p0 = lane < m ? S.Pz[lane] : make_double2(0, 0);
-  const double2 p1 = lane + 32 < m ? S.Pz[lane + 32] : make_double2(0, 0);
-  double2 a0 = make_double2(0, 0), a1 = make_double2(0, 0);
-  for (int k = 0; k < n; ++k) {
-    const double2 yk = make_double2(__shfl_sync(0xffffffffu, y.x, k), __shfl_sync(0xffffffffu, y.y, k));
-    const double2 ek = S.E[k];
-    a0 = a0 + cmul_conj_a(ek * p0, yk);
-    a1 = a1 + cmul_conj_a(ek * p1, yk);
-  }
-  v0 = rs * a0;
-  v1 = rs * a1;
-}
-
-// s_k = rs sum_l A^_kl t_l, t in S.t (lane k < n)
-__device__ double2 apply_A(const WarpMem& S, int n, int m, int lane, double rs) {
-  const double2 ek = lane < n ? S.E[lane] : make_double2(0, 0);
-  double2 acc = make_double2(0, 0);
-  for (int l = 0; l < m; ++l) acc = acc + (ek * S.Pz[l]) * S.t[l];
-  return rs * acc;
-}
-
-// g (F + B) with F_l = sum_{l' <= l} q^(l-l') x_l', B_l = sum_{l' > l} q^(l'-l) x_l',
-// x in S.v; returns the entries l = lane, lane + 32.  Full warp.
-__device__ void toeplitz(WarpMem& S, int m, int lane, double2 q, double2 g, double2& o0, double2& o1) {
-  affine_scan64(S.v, m, q, S.F);
-  for (int r = lane; r < m; r += 32) S.t[r] = r == 0 ? make_double2(0, 0) : q * S.v[m - r];
-  __syncwarp();
-  affine_scan64(S.t, m, q, S.B);
-  __syncwarp();
-  o0 = lane < m ? g * (S.F[lane] + S.B[m - 1 - lane]) : make_double2(0, 0);
-  o1 = lane + 32 < m ? g * (S.F[lane + 32] + S.B[m - 33 - lane]) : make_double2(0, 0);
-  __syncwarp();
-}
-
-__device__ __forceinline__ void put_v(WarpMem& S, int m, int lane, double2 v0, double2 v1) {
-  if (lane < m) S.v[lane] = v0;
-  if (lane + 32 < m) S.v[lane + 32] = v1;
-  __syncwarp();
 }
 
 // incident field of mode 0: U~0_l = N^2 e^{-i k0 z'_l}
-__device__ __forceinline__ double2 incident(const Problem& P, int om, int l) {
-  double s, c;
-  sincos(-(P.omega[om] / P.c0) * (P.z1 + (l + 0.5) * P.hz), &s, &c);
-  const double n2 = (double)P.n * P.n;
-  return make_double2(n2 * c, n2 * s);
+__global__ void k_diff_incident(Problem P, double2* __restrict__ inc) {
+  const int om = blockIdx.x;
+  for (int l = threadIdx.x; l < P.m; l += blockDim.x) {
+    double s, c;
+    sincos(-P.k0[om] * (P.z1 + (l + 0.5) * P.hz), &s, &c);
+    const double n2 = (double)P.n * P.n;
+    inc[om * P.m + l] = make_double2(n2 * c, n2 * s);
+  }
+}
+
+// log alpha -> the tape's log alpha and alpha
+__global__ void k_diff_alpha(const double* __restrict__ log_alpha, int F, double* __restrict__ la) {
+  const int om = threadIdx.x;
+  if (om < F) {
+    la[om] = log_alpha[om];
+    la[F + om] = exp(log_alpha[om]);
+  }
+}
+
+// the scalars of one mode at alpha
+struct ModeScalars { double eta, mu, kappa; };
+__device__ __forceinline__ ModeScalars mode_scalars(double tr, double ne, double alpha) {
+  ModeScalars s{0.0, 0.0, 1.0};
+  if (tr > 0.0 && alpha < AP_MAX * tr) {
+    const double r = rcp64(tr + alpha);
+    s.eta = fabs(ne) * r;
+    s.mu = tr * r;
+    s.kappa = alpha * r;
+  }
+  return s;
+}
+
+// P_l and T_l of the planes of block a, handed to f(l, P, T, l-th index j): real (an
+// evanescent mode: P and T real) or complex.
+template <typename R, typename F>
+__device__ __forceinline__ void planes_real(const DiffTables<R>& tab, long long at, long long ab, int a, int m, F f) {
+  using W = Wide<R>;
+  using T = typename W::T;
+  const T q = W::ld(&tab.q[at].x), g = W::ld(tab.g + at);
+  const T q2 = W::mul(q, q);
+  const int top = min(PB * a + PB, m) - 1;
+  T p[PB];
+  T cur = W::ld(tab.pr + ab);
+#pragma unroll
+  for (int j = PB - 1; j >= 0; --j) {
+    const int l = PB * a + j;
+    if (l < top) cur = W::mul(cur, q);
+    p[j] = cur;
+  }
+  T h = W::ld(tab.sr + ab);
+#pragma unroll
+  for (int j = 0; j < PB; ++j) {
+    const int l = PB * a + j;
+    if (l <= top) f(l, j, p[j], W::fmar(g, (R)(m - 1 - l), h));
+    h = W::fma(q2, h, g);
+  }
+}
+template <typename R, typename F>
+__device__ __forceinline__ void planes_cplx(const DiffTables<R>& tab, long long at, long long ab, int a, int m,
+                                            bool prop, F f) {
+  using W = Wide<R>;
+  using T = typename W::T;
+  using C = WC<T>;
+  const T zero = W::from(0.0);
+  const C q = C{W::ld(&tab.q[at].x), W::ld(&tab.q[at].y)};
+  const T g = W::ld(tab.g + at);
+  const C q2 = C{W::fma(q.re, q.re, W::neg(W::mul(q.im, q.im))), W::mulr(W::mul(q.re, q.im), (R)2)};
+  const int top = min(PB * a + PB, m) - 1;
+  C p = C{W::ld(tab.pr + ab), W::ld(tab.pi + ab)};
+  C s = C{W::ld(tab.sr + ab), W::ld(tab.si + ab)};
+  if (prop) {  // both from the block's top plane down
+#pragma unroll 1
+    for (int l = top; l >= PB * a; --l) {
+      if (l < top) {
+        p = C{W::fma(p.re, q.re, W::neg(W::mul(p.im, q.im))), W::fma(p.re, q.im, W::mul(p.im, q.re))};
+        const C t = C{s.re, W::add(s.im, g)};  // gamma = i g
+        s = C{W::fma(q2.re, t.re, W::neg(W::mul(q2.im, t.im))), W::fma(q2.re, t.im, W::mul(q2.im, t.re))};
+      }
+      f(l, p, C{s.re, W::fmar(g, (R)(l + 1), s.im)});
+    }
+  } else {  // an evanescent mode in a warp that also holds propagating ones
+    T pv[PB];
+    T cur = p.re;
+#pragma unroll
+    for (int j = PB - 1; j >= 0; --j) {
+      if (PB * a + j < top) cur = W::mul(cur, q.re);
+      pv[j] = cur;
+    }
+    T h = s.re;
+#pragma unroll
+    for (int j = 0; j < PB; ++j) {
+      const int l = PB * a + j;
+      if (l <= top) f(l, C{pv[j], zero}, C{W::fmar(g, (R)(m - 1 - l), h), zero});
+      h = W::fma(q2.re, h, g);
+    }
+  }
 }
 
 // block sum of one double per warp (lane 0's value) -> partial[slot]
@@ -229,241 +365,375 @@ __device__ __forceinline__ void block_partial(double v, double* red, double* par
   __syncthreads();
   if (threadIdx.x == 0) {
     double s = 0.0;
-    for (int w = 0; w < DW; ++w) s += red[w];
+    for (int w = 0; w < DG; ++w) s += red[w];
     partial[slot] = s;
   }
-  __syncthreads();
 }
 
 // ---------------------------------------------------------------------------
-// normal matrices G^ = A^ A^^H, one block per mode (A^ staged in shared memory)
-// ---------------------------------------------------------------------------
-struct GramMem {
-  double2 A[DENSE_M1][DENSE_M + 1];
-  double2 E[DENSE_M1], Pz[DENSE_M];  // filled by warp 0 (mode_setup)
-  int usable;
-};
-
-__global__ void __launch_bounds__(GT) k_diff_gram(Problem P, double2* __restrict__ gram) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  GramMem& S = *reinterpret_cast<GramMem*>(smem_raw);
-  const int n = P.m1, m = P.m;
-  const int P1 = n * (n + 1) / 2;
-  const long long N2 = (long long)P.n * P.n, total = N2 * P.n_omega;
-  for (long long item = blockIdx.x; item < total; item += gridDim.x) {
-    const int om = (int)(item / N2);
-    const long long nu = item - (long long)om * N2;
-    if (threadIdx.x < 32) {
-      const ModeGeo g = mode_setup(P, om, nu, S.E, S.Pz);
-      if (threadIdx.x == 0) S.usable = g.usable;
-    }
-    __syncthreads();
-    const bool usable = S.usable;
-    if (usable)
-      for (int e = threadIdx.x; e < n * m; e += GT) {
-        const int k = e / m, l = e - k * m;
-        S.A[k][l] = S.E[k] * S.Pz[l];
-      }
-    __syncthreads();
-    double2* out = gram + item * P1;
-    for (int e = threadIdx.x; e < P1; e += GT) {
-      int j = 0;
-      while (col_off(j + 1, n) <= e) ++j;
-      const int k = j + (int)(e - col_off(j, n));
-      double2 acc = make_double2(0, 0);
-      if (usable) {
-        for (int l = 0; l < m; ++l) acc = acc + mulc(S.A[k][l], S.A[j][l]);
-        if (k == j) acc.y = 0.0;
-      }
-      out[e] = acc;
-    }
-    __syncthreads();
-  }
-}
-
-// ---------------------------------------------------------------------------
-// forward: factor, solve, eq. (9); tape <- L, y' (or b), V~/U~ planes
+// forward: tape <- c, g; V~/U~ planes; block partials of Phi
 // ---------------------------------------------------------------------------
 template <typename R>
-__global__ void __launch_bounds__(DW * 32)
-k_diff_forward(Problem P, const double2* __restrict__ gram, const cx<R>* __restrict__ wt,
-               const double* __restrict__ log_alpha, double2* __restrict__ Ls, double2* __restrict__ ys,
-               cx<R>* __restrict__ vt, cx<R>* __restrict__ ut, double* __restrict__ partial,
-               unsigned long long* __restrict__ ctr) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double red[DW];
-  __shared__ unsigned short rc[MAX_P1];
-  WarpMem& S = reinterpret_cast<WarpMem*>(smem_raw)[threadIdx.x >> 5];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__global__ void __launch_bounds__(DT)
+k_diff_forward(Problem P, DiffTables<R> tab, const cx<R>* __restrict__ wt, const double* __restrict__ alpha_arr,
+               double2* __restrict__ cs, typename Wide<R>::SC* __restrict__ gs, cx<R>* __restrict__ vt,
+               cx<R>* __restrict__ ut, double* __restrict__ partial, unsigned long long* __restrict__ ctr) {
+  using W = Wide<R>;
+  using T = typename W::T;
+  __shared__ WC<T> sc[DG][32];
+  __shared__ Factor<R> cv_s[32];
+  __shared__ WC<T> f_s[32];
+  __shared__ double red[DG];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int om = blockIdx.y, n = P.m1, m = P.m;
-  const int P1 = n * (n + 1) / 2;
   const long long N2 = (long long)P.n * P.n;
-  const double alpha = exp(log_alpha[om]);
-  build_rc(rc, n);
-  __syncthreads();
-  double phi = 0.0;
-  bool bad = false;
-  for (long long nu = (long long)blockIdx.x * DW + warp; nu < N2; nu += (long long)gridDim.x * DW) {
-    const long long mode = om * N2 + nu;
-    const ModeGeo g = mode_setup(P, om, nu, S.E, S.Pz);
-    const double2 b = lane < n ? to_d(wt[((long long)om * n + lane) * N2 + nu]) : make_double2(0, 0);
-    const double ap = alpha * g.rs * g.rs;
-    double2 v0 = make_double2(0, 0), v1 = make_double2(0, 0), u0 = v0, u1 = v0;
-    if (g.usable && ap < AP_MAX) {
-      load_lower(S, gram + mode * P1, n, lane);
-      if (lane < n) S.H[lane][lane].x += ap;
-      __syncwarp();
-      cholesky(S, n, lane, rc, bad);
-      store_lower(Ls + mode * P1, S, n, lane);
-      const double2 y = chol_solve(S, n, lane, b);
-      if (lane < n) ys[mode * n + lane] = y;
-      phi += ap * ap * warp_sum(abs2(y));
-      apply_AH(S, n, m, lane, y, g.rs, v0, v1);
-      put_v(S, m, lane, v0, v1);
-      toeplitz(S, m, lane, g.q, g.gamma, u0, u1);
-    } else {
-      if (lane < n) ys[mode * n + lane] = b;
-      phi += warp_sum(abs2(b));
-    }
-    if (nu == 0) {
-      if (lane < m) u0 = u0 + incident(P, om, lane);
-      if (lane + 32 < m) u1 = u1 + incident(P, om, lane + 32);
-    }
-    if (lane < m) {
-      vt[((long long)om * m + lane) * N2 + nu] = from_d<R>(v0);
-      ut[((long long)om * m + lane) * N2 + nu] = from_d<R>(u0);
-    }
-    if (lane + 32 < m) {
-      vt[((long long)om * m + lane + 32) * N2 + nu] = from_d<R>(v1);
-      ut[((long long)om * m + lane + 32) * N2 + nu] = from_d<R>(u1);
+  const long long nu = (long long)blockIdx.x * 32 + lane;
+  const bool valid = nu < N2;
+  const long long at = (long long)om * N2 + (valid ? nu : 0);
+  const double ne = tab.ne[at];
+  const bool prop = signbit(ne);
+  const bool cplx = __any_sync(0xffffffffu, prop);
+  const T zero = W::from(0.0);
+  cx<R> b[KC];
+  WC<T> e[KC];
+  WC<T> c = WC<T>{zero, zero};
+  R big = R(0);
+#pragma unroll
+  for (int i = 0; i < KC; ++i) {
+    const int k = w + DG * i;
+    const long long ak = ((long long)om * n + k) * N2 + nu;
+    const bool on = valid && k < n;
+    b[i] = on ? wt[ak] : czero<R>();
+    e[i].re = on ? W::ld(tab.er + ak) : zero;
+    e[i].im = on && cplx ? W::ld(tab.ei + ak) : zero;
+    big = fmax(big, fmax(fabs(b[i].x), fabs(b[i].y)));
+  }
+#pragma unroll
+  for (int i = 0; i < KC; ++i) {  // c = e^H b
+    c.re = W::fmar(e[i].re, b[i].x, c.re);
+    c.im = W::fmar(e[i].re, b[i].y, c.im);
+    if (cplx) {
+      c.re = W::fmar(e[i].im, b[i].y, c.re);
+      c.im = W::fmar(W::neg(e[i].im), b[i].x, c.im);
     }
   }
-  if (bad && lane == 0) atomicAdd(ctr + C_NONFINITE, 1ull);
+  sc[w][lane] = c;
+  __syncthreads();
+  double phi = 0.0;
+  if (w == 0) {
+    for (int i = 1; i < DG; ++i) c = WC<T>{W::add(c.re, sc[i][lane].re), W::add(c.im, sc[i][lane].im)};
+    const double tr = tab.tr[at], alpha = alpha_arr[om];
+    const ModeScalars s = mode_scalars(tr, ne, alpha);
+    const double2 cd = make_double2(W::d(c.re), W::d(c.im));
+    const double nu1 = s.mu * (1.0 + s.kappa);  // 1 - kappa^2
+    cv_s[lane] = Factor<R>::make(s.eta * cd);
+    const double2 fd = nu1 * cd;
+    f_s[lane] = WC<T>{W::from(fd.x), W::from(fd.y)};
+    if (valid) {
+      cs[at] = cd;
+      phi = s.kappa * s.kappa * nu1 * abs2(cd);
+    }
+    phi = warp_sum(phi);
+    // alpha = 0 (log alpha = -inf): the regularised matrix is singular
+    const bool bad = valid && tr > 0.0 && !(alpha > 0.0) && alpha < AP_MAX;
+    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicAdd(ctr + C_NONFINITE, 1ull);
+  }
+  __syncthreads();
+  const WC<T> f = f_s[lane];
+  const int ex = warp_exponent(big);
+  T gg = zero;
+#pragma unroll
+  for (int i = 0; i < KC; ++i) {  // g = b - (1 - kappa^2) c e, ||g||^2
+    const int k = w + DG * i;
+    if (k < n) {
+      T gr = W::add(W::from_r(b[i].x), W::neg(W::mul(f.re, e[i].re)));
+      T gi = W::add(W::from_r(b[i].y), W::neg(W::mul(f.im, e[i].re)));
+      if (cplx) {
+        gr = W::fma(f.im, e[i].im, gr);
+        gi = W::add(gi, W::neg(W::mul(f.re, e[i].im)));
+      }
+      if (valid) gs[((long long)om * n + k) * N2 + nu] = W::pack(gr, gi);
+      const T xr = scale_by(gr, -ex), xi = scale_by(gi, -ex);
+      gg = W::fma(xr, xr, gg);
+      gg = W::fma(xi, xi, gg);
+    }
+  }
+  gg = W::wsum(gg);
+  phi += W::d(gg) * (pow2d(ex) * pow2d(ex));
+  const Factor<R> cv = cv_s[lane];
+  for (int a = w; a < tab.nb; a += DG) {
+    if (!valid) break;
+    const long long ab = ((long long)om * tab.nb + a) * N2 + nu;
+    const long long o0 = (long long)om * m * N2 + nu;
+    const bool inc = nu == 0;
+    auto put = [&](int l, T vr, T vi, T ur, T ui) {
+      vt[o0 + l * N2] = mk<R>(cv.out(vr), cv.out(vi));
+      if (inc) {
+        const double2 z = tab.inc[om * m + l];
+        ut[o0 + l * N2] = mk<R>((R)((double)cv.out(ur) + z.x), (R)((double)cv.out(ui) + z.y));
+      } else {
+        ut[o0 + l * N2] = mk<R>(cv.out(ur), cv.out(ui));
+      }
+    };
+    if (!cplx) {
+      planes_real<R>(tab, at, ab, a, m, [&](int l, int, T p, T t) {
+        const T vr = W::mul(p, cv.re), vi = W::mul(p, cv.im);
+        put(l, vr, vi, W::mul(t, vr), W::mul(t, vi));
+      });
+    } else {
+      planes_cplx<R>(tab, at, ab, a, m, prop, [&](int l, WC<T> p, WC<T> t) {
+        const T vr = W::fma(p.re, cv.re, W::mul(p.im, cv.im));  // conj(P) c
+        const T vi = W::fma(p.re, cv.im, W::neg(W::mul(p.im, cv.re)));
+        put(l, vr, vi, W::fma(t.re, vr, W::neg(W::mul(t.im, vi))), W::fma(t.re, vi, W::mul(t.im, vr)));
+      });
+    }
+  }
   block_partial(phi, red, partial, (long long)om * gridDim.x + blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
-// VJP: b-bar per mode (written as N^2 b-bar for the inverse transform) and the
-// lnalpha-bar partials.  vbt/ubt (the forward transforms of V-bar, u-bar) may
+// VJP: N^2 b-bar per mode (for the inverse transform) and the lnalpha-bar partials.
+// vbt/ubt (the forward transforms of V-bar, u-bar; the adjoint of F^-1 is F / N^2) may
 // be null when xi carries no cotangent; wbt may be null when W needs no gradient.
 // ---------------------------------------------------------------------------
 template <typename R>
-__global__ void __launch_bounds__(DW * 32)
-k_diff_vjp(Problem P, const double2* __restrict__ Ls, const double2* __restrict__ ys,
-           const cx<R>* __restrict__ vbt, const cx<R>* __restrict__ ubt, const double* __restrict__ log_alpha,
+__global__ void __launch_bounds__(DT)
+k_diff_vjp(Problem P, DiffTables<R> tab, const double2* __restrict__ cs, const typename Wide<R>::SC* __restrict__ gs,
+           const cx<R>* __restrict__ vbt, const cx<R>* __restrict__ ubt, const double* __restrict__ alpha_arr,
            const double* __restrict__ grad_phi, cx<R>* __restrict__ wbt, double* __restrict__ partial) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double red[DW];
-  WarpMem& S = reinterpret_cast<WarpMem*>(smem_raw)[threadIdx.x >> 5];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  using W = Wide<R>;
+  using T = typename W::T;
+  __shared__ WC<T> sc[DG][32];
+  __shared__ Factor<R> t_s[32];
+  __shared__ Factor<R> gf_s;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int om = blockIdx.y, n = P.m1, m = P.m;
-  const int P1 = n * (n + 1) / 2;
   const long long N2 = (long long)P.n * P.n;
-  const double inv_n2 = 1.0 / (double)N2;
-  const double alpha = exp(log_alpha[om]);
+  const long long nu = (long long)blockIdx.x * 32 + lane;
+  const bool valid = nu < N2;
+  const long long at = (long long)om * N2 + (valid ? nu : 0);
+  const double ne = tab.ne[at];
+  const bool prop = signbit(ne);
+  const bool cplx = __any_sync(0xffffffffu, prop);
+  const T zero = W::from(0.0);
   const double gphi = grad_phi ? grad_phi[om] : 0.0;
-  double lbar = 0.0;
-  for (long long nu = (long long)blockIdx.x * DW + warp; nu < N2; nu += (long long)gridDim.x * DW) {
-    const long long mode = om * N2 + nu;
-    const ModeGeo g = mode_setup(P, om, nu, S.E, S.Pz);
-    const double2 y = lane < n ? ys[mode * n + lane] : make_double2(0, 0);
-    const double ap = alpha * g.rs * g.rs;
-    double2 bb;
-    if (g.usable && ap < AP_MAX) {
-      load_lower(S, Ls + mode * P1, n, lane);
-      set_dinv(S, n, lane);
-      double2 s = make_double2(0, 0);
-      if (vbt) {
-        // t = V~-bar + conj(gamma) (scans with conj(q)) of U~-bar;  F^-1 adjoint = F / N^2
-        double2 a0 = make_double2(0, 0), a1 = a0;
-        if (lane < m) a0 = inv_n2 * to_d(ubt[((long long)om * m + lane) * N2 + nu]);
-        if (lane + 32 < m) a1 = inv_n2 * to_d(ubt[((long long)om * m + lane + 32) * N2 + nu]);
-        put_v(S, m, lane, a0, a1);
-        double2 t0, t1;
-        toeplitz(S, m, lane, conjx(g.q), conjx(g.gamma), t0, t1);
-        if (lane < m) S.t[lane] = t0 + inv_n2 * to_d(vbt[((long long)om * m + lane) * N2 + nu]);
-        if (lane + 32 < m) S.t[lane + 32] = t1 + inv_n2 * to_d(vbt[((long long)om * m + lane + 32) * N2 + nu]);
-        __syncwarp();
-        s = apply_A(S, n, m, lane, g.rs);
-        __syncwarp();
+  T tr_ = zero, ti_ = zero;
+  if (vbt && valid) {
+    for (int a = w; a < tab.nb; a += DG) {
+      const long long ab = ((long long)om * tab.nb + a) * N2 + nu;
+      const long long o0 = (long long)om * m * N2 + nu;
+      if (!cplx) {
+        cx<R> vb[PB], ub[PB];
+#pragma unroll
+        for (int j = 0; j < PB; ++j) {  // the block's loads in flight together
+          const int l = PB * a + j;
+          vb[j] = l < m ? vbt[o0 + l * N2] : czero<R>();
+          ub[j] = l < m ? ubt[o0 + l * N2] : czero<R>();
+        }
+        planes_real<R>(tab, at, ab, a, m, [&](int l, int j, T p, T t) {
+          tr_ = W::fma(p, W::fmar(t, ub[j].x, W::from_r(vb[j].x)), tr_);
+          ti_ = W::fma(p, W::fmar(t, ub[j].y, W::from_r(vb[j].y)), ti_);
+        });
+      } else {
+        planes_cplx<R>(tab, at, ab, a, m, prop, [&](int l, WC<T> p, WC<T> t) {
+          const cx<R> v = vbt[o0 + l * N2], u = ubt[o0 + l * N2];
+          // V-bar + conj(T) U-bar
+          const T xr = W::fmar(t.im, u.y, W::fmar(t.re, u.x, W::from_r(v.x)));
+          const T xi = W::fmar(W::neg(t.im), u.x, W::fmar(t.re, u.y, W::from_r(v.y)));
+          tr_ = W::add(tr_, W::fma(p.re, xr, W::neg(W::mul(p.im, xi))));
+          ti_ = W::add(ti_, W::fma(p.re, xi, W::mul(p.im, xr)));
+        });
       }
-      s = s + (2.0 * ap * ap * gphi) * y;
-      bb = chol_solve(S, n, lane, s);
-      lbar += -ap * warp_sum(bb.x * y.x + bb.y * y.y) + 2.0 * gphi * ap * ap * warp_sum(abs2(y));
-    } else {
-      bb = (2.0 * gphi) * y;  // the slot holds b: Phi_nu = ||b||^2
     }
-    if (wbt && lane < n) wbt[((long long)om * n + lane) * N2 + nu] = from_d<R>((double)N2 * bb);
   }
-  block_partial(lbar, red, partial, (long long)om * gridDim.x + blockIdx.x);
+  sc[w][lane] = WC<T>{tr_, ti_};
+  __syncthreads();
+  if (w == 0) {
+    for (int i = 1; i < DG; ++i) {
+      tr_ = W::add(tr_, sc[i][lane].re);
+      ti_ = W::add(ti_, sc[i][lane].im);
+    }
+    const ModeScalars s = mode_scalars(tab.tr[at], ne, alpha_arr[om]);
+    const double2 c = cs[at];
+    const double2 t = s.eta * make_double2(W::d(tr_), W::d(ti_));  // N^2 eta tau
+    t_s[lane] = Factor<R>::make(t);
+    double lbar = 0.0;
+    if (valid) {
+      lbar = -s.kappa * P.inv_n2 * (t.x * c.x + t.y * c.y);
+      if (grad_phi) lbar += 2.0 * gphi * s.kappa * s.kappa * s.mu * abs2(c);
+    }
+    lbar = warp_sum(lbar);
+    if (lane == 0) {
+      partial[(long long)om * gridDim.x + blockIdx.x] = lbar;
+      gf_s = Factor<R>::make(make_double2(2.0 * gphi * (double)N2, 0.0));
+    }
+  }
+  if (!wbt) return;
+  __syncthreads();
+  const Factor<R> t = t_s[lane], gf = gf_s;
+#pragma unroll
+  for (int i = 0; i < KC; ++i) {
+    const int k = w + DG * i;
+    if (valid && k < n) {
+      const long long ak = ((long long)om * n + k) * N2 + nu;
+      R br = R(0), bi = R(0);
+      const T er = W::ld(tab.er + ak), ei = cplx ? W::ld(tab.ei + ak) : zero;
+      T xr = W::mul(er, t.re), xi = W::mul(er, t.im);
+      if (cplx) {
+        xr = W::add(xr, W::neg(W::mul(ei, t.im)));
+        xi = W::fma(ei, t.re, xi);
+      }
+      br = t.out(xr);
+      bi = t.out(xi);
+      if (grad_phi) {
+        T gr, gi;
+        W::unpack(gs[ak], gr, gi);
+        br += gf.out(W::mul(gr, gf.re));
+        bi += gf.out(W::mul(gi, gf.re));
+      }
+      wbt[ak] = mk<R>(br, bi);
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
-// JVP for nd <= JVP_CHUNK directions at once (L loaded once per mode)
+// JVP for nd <= JVP_CHUNK directions at once, JG of them per pass over the planes
 // dwt: [nd][n_omega][M1][N2]; dvt, dut: [nd][n_omega][M][N2]
 // ---------------------------------------------------------------------------
 template <typename R>
-__global__ void __launch_bounds__(DW * 32)
-k_diff_jvp(Problem P, int nd, const double2* __restrict__ Ls, const double2* __restrict__ ys,
-           const cx<R>* __restrict__ dwt, const double* __restrict__ log_alpha,
-           const double* __restrict__ dlog_alpha, cx<R>* __restrict__ dvt, cx<R>* __restrict__ dut,
-           double* __restrict__ partial) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double red[DW];
-  WarpMem& S = reinterpret_cast<WarpMem*>(smem_raw)[threadIdx.x >> 5];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__global__ void __launch_bounds__(DT)
+k_diff_jvp(Problem P, DiffTables<R> tab, int nd, const double2* __restrict__ cs,
+           const typename Wide<R>::SC* __restrict__ gs, const cx<R>* __restrict__ dwt,
+           const double* __restrict__ alpha_arr, const double* __restrict__ dlog_alpha, cx<R>* __restrict__ dvt,
+           cx<R>* __restrict__ dut, double* __restrict__ partial) {
+  using W = Wide<R>;
+  using T = typename W::T;
+  __shared__ WC<T> sc[JG][DG][32];
+  __shared__ Factor<R> cv_s[JG][32];
+  __shared__ double ps[JG][DG], pe[JG];  // Phi-dot: the warps' sums and the scalar part
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int om = blockIdx.y, n = P.m1, m = P.m, F = P.n_omega;
-  const int P1 = n * (n + 1) / 2;
   const long long N2 = (long long)P.n * P.n;
-  const double alpha = exp(log_alpha[om]);
-  __shared__ double acc[DW][JVP_CHUNK];  // per-warp Phi-dot sums (lane 0 adds)
-  if (lane < JVP_CHUNK) acc[warp][lane] = 0.0;
-  __syncwarp();
-  for (long long nu = (long long)blockIdx.x * DW + warp; nu < N2; nu += (long long)gridDim.x * DW) {
-    const long long mode = om * N2 + nu;
-    const ModeGeo g = mode_setup(P, om, nu, S.E, S.Pz);
-    const double2 y = lane < n ? ys[mode * n + lane] : make_double2(0, 0);
-    const double ap = alpha * g.rs * g.rs;
-    const bool solve = g.usable && ap < AP_MAX;
-    double yy = 0.0;
-    if (solve) {
-      load_lower(S, Ls + mode * P1, n, lane);
-      set_dinv(S, n, lane);
-      yy = warp_sum(abs2(y));
+  const long long nu = (long long)blockIdx.x * 32 + lane;
+  const bool valid = nu < N2;
+  const long long at = (long long)om * N2 + (valid ? nu : 0);
+  const double ne = tab.ne[at];
+  const bool prop = signbit(ne);
+  const bool cplx = __any_sync(0xffffffffu, prop);
+  const T zero = W::from(0.0);
+  WC<T> e[KC], g[KC];
+  R big = R(0);
+#pragma unroll
+  for (int i = 0; i < KC; ++i) {
+    const int k = w + DG * i;
+    const long long ak = ((long long)om * n + k) * N2 + nu;
+    const bool on = valid && k < n;
+    e[i] = WC<T>{zero, zero};
+    g[i] = WC<T>{zero, zero};
+    if (on) {
+      e[i].re = W::ld(tab.er + ak);
+      if (cplx) e[i].im = W::ld(tab.ei + ak);
+      W::unpack(gs[ak], g[i].re, g[i].im);
     }
-#pragma unroll 1
-    for (int d = 0; d < nd; ++d) {
-      const double2 db =
-          lane < n ? to_d(dwt[(((long long)d * F + om) * n + lane) * N2 + nu]) : make_double2(0, 0);
-      const double dla = dlog_alpha ? dlog_alpha[d * F + om] : 0.0;
-      double2 v0 = make_double2(0, 0), v1 = v0, u0 = v0, u1 = v0;
-      double dp;
-      if (solve) {
-        const double2 dy = chol_solve(S, n, lane, db - (dla * ap) * y);
-        dp = 2.0 * ap * ap * (dla * yy + warp_sum(y.x * dy.x + y.y * dy.y));
-        apply_AH(S, n, m, lane, dy, g.rs, v0, v1);
-        put_v(S, m, lane, v0, v1);
-        toeplitz(S, m, lane, g.q, g.gamma, u0, u1);
-      } else {
-        dp = 2.0 * warp_sum(y.x * db.x + y.y * db.y);  // Phi_nu = ||b||^2
-      }
-      if (lane == 0) acc[warp][d] += dp;
-      const long long base = ((long long)d * F + om) * m;
-      if (lane < m) {
-        dvt[(base + lane) * N2 + nu] = from_d<R>(v0);
-        dut[(base + lane) * N2 + nu] = from_d<R>(u0);
-      }
-      if (lane + 32 < m) {
-        dvt[(base + lane + 32) * N2 + nu] = from_d<R>(v1);
-        dut[(base + lane + 32) * N2 + nu] = from_d<R>(u1);
-      }
-    }
+    big = fmax(big, fmax(fabs(W::r(g[i].re)), fabs(W::r(g[i].im))));
   }
-  __syncthreads();
-  if (threadIdx.x < nd) {
-    double t = 0.0;
-    for (int w = 0; w < DW; ++w) t += acc[w][threadIdx.x];
-    partial[((long long)threadIdx.x * F + om) * gridDim.x + blockIdx.x] = t;
+  const int eg = warp_exponent(big);
+#pragma unroll
+  for (int i = 0; i < KC; ++i) g[i] = WC<T>{scale_by(g[i].re, -eg), scale_by(g[i].im, -eg)};
+  ModeScalars s{0.0, 0.0, 1.0};
+  double2 c0 = make_double2(0.0, 0.0);
+  if (w < JG) {
+    s = mode_scalars(tab.tr[at], ne, alpha_arr[om]);
+    c0 = cs[at];
+  }
+#pragma unroll 1
+  for (int d0 = 0; d0 < nd; d0 += JG) {
+#pragma unroll 1
+    for (int jd = 0; jd < JG; ++jd) {
+      const int d = d0 + jd;
+      if (d >= nd) break;
+      cx<R> db[KC];
+      R bb = R(0);
+#pragma unroll
+      for (int i = 0; i < KC; ++i) {
+        const int k = w + DG * i;
+        db[i] = valid && k < n ? dwt[(((long long)d * F + om) * n + k) * N2 + nu] : czero<R>();
+        bb = fmax(bb, fmax(fabs(db[i].x), fabs(db[i].y)));
+      }
+      const int eb = warp_exponent(bb);
+      WC<T> c = WC<T>{zero, zero};
+      T dp = zero;
+#pragma unroll
+      for (int i = 0; i < KC; ++i) {
+        c.re = W::fmar(e[i].re, db[i].x, c.re);
+        c.im = W::fmar(e[i].re, db[i].y, c.im);
+        if (cplx) {
+          c.re = W::fmar(e[i].im, db[i].y, c.re);
+          c.im = W::fmar(W::neg(e[i].im), db[i].x, c.im);
+        }
+        dp = W::fmar(g[i].re, scale_by(db[i].x, -eb), dp);
+        dp = W::fmar(g[i].im, scale_by(db[i].y, -eb), dp);
+      }
+      sc[jd][w][lane] = c;
+      dp = W::wsum(dp);
+      if (lane == 0) ps[jd][w] = 2.0 * W::d(dp) * (pow2d(eb) * pow2d(eg));
+    }
+    __syncthreads();
+    if (w < JG && d0 + w < nd) {  // warp w: the scalars of direction d0 + w
+      const int d = d0 + w;
+      T cr = sc[w][0][lane].re, ci = sc[w][0][lane].im;
+      for (int i = 1; i < DG; ++i) {
+        cr = W::add(cr, sc[w][i][lane].re);
+        ci = W::add(ci, sc[w][i][lane].im);
+      }
+      const double dla = dlog_alpha ? dlog_alpha[d * F + om] : 0.0;
+      const double kd = -s.kappa * dla;
+      cv_s[w][lane] =
+          Factor<R>::make(s.eta * make_double2(W::d(cr) + kd * c0.x, W::d(ci) + kd * c0.y));
+      double x = 0.0;
+      if (dlog_alpha) x = warp_sum(valid ? 2.0 * s.kappa * s.kappa * s.mu * dla * abs2(c0) : 0.0);
+      if (lane == 0) pe[w] = x;
+    }
+    __syncthreads();
+    if (threadIdx.x < JG && d0 + threadIdx.x < nd) {
+      double t = pe[threadIdx.x];
+      for (int i = 0; i < DG; ++i) t += ps[threadIdx.x][i];
+      partial[((long long)(d0 + threadIdx.x) * F + om) * gridDim.x + blockIdx.x] = t;
+    }
+    if (valid) {
+      for (int a = w; a < tab.nb; a += DG) {
+        const long long ab = ((long long)om * tab.nb + a) * N2 + nu;
+        const int jn = min(JG, nd - d0);
+        if (!cplx) {
+          planes_real<R>(tab, at, ab, a, m, [&](int l, int, T p, T t) {
+            const T pt = W::mul(p, t);
+#pragma unroll
+            for (int jd = 0; jd < JG; ++jd) {
+              if (jd < jn) {
+                const Factor<R>& cv = cv_s[jd][lane];
+                const long long o = (((long long)(d0 + jd) * F + om) * m + l) * N2 + nu;
+                dvt[o] = mk<R>(cv.out(W::mul(p, cv.re)), cv.out(W::mul(p, cv.im)));
+                dut[o] = mk<R>(cv.out(W::mul(pt, cv.re)), cv.out(W::mul(pt, cv.im)));
+              }
+            }
+          });
+        } else {
+          planes_cplx<R>(tab, at, ab, a, m, prop, [&](int l, WC<T> p, WC<T> t) {
+#pragma unroll 1
+            for (int jd = 0; jd < jn; ++jd) {
+              const Factor<R>& cv = cv_s[jd][lane];
+              const T vr = W::fma(p.re, cv.re, W::mul(p.im, cv.im));  // conj(P) c
+              const T vi = W::fma(p.re, cv.im, W::neg(W::mul(p.im, cv.re)));
+              const long long o = (((long long)(d0 + jd) * F + om) * m + l) * N2 + nu;
+              dvt[o] = mk<R>(cv.out(vr), cv.out(vi));
+              dut[o] = mk<R>(cv.out(W::fma(t.re, vr, W::neg(W::mul(t.im, vi)))),
+                             cv.out(W::fma(t.re, vi, W::mul(t.im, vr))));
+            }
+          });
+        }
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -535,19 +805,15 @@ __global__ void k_diff_jvp_point(Problem P, int nd, const cx<R>* __restrict__ Vx
   }
 }
 
-// out[r] = sum_c partial[r cols + c], fixed order
+// out[r] = sum_c partial[r cols + c]: one warp per row, lanes over the columns, then a
+// tree over the lanes (a fixed order)
 __global__ void k_reduce_rows(const double* __restrict__ partial, int rows, int cols, double* __restrict__ out) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= rows) return;
   double s = 0.0;
-  for (int c = 0; c < cols; ++c) s += partial[(long long)r * cols + c];
-  out[r] = s;
-}
-
-// opt in to more than 48 KB of dynamic shared memory, once per kernel and device
-// (the flag is per call site: each caller below launches a distinct kernel)
-template <typename K> cudaError_t allow_smem(K kernel, size_t bytes, SmemOptIn& flag) {
-  return opt_in_smem(flag, (const void*)kernel, bytes);
+  for (int c = lane; c < cols; c += 32) s += partial[(long long)r * cols + c];
+  s = warp_sum(s);
+  if (lane == 0) out[r] = s;
 }
 
 unsigned point_grid(long long n) {
@@ -558,60 +824,74 @@ unsigned point_grid(long long n) {
 
 }  // namespace
 
-int diff_blocks_per_omega(int n, int n_omega) {
-  const long long N2 = (long long)n * n;
-  const long long want = (N2 + DW - 1) / DW;
-  long long cap = (3LL * sm_count() + n_omega - 1) / n_omega;
-  if (cap < 1) cap = 1;
-  return (int)(want < cap ? want : cap);
+int diff_blocks_per_omega(int n) { return (int)(((long long)n * n + 31) / 32); }
+
+template <typename R>
+size_t diff_tables(const Problem& P, void* base, DiffTables<R>* tab, DiffTablesOut<R>* out) {
+  using S = typename DiffTables<R>::S;
+  const size_t F = P.n_omega, N2 = (size_t)P.n * P.n, nb = (P.m + DIFF_PB - 1) / DIFF_PB;
+  char* b = (char*)base;
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    char* p = b + off;
+    off = (off + bytes + 255) & ~(size_t)255;
+    return p;
+  };
+  DiffTablesOut<R> o;
+  o.er = (S*)take(sizeof(S) * F * P.m1 * N2);
+  o.ei = (S*)take(sizeof(S) * F * P.m1 * N2);
+  o.pr = (S*)take(sizeof(S) * F * nb * N2);
+  o.pi = (S*)take(sizeof(S) * F * nb * N2);
+  o.sr = (S*)take(sizeof(S) * F * nb * N2);
+  o.si = (S*)take(sizeof(S) * F * nb * N2);
+  o.q = (typename DiffTables<R>::S2*)take(2 * sizeof(S) * F * N2);
+  o.g = (S*)take(sizeof(S) * F * N2);
+  o.tr = (double*)take(8 * F * N2);
+  o.ne = (double*)take(8 * F * N2);
+  o.inc = (double2*)take(16 * F * P.m);
+  if (out) *out = o;
+  if (tab) *tab = DiffTables<R>{o.er, o.ei, o.pr, o.pi, o.sr, o.si, o.q, o.g, o.tr, o.ne, o.inc, (int)nb};
+  return off;
 }
 
-cudaError_t launch_diff_gram(const Problem& P, double2* gram, cudaStream_t s) {
-  const size_t smem = sizeof(GramMem);
-  static SmemOptIn done;
-  cudaError_t e = allow_smem(k_diff_gram, smem, done);
-  if (e != cudaSuccess) return e;
-  const long long total = (long long)P.n * P.n * P.n_omega;
-  const long long cap = 4LL * sm_count();
-  k_diff_gram<<<(unsigned)(total < cap ? total : cap), GT, smem, s>>>(P, gram);
+template <typename R>
+cudaError_t launch_diff_tables(const Problem& P, const DiffTables<R>& tab, const DiffTablesOut<R>& out,
+                               cudaStream_t s) {
+  k_diff_tables<R><<<dim3(diff_blocks_per_omega(P.n), P.n_omega), DT, 0, s>>>(P, tab, out);
+  k_diff_incident<<<P.n_omega, 64, 0, s>>>(P, out.inc);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_diff_alpha(const double* log_alpha, int F, double* la, cudaStream_t s) {
+  k_diff_alpha<<<1, MAX_OMEGA, 0, s>>>(log_alpha, F, la);
   return cudaGetLastError();
 }
 
 template <typename R>
-cudaError_t launch_diff_forward(const Problem& P, int gb, const double2* gram, const cx<R>* wt,
-                                const double* log_alpha, double2* Ls, double2* ys, cx<R>* vt, cx<R>* ut,
-                                double* partial, unsigned long long* ctr, cudaStream_t s) {
-  const size_t smem = sizeof(WarpMem) * DW;
-  static SmemOptIn done;
-  cudaError_t e = allow_smem(k_diff_forward<R>, smem, done);
-  if (e != cudaSuccess) return e;
-  k_diff_forward<R><<<dim3(gb, P.n_omega), DW * 32, smem, s>>>(P, gram, wt, log_alpha, Ls, ys, vt, ut, partial, ctr);
+cudaError_t launch_diff_forward(const Problem& P, const DiffTables<R>& tab, const cx<R>* wt, const double* alpha,
+                                double2* cs, void* gs, cx<R>* vt, cx<R>* ut, double* partial,
+                                unsigned long long* ctr, cudaStream_t s) {
+  k_diff_forward<R><<<dim3(diff_blocks_per_omega(P.n), P.n_omega), DT, 0, s>>>(
+      P, tab, wt, alpha, cs, (typename Wide<R>::SC*)gs, vt, ut, partial, ctr);
   return cudaGetLastError();
 }
 
 template <typename R>
-cudaError_t launch_diff_vjp(const Problem& P, int gb, const double2* Ls, const double2* ys, const cx<R>* vbt,
-                            const cx<R>* ubt, const double* log_alpha, const double* grad_phi, cx<R>* wbt,
+cudaError_t launch_diff_vjp(const Problem& P, const DiffTables<R>& tab, const double2* cs, const void* gs,
+                            const cx<R>* vbt, const cx<R>* ubt, const double* alpha, const double* grad_phi,
+                            cx<R>* wbt, double* partial, cudaStream_t s) {
+  k_diff_vjp<R><<<dim3(diff_blocks_per_omega(P.n), P.n_omega), DT, 0, s>>>(
+      P, tab, cs, (const typename Wide<R>::SC*)gs, vbt, ubt, alpha, grad_phi, wbt, partial);
+  return cudaGetLastError();
+}
+
+template <typename R>
+cudaError_t launch_diff_jvp(const Problem& P, const DiffTables<R>& tab, int nd, const double2* cs, const void* gs,
+                            const cx<R>* dwt, const double* alpha, const double* dlog_alpha, cx<R>* dvt, cx<R>* dut,
                             double* partial, cudaStream_t s) {
-  const size_t smem = sizeof(WarpMem) * DW;
-  static SmemOptIn done;
-  cudaError_t e = allow_smem(k_diff_vjp<R>, smem, done);
-  if (e != cudaSuccess) return e;
-  k_diff_vjp<R><<<dim3(gb, P.n_omega), DW * 32, smem, s>>>(P, Ls, ys, vbt, ubt, log_alpha, grad_phi, wbt, partial);
-  return cudaGetLastError();
-}
-
-template <typename R>
-cudaError_t launch_diff_jvp(const Problem& P, int gb, int nd, const double2* Ls, const double2* ys,
-                            const cx<R>* dwt, const double* log_alpha, const double* dlog_alpha, cx<R>* dvt,
-                            cx<R>* dut, double* partial, cudaStream_t s) {
   if (nd < 1 || nd > JVP_CHUNK) return cudaErrorInvalidValue;
-  const size_t smem = sizeof(WarpMem) * DW;
-  static SmemOptIn done;
-  cudaError_t e = allow_smem(k_diff_jvp<R>, smem, done);
-  if (e != cudaSuccess) return e;
-  k_diff_jvp<R><<<dim3(gb, P.n_omega), DW * 32, smem, s>>>(P, nd, Ls, ys, dwt, log_alpha, dlog_alpha, dvt, dut,
-                                                          partial);
+  k_diff_jvp<R><<<dim3(diff_blocks_per_omega(P.n), P.n_omega), DT, 0, s>>>(
+      P, tab, nd, cs, (const typename Wide<R>::SC*)gs, dwt, alpha, dlog_alpha, dvt, dut, partial);
   return cudaGetLastError();
 }
 
@@ -637,25 +917,28 @@ cudaError_t launch_diff_jvp_point(const Problem& P, int nd, const cx<R>* Vx, con
 }
 
 cudaError_t launch_reduce_rows(const double* partial, int rows, int cols, double* out, cudaStream_t s) {
-  k_reduce_rows<<<(rows + 127) / 128, 128, 0, s>>>(partial, rows, cols, out);
+  k_reduce_rows<<<(rows + 3) / 4, 128, 0, s>>>(partial, rows, cols, out);
   return cudaGetLastError();
 }
 
-#define FL_DIFF_INST(R)                                                                                         \
-  template cudaError_t launch_diff_forward<R>(const Problem&, int, const double2*, const cx<R>*, const double*,  \
-                                              double2*, double2*, cx<R>*, cx<R>*, double*, unsigned long long*,  \
-                                              cudaStream_t);                                                    \
-  template cudaError_t launch_diff_vjp<R>(const Problem&, int, const double2*, const double2*, const cx<R>*,     \
-                                          const cx<R>*, const double*, const double*, cx<R>*, double*,          \
-                                          cudaStream_t);                                                        \
-  template cudaError_t launch_diff_jvp<R>(const Problem&, int, int, const double2*, const double2*,             \
-                                          const cx<R>*, const double*, const double*, cx<R>*, cx<R>*, double*,  \
-                                          cudaStream_t);                                                        \
-  template cudaError_t launch_diff_combine<R>(const Problem&, const cx<R>*, const cx<R>*, R*, R*, R*,            \
-                                              cudaStream_t);                                                    \
-  template cudaError_t launch_diff_vjp_point<R>(const Problem&, const R*, const cx<R>*, const cx<R>*, const R*,  \
-                                                cx<R>*, cx<R>*, cudaStream_t);                                  \
-  template cudaError_t launch_diff_jvp_point<R>(const Problem&, int, const cx<R>*, const cx<R>*, const R*,       \
+#define FL_DIFF_INST(R)                                                                                            \
+  template size_t diff_tables<R>(const Problem&, void*, DiffTables<R>*, DiffTablesOut<R>*);                         \
+  template cudaError_t launch_diff_tables<R>(const Problem&, const DiffTables<R>&, const DiffTablesOut<R>&,         \
+                                             cudaStream_t);                                                        \
+  template cudaError_t launch_diff_forward<R>(const Problem&, const DiffTables<R>&, const cx<R>*, const double*,    \
+                                              double2*, void*, cx<R>*, cx<R>*, double*, unsigned long long*,       \
+                                              cudaStream_t);                                                       \
+  template cudaError_t launch_diff_vjp<R>(const Problem&, const DiffTables<R>&, const double2*, const void*,        \
+                                          const cx<R>*, const cx<R>*, const double*, const double*, cx<R>*,        \
+                                          double*, cudaStream_t);                                                  \
+  template cudaError_t launch_diff_jvp<R>(const Problem&, const DiffTables<R>&, int, const double2*, const void*,   \
+                                          const cx<R>*, const double*, const double*, cx<R>*, cx<R>*, double*,     \
+                                          cudaStream_t);                                                           \
+  template cudaError_t launch_diff_combine<R>(const Problem&, const cx<R>*, const cx<R>*, R*, R*, R*,               \
+                                              cudaStream_t);                                                       \
+  template cudaError_t launch_diff_vjp_point<R>(const Problem&, const R*, const cx<R>*, const cx<R>*, const R*,     \
+                                                cx<R>*, cx<R>*, cudaStream_t);                                     \
+  template cudaError_t launch_diff_jvp_point<R>(const Problem&, int, const cx<R>*, const cx<R>*, const R*,          \
                                                 const cx<R>*, const cx<R>*, R*, cudaStream_t);
 FL_DIFF_INST(double)
 FL_DIFF_INST(float)

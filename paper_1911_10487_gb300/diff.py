@@ -39,7 +39,7 @@ class Tape:
 
 
 class DiffPlan:
-    """Normal matrices of one geometry / frequency list / precision, plus buffers."""
+    """Mode tables of one geometry / frequency list / precision, plus buffers."""
 
     def __init__(self, rc, geom, omega, precision: str = "fp64", c0: float = 1.0, eps_u: float = 1e-8):
         import torch

@@ -57,9 +57,9 @@ def test_derivatives_at_the_edges_of_the_split(shape, precision, tol):
     rW, ra = adjoint.vjp(t, gxi, gphi)
     rW0, _ = adjoint.vjp(t, gxi, np.zeros(len(om)))
     err = {"xi": _rel(xi, t.xi), "phi": _rel(phi, t.phi), "gW": _rel(gW, rW), "gW0": _rel(gW0, rW0), "gla": _rel(gla, ra)}
-    for d in {0, dW.shape[0] - 1}:
-        rx, rp = adjoint.jvp(t, dW[d], dla[d])
-        err[f"dxi{d}"], err[f"dphi{d}"] = _rel(dxi[d], rx), _rel(dphi[d], rp)
+    ref = [adjoint.jvp(t, dW[d], dla[d]) for d in range(dW.shape[0])]
+    # over all directions together: one direction's Phi-dot is a sum that may cancel
+    err["dxi"], err["dphi"] = _rel(dxi, np.stack([r[0] for r in ref])), _rel(dphi, np.stack([r[1] for r in ref]))
     plan.close()
     rc.close()
     print(shape, precision, {k: f"{v:.1e}" for k, v in err.items()})
