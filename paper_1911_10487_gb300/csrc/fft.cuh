@@ -83,8 +83,12 @@ template <typename R, bool INV> struct Dft {
     v[0] = s02 + s13; v[2] = s02 - s13;
     v[1] = d02 + d13; v[3] = d02 - d13;
   }
-  // x w16^e, w16 = exp(-2 pi i/16) (conjugated for the inverse); e is a constant
+  // x w16^e, w16 = exp(-2 pi i/16) (conjugated for the inverse); e is a constant (w16^0
+  // and w16^4 = -i cost no arithmetic: 10 of 170 FP64 operations of a 16-point DFT, on a
+  // GPU where those bound the FP64 passes)
   __device__ __forceinline__ static C tw16(C x, int e) {
+    if (e == 0) return x;
+    if (e == 4) return rot90<INV>(x);
     const R c = R(cos16(e)), sn = INV ? R(sin16(e)) : -R(sin16(e));
     return mk<R>(x.x * c - x.y * sn, x.x * sn + x.y * c);
   }
@@ -126,10 +130,44 @@ template <typename R, bool INV> struct Dft {
   __device__ __forceinline__ static void d3(C* v) {
     // y1,2 = a0 - (a1+a2)/2 -/+ i (sqrt(3)/2)(a1 - a2)  (forward; signs swap for the inverse)
     const R h = R(0.86602540378443864676);
+    if constexpr (sizeof(R) == 8) {  // 12 operations, the products fused into the sums
+      const C s = v[1] + v[2], e = rot90<INV>(v[1] - v[2]);
+      const C t = mk<R>(fma(R(-0.5), s.x, v[0].x), fma(R(-0.5), s.y, v[0].y));
+      v[0] = v[0] + s;
+      v[1] = mk<R>(fma(h, e.x, t.x), fma(h, e.y, t.y));
+      v[2] = mk<R>(fma(-h, e.x, t.x), fma(-h, e.y, t.y));
+      return;
+    }
     C s = v[1] + v[2];
     C t = v[0] - R(0.5) * s;
     C d = h * rot90<INV>(v[1] - v[2]);
     v[0] = v[0] + s; v[1] = t + d; v[2] = t - d;
+  }
+  // 12 points as 3 x 4 without twiddles (Good-Thomas): n = 4 n1 + 3 n2, k = 4 k1 + 9 k2
+  // (mod 12) gives n k = 4 n1 k1 + 3 n2 k2 (mod 12)
+  __device__ __forceinline__ static void d12(C* v) {
+    C y[4][3];
+#pragma unroll
+    for (int n2 = 0; n2 < 4; ++n2) {
+#pragma unroll
+      for (int n1 = 0; n1 < 3; ++n1) y[n2][n1] = v[(4 * n1 + 3 * n2) % 12];
+      d3(y[n2]);
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) {
+      C z[4] = {y[0][k1], y[1][k1], y[2][k1], y[3][k1]};
+      d4(z);
+#pragma unroll
+      for (int k2 = 0; k2 < 4; ++k2) v[(4 * k1 + 9 * k2) % 12] = z[k2];
+    }
+  }
+  template <int RAD> __device__ __forceinline__ static void run(C* v) {
+    if constexpr (RAD == 2) d2(v);
+    else if constexpr (RAD == 3) d3(v);
+    else if constexpr (RAD == 4) d4(v);
+    else if constexpr (RAD == 8) d8(v);
+    else if constexpr (RAD == 12) d12(v);
+    else d16(v);
   }
 };
 
@@ -258,6 +296,157 @@ struct FftStagesPP {
 template <typename R, int N, bool INV, int LINES, int THREADS, Lay L, int MAXR, int SKEW = 0>
 __device__ __forceinline__ cx<R>* fft_lines_pp(cx<R>* a, cx<R>* b, const cx<R>* tw) {
   return FftStagesPP<R, N, INV, LINES, THREADS, L, SKEW, MAXR, 0, 1>::run(a, b, tw);
+}
+
+// ---- transforms between global memory and registers ---------------------------
+// The passes below hold a line in registers at both ends: the first stage's inputs are
+// loaded straight from global memory in butterfly order (element j + r N/RAD, neighbouring
+// threads on neighbouring elements), the last stage's outputs (element k + r N/RAD) leave
+// from registers.  A two-stage length crosses shared memory once and meets one barrier;
+// staging the tile in shared memory first and last took three crossings and four barriers.
+
+// Plans of these passes.  3-smooth lengths end in a 12-point stage (no inner twiddles):
+// 192 = 16 x 12, one crossing, where 3 x 16 x 4 takes two and 20% more operations.
+// DENSE32 keeps FftPlan's factors: the FP32 transforms of the derivatives, whose FP64
+// sums (Phi) follow the rounding of the transform.
+template <int N, int MAXR, bool DENSE32> struct IoPlan {
+  static constexpr bool R12 = !DENSE32 && N % 12 == 0 && N / 12 <= MAXR && (N / 12 & (N / 12 - 1)) == 0;
+  static constexpr int stages = R12 ? (N > 12 ? 2 : 1) : FftPlan<N, MAXR>::stages;
+  __host__ __device__ static constexpr int radix(int s) {
+    return R12 ? (s == stages - 1 ? 12 : N / 12) : FftPlan<N, MAXR>::radix(s);
+  }
+  // product of the radices before stage s
+  __host__ __device__ static constexpr int ns(int s) { return s == 0 ? 1 : ns(s - 1) * radix(s - 1); }
+  // twiddles by stage: entry r NS + k of stage s >= 1 at off(s), w^(r k N/(NS RAD)) -- a row of
+  // consecutive k per r, so that neighbouring butterflies read neighbouring entries
+  __host__ __device__ static constexpr int off(int s) { return s <= 1 ? 0 : off(s - 1) + ns(s - 1) * radix(s - 1); }
+  static constexpr int tw_elems = stages > 1 ? off(stages - 1) + ns(stages - 1) * radix(stages - 1) : 1;
+};
+
+template <typename R, class PL, int N, int THREADS, int S = 1>
+__device__ __forceinline__ void load_stage_twiddles(cx<R>* tws, const cx<R>* __restrict__ tw) {
+  if constexpr (S < PL::stages) {
+    constexpr int NS = PL::ns(S), RAD = PL::radix(S), ST = N / (NS * RAD);
+    for (int e = threadIdx.x; e < NS * RAD; e += THREADS) tws[PL::off(S) + e] = tw[(e / NS) * (e % NS) * ST];
+    load_stage_twiddles<R, PL, N, THREADS, S + 1>(tws, tw);
+  }
+}
+
+// the RAD inputs of butterfly j of line b at stage S >= 1 from the tile, twiddled and transformed
+template <typename R, class PL, int N, bool INV, int LINES, Lay L, int SKEW, int S>
+__device__ __forceinline__ void io_butterfly(const cx<R>* buf, const cx<R>* tws, int b, int j, cx<R>* v) {
+  using IX = LayIdx<L, N, LINES, SKEW>;
+  constexpr int RAD = PL::radix(S), NS = PL::ns(S), NB = N / RAD;
+  const int k = j % NS;
+#pragma unroll
+  for (int r = 0; r < RAD; ++r) {
+    cx<R> x = buf[IX::at(b, j + r * NB)];
+    if (r > 0) {
+      cx<R> w = tws[PL::off(S) + r * NS + k];
+      if (INV) w.y = -w.y;
+      x = x * w;
+    }
+    v[r] = x;
+  }
+  Dft<R, INV>::template run<RAD>(v);
+}
+
+// stages S .. stages - 2 in place in the tile
+template <typename R, class PL, int N, bool INV, int LINES, int THREADS, Lay L, int SKEW, int S>
+__device__ __forceinline__ void io_middle(cx<R>* buf, const cx<R>* tws) {
+  if constexpr (S < PL::stages - 1) {
+    using IX = LayIdx<L, N, LINES, SKEW>;
+    constexpr int RAD = PL::radix(S), NS = PL::ns(S), NB = N / RAD, TOTAL = LINES * NB;
+    constexpr int PER = (TOTAL + THREADS - 1) / THREADS;
+    cx<R> v[PER][RAD];
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      const int t = threadIdx.x + p * THREADS;
+      if (TOTAL % THREADS == 0 || t < TOTAL) {
+        int b, j;
+        IX::map(t, NB, b, j);
+        io_butterfly<R, PL, N, INV, LINES, L, SKEW, S>(buf, tws, b, j, v[p]);
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      const int t = threadIdx.x + p * THREADS;
+      if (TOTAL % THREADS == 0 || t < TOTAL) {
+        int b, j;
+        IX::map(t, NB, b, j);
+        const int o = (j / NS) * NS * RAD + j % NS;
+#pragma unroll
+        for (int r = 0; r < RAD; ++r) buf[IX::at(b, o + r * NS)] = v[p][r];
+      }
+    }
+    __syncthreads();
+    io_middle<R, PL, N, INV, LINES, THREADS, L, SKEW, S + 1>(buf, tws);
+  }
+}
+
+// First stage: ld(b, i) gives element i of line b; its outputs go to the tile (then a
+// barrier and the middle stages), ready for the last stage.  Only for plans of two stages
+// or more.
+template <typename R, class PL, int N, bool INV, int LINES, int THREADS, Lay L, int SKEW, class Ld>
+__device__ __forceinline__ void io_first(cx<R>* buf, const cx<R>* tws, Ld ld) {
+  using IX = LayIdx<L, N, LINES, SKEW>;
+  constexpr int RAD = PL::radix(0), NB = N / RAD, TOTAL = LINES * NB;
+  constexpr int PER = (TOTAL + THREADS - 1) / THREADS;
+  cx<R> v[PER][RAD];
+#pragma unroll
+  for (int p = 0; p < PER; ++p) {  // every load of the thread first
+    const int t = threadIdx.x + p * THREADS;
+    if (TOTAL % THREADS == 0 || t < TOTAL) {
+      int b, j;
+      IX::map(t, NB, b, j);
+#pragma unroll
+      for (int r = 0; r < RAD; ++r) v[p][r] = ld(b, j + r * NB);
+    }
+  }
+#pragma unroll
+  for (int p = 0; p < PER; ++p) {
+    const int t = threadIdx.x + p * THREADS;
+    if (TOTAL % THREADS == 0 || t < TOTAL) {
+      int b, j;
+      IX::map(t, NB, b, j);
+      Dft<R, INV>::template run<RAD>(v[p]);
+#pragma unroll
+      for (int r = 0; r < RAD; ++r) buf[IX::at(b, j * RAD + r)] = v[p][r];
+    }
+  }
+  __syncthreads();
+  io_middle<R, PL, N, INV, LINES, THREADS, L, SKEW, 1>(buf, tws);
+}
+
+// Transform LINES lines: ld(b, i) -> element i of line b, st(b, i, value) takes the results.
+// Called by all THREADS threads; the twiddles tws (load_stage_twiddles) need no barrier
+// before it when the plan has a barrier (two stages or more).  Safe in place: every load is
+// made before the barrier, every store after it (one stage: a thread owns whole lines).
+template <typename R, class PL, int N, bool INV, int LINES, int THREADS, Lay L, int SKEW, class Ld, class St>
+__device__ __forceinline__ void fft_lines_io(cx<R>* buf, const cx<R>* tws, Ld ld, St st) {
+  using IX = LayIdx<L, N, LINES, SKEW>;
+  constexpr int S = PL::stages - 1, RAD = PL::radix(S), NB = N / RAD, TOTAL = LINES * NB;
+  if constexpr (S == 0) {
+    for (int b = threadIdx.x; b < LINES; b += THREADS) {
+      cx<R> v[RAD];
+#pragma unroll
+      for (int r = 0; r < RAD; ++r) v[r] = ld(b, r);
+      Dft<R, INV>::template run<RAD>(v);
+#pragma unroll
+      for (int r = 0; r < RAD; ++r) st(b, r, v[r]);
+    }
+  } else {
+    io_first<R, PL, N, INV, LINES, THREADS, L, SKEW>(buf, tws, ld);
+    for (int t = threadIdx.x; t < TOTAL; t += THREADS) {
+      int b, j;
+      IX::map(t, NB, b, j);
+      cx<R> v[RAD];
+      io_butterfly<R, PL, N, INV, LINES, L, SKEW, S>(buf, tws, b, j, v);
+#pragma unroll
+      for (int r = 0; r < RAD; ++r) st(b, j + r * NB, v[r]);
+    }
+  }
 }
 
 }  // namespace fl

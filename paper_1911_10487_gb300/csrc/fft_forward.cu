@@ -117,19 +117,37 @@ cudaError_t fwd_plane(const cx<R>* W, const Problem& P, const Work<R>& w, cudaSt
   return launch_mode_norms<R>(P, w, s);
 }
 
+template <typename R, int N, bool INV, typename TI, int T, bool D32>
+cudaError_t rows_launch(const TI* in, cx<R>* out, long long nrows, const cx<R>* tw, R scale, cudaStream_t s) {
+  using DP = DensePass<R, N, T>;
+  return launch_pdl(k_fft_rows<R, N, INV, TI, T, D32>, dim3((unsigned)((nrows + DP::LINES - 1) / DP::LINES)),
+                    dim3(DP::RT), 0, s, in, out, nrows, tw, scale);
+}
+
+template <typename R, int N, bool INV, int T, bool D32>
+cudaError_t cols_launch(const cx<R>* in, cx<R>* out, long long planes, const cx<R>* tw, unsigned* clear, int nclear,
+                        cudaStream_t s) {
+  using DP = DensePass<R, N, T>;
+  constexpr long long MAX_Y = 32768;  // planes per launch (grid y <= 65535)
+  for (long long p0 = 0; p0 < planes; p0 += MAX_Y) {
+    const long long np = planes - p0 < MAX_Y ? planes - p0 : MAX_Y;
+    const cudaError_t e = launch_pdl(k_fft_cols<R, N, INV, T, D32>, dim3((N + DP::COLS - 1) / DP::COLS, (unsigned)np),
+                                     dim3(DP::CT), 0, s, in + p0 * N * N, out + p0 * N * N, tw, clear, nclear);
+    if (e != cudaSuccess) return e;
+    clear = nullptr;
+  }
+  return cudaSuccess;
+}
+
 // W (complex64) -> W~ (complex128 in w.wt64) and the norms: the forward transform
 // of the mixed truncated-SVD route, in FP64
 template <int N>
 cudaError_t fwd_wide_impl(const float2* W, const Problem& P, const Work<float>& w, cudaStream_t s, cudaEvent_t mid) {
-  constexpr int LINES = row_lines<double, N, 0>();
-  const long long nrows = (long long)P.n_omega * P.m1 * N;
-  const long long nblk = (nrows + LINES - 1) / LINES;
-  cudaError_t e = launch_pdl(k_fft_rows<double, N, false, float2>, dim3((unsigned)nblk), dim3(THREADS), 0, s, W,
-                             w.wt64, nrows, w.tw64, 1.0);
+  const long long planes = (long long)P.n_omega * P.m1;
+  cudaError_t e = rows_launch<double, N, false, float2, 0, false>(W, w.wt64, planes * N, w.tw64, 1.0, s);
   if (e != cudaSuccess) return e;
   if (mid) cudaEventRecord(mid, s);
-  const dim3 g2((N + tile_cols<double, 0>() - 1) / tile_cols<double, 0>(), (unsigned)(P.n_omega * P.m1));
-  e = launch_pdl(k_fft_cols<double, N, false>, g2, dim3(THREADS), 0, s, w.wt64, w.tw64, (unsigned*)nullptr, 0);
+  e = cols_launch<double, N, false, 0, false>(w.wt64, w.wt64, planes, w.tw64, nullptr, 0, s);
   if (e != cudaSuccess) return e;
   const dim3 gn((unsigned)w.n_partial, (unsigned)P.n_omega);
   e = launch_pdl(k_mode_norms<double>, gn, dim3(NORM_T), 0, s, (const double2*)w.wt64, w.norms, w.partial, P.m1,
@@ -141,17 +159,12 @@ cudaError_t fwd_wide_impl(const float2* W, const Problem& P, const Work<float>& 
 template <typename R, int N, int T>
 cudaError_t fwd_tiled(const cx<R>* W, const Problem& P, const Work<R>& w, cudaStream_t s, cudaEvent_t mid,
                       bool norms) {
-  constexpr int LINES = row_lines<R, N, T>();
-  const long long nrows = (long long)P.n_omega * P.m1 * N;
-  const long long nblk = (nrows + LINES - 1) / LINES;
-  cudaError_t e = launch_pdl(k_fft_rows<R, N, false, cx<R>, T>, dim3((unsigned)nblk), dim3(THREADS), 0, s, W, w.wt,
-                             nrows, (const cx<R>*)w.tw, R(1));
+  const long long planes = (long long)P.n_omega * P.m1;
+  cudaError_t e = rows_launch<R, N, false, cx<R>, T, false>(W, w.wt, planes * N, (const cx<R>*)w.tw, R(1), s);
   if (e != cudaSuccess) return e;
   if (mid) cudaEventRecord(mid, s);
-  constexpr int TC = tile_cols<R, T>();
-  const dim3 g2((N + TC - 1) / TC, (unsigned)(P.n_omega * P.m1));
-  e = launch_pdl(k_fft_cols<R, N, false, T>, g2, dim3(THREADS), 0, s, w.wt, (const cx<R>*)w.tw,
-                 norms ? (unsigned*)nullptr : w.bar, P.n_omega);
+  e = cols_launch<R, N, false, T, false>(w.wt, w.wt, planes, (const cx<R>*)w.tw, norms ? (unsigned*)nullptr : w.bar,
+                                         P.n_omega, s);
   if (e != cudaSuccess) return e;
   if (!norms) return cudaGetLastError();
   return launch_mode_norms<R>(P, w, s);
@@ -173,27 +186,15 @@ cudaError_t fwd_impl(const cx<R>* W, const Problem& P, const Work<R>& w, cudaStr
 }
 
 template <typename R, int N>
-cudaError_t dense_impl(cx<R>* in, cx<R>* out, long long planes, bool inverse, const cx<R>* tw, cudaStream_t s) {
-  constexpr int LINES = row_lines<R, N, 0>();
-  constexpr long long MAX_Y = 32768;  // planes per column launch (grid y <= 65535)
-  const long long nrows = planes * N;
-  const unsigned nblk = (unsigned)((nrows + LINES - 1) / LINES);
-  auto cols = [&](cx<R>* buf, bool inv) {
-    for (long long p0 = 0; p0 < planes; p0 += MAX_Y) {
-      const long long np = planes - p0 < MAX_Y ? planes - p0 : MAX_Y;
-      const dim3 gc((N + tile_cols<R, 0>() - 1) / tile_cols<R, 0>(), (unsigned)np);
-      if (inv) k_fft_cols<R, N, true><<<gc, THREADS, 0, s>>>(buf + p0 * N * N, tw, nullptr, 0);
-      else k_fft_cols<R, N, false><<<gc, THREADS, 0, s>>>(buf + p0 * N * N, tw, nullptr, 0);
-    }
-  };
+cudaError_t dense_impl(const cx<R>* in, cx<R>* out, long long planes, bool inverse, const cx<R>* tw, cudaStream_t s) {
+  constexpr bool D32 = sizeof(R) == 4;
+  cudaError_t e;
   if (!inverse) {
-    k_fft_rows<R, N, false><<<nblk, THREADS, 0, s>>>(in, out, nrows, tw, R(1));
-    cols(out, false);
-  } else {
-    cols(in, true);
-    k_fft_rows<R, N, true><<<nblk, THREADS, 0, s>>>(in, out, nrows, tw, R(1.0 / ((double)N * N)));
+    if ((e = rows_launch<R, N, false, cx<R>, 0, D32>(in, out, planes * N, tw, R(1), s)) != cudaSuccess) return e;
+    return cols_launch<R, N, false, 0, D32>(out, out, planes, tw, nullptr, 0, s);
   }
-  return cudaGetLastError();
+  if ((e = cols_launch<R, N, true, 0, D32>(in, out, planes, tw, nullptr, 0, s)) != cudaSuccess) return e;
+  return rows_launch<R, N, true, cx<R>, 0, D32>(out, out, planes * N, tw, R(1.0 / ((double)N * N)), s);
 }
 
 }  // namespace
@@ -228,7 +229,7 @@ cudaError_t launch_fft2_forward(const cx<R>* W, const Problem& P, const Work<R>&
 }
 
 template <typename R>
-cudaError_t launch_fft2_dense(cx<R>* in, cx<R>* out, int n, long long planes, bool inverse, const cx<R>* tw,
+cudaError_t launch_fft2_dense(const cx<R>* in, cx<R>* out, int n, long long planes, bool inverse, const cx<R>* tw,
                               cudaStream_t s) {
   switch (n) {
 #define FL_CASE(K) case K: return dense_impl<R, K>(in, out, planes, inverse, tw, s);
@@ -237,8 +238,8 @@ cudaError_t launch_fft2_dense(cx<R>* in, cx<R>* out, int n, long long planes, bo
     default: return cudaErrorInvalidValue;
   }
 }
-template cudaError_t launch_fft2_dense<double>(double2*, double2*, int, long long, bool, const double2*, cudaStream_t);
-template cudaError_t launch_fft2_dense<float>(float2*, float2*, int, long long, bool, const float2*, cudaStream_t);
+template cudaError_t launch_fft2_dense<double>(const double2*, double2*, int, long long, bool, const double2*, cudaStream_t);
+template cudaError_t launch_fft2_dense<float>(const float2*, float2*, int, long long, bool, const float2*, cudaStream_t);
 
 template <typename R>
 cudaError_t launch_twiddles(cx<R>* tw, int n, cudaStream_t s) {

@@ -16,23 +16,18 @@ namespace fl {
 
 namespace {
 
-// Tile shapes of the transform passes (fs_options.fft_tile, chosen by the batch tuner):
-//   0  shared-memory tiles of 2048 elements, 16 (FP32) or 8 (FP64) columns per column
-//      tile, radix cap 16 (8 in the recovery pass) -- measured best on one 128^2 problem;
-//   1  tiles of 1024 elements, 8 or 4 columns, radix cap 8: twice the blocks with half
-//      the shared memory each, for many concurrent problems.
-// Row tiles are padded after every SKEW elements (LayIdx): the first (radix-SKEW) stage
-// of a row pass writes with that stride.
+// Tile shapes of the gather and recovery passes (fs_options.fft_tile, chosen by the batch
+// tuner): 0 -- tiles of 2048 elements, 16 (FP32) or 8 (FP64) columns per column tile, radix
+// cap 16 (8 in the recovery pass); 1 -- tiles of 1024 elements, 8 or 4 columns, radix cap 8.
+// Row tiles are padded after every SKEW elements (LayIdx).
 template <int T> struct Tile;
 template <> struct Tile<0> {
   static constexpr int ELEMS = 2048, TC32 = 16, TC64 = 8;
-  static constexpr int RADIX_ROWS = 16, RADIX_COLS = 16, RADIX_GATHER = 16, RADIX_RECOVER = 8;
-  static constexpr int SKEW_ROWS = 16, SKEW_RECOVER = 8;
+  static constexpr int RADIX_GATHER = 16, RADIX_RECOVER = 8, SKEW_RECOVER = 8;
 };
 template <> struct Tile<1> {
   static constexpr int ELEMS = 1024, TC32 = 8, TC64 = 4;
-  static constexpr int RADIX_ROWS = 8, RADIX_COLS = 8, RADIX_GATHER = 8, RADIX_RECOVER = 8;
-  static constexpr int SKEW_ROWS = 8, SKEW_RECOVER = 8;
+  static constexpr int RADIX_GATHER = 8, RADIX_RECOVER = 8, SKEW_RECOVER = 8;
 };
 template <typename R, int T> __host__ __device__ constexpr int tile_cols() {
   return sizeof(R) == 4 ? Tile<T>::TC32 : Tile<T>::TC64;
@@ -40,14 +35,26 @@ template <typename R, int T> __host__ __device__ constexpr int tile_cols() {
 
 constexpr int THREADS = 256;
 
-// rows of one tile of the dense row pass: the tile's elements over N; FP32 at N = 256
-// with the default tile: 4096 elements (16 rows), fewer CTAs with less fixed cost
-// (measured: the row pass of 256^2 x 64 with 19 planes and 8 frequencies 61.5 -> 55.5 us;
-// at 192, 21 rows a tile, slower: 53.6 -> 57.8 us)
-template <typename R, int N, int T> __host__ __device__ constexpr int row_lines() {
-  constexpr int E = (sizeof(R) == 4 && T == 0 && N >= 256) ? 4096 : Tile<T>::ELEMS;
-  return E / N > 0 ? E / N : 1;
-}
+// ---- shapes of the dense passes --------------------------------------------------
+// One butterfly of 16 (12) elements per thread in the first stage.  FP32 (bound by memory):
+// tiles of up to 2048 elements in 128 threads, 16 loads in flight per thread and many CTAs
+// per SM.  FP64 (bound by the FP64 pipe, which one warp per SM quarter fills): small tiles
+// of 1-4 warps, so that the CTAs of a small problem spread over the SMs, and line counts
+// that give every stage whole warps (a half-empty warp costs a whole one).
+// T: fs_options.fft_tile (1: half the lines, radix cap 8)
+constexpr int round32(int x) { return x <= 32 ? 32 : (x + 31) / 32 * 32; }
+template <typename R, int N, int T> struct DensePass {
+  static constexpr bool F32 = sizeof(R) == 4;
+  static constexpr int MAXR = T == 0 ? 16 : 8;
+  static constexpr int ROWS0 = F32 ? (N <= 16 ? 64 : N <= 32 ? 32 : N <= 128 ? 16 : 8)
+                                   : (N == 8 ? 64 : N <= 16 ? 32 : N <= 32 ? 16 : N <= 192 ? 8 : 4);
+  static constexpr int LINES = T == 0 ? ROWS0 : ROWS0 / 2;                            // rows per tile
+  static constexpr int COLS = T == 0 ? (F32 || N <= 32 ? 16 : 8) : (F32 ? 8 : 4);     // columns per tile
+  static constexpr int PT = T == 0 ? (N % 3 == 0 ? 12 : 16) : 8;                      // elements per thread
+  static constexpr int threads(int lines) { return round32(lines * N / PT) < 256 ? round32(lines * N / PT) : 256; }
+  static constexpr int RT = threads(LINES), CT = threads(COLS);
+  static constexpr int SKEW = MAXR;
+};
 
 // CTAs per plane of the single-pass (cluster) transforms: the smallest power of two,
 // at most 8 (the portable cluster size), that leaves each CTA at most 16 rows (24 for
@@ -68,65 +75,60 @@ __device__ __forceinline__ void load_twiddles(cx<R>* tw_s, const cx<R>* __restri
 }
 
 // ---- dense pass along x (rows): forward, or inverse with 1/N^2 scaling --------
-// TI: element type of `in` (cx<R>, or float2 read into an FP64 transform)
-template <typename R, int N, bool INV, typename TI = cx<R>, int T = 0>
-__global__ void __launch_bounds__(THREADS)
-k_fft_rows(const TI* __restrict__ in, cx<R>* __restrict__ out, long long nrows,
-           const cx<R>* __restrict__ tw, R scale) {
-  constexpr int LINES = row_lines<R, N, T>();
-  using IX = LayIdx<Lay::ROW, N, LINES, Tile<T>::SKEW_ROWS>;
-  __shared__ cx<R> buf[IX::ELEMS];
-  __shared__ cx<R> tw_s[N];
-  load_twiddles<R, N>(tw_s, tw);  // a constant table: read while the predecessor drains
+// TI: element type of `in` (cx<R>, or float2 read into an FP64 transform); D32: FftPlan's
+// factors in FP32 (IoPlan)
+template <typename R, int N, bool INV, typename TI = cx<R>, int T = 0, bool D32 = false>
+__global__ void __launch_bounds__((DensePass<R, N, T>::RT))
+k_fft_rows(const TI* __restrict__ in, cx<R>* out, long long nrows, const cx<R>* __restrict__ tw, R scale) {
+  using DP = DensePass<R, N, T>;
+  using PL = IoPlan<N, DP::MAXR, D32>;
+  constexpr int LINES = DP::LINES;
+  __shared__ cx<R> buf[PL::stages > 1 ? LayIdx<Lay::ROW, N, LINES, DP::SKEW>::ELEMS : 1];
+  __shared__ cx<R> tws[PL::tw_elems];
+  load_stage_twiddles<R, PL, N, DP::RT>(tws, tw);  // a constant table: read while the predecessor drains
   pdl_wait();
   pdl_trigger();
   const long long row0 = (long long)blockIdx.x * LINES;
-  const long long base = row0 * N;
-  const long long limit = nrows * N;
-  for (int e = threadIdx.x; e < LINES * N; e += THREADS) {
-    cx<R> v = czero<R>();
-    if (base + e < limit) {
-      if constexpr (std::is_same<TI, cx<R>>::value) v = in[base + e];
-      else v = from_d<R>(to_d(in[base + e]));
-    }
-    buf[IX::at(e / N, e % N)] = v;
-  }
-  __syncthreads();
-  fft_lines<R, N, INV, LINES, THREADS, Lay::ROW, Tile<T>::RADIX_ROWS, Tile<T>::SKEW_ROWS>(buf, tw_s);
-  for (int e = threadIdx.x; e < LINES * N; e += THREADS)
-    if (base + e < limit) {
-      const cx<R> v = buf[IX::at(e / N, e % N)];
-      out[base + e] = INV ? scale * v : v;
-    }
+  const int rows = (int)(nrows - row0 < LINES ? nrows - row0 : LINES);
+  const TI* src = in + row0 * N;
+  cx<R>* dst = out + row0 * N;
+  fft_lines_io<R, PL, N, INV, LINES, DP::RT, Lay::ROW, DP::SKEW>(
+      buf, tws,
+      [&](int b, int i) {
+        if (b >= rows) return czero<R>();
+        if constexpr (std::is_same<TI, cx<R>>::value) return src[b * N + i];
+        else return from_d<R>(to_d(src[b * N + i]));
+      },
+      [&](int b, int i, cx<R> v) {
+        if (b < rows) dst[b * N + i] = INV ? scale * v : v;
+      });
 }
 
-// ---- dense pass along y (columns), in place; grid (ceil(N/TC), planes) ---------
+// ---- dense pass along y (columns); grid (ceil(N/TC), planes); in == out is allowed ---
 // clear (may be null): nclear counters zeroed by block (0, 0) -- the barrier counters
 // of the classification kernel that follows
-template <typename R, int N, bool INV, int T = 0>
-__global__ void __launch_bounds__(THREADS)
-k_fft_cols(cx<R>* __restrict__ data, const cx<R>* __restrict__ tw, unsigned* __restrict__ clear, int nclear) {
-  constexpr int TC = tile_cols<R, T>();
-  constexpr int E = N * TC;
-  __shared__ cx<R> buf[E];
-  __shared__ cx<R> tw_s[N];
-  load_twiddles<R, N>(tw_s, tw);  // a constant table: read while the predecessor drains
+template <typename R, int N, bool INV, int T = 0, bool D32 = false>
+__global__ void __launch_bounds__((DensePass<R, N, T>::CT))
+k_fft_cols(const cx<R>* in, cx<R>* out, const cx<R>* __restrict__ tw, unsigned* __restrict__ clear, int nclear) {
+  using DP = DensePass<R, N, T>;
+  using PL = IoPlan<N, DP::MAXR, D32>;
+  constexpr int TC = DP::COLS;
+  __shared__ cx<R> buf[PL::stages > 1 ? N * TC : 1];
+  __shared__ cx<R> tws[PL::tw_elems];
+  load_stage_twiddles<R, PL, N, DP::CT>(tws, tw);  // a constant table: read while the predecessor drains
   pdl_wait();
   pdl_trigger();
   if (clear && blockIdx.x == 0 && blockIdx.y == 0)
-    for (int i = threadIdx.x; i < nclear; i += THREADS) clear[i] = 0u;
+    for (int i = threadIdx.x; i < nclear; i += DP::CT) clear[i] = 0u;
   const int c0 = blockIdx.x * TC;
-  cx<R>* pl = data + (long long)blockIdx.y * N * N;
-  for (int e = threadIdx.x; e < E; e += THREADS) {
-    const int i = e / TC, b = e % TC;
-    buf[e] = (c0 + b < N) ? pl[(long long)i * N + c0 + b] : czero<R>();
-  }
-  __syncthreads();
-  fft_lines<R, N, INV, TC, THREADS, Lay::COL, Tile<T>::RADIX_COLS>(buf, tw_s);
-  for (int e = threadIdx.x; e < E; e += THREADS) {
-    const int i = e / TC, b = e % TC;
-    if (c0 + b < N) pl[(long long)i * N + c0 + b] = buf[e];
-  }
+  const long long o = (long long)blockIdx.y * N * N + c0;
+  const cx<R>* src = in + o;
+  cx<R>* dst = out + o;
+  fft_lines_io<R, PL, N, INV, TC, DP::CT, Lay::COL, 0>(
+      buf, tws, [&](int b, int i) { return N % TC == 0 || c0 + b < N ? src[i * N + b] : czero<R>(); },
+      [&](int b, int i, cx<R> v) {
+        if (N % TC == 0 || c0 + b < N) dst[i * N + b] = v;
+      });
 }
 
 // ---- per-mode norms ||W~_nu||^2 = sum_k |W~_k(nu)|^2 ----------------------------

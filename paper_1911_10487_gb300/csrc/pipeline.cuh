@@ -236,10 +236,10 @@ cudaError_t launch_recover(const Problem& P, const Work<R>& w, R* xi, R* c, cuda
                            cudaEvent_t mid = nullptr);
 template <typename R>
 cudaError_t launch_twiddles(cx<R>* tw, int n, cudaStream_t s);
-// dense 2D FFT of `planes` N x N planes: forward (unnormalised) in -> out, or
-// inverse (with 1/N^2) transforming `in` in place along y, then in -> out along x
+// dense 2D FFT of `planes` N x N planes, in -> out (in == out is allowed): forward
+// (unnormalised) along x then y, or inverse (with 1/N^2) along y then x
 template <typename R>
-cudaError_t launch_fft2_dense(cx<R>* in, cx<R>* out, int n, long long planes, bool inverse, const cx<R>* tw,
+cudaError_t launch_fft2_dense(const cx<R>* in, cx<R>* out, int n, long long planes, bool inverse, const cx<R>* tw,
                               cudaStream_t s);
 // the sampled-G kernel tables of one frequency (kernel_plan.cu): G sampled on the grid
 // offsets, its 2D FFT, packed mode-major with omega^2 h_z applied and the traces;
