@@ -48,6 +48,9 @@ struct fs_ctx {
   void* tw[2][N_SIZES] = {};  // [fp64?][size]
   unsigned long long* ctr = nullptr;
   unsigned long long* ctr_host = nullptr;
+  // the stopping test of fs_forward: its value (mapped page-locked memory) and event
+  double* fwd_host = nullptr;
+  cudaEvent_t fwd_ev = nullptr;
   // staging for fs_reconstruct_host
   void* stage = nullptr;
   size_t stage_bytes = 0;
@@ -509,6 +512,8 @@ void fs_destroy(fs_ctx* ctx) {
       if (p) cudaFree(p);
   if (ctx->ctr) cudaFree(ctx->ctr);
   if (ctx->ctr_host) cudaFreeHost(ctx->ctr_host);
+  if (ctx->fwd_host) cudaFreeHost(ctx->fwd_host);
+  if (ctx->fwd_ev) cudaEventDestroy(ctx->fwd_ev);
   for (auto& e : ctx->ev)
     if (e) cudaEventDestroy(e);
   for (int k = 0; k < fs_ctx::MAX_SIDE; ++k) {
@@ -808,17 +813,27 @@ fs_status fs_forward(fs_ctx* ctx, const fs_geometry* g, fs_precision prec, const
   const bool fp64 = prec == FS_FP64;
   const size_t need = fp64 ? forward_bytes<double>(P) : forward_bytes<float>(P);
   if ((st = ensure_workspace(ctx, need)) != FS_OK) return st;
+  if (!ctx->fwd_ev && (e = cudaEventCreateWithFlags(&ctx->fwd_ev, cudaEventDisableTiming)) != cudaSuccess) {
+    ctx->fwd_ev = nullptr;
+    return cuda_fail(ctx, e, "forward event");
+  }
+  if (!ctx->fwd_host && cudaMallocHost(&ctx->fwd_host, sizeof(double)) != cudaSuccess) {
+    ctx->fwd_host = nullptr;
+    return fail(ctx, FS_ENOMEM, "page-locked memory of the forward solve");
+  }
   std::vector<int> it(n_omega, 0), conv(n_omega, 0);
   if (fp64) {
     const double2* tw = nullptr;
     if ((st = ensure_twiddles<double>(ctx, g->n, &tw)) != FS_OK) return st;
     e = forward_solve<double>(P, (const double*)xi, (const double2*)incident, (double2*)W, (double2*)u, ctx->ws,
-                              (int)method, rtol, max_iter, tw, ctx->stream, it.data(), conv.data());
+                              (int)method, rtol, max_iter, tw, ctx->stream, ctx->fwd_host, ctx->fwd_ev, it.data(),
+                              conv.data());
   } else {
     const float2* tw = nullptr;
     if ((st = ensure_twiddles<float>(ctx, g->n, &tw)) != FS_OK) return st;
     e = forward_solve<float>(P, (const float*)xi, (const float2*)incident, (float2*)W, (float2*)u, ctx->ws,
-                             (int)method, rtol, max_iter, tw, ctx->stream, it.data(), conv.data());
+                             (int)method, rtol, max_iter, tw, ctx->stream, ctx->fwd_host, ctx->fwd_ev, it.data(),
+                              conv.data());
   }
   if (e != cudaSuccess) return cuda_fail(ctx, e, "forward");
   if (iterations)

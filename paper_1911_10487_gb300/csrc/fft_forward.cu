@@ -117,6 +117,76 @@ cudaError_t fwd_plane(const cx<R>* W, const Problem& P, const Work<R>& w, cudaSt
   return launch_mode_norms<R>(P, w, s);
 }
 
+// ---- rows of pairs of real planes ------------------------------------------------
+// The forward transform along x of M real planes, two to a complex plane: pair p holds
+// planes 2p - off and 2p + 1 - off (off = M mod 2; plane -1 is zero) in its real and
+// imaginary part; the reader separates them by their symmetry (k_apply_data).
+template <typename R, int N>
+__global__ void __launch_bounds__((DensePass<R, N, 0>::RT))
+k_fft_rows_pairs(const R* __restrict__ xi, cx<R>* __restrict__ out, long long nrows, int off,
+                 const cx<R>* __restrict__ tw) {
+  using DP = DensePass<R, N, 0>;
+  using PL = IoPlan<N, DP::MAXR, false>;
+  constexpr int LINES = DP::LINES;
+  __shared__ cx<R> buf[PL::stages > 1 ? LayIdx<Lay::ROW, N, LINES, DP::SKEW>::ELEMS : 1];
+  __shared__ cx<R> tws[PL::tw_elems];
+  load_stage_twiddles<R, PL, N, DP::RT>(tws, tw);
+  pdl_wait();
+  pdl_trigger();
+  const long long row0 = (long long)blockIdx.x * LINES;
+  fft_lines_io<R, PL, N, false, LINES, DP::RT, Lay::ROW, DP::SKEW>(
+      buf, tws,
+      [&](int b, int i) {
+        const long long row = row0 + b;
+        if (row >= nrows) return czero<R>();
+        const long long p = row / N, y = row - p * N, l = 2 * p - off;
+        const R re = l >= 0 ? xi[(l * N + y) * N + i] : R(0);
+        return mk<R>(re, xi[((l + 1) * N + y) * N + i]);
+      },
+      [&](int b, int i, cx<R> v) {
+        if (row0 + b < nrows) out[(row0 + b) * N + i] = v;
+      });
+}
+
+// ---- rows: inverse along x, times xi, forward along x --------------------------------
+// The middle of F[xi F^-1 U~]: between the two column passes everything happens within a
+// row, so one kernel reads and writes the planes once (three kernels before: inverse rows,
+// the product, forward rows; 128^2 x 64 FP64 per iteration 116 us -> 113 us, bound by the FP64
+// pipe; FP32 by memory, where the passes saved count).
+template <typename R, int N>
+__global__ void __launch_bounds__((DensePass<R, N, 0>::RT))
+k_rows_xi(cx<R>* __restrict__ data, const R* __restrict__ xi, long long nrows, const cx<R>* __restrict__ tw,
+          R scale) {
+  using DP = DensePass<R, N, 0>;
+  using PL = IoPlan<N, DP::MAXR, sizeof(R) == 4>;
+  constexpr int LINES = DP::LINES;
+  using IX = LayIdx<Lay::ROW, N, LINES, DP::SKEW>;
+  extern __shared__ __align__(16) unsigned char rows_xi_smem[];  // 2 IX::ELEMS elements
+  cx<R>* buf = reinterpret_cast<cx<R>*>(rows_xi_smem);
+  cx<R>* mid = buf + IX::ELEMS;
+  __shared__ cx<R> tws[PL::tw_elems];
+  load_stage_twiddles<R, PL, N, DP::RT>(tws, tw);
+  pdl_wait();
+  pdl_trigger();
+  const long long row0 = (long long)blockIdx.x * LINES;
+  const int rows = (int)(nrows - row0 < LINES ? nrows - row0 : LINES);
+  cx<R>* d = data + row0 * N;
+  const R* x = xi + row0 * N;
+  fft_lines_io<R, PL, N, true, LINES, DP::RT, Lay::ROW, DP::SKEW>(
+      buf, tws, [&](int b, int i) { return b < rows ? d[b * N + i] : czero<R>(); },
+      [&](int b, int i, cx<R> v) {
+        const R f = b < rows ? x[b * N + i] : R(0);
+        v = scale * v;
+        mid[IX::at(b, i)] = mk<R>(f * v.x, f * v.y);
+      });
+  __syncthreads();
+  fft_lines_io<R, PL, N, false, LINES, DP::RT, Lay::ROW, DP::SKEW>(
+      buf, tws, [&](int b, int i) { return mid[IX::at(b, i)]; },
+      [&](int b, int i, cx<R> v) {
+        if (b < rows) d[b * N + i] = v;
+      });
+}
+
 template <typename R, int N, bool INV, typename TI, int T, bool D32>
 cudaError_t rows_launch(const TI* in, cx<R>* out, long long nrows, const cx<R>* tw, R scale, cudaStream_t s) {
   using DP = DensePass<R, N, T>;
@@ -197,6 +267,34 @@ cudaError_t dense_impl(const cx<R>* in, cx<R>* out, long long planes, bool inver
   return rows_launch<R, N, true, cx<R>, 0, D32>(out, out, planes * N, tw, R(1.0 / ((double)N * N)), s);
 }
 
+// F[xi F^-1 ut] -> out, M planes
+template <typename R, int N>
+cudaError_t xi_impl(const cx<R>* ut, cx<R>* out, const R* xi, long long planes, const cx<R>* tw, cudaStream_t s) {
+  using DP = DensePass<R, N, 0>;
+  constexpr bool D32 = sizeof(R) == 4;
+  cudaError_t e = cols_launch<R, N, true, 0, D32>(ut, out, planes, tw, nullptr, 0, s);
+  if (e != cudaSuccess) return e;
+  const long long nrows = planes * N;
+  constexpr size_t smem = 2 * sizeof(cx<R>) * LayIdx<Lay::ROW, N, DP::LINES, DP::SKEW>::ELEMS;
+  static SmemOptIn attr;
+  if ((e = opt_in_smem(attr, (const void*)k_rows_xi<R, N>, smem)) != cudaSuccess) return e;
+  e = launch_pdl(k_rows_xi<R, N>, dim3((unsigned)((nrows + DP::LINES - 1) / DP::LINES)), dim3(DP::RT), smem, s, out,
+                 xi, nrows, tw, R(1.0 / ((double)N * N)));
+  if (e != cudaSuccess) return e;
+  return cols_launch<R, N, false, 0, D32>(out, out, planes, tw, nullptr, 0, s);
+}
+
+template <typename R, int N>
+cudaError_t pairs_impl(const R* xi, cx<R>* out, int m, const cx<R>* tw, cudaStream_t s) {
+  using DP = DensePass<R, N, 0>;
+  const int np = (m + 1) / 2;
+  const long long nrows = (long long)np * N;
+  cudaError_t e = launch_pdl(k_fft_rows_pairs<R, N>, dim3((unsigned)((nrows + DP::LINES - 1) / DP::LINES)),
+                             dim3(DP::RT), 0, s, xi, out, nrows, m & 1, tw);
+  if (e != cudaSuccess) return e;
+  return cols_launch<R, N, false, 0, false>(out, out, np, tw, nullptr, 0, s);
+}
+
 }  // namespace
 
 bool fft_size_supported(int n) {
@@ -240,6 +338,33 @@ cudaError_t launch_fft2_dense(const cx<R>* in, cx<R>* out, int n, long long plan
 }
 template cudaError_t launch_fft2_dense<double>(const double2*, double2*, int, long long, bool, const double2*, cudaStream_t);
 template cudaError_t launch_fft2_dense<float>(const float2*, float2*, int, long long, bool, const float2*, cudaStream_t);
+
+template <typename R>
+cudaError_t launch_xi_transform(const cx<R>* ut, cx<R>* out, const R* xi, int n, long long planes, const cx<R>* tw,
+                                cudaStream_t s) {
+  switch (n) {
+#define FL_CASE(K) case K: return xi_impl<R, K>(ut, out, xi, planes, tw, s);
+    FL_SIZES(FL_CASE)
+#undef FL_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+template cudaError_t launch_xi_transform<double>(const double2*, double2*, const double*, int, long long,
+                                                 const double2*, cudaStream_t);
+template cudaError_t launch_xi_transform<float>(const float2*, float2*, const float*, int, long long, const float2*,
+                                                cudaStream_t);
+
+template <typename R>
+cudaError_t launch_fft2_pairs(const R* xi, cx<R>* out, int n, int m, const cx<R>* tw, cudaStream_t s) {
+  switch (n) {
+#define FL_CASE(K) case K: return pairs_impl<R, K>(xi, out, m, tw, s);
+    FL_SIZES(FL_CASE)
+#undef FL_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+template cudaError_t launch_fft2_pairs<double>(const double*, double2*, int, int, const double2*, cudaStream_t);
+template cudaError_t launch_fft2_pairs<float>(const float*, float2*, int, int, const float2*, cudaStream_t);
 
 template <typename R>
 cudaError_t launch_twiddles(cx<R>* tw, int n, cudaStream_t s) {

@@ -51,6 +51,13 @@ __device__ __forceinline__ double rsqrt64(double x) {
   return __longlong_as_double(yb - ((long long)h << 52));
 }
 
+// sqrt(x) from r = rsqrt64(x): x r, corrected by its residual to within rounding of the exact
+// root (phases k_z d of tens of radians carry the relative error of k_z)
+__device__ __forceinline__ double sqrt_from_rsqrt(double x, double r) {
+  const double s = x * r;
+  return fma(fma(-s, s, x), 0.5 * r, s);
+}
+
 // 1/sqrt(x) and 1/x of a positive normal double to FP32 accuracy (~2e-7 relative)
 // at any exponent: the FP32 reciprocal (square root) of the mantissa, the exponent on
 // the bit pattern.  No FP64 arithmetic.

@@ -241,6 +241,14 @@ cudaError_t launch_twiddles(cx<R>* tw, int n, cudaStream_t s);
 template <typename R>
 cudaError_t launch_fft2_dense(const cx<R>* in, cx<R>* out, int n, long long planes, bool inverse, const cx<R>* tw,
                               cudaStream_t s);
+// F[xi F^-1 ut] -> out for `planes` planes (xi [planes][N][N]; out must not be ut)
+template <typename R>
+cudaError_t launch_xi_transform(const cx<R>* ut, cx<R>* out, const R* xi, int n, long long planes, const cx<R>* tw,
+                                cudaStream_t s);
+// forward 2D FFT of m real planes, two to a complex plane: (m + 1) / 2 planes out, pair p
+// the planes 2p - m % 2 (real part; zero for plane -1) and 2p + 1 - m % 2 (imaginary part)
+template <typename R>
+cudaError_t launch_fft2_pairs(const R* xi, cx<R>* out, int n, int m, const cx<R>* tw, cudaStream_t s);
 // the sampled-G kernel tables of one frequency (kernel_plan.cu): G sampled on the grid
 // offsets, its 2D FFT, packed mode-major with omega^2 h_z applied and the traces;
 // gs and ft are scratch of D N^2 complex128 each, tw64 the FP64 twiddles of N
@@ -264,14 +272,15 @@ cudaError_t launch_point_sources(const Problem& P, const double* spec, int n_src
 // 1: restarted GMRES on u - omega^2 T(xi u) = u0; 2: Algorithm 1, GMRES where it does
 // not converge -- then the data of eq. (7).  iters and converged (host arrays of
 // n_omega, may be null) report each frequency.  ws holds forward_bytes(P) bytes.
-// Synchronises the stream at each stopping test and inner product.
+// host: mapped page-locked memory for the stopping test's value, ev an event, both the
+// caller's.  The host waits at each stopping test and inner product.
 template <typename R>
 size_t forward_bytes(const Problem& P);
 // incident: u0 [n_omega][M][N][N] on X, or null for the plane wave
 template <typename R>
 cudaError_t forward_solve(const Problem& P, const R* xi, const cx<R>* incident, cx<R>* W, cx<R>* u_out, void* ws,
-                          int method, double rtol, int max_iter, const cx<R>* tw, cudaStream_t s, int* iters,
-                          int* converged);
+                          int method, double rtol, int max_iter, const cx<R>* tw, cudaStream_t s, double* host,
+                          cudaEvent_t ev, int* iters, int* converged);
 
 bool fft_size_supported(int n);
 
