@@ -142,10 +142,9 @@ typedef struct {
                           Results are identical up to the rounding of the sum ||W||^2 (its
                           terms are grouped differently).                                  */
   int fft_tile;        /* tile shape of the transform passes, a tuning knob: 0 (default)
-                          shared-memory tiles of 2048 elements, 16 (FP32) / 8 (FP64) columns
-                          per column tile, radix cap 16; 1: tiles of 1024 elements, 8 / 4
-                          columns, radix cap 8 (twice the blocks, half the shared memory
-                          each).  Applies to the two-pass transforms.  Results agree to
+                          up to 16 (FP32) / 8 (FP64) rows or columns per tile, radix cap
+                          16; 1: half as many, radix cap 8 (twice the blocks, half the
+                          shared memory each).  Applies to the two-pass transforms.  Results agree to
                           rounding.                                                      */
   int forward_single_pass; /* FS_MIXED, N <= 128: 1 (default): the forward 2D transform of W in one pass,
                           a cluster of CTAs per data plane exchanging rows and columns

@@ -135,7 +135,9 @@ Layout layout(int n, int m, int m1, int n_omega, bool fp64) {
   L.blkgz = off; off = align_up(off + 4 * cb);
   L.colblk = off; off = align_up(off + 4 * cb * 8);
   L.cols = off; off = align_up(off + 4 * (size_t)n_omega * n);
+  L.colpos = off; off = align_up(off + 4 * (size_t)n_omega * n);
   L.ncol = off; off = align_up(off + 4 * (size_t)n_omega);
+  L.colseg = off; off = align_up(off + 4 * (size_t)n_omega);
   L.count = off; off = align_up(off + 4 * (size_t)n_omega);
   L.dnu = off; off = align_up(off + 8 * (size_t)n_omega);
   L.bar = off; off = align_up(off + 4 * (size_t)n_omega);
@@ -270,7 +272,9 @@ Work<R> carve_work(void* base, const Layout& L, unsigned long long* ctr, const c
   w.blkgz = (int*)(b + L.blkgz);
   w.colblk = (unsigned*)(b + L.colblk);
   w.cols = (int*)(b + L.cols);
+  w.colpos = (int*)(b + L.colpos);
   w.ncol = (int*)(b + L.ncol);
+  w.colseg = (int*)(b + L.colseg);
   w.count = (int*)(b + L.count);
   w.dnu = (double*)(b + L.dnu);
   w.bar = (unsigned*)(b + L.bar);

@@ -127,6 +127,31 @@ template <typename R, bool INV> struct Dft {
       for (int k2 = 0; k2 < 4; ++k2) v[k1 + 4 * k2] = z[k2];
     }
   }
+  // 16 points of which only the first E and the last E (1 or 2) are not zero, as d16 would
+  // transform them (the same operations on the same values, those with zeros left out: 44 or
+  // 96 of 160)
+  template <int E> __device__ __forceinline__ static void d16_edge(C* v) {
+    const C a0 = v[0], b1 = v[15], a1 = E > 1 ? v[1] : v[0], b0 = E > 1 ? v[14] : v[15];
+    C p0 = b0, p1 = b1;  // w4^(3 k1) b
+#pragma unroll
+    for (int k1 = 0; k1 < 4; ++k1) {
+      const C t1 = tw16(a1, k1), t2 = tw16(p0, 2 * k1), t3 = tw16(p1, 3 * k1);
+      if constexpr (E > 1) {
+        C z[4] = {a0, t1, t2, t3};
+        d4(z);
+#pragma unroll
+        for (int k2 = 0; k2 < 4; ++k2) v[k1 + 4 * k2] = z[k2];
+      } else {
+        const C d = rot90<INV>(mk<R>(-t3.x, -t3.y));
+        v[k1] = a0 + t3;
+        v[k1 + 8] = a0 - t3;
+        v[k1 + 4] = a0 + d;
+        v[k1 + 12] = a0 - d;
+      }
+      p0 = rot90<!INV>(p0);  // w4^3 = conj(w4)
+      p1 = rot90<!INV>(p1);
+    }
+  }
   __device__ __forceinline__ static void d3(C* v) {
     // y1,2 = a0 - (a1+a2)/2 -/+ i (sqrt(3)/2)(a1 - a2)  (forward; signs swap for the inverse)
     const R h = R(0.86602540378443864676);
@@ -239,65 +264,6 @@ __device__ __forceinline__ void fft_lines(cx<R>* buf, const cx<R>* tw) {
   FftStages<R, N, INV, LINES, THREADS, L, SKEW, MAXR, 0, 1>::run(buf, tw);
 }
 
-// Out-of-place form of a stage: reads `src`, writes `dst`, one butterfly of a thread
-// at a time (few values live, for tiles with many butterflies per thread, where the
-// in-place form would hold them all in registers); one barrier per stage.
-template <typename R, int N, bool INV, int LINES, int THREADS, Lay L, int SKEW, int RAD, int NS>
-__device__ __forceinline__ void fft_stage_pp(const cx<R>* src, cx<R>* dst, const cx<R>* tw) {
-  using C = cx<R>;
-  using IX = LayIdx<L, N, LINES, SKEW>;
-  constexpr int NB = N / RAD;
-  constexpr int TOTAL = LINES * NB;
-  constexpr int STRIDE_TW = N / (NS * RAD);
-#pragma unroll 1
-  for (int t = threadIdx.x; t < TOTAL; t += THREADS) {
-    int b, j;
-    IX::map(t, NB, b, j);
-    const int k = j % NS;
-    C v[RAD];
-#pragma unroll
-    for (int r = 0; r < RAD; ++r) {
-      C x = src[IX::at(b, j + r * NB)];
-      if (r > 0 && NS > 1) {
-        C w = tw[r * k * STRIDE_TW];
-        if (INV) w.y = -w.y;
-        x = x * w;
-      }
-      v[r] = x;
-    }
-    if constexpr (RAD == 2) Dft<R, INV>::d2(v);
-    else if constexpr (RAD == 4) Dft<R, INV>::d4(v);
-    else if constexpr (RAD == 8) Dft<R, INV>::d8(v);
-    else if constexpr (RAD == 16) Dft<R, INV>::d16(v);
-    else Dft<R, INV>::d3(v);
-    const int oi = (j / NS) * NS * RAD + k;
-#pragma unroll
-    for (int r = 0; r < RAD; ++r) dst[IX::at(b, oi + r * NS)] = v[r];
-  }
-  __syncthreads();
-}
-
-template <typename R, int N, bool INV, int LINES, int THREADS, Lay L, int SKEW, int MAXR, int S, int NS>
-struct FftStagesPP {
-  __device__ __forceinline__ static cx<R>* run(cx<R>* a, cx<R>* b, const cx<R>* tw) {
-    if constexpr (S < FftPlan<N, MAXR>::stages) {
-      constexpr int RAD = FftPlan<N, MAXR>::radix(S);
-      fft_stage_pp<R, N, INV, LINES, THREADS, L, SKEW, RAD, NS>(a, b, tw);
-      return FftStagesPP<R, N, INV, LINES, THREADS, L, SKEW, MAXR, S + 1, NS * RAD>::run(b, a, tw);
-    } else {
-      return a;
-    }
-  }
-};
-
-// Transform the LINES lines of tile `a` through `b` (same layout); returns the one
-// that holds the result (a after an even number of stages, b after an odd one).  The
-// input tile must be complete before the call (a barrier), as for fft_lines.
-template <typename R, int N, bool INV, int LINES, int THREADS, Lay L, int MAXR, int SKEW = 0>
-__device__ __forceinline__ cx<R>* fft_lines_pp(cx<R>* a, cx<R>* b, const cx<R>* tw) {
-  return FftStagesPP<R, N, INV, LINES, THREADS, L, SKEW, MAXR, 0, 1>::run(a, b, tw);
-}
-
 // ---- transforms between global memory and registers ---------------------------
 // The passes below hold a line in registers at both ends: the first stage's inputs are
 // loaded straight from global memory in butterfly order (element j + r N/RAD, neighbouring
@@ -387,21 +353,39 @@ __device__ __forceinline__ void io_middle(cx<R>* buf, const cx<R>* tws) {
 
 // First stage: ld(b, i) gives element i of line b; its outputs go to the tile (then a
 // barrier and the middle stages), ready for the last stage.  Only for plans of two stages
-// or more.
-template <typename R, class PL, int N, bool INV, int LINES, int THREADS, Lay L, int SKEW, class Ld>
+// or more.  PRE: an index load first: the thread's ld.pre(b, i) (ints), then its ld(b, i, index).
+template <typename R, class PL, int N, bool INV, int LINES, int THREADS, Lay L, int SKEW, bool PRE = false, class Ld>
 __device__ __forceinline__ void io_first(cx<R>* buf, const cx<R>* tws, Ld ld) {
   using IX = LayIdx<L, N, LINES, SKEW>;
   constexpr int RAD = PL::radix(0), NB = N / RAD, TOTAL = LINES * NB;
   constexpr int PER = (TOTAL + THREADS - 1) / THREADS;
   cx<R> v[PER][RAD];
+  {  // every load of the thread first
+    int at[PRE ? PER : 1][PRE ? RAD : 1];
+    if constexpr (PRE) {
 #pragma unroll
-  for (int p = 0; p < PER; ++p) {  // every load of the thread first
-    const int t = threadIdx.x + p * THREADS;
-    if (TOTAL % THREADS == 0 || t < TOTAL) {
-      int b, j;
-      IX::map(t, NB, b, j);
+      for (int p = 0; p < PER; ++p) {
+        const int t = threadIdx.x + p * THREADS;
+        if (TOTAL % THREADS == 0 || t < TOTAL) {
+          int b, j;
+          IX::map(t, NB, b, j);
 #pragma unroll
-      for (int r = 0; r < RAD; ++r) v[p][r] = ld(b, j + r * NB);
+          for (int r = 0; r < RAD; ++r) at[p][r] = ld.pre(b, j + r * NB);
+        }
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      const int t = threadIdx.x + p * THREADS;
+      if (TOTAL % THREADS == 0 || t < TOTAL) {
+        int b, j;
+        IX::map(t, NB, b, j);
+#pragma unroll
+        for (int r = 0; r < RAD; ++r) {
+          if constexpr (PRE) v[p][r] = ld(b, j + r * NB, at[p][r]);
+          else v[p][r] = ld(b, j + r * NB);
+        }
+      }
     }
   }
 #pragma unroll
@@ -419,11 +403,27 @@ __device__ __forceinline__ void io_first(cx<R>* buf, const cx<R>* tws, Ld ld) {
   io_middle<R, PL, N, INV, LINES, THREADS, L, SKEW, 1>(buf, tws);
 }
 
+// The last stage: st(b, i, value) takes the results (its own inputs' places in the tile are free).
+template <typename R, class PL, int N, bool INV, int LINES, int THREADS, Lay L, int SKEW, class St>
+__device__ __forceinline__ void io_last(const cx<R>* buf, const cx<R>* tws, St st) {
+  using IX = LayIdx<L, N, LINES, SKEW>;
+  constexpr int S = PL::stages - 1, RAD = PL::radix(S), NB = N / RAD, TOTAL = LINES * NB;
+  for (int t = threadIdx.x; t < TOTAL; t += THREADS) {
+    int b, j;
+    IX::map(t, NB, b, j);
+    cx<R> v[RAD];
+    io_butterfly<R, PL, N, INV, LINES, L, SKEW, S>(buf, tws, b, j, v);
+#pragma unroll
+    for (int r = 0; r < RAD; ++r) st(b, j + r * NB, v[r]);
+  }
+}
+
 // Transform LINES lines: ld(b, i) -> element i of line b, st(b, i, value) takes the results.
 // Called by all THREADS threads; the twiddles tws (load_stage_twiddles) need no barrier
 // before it when the plan has a barrier (two stages or more).  Safe in place: every load is
 // made before the barrier, every store after it (one stage: a thread owns whole lines).
-template <typename R, class PL, int N, bool INV, int LINES, int THREADS, Lay L, int SKEW, class Ld, class St>
+template <typename R, class PL, int N, bool INV, int LINES, int THREADS, Lay L, int SKEW, bool PRE = false, class Ld,
+          class St>
 __device__ __forceinline__ void fft_lines_io(cx<R>* buf, const cx<R>* tws, Ld ld, St st) {
   using IX = LayIdx<L, N, LINES, SKEW>;
   constexpr int S = PL::stages - 1, RAD = PL::radix(S), NB = N / RAD, TOTAL = LINES * NB;
@@ -431,21 +431,17 @@ __device__ __forceinline__ void fft_lines_io(cx<R>* buf, const cx<R>* tws, Ld ld
     for (int b = threadIdx.x; b < LINES; b += THREADS) {
       cx<R> v[RAD];
 #pragma unroll
-      for (int r = 0; r < RAD; ++r) v[r] = ld(b, r);
+      for (int r = 0; r < RAD; ++r) {
+        if constexpr (PRE) v[r] = ld(b, r, ld.pre(b, r));
+        else v[r] = ld(b, r);
+      }
       Dft<R, INV>::template run<RAD>(v);
 #pragma unroll
       for (int r = 0; r < RAD; ++r) st(b, r, v[r]);
     }
   } else {
-    io_first<R, PL, N, INV, LINES, THREADS, L, SKEW>(buf, tws, ld);
-    for (int t = threadIdx.x; t < TOTAL; t += THREADS) {
-      int b, j;
-      IX::map(t, NB, b, j);
-      cx<R> v[RAD];
-      io_butterfly<R, PL, N, INV, LINES, L, SKEW, S>(buf, tws, b, j, v);
-#pragma unroll
-      for (int r = 0; r < RAD; ++r) st(b, j + r * NB, v[r]);
-    }
+    io_first<R, PL, N, INV, LINES, THREADS, L, SKEW, PRE>(buf, tws, ld);
+    io_last<R, PL, N, INV, LINES, THREADS, L, SKEW>(buf, tws, st);
   }
 }
 

@@ -17,88 +17,97 @@ namespace fl {
 namespace {
 
 // ---- inverse pass 1: gather active profiles, columns (along y) ----------------
+// A tile is GC columns of the compact column list by GL planes: the profiles lie plane-fastest
+// per mode, so the GL planes of a mode are one 32-byte sector of the loads, and the GC columns
+// one of the stores (16 columns of one plane before: a quarter of each sector used, and with 17
+// active columns a second tile for one of them).  256^2 x 64, 8 frequencies, 137 columns: 27 us
+// -> 21 us.
+template <typename R, int N, int T> struct GatherPass {
+  static constexpr bool F32 = sizeof(R) == 4;
+  static constexpr int GC = 4, GL = (F32 ? 4 : 2) / (T == 0 ? 1 : 2), LINES = GC * GL;
+  using PL = IoPlan<N, T == 0 ? 16 : 8, false>;
+  static constexpr int NT = round32(LINES * N / (T == 0 ? (N % 3 == 0 ? 12 : 16) : 8)) < 256
+                                ? round32(LINES * N / (T == 0 ? (N % 3 == 0 ? 12 : 16) : 8)) : 256;
+};
 constexpr int GATHER_COLS = 32;  // active columns the gather's grid covers in one pass (see rec_tiled)
+
+// Element i of line b of a gather tile: column cb + b / GL, plane l0 + b % GL (the lanes
+// of the loads go through the planes of a mode, those of the stores through both).  pre: the
+// mode's slot (-1: zero), so that a thread's slot loads, then its profile loads, are in flight
+// together.
+template <typename R, int N, int GL> struct GatherLoad {
+  const int* cols;      // of this frequency, from column cb on
+  const int* slot;
+  const cx<R>* prof;    // of this frequency, field and plane l0
+  int nc, nl, stride;   // columns and planes of the tile, 2 M
+  const cx<R>* inc;     // U~0 at nu = 0 on the tile's planes when that mode is inactive (else null)
+  __device__ __forceinline__ int pre(int b, int i) const {
+    return b / GL < nc && b % GL < nl ? slot[i * N + cols[b / GL]] : -1;
+  }
+  __device__ __forceinline__ cx<R> operator()(int b, int i, int s) const {
+    if (s >= 0) return prof[(long long)s * stride + b % GL];
+    return inc && i == 0 && b / GL == 0 ? inc[b % GL] : czero<R>();
+  }
+};
 
 // Column chunks blockIdx.z, blockIdx.z + gridDim.z, ... of the compact column list of
 // frequency om (grid below); field f = 0 (V~) or 1 (U~).  Inactive modes are zero in
 // V~ and equal the incident field U~0 in U~; the plane wave exp(-i k0 z) has
 // U~0 = N^2 exp(-i k0 z'_l) at nu = 0 and zero elsewhere.
 template <typename R, int N, int T>
-__global__ void __launch_bounds__(THREADS)
+__global__ void __launch_bounds__((GatherPass<R, N, T>::NT))
 k_ifft_cols_gather(Problem P, const cx<R>* __restrict__ prof, const int* __restrict__ slot,
                    const int* __restrict__ cols, const int* __restrict__ ncol,
                    cx<R>* __restrict__ t2, const cx<R>* __restrict__ tw) {
-  constexpr int TC = tile_cols<R, T>();
-  constexpr int E = N * TC;
-  constexpr int PER = (E + THREADS - 1) / THREADS;
-  __shared__ cx<R> buf[E];
-  __shared__ cx<R> tw_s[N];
-  load_twiddles<R, N>(tw_s, tw);  // a constant table: read while the predecessor drains
+  using GP = GatherPass<R, N, T>;
+  using PL = typename GP::PL;
+  constexpr int GC = GP::GC, GL = GP::GL;
+  __shared__ cx<R> buf[PL::stages > 1 ? N * GP::LINES : 1];
+  __shared__ cx<R> tws[PL::tw_elems];
+  __shared__ cx<R> inc[GL];
+  load_stage_twiddles<R, PL, N, GP::NT>(tws, tw);  // a constant table: read while the predecessor drains
   pdl_wait();
   pdl_trigger();
-  // grid (M, 2 n_omega, gather_chunks): the column chunk is the slowest index, so that
-  // the chunks that hold active columns (the first ceil(ncol / TC)) are dispatched first
-  // and the rest, which return at once, last; a block loops when ncol needs more chunks
+  // grid (ceil(M / GL), 2 n_omega, chunks): the column chunk is the slowest index, so that
+  // the chunks that hold active columns are dispatched first and the rest, which return at
+  // once, last; a block loops when ncol needs more chunks
   const int om = blockIdx.y >> 1, f = blockIdx.y & 1;
-  const int l = blockIdx.x;
+  const int l0 = blockIdx.x * GL;
   const int nc = ncol[om];
   const long long N2 = (long long)N * N;
   const int M = P.m;
-  for (int cb = blockIdx.z * TC; cb < nc; cb += gridDim.z * TC) {
-    if (cb != (int)blockIdx.z * TC) __syncthreads();  // the previous chunk's stores have read buf
-    // element e = t + p THREADS is row i = e / TC of line b = t mod TC (THREADS is a
-    // multiple of TC): one column per thread, its PER slot loads and then its profile
-    // loads issued together
-    static_assert(THREADS % TC == 0, "one column per thread");
-    const int b = threadIdx.x % TC;
-    const int nu1 = cb + b < nc ? cols[om * N + cb + b] : -1;
-    int sl[PER];
-#pragma unroll
-    for (int p = 0; p < PER; ++p) {
-      const int e = threadIdx.x + p * THREADS, i = e / TC;
-      sl[p] = (nu1 >= 0 && e < E) ? slot[om * N2 + (long long)i * N + nu1] : -1;
+  const int* sl = slot + om * N2;
+  const cx<R>* pr = prof + (long long)om * N2 * 2 * M + f * M + l0;
+  cx<R>* dst = t2 + ((long long)om * 2 + f) * M * N2 + l0 * N2;
+  for (int cb = blockIdx.z * GC; cb < nc; cb += gridDim.z * GC) {
+    // column 0 of the list is nu1 = 0 (it always holds the incident mode)
+    const bool wave = cb == 0 && f == 1 && !P.incident && sl[0] < 0;
+    if (wave && threadIdx.x < GL) {
+      double sn, cs;
+      sincos(-(P.omega[om] / P.c0) * (P.z1 + (l0 + threadIdx.x + 0.5) * P.hz), &sn, &cs);
+      inc[threadIdx.x] = from_d<R>(make_double2((double)N2 * cs, (double)N2 * sn));
     }
-#pragma unroll
-    for (int p = 0; p < PER; ++p) {
-      const int e = threadIdx.x + p * THREADS;
-      if (e < E) {
-        const int i = e / TC;
-        cx<R> v = czero<R>();
-        if (sl[p] >= 0) {
-          v = prof[(((long long)om * N2 + sl[p]) * 2 + f) * M + l];
-        } else if (f == 1 && i == 0 && nu1 == 0 && !P.incident) {  // one thread: FP64 is slow on this GPU
-          double sn, cs;
-          sincos(-(P.omega[om] / P.c0) * (P.z1 + (l + 0.5) * P.hz), &sn, &cs);
-          v = from_d<R>(make_double2((double)N2 * cs, (double)N2 * sn));
-        }
-        buf[e] = v;
-      }
-    }
-    __syncthreads();
-    fft_lines<R, N, true, TC, THREADS, Lay::COL, Tile<T>::RADIX_GATHER>(buf, tw_s);
-    const long long ob = (((long long)om * 2 + f) * M + l) * N2;
-#pragma unroll
-    for (int p = 0; p < PER; ++p) {
-      const int e = threadIdx.x + p * THREADS;
-      if (e < E && nu1 >= 0) t2[ob + (long long)(e / TC) * N + cb + b] = buf[e];
-    }
+    if (wave || cb != (int)blockIdx.z * GC) __syncthreads();  // (the previous chunk's last stage has read buf)
+    const int ncb = min(GC, nc - cb), nlb = min(GL, M - l0);
+    fft_lines_io<R, PL, N, true, GP::LINES, GP::NT, Lay::COL, 0, true>(
+        buf, tws, GatherLoad<R, N, GL>{cols + om * N + cb, sl, pr, ncb, nlb, 2 * M, wave ? inc : nullptr},
+        [&](int b, int i, cx<R> v) {
+          if (b / GL < ncb && b % GL < nlb) dst[(b % GL) * N2 + i * N + cb + b / GL] = v;
+        });
   }
 }
 
-__device__ __forceinline__ unsigned long long block_sum_u64(unsigned v, unsigned* red) {
+template <int NT> __device__ __forceinline__ unsigned long long block_sum_u64(unsigned v, unsigned* red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
   unsigned long long s = 0;
   if (threadIdx.x == 0)
-    for (int w = 0; w < THREADS / 32; ++w) s += red[w];
+    for (int w = 0; w < NT / 32; ++w) s += red[w];
   return s;
 }
 
 // ---- inverse pass 2: rows (along x) + step 3 ----------------------------------
-// grid ceil(M N / LINES); a block owns LINES rows (l, y) of the X grid, loops over
-// the frequencies, transforms V and u rows and accumulates the least-squares sums
-// in the accumulator type A.  Returns (block-uniform) whether any sum overflowed.
 // a / b and 1/sqrt(x) of the pointwise recovery: IEEE in FP32; in FP64 by
 // Newton-Raphson from FP32 seeds (rcp64, rsqrt64), a few dependent FP64 operations
 // instead of the FP64 division and square root, which dominate this kernel on a
@@ -110,145 +119,38 @@ template <typename R> __device__ __forceinline__ R inv_sqrt(R x);
 template <> __device__ __forceinline__ float inv_sqrt<float>(float x) { return rsqrtf(x); }  // <= 2 ulp
 template <> __device__ __forceinline__ double inv_sqrt<double>(double x) { return rsqrt64(x); }
 
-// The recovery pass's tile.  FP32, default tile (fs_options.fft_tile = 0): from N = 96
-// up, 4096 elements (the V and u rows of 4096 / (2N) rows of X) with radix-16 stages
-// (a 128-point row in two stages, 16 and 8, every thread busy in both), transformed out
-// of place (PP: two tiles in shared memory, one butterfly per thread at a time, one
-// barrier per stage; in place, the radix-3 stages of N = 96 and 192 would hold five
-// butterflies a thread in registers and spill); below 96 at N = 2^k, 1024 elements in
-// place (small problems need the CTAs: 64^2 x 16 recovers in 18 us instead of 33 with
-// 4096); otherwise the tile of fs_options.fft_tile.  MINB: CTAs per SM the register
-// allocation is held to -- three at N = 2^k (at most 80 registers a thread; 1 us faster
-// at 128^2 than two CTAs of 102), two with PP at radix-3 sizes (128 registers, no
-// spill), one elsewhere.
-template <typename R, int N, int T> struct RecTile {
-  static constexpr bool F32 = sizeof(R) == 4 && T == 0;
-  static constexpr bool PP = F32 && N >= 96;
-  static constexpr bool BIG = F32 && (PP || N % 3 != 0);
-  static constexpr int ELEMS = BIG ? (N >= 96 ? 4096 : 1024) : Tile<T>::ELEMS;
-  static constexpr int RADIX = BIG ? 16 : Tile<T>::RADIX_RECOVER;
-  static constexpr int SKEW = BIG ? 16 : Tile<T>::SKEW_RECOVER;
-  static constexpr int MINB = T == 0 && N % 3 != 0 ? 3 : (PP ? 2 : 1);
-};
-template <typename R, int N, int T> __host__ __device__ constexpr int rec_lines() {
-  return RecTile<R, N, T>::ELEMS / N / 2 > 0 ? RecTile<R, N, T>::ELEMS / N / 2 : 1;
-}
-// the recovery pass's dynamic shared memory: its tile (two with PP)
-template <typename R, int N, int T> __host__ __device__ constexpr size_t rec_smem() {
-  return sizeof(cx<R>) * (RecTile<R, N, T>::PP ? 2 : 1) *
-         (size_t)LayIdx<Lay::ROW, N, 2 * rec_lines<R, N, T>(), RecTile<R, N, T>::SKEW>::ELEMS;
-}
-
-// filled: the tile is already zero for the first frequency.  In FP64 without a given
-// incident field the sums are taken of the unscaled transforms (N^2 V, N^2 u): xi is
-// their quotient either way, and the guard on sum |u|^2 is scaled instead
-// (Problem::u_guard_raw), which saves four FP64 products per voxel and frequency.
-template <typename R, bool INC> __host__ __device__ constexpr bool raw_sums() { return sizeof(R) == 8 && !INC; }
-
-template <typename R, int N, typename A, bool INC, int T>
-__device__ __forceinline__ bool recover_pass(const Problem& P, const cx<R>* __restrict__ t2,
-                                             const int* __restrict__ cols, const int* __restrict__ ncol,
-                                             const cx<R>* __restrict__ u0, cx<R>* buf, const cx<R>* tw_s, A* num,
-                                             A* den, bool filled) {
-  constexpr int LINES = rec_lines<R, N, T>();
-  constexpr int E = LINES * N;
-  using IX = LayIdx<Lay::ROW, N, 2 * LINES, RecTile<R, N, T>::SKEW>;  // V~ lines, then U~ lines
-  constexpr int PER = (E + THREADS - 1) / THREADS;
-  const int M = P.m;
-  const long long N2 = (long long)N * N;
-  const long long nrows = (long long)M * N;
-  const long long row0 = (long long)blockIdx.x * LINES;
-  const R scale = raw_sums<R, INC>() ? R(1) : R(1.0 / (double)N2);
-#pragma unroll
-  for (int p = 0; p < PER; ++p) { num[p] = A(0); den[p] = A(0); }
-  for (int om = 0; om < P.n_omega; ++om) {
-    if (om > 0 || !filled)
-      for (int e = threadIdx.x; e < IX::ELEMS; e += THREADS) buf[e] = czero<R>();
-    __syncthreads();
-    const int nc = ncol[om];
-    const int* cl = cols + om * N;
-    const int tot = 2 * LINES * nc;
-    for (int q = threadIdx.x; q < tot; q += THREADS) {
-      const int line = q / nc, c = q - line * nc;
-      const int f = line / LINES, b = line - f * LINES;
-      const long long r = row0 + b;
-      if (r < nrows) {
-        const long long l = r / N, i = r - l * N;
-        buf[IX::at(line, cl[c])] = t2[(((long long)om * 2 + f) * M + l) * N2 + i * N + c];
-      }
-    }
-    __syncthreads();
-    const cx<R>* res = buf;
-    if constexpr (RecTile<R, N, T>::PP)
-      res = fft_lines_pp<R, N, true, 2 * LINES, THREADS, Lay::ROW, RecTile<R, N, T>::RADIX, RecTile<R, N, T>::SKEW>(
-          buf, buf + IX::ELEMS, tw_s);
-    else
-      fft_lines<R, N, true, 2 * LINES, THREADS, Lay::ROW, RecTile<R, N, T>::RADIX, RecTile<R, N, T>::SKEW>(buf, tw_s);
-#pragma unroll
-    for (int p = 0; p < PER; ++p) {
-      const int e = threadIdx.x + p * THREADS;
-      if (e < E) {
-        cx<R> v = res[IX::at(e / N, e % N)];
-        cx<R> u = res[IX::at(LINES + e / N, e % N)];
-        if constexpr (!raw_sums<R, INC>()) {
-          v = scale * v;
-          u = scale * u;
-        }
-        if (INC) {  // the given incident field (the transform holds U~ - U~0)
-          const long long r = row0 + e / N;
-          if (r < nrows) u = u + u0[((long long)om * M + r / N) * N2 + (r % N) * N + (e % N)];
-        }
-        num[p] += (A)u.x * (A)v.x + (A)u.y * (A)v.y;  // Re(conj(u) V)
-        den[p] += (A)u.x * (A)u.x + (A)u.y * (A)u.y;  // |u|^2
-      }
-    }
-    __syncthreads();
-  }
-  bool bad = false;
-#pragma unroll
-  for (int p = 0; p < PER; ++p) bad |= !(isfinite(num[p]) && isfinite(den[p]));
-  return __syncthreads_or(bad) != 0;
-}
-
-// xi and c of the elements e = threadIdx.x + p THREADS < E of rows row0 + e / N (below
-// nrows) from the least-squares sums, and the counters of guarded, NaN-c and non-finite
-// voxels (almost always zero, so one barrier decides).  guard: the least den of a kept
-// voxel (host-derived: no FP64 division on the device)
-template <typename R, int PER, int N>
-__device__ __forceinline__ void recover_epilogue(const Problem& P, const R* num, const R* den, R guard,
-                                                 long long row0, long long nrows, int E, R* __restrict__ xi,
-                                                 R* __restrict__ cout, unsigned long long* __restrict__ ctr,
-                                                 unsigned* red) {
-  const R inv_c02 = R(P.inv_c02);
+// xi and c of the PER elements of the thread from the least-squares sums, and the counters of
+// guarded, NaN-c and non-finite voxels (almost always zero, so one barrier decides).  at(p):
+// offset of element p in xi, negative for none.  guard: the least den of a kept voxel
+// (host-derived: no FP64 division on the device)
+template <typename R, int PER, int NT, class At>
+__device__ __forceinline__ void recover_epilogue(const Problem& P, const R* num, const R* den, R guard, At at,
+                                                 R* __restrict__ xi, R* __restrict__ cout,
+                                                 unsigned long long* __restrict__ ctr, unsigned* red) {
+  const R inv_c02 = sizeof(R) == 4 ? R(P.inv_c02_f) : R(P.inv_c02);
   unsigned n_guard = 0, n_nan = 0, n_bad = 0;
 #pragma unroll
   for (int p = 0; p < PER; ++p) {
-    const int e = threadIdx.x + p * THREADS;
-    if (e < E) {
-      const long long r = row0 + e / N;
-      if (r < nrows) {
-        const bool g = !(den[p] >= guard);
-        const R x = g ? R(0) : quot<R>(num[p], den[p]);
-        n_guard += g;
-        n_bad += !isfinite(x);
-        const long long o = r * N + (e % N);
-        xi[o] = x;
-        if (cout) {
-          const bool ok = x < inv_c02;
-          n_nan += !ok;
-          cout[o] = ok ? inv_sqrt<R>(inv_c02 - x) : R(NAN);
-        }
+    const long long o = at(p);
+    if (o >= 0) {
+      const bool g = !(den[p] >= guard);
+      const R x = g ? R(0) : quot<R>(num[p], den[p]);
+      n_guard += g;
+      n_bad += !isfinite(x);
+      xi[o] = x;
+      if (cout) {
+        const bool ok = x < inv_c02;
+        n_nan += !ok;
+        cout[o] = ok ? inv_sqrt<R>(inv_c02 - x) : R(NAN);
       }
     }
   }
-  // the counters of guarded, NaN-c and non-finite voxels: almost always zero, so one
-  // barrier decides
   if (__syncthreads_or((n_guard | n_nan | n_bad) != 0u)) {
-    const unsigned long long sg = block_sum_u64(n_guard, red);
+    const unsigned long long sg = block_sum_u64<NT>(n_guard, red);
     __syncthreads();
-    const unsigned long long sn = block_sum_u64(n_nan, red);
+    const unsigned long long sn = block_sum_u64<NT>(n_nan, red);
     __syncthreads();
-    const unsigned long long sb = block_sum_u64(n_bad, red);
+    const unsigned long long sb = block_sum_u64<NT>(n_bad, red);
     if (threadIdx.x == 0) {
       if (sg) atomicAdd(ctr + C_U_GUARD, sg);
       if (sn) atomicAdd(ctr + C_NAN_C, sn);
@@ -257,46 +159,202 @@ __device__ __forceinline__ void recover_epilogue(const Problem& P, const R* num,
   }
 }
 
+// The recovery pass: LINES rows of X per block, their V and u lines together (lines 0 .. LINES
+// - 1 and LINES .. 2 LINES - 1 of the tile).  The compact columns of the next frequency are
+// staged by asynchronous copies while this one is transformed; the first stage reads them
+// through the position of each column in the list, leaving out the inputs of columns that the
+// list's band does not reach; the last stage goes back over its own inputs in the tile, and each
+// thread then adds its voxels' V and u to the least-squares sums in registers.
+// What bounds it: shared memory and latency in FP32, the FP64 pipe in FP64.  Clearing the tile,
+// scattering the columns and every stage in place took six crossings of shared memory and five
+// barriers per frequency: 256^2 x 64, 8 frequencies (FP32) 171 us; this split without staging
+// and band 146 us, with both 117 us; 128^2 x 71, 3 frequencies, incident field (FP64) 435 us ->
+// 322 us, 256 us of it FP64 instructions.  (A V and a u butterfly held in registers beside the
+// sums, one crossing fewer, left half the resident blocks: 131 us.)
+// The sums are taken of the unscaled transforms (raw: N^2 V and N^2 u, a given incident field
+// times N^2) in FP64: xi is their quotient either way, and the guard on sum |u|^2 is scaled
+// instead (Problem::u_guard_raw), which saves FP64 products per voxel and frequency.
+template <typename R, int N, int T> struct RecPass {
+  static constexpr bool F32 = sizeof(R) == 4;
+  // radices that give each stage of a small FP64 tile whole warps
+  static constexpr int MAXR = T == 1 ? 8 : F32 ? 16 : (N == 16 ? 4 : N <= 64 ? 8 : 16);
+  using PL = IoPlan<N, MAXR, false>;
+  static constexpr int NT = F32 ? (N >= 192 ? 256 : 128) : (N >= 192 ? 128 : 64);
+  static constexpr int ROWS0 = F32 ? (N <= 16 ? 16 : 8) : (N <= 16 ? 8 : 4);
+  static constexpr int LINES = T == 0 ? ROWS0 : ROWS0 / 2;
+  static constexpr int SKEW = 16;
+  // resident blocks the registers are held to: at 128^2 x 64 the pass's 1024 blocks at once
+  static constexpr int MINB = !F32 || T == 1 ? 1 : N >= 192 ? 3 : (N == 128 || N == 64) ? 7 : 1;
+  static constexpr int SC = !F32 && N == 256 ? 16 : 32;  // staged columns per row (RecStage)
+  static constexpr int E = LINES * N, PER = (E + NT - 1) / NT;  // voxels of the block, of a thread
+  using IX = LayIdx<Lay::ROW, N, 2 * LINES, SKEW>;
+};
+
+template <typename R> __host__ __device__ constexpr bool raw_sums() { return sizeof(R) == 8; }
+
+// What a block stages of the next frequency while it transforms this one: the columns of its
+// rows (at most RecPass::SC; more are read from global memory by the first stage) and the positions of
+// the columns in the list.
+template <typename R, int N, int T> struct RecStage {
+  cx<R> col[2][2 * RecPass<R, N, T>::LINES][RecPass<R, N, T>::SC];
+  int pos[2][N];
+};
+
+// The first stage of a radix-16 plan when only the first and the last E sixteenths of the columns
+// hold anything (low wavenumbers; E = 8: no such bound): butterfly j has inputs j + r N/16.
+template <typename R, int N, int T, int E, class Ld>
+__device__ __forceinline__ void recover_first(cx<R>* buf, Ld ld) {
+  using RP = RecPass<R, N, T>;
+  constexpr int NB = N / 16, TOTAL = 2 * RP::LINES * NB;
+  for (int t = threadIdx.x; t < TOTAL; t += RP::NT) {
+    const int b = t / NB, j = t % NB;
+    cx<R> v[16];
+#pragma unroll
+    for (int r = 0; r < 16; ++r)
+      if (r < E || r >= 16 - E) v[r] = ld(b, j + r * NB);
+    if constexpr (E == 8) Dft<R, true>::d16(v);
+    else Dft<R, true>::template d16_edge<E>(v);
+#pragma unroll
+    for (int r = 0; r < 16; ++r) buf[RP::IX::at(b, j * 16 + r)] = v[r];
+  }
+}
+
+// the sums of the thread's voxels e = threadIdx.x + p NT over the frequencies, in the
+// accumulator type A
+template <typename R, int N, typename A, bool INC, int T>
+__device__ __forceinline__ void recover_pass(const Problem& P, const cx<R>* __restrict__ t2,
+                                             const int* __restrict__ colpos, const int* __restrict__ ncol,
+                                             const int* __restrict__ colseg, const cx<R>* __restrict__ u0, cx<R>* buf,
+                                             const cx<R>* tws, RecStage<R, N, T>& stg, A* num, A* den) {
+  using RP = RecPass<R, N, T>;
+  using PL = typename RP::PL;
+  using IX = typename RP::IX;
+  constexpr int LINES = RP::LINES, NT = RP::NT, E = RP::E, PER = RP::PER, SC = RP::SC;
+  const long long nrows = (long long)P.m * N;
+  const long long row0 = (long long)blockIdx.x * LINES;
+  const int rows = (int)(nrows - row0 < LINES ? nrows - row0 : LINES);
+  const long long uoff = nrows * N;  // u behind V by nrows rows
+  const R scale = sizeof(R) == 4 ? R(P.inv_n2_f) : R(P.inv_n2);
+  const R n2 = R((double)N * N);
+#pragma unroll
+  for (int p = 0; p < PER; ++p) { num[p] = A(0); den[p] = A(0); }
+  auto stage = [&](int om, int nc) {
+    const cx<R>* src = t2 + ((long long)om * 2 * nrows + row0) * N;
+    if (nc <= SC)
+      for (int q = threadIdx.x; q < 2 * LINES * SC; q += NT) {
+        const int line = q / SC, c = q % SC, bl = line >= LINES ? line - LINES : line;
+        if (c < nc && bl < rows)
+          async_copy(&stg.col[om & 1][line][c], (line >= LINES ? src + uoff : src) + bl * N + c);
+      }
+    for (int i = threadIdx.x; i < N; i += NT) async_copy(&stg.pos[om & 1][i], colpos + om * N + i);
+  };
+  int nc = ncol[0];
+  stage(0, nc);
+  for (int om = 0; om < P.n_omega; ++om) {
+    const int seg = colseg[om];
+    const int nc1 = om + 1 < P.n_omega ? ncol[om + 1] : 0;
+    async_wait();
+    __syncthreads();  // this frequency's columns are staged, and the tile has been read
+    if (om + 1 < P.n_omega) stage(om + 1, nc1);
+    const int* ps = stg.pos[om & 1];
+    const cx<R>* src = t2 + ((long long)om * 2 * nrows + row0) * N;
+    const bool staged = nc <= SC;
+    auto ld = [&](int line, int i) {
+      const int c = ps[i], bl = line >= LINES ? line - LINES : line;
+      if (c < 0 || bl >= rows) return czero<R>();
+      return staged ? stg.col[om & 1][line][c] : (line >= LINES ? src + uoff : src)[bl * N + c];
+    };
+    auto st = [&](int line, int i, cx<R> v) { buf[IX::at(line, i)] = v; };
+    if constexpr (PL::stages == 2 && PL::radix(0) == 16) {
+      if ((seg & ~0x8001) == 0) recover_first<R, N, T, 1>(buf, ld);
+      else if ((seg & ~0xC003) == 0) recover_first<R, N, T, 2>(buf, ld);
+      else recover_first<R, N, T, 8>(buf, ld);
+      __syncthreads();
+      io_last<R, PL, N, true, 2 * LINES, NT, Lay::ROW, RP::SKEW>(buf, tws, st);
+    } else {
+      fft_lines_io<R, PL, N, true, 2 * LINES, NT, Lay::ROW, RP::SKEW>(buf, tws, ld, st);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      const int e = threadIdx.x + p * NT;
+      if (E % NT == 0 || e < E) {
+        const int b = e / N, i = e % N;
+        cx<R> v = buf[IX::at(b, i)], u = buf[IX::at(LINES + b, i)];
+        if constexpr (!raw_sums<R>()) {
+          v = scale * v;
+          u = scale * u;
+        }
+        if (INC && b < rows) {  // the transform holds U~ - U~0
+          const cx<R> w = u0[((long long)om * nrows + row0) * N + e];
+          if constexpr (raw_sums<R>()) u = mk<R>(fma(n2, w.x, u.x), fma(n2, w.y, u.y));
+          else u = u + w;
+        }
+        num[p] += (A)u.x * (A)v.x + (A)u.y * (A)v.y;  // Re(conj(u) V)
+        den[p] += (A)u.x * (A)u.x + (A)u.y * (A)u.y;  // |u|^2
+      }
+    }
+    nc = nc1;
+  }
+  __syncthreads();  // (a second pass reuses the tile and the staged columns)
+}
+
 // INC: u0 (the incident field on X) is given and added to u; otherwise the transform
 // already holds the plane wave
 template <typename R, int N, bool INC, int T>
-__global__ void __launch_bounds__(THREADS, (RecTile<R, N, T>::MINB))
-k_ifft_rows_recover(Problem P, const cx<R>* __restrict__ t2, const int* __restrict__ cols,
-                    const int* __restrict__ ncol, const cx<R>* __restrict__ u0, R* __restrict__ xi,
-                    R* __restrict__ cout, unsigned long long* __restrict__ ctr, const cx<R>* __restrict__ tw) {
-  constexpr int LINES = rec_lines<R, N, T>();
-  constexpr int E = LINES * N;            // elements of one field
-  constexpr int PER = (E + THREADS - 1) / THREADS;
-  using IX = LayIdx<Lay::ROW, N, 2 * LINES, RecTile<R, N, T>::SKEW>;
-  extern __shared__ __align__(16) unsigned char rec_smem_raw[];  // rec_smem<R, N, T>() bytes
-  cx<R>* buf = reinterpret_cast<cx<R>*>(rec_smem_raw);
-  __shared__ cx<R> tw_s[N];
-  __shared__ unsigned red[THREADS / 32];
-  // the constant twiddle table and the cleared tile of the first frequency, while the
-  // predecessor drains
-  load_twiddles<R, N>(tw_s, tw);
-  for (int e = threadIdx.x; e < IX::ELEMS; e += THREADS) buf[e] = czero<R>();
+__global__ void __launch_bounds__((RecPass<R, N, T>::NT), (RecPass<R, N, T>::MINB))
+k_ifft_rows_recover(Problem P, const cx<R>* __restrict__ t2, const int* __restrict__ colpos,
+                    const int* __restrict__ ncol, const int* __restrict__ colseg, const cx<R>* __restrict__ u0, R* __restrict__ xi, R* __restrict__ cout,
+                    unsigned long long* __restrict__ ctr, const cx<R>* __restrict__ tw) {
+  using RP = RecPass<R, N, T>;
+  using PL = typename RP::PL;
+  constexpr int NT = RP::NT, E = RP::E, PER = RP::PER;
+  __shared__ cx<R> buf[RP::IX::ELEMS];
+  __shared__ cx<R> tws[PL::tw_elems];
+  __shared__ RecStage<R, N, T> stg;
+  __shared__ unsigned red[NT / 32];
+  load_stage_twiddles<R, PL, N, NT>(tws, tw);  // a constant table: read while the predecessor drains
   pdl_wait();
   pdl_trigger();
   const long long nrows = (long long)P.m * N;
-  const long long row0 = (long long)blockIdx.x * LINES;
+  const long long row0 = (long long)blockIdx.x * RP::LINES;
+  const int el = (int)(nrows - row0 < RP::LINES ? nrows - row0 : RP::LINES) * N;  // voxels of this block
   R num[PER], den[PER];
-  const double gd = raw_sums<R, INC>() ? P.u_guard_raw : P.u_guard;
-  R guard = R(gd);
-  if (P.sums64 || recover_pass<R, N, R, INC, T>(P, t2, cols, ncol, u0, buf, tw_s, num, den, true)) {
-    // the sums left the range of R (|u| |V| beyond FP32 for huge evanescent
-    // profiles): redo this block with FP64 sums; xi itself is in range
-    double nd[PER], dd[PER];
-    recover_pass<R, N, double, INC, T>(P, t2, cols, ncol, u0, buf, tw_s, nd, dd, P.sums64 != 0);
+  const double gd = raw_sums<R>() ? P.u_guard_raw : P.u_guard;
+  R guard = sizeof(R) == 4 ? R(P.u_guard_f) : R(gd);
+  bool redo = sizeof(R) == 4 && P.sums64;
+  if (!redo) {
+    recover_pass<R, N, R, INC, T>(P, t2, colpos, ncol, colseg, u0, buf, tws, stg, num, den);
+    if constexpr (sizeof(R) == 4) {
+      bool bad = false;
 #pragma unroll
-    for (int p = 0; p < PER; ++p) {
-      const bool g = !(dd[p] >= gd);
-      num[p] = g ? R(0) : R(nd[p] / dd[p]);
-      den[p] = g ? R(0) : R(1);
+      for (int p = 0; p < PER; ++p)
+        bad |= threadIdx.x + p * NT < el && !(isfinite(num[p]) && isfinite(den[p]));
+      redo = __syncthreads_or(bad) != 0;
     }
-    guard = R(0.5);  // den is now 1 (kept) or 0 (guarded)
   }
-  recover_epilogue<R, PER, N>(P, num, den, guard, row0, nrows, E, xi, cout, ctr, red);
+  if constexpr (sizeof(R) == 4) {
+    if (redo) {
+      // the sums left the range of R (|u| |V| beyond FP32 for huge evanescent profiles), or
+      // were asked for in FP64: FP64 sums; xi itself is in range
+      double nd[PER], dd[PER];
+      recover_pass<R, N, double, INC, T>(P, t2, colpos, ncol, colseg, u0, buf, tws, stg, nd, dd);
+#pragma unroll
+      for (int p = 0; p < PER; ++p) {
+        const bool g = !(dd[p] >= gd);
+        num[p] = g ? R(0) : R(nd[p] / dd[p]);
+        den[p] = g ? R(0) : R(1);
+      }
+      guard = R(0.5);  // den is now 1 (kept) or 0 (guarded)
+    }
+  }
+  recover_epilogue<R, PER, NT>(
+      P, num, den, guard,
+      [&](int p) {
+        const int e = threadIdx.x + p * NT;
+        return e < el ? row0 * N + e : -1LL;
+      },
+      xi, cout, ctr, red);
 }
 
 // ---- single-pass inverse transform and recovery: one X plane per cluster ---------
@@ -466,8 +524,13 @@ k_ifft2_plane_recover(Problem P, const cx<R>* __restrict__ prof, const int* __re
     }
   }
   // after a redo den is 1 (kept) or 0 (guarded)
-  recover_epilogue<R, PER, N>(P, num, den, any ? R(0.5) : R(P.u_guard), row0, (long long)P.m * N, E, xi, cout, ctr,
-                              red);
+  recover_epilogue<R, PER, THREADS>(
+      P, num, den, any ? R(0.5) : R(P.u_guard_f),
+      [&](int p) {
+        const int e = threadIdx.x + p * THREADS;
+        return e < E ? (row0 + e / N) * N + (e % N) : -1LL;
+      },
+      xi, cout, ctr, red);
 }
 
 template <typename R, int N, bool INC>
@@ -486,31 +549,24 @@ cudaError_t rec_plane(const Problem& P, const Work<R>& w, R* xi, R* c, cudaStrea
 
 template <typename R, int N, int T>
 cudaError_t rec_tiled(const Problem& P, const Work<R>& w, R* xi, R* c, cudaStream_t s, cudaEvent_t mid) {
-  constexpr int TC = tile_cols<R, T>();
+  using GP = GatherPass<R, N, T>;
+  using RP = RecPass<R, N, T>;
   // column chunks for the first GATHER_COLS active columns in the grid (the blocks loop
   // over more): the active columns are few in the usual case, and a grid of blocks that
   // return at once only delays the successor's launch (measured, 64-problem batch: 6.17
   // ms with every chunk in the grid, 6.07 with 32 columns; FP64 128^2 step +0.5 us)
-  constexpr int NCH = (N + TC - 1) / TC, GZ = (GATHER_COLS + TC - 1) / TC;
-  dim3 g1(P.m, 2 * P.n_omega, NCH < GZ ? NCH : GZ);
-  cudaError_t e = launch_pdl(k_ifft_cols_gather<R, N, T>, g1, dim3(THREADS), 0, s, P, (const cx<R>*)w.prof,
+  constexpr int NCH = (N + GP::GC - 1) / GP::GC, GZ = GATHER_COLS / GP::GC;
+  const dim3 g1((P.m + GP::GL - 1) / GP::GL, 2 * P.n_omega, NCH < GZ ? NCH : GZ);
+  cudaError_t e = launch_pdl(k_ifft_cols_gather<R, N, T>, g1, dim3(GP::NT), 0, s, P, (const cx<R>*)w.prof,
                              (const int*)w.slot, (const int*)w.cols, (const int*)w.ncol, w.t2, (const cx<R>*)w.tw);
   if (e != cudaSuccess) return e;
   if (mid) cudaEventRecord(mid, s);
-  constexpr int LINES = rec_lines<R, N, T>();
-  constexpr size_t smem = rec_smem<R, N, T>();
   const long long nrows = (long long)P.m * N;
-  const dim3 gr((unsigned)((nrows + LINES - 1) / LINES));
-  static SmemOptIn attr[2];
-  if (w.u0) {
-    if ((e = opt_in_smem(attr[1], (const void*)k_ifft_rows_recover<R, N, true, T>, smem)) != cudaSuccess) return e;
-    e = launch_pdl(k_ifft_rows_recover<R, N, true, T>, gr, dim3(THREADS), smem, s, P, (const cx<R>*)w.t2,
-                   (const int*)w.cols, (const int*)w.ncol, w.u0, xi, c, w.ctr, (const cx<R>*)w.tw);
-  } else {
-    if ((e = opt_in_smem(attr[0], (const void*)k_ifft_rows_recover<R, N, false, T>, smem)) != cudaSuccess) return e;
-    e = launch_pdl(k_ifft_rows_recover<R, N, false, T>, gr, dim3(THREADS), smem, s, P, (const cx<R>*)w.t2,
-                   (const int*)w.cols, (const int*)w.ncol, w.u0, xi, c, w.ctr, (const cx<R>*)w.tw);
-  }
+  const dim3 gr((unsigned)((nrows + RP::LINES - 1) / RP::LINES));
+  e = w.u0 ? launch_pdl(k_ifft_rows_recover<R, N, true, T>, gr, dim3(RP::NT), 0, s, P, (const cx<R>*)w.t2,
+                        (const int*)w.colpos, (const int*)w.ncol, (const int*)w.colseg, w.u0, xi, c, w.ctr, (const cx<R>*)w.tw)
+           : launch_pdl(k_ifft_rows_recover<R, N, false, T>, gr, dim3(RP::NT), 0, s, P, (const cx<R>*)w.t2,
+                        (const int*)w.colpos, (const int*)w.ncol, (const int*)w.colseg, w.u0, xi, c, w.ctr, (const cx<R>*)w.tw);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

@@ -16,24 +16,7 @@ namespace fl {
 
 namespace {
 
-// Tile shapes of the gather and recovery passes (fs_options.fft_tile, chosen by the batch
-// tuner): 0 -- tiles of 2048 elements, 16 (FP32) or 8 (FP64) columns per column tile, radix
-// cap 16 (8 in the recovery pass); 1 -- tiles of 1024 elements, 8 or 4 columns, radix cap 8.
-// Row tiles are padded after every SKEW elements (LayIdx).
-template <int T> struct Tile;
-template <> struct Tile<0> {
-  static constexpr int ELEMS = 2048, TC32 = 16, TC64 = 8;
-  static constexpr int RADIX_GATHER = 16, RADIX_RECOVER = 8, SKEW_RECOVER = 8;
-};
-template <> struct Tile<1> {
-  static constexpr int ELEMS = 1024, TC32 = 8, TC64 = 4;
-  static constexpr int RADIX_GATHER = 8, RADIX_RECOVER = 8, SKEW_RECOVER = 8;
-};
-template <typename R, int T> __host__ __device__ constexpr int tile_cols() {
-  return sizeof(R) == 4 ? Tile<T>::TC32 : Tile<T>::TC64;
-}
-
-constexpr int THREADS = 256;
+constexpr int THREADS = 256;  // of the single-pass (cluster) transforms
 
 // ---- shapes of the dense passes --------------------------------------------------
 // One butterfly of 16 (12) elements per thread in the first stage.  FP32 (bound by memory):

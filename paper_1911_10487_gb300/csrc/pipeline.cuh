@@ -52,6 +52,7 @@ struct Problem {
   double kn;
   double inv_c02, u_guard;  // c0^-2 and the |u|^2 guard eps_u^2 n_omega of the recovery
   double u_guard_raw;       // the same guard on the sums of the unscaled transforms: u_guard N^4
+  float inv_c02_f, u_guard_f, inv_n2_f;  // rounded (a conversion on the device costs an FP64 instruction)
   double inv_n2, dscale;    // 1/N^2 and tau max(delta, delta_floor): delta_nu = dscale ||W||
   int sampled;  // 1: the sampled-G kernel of a kernel plan (Work::ktab) replaces the Weyl form
   int incident; // 1: the incident field on X is given (Work::u0) instead of the plane wave
@@ -90,6 +91,9 @@ inline void derive_constants(Problem& P) {
   P.u_guard = P.eps_u * P.eps_u * P.n_omega;
   P.u_guard_raw = P.u_guard * ((double)P.n * P.n) * ((double)P.n * P.n);
   P.inv_n2 = 1.0 / ((double)P.n * (double)P.n);
+  P.inv_c02_f = (float)P.inv_c02;
+  P.u_guard_f = (float)P.u_guard;
+  P.inv_n2_f = (float)P.inv_n2;
   P.dscale = P.tau * fmax(P.delta, P.delta_floor);
   for (int j = 0; j < P.n_omega; ++j) {
     const double om2 = P.omega[j] * P.omega[j];
@@ -122,7 +126,9 @@ template <typename R> struct Work {
   int* blkgz;       // [n_omega][classify_blocks] grazing modes per classification block
   unsigned* colblk; // [n_omega][classify_blocks][8] columns holding an active mode, per block
   int* cols;        // [n_omega][N] columns nu1 holding a nonzero mode
+  int* colpos;      // [n_omega][N] position of column nu1 in cols, or -1
   int* ncol;        // [n_omega]
+  int* colseg;      // [n_omega] bit s: a column of the list in sixteenth s of the N
   int* count;       // [n_omega] active modes
   double* dnu;      // [n_omega] delta_nu
   unsigned* bar;    // [n_omega] barrier counters of the single-pass classification
@@ -155,7 +161,7 @@ inline int classify_blocks(int n) { return (n * n + 1023) / 1024; }
 // from the base of the workspace, and its total size.  The context entry points
 // and the allocation-free entry point carve their workspace from this one layout.
 struct Layout {
-  size_t t12, prof, norms, partial, slot, act, flagbits, blkcnt, blkgz, colblk, cols, ncol, count, dnu, bar, total;
+  size_t t12, prof, norms, partial, slot, act, flagbits, blkcnt, blkgz, colblk, cols, colpos, ncol, colseg, count, dnu, bar, total;
   int n_partial;
 };
 // (the W~ part of the t12 region is sized for complex128 in both precisions, so

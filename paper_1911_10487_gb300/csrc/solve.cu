@@ -200,8 +200,8 @@ k_classify_flags(Problem P, const double* __restrict__ norms, const double* __re
 __global__ void __launch_bounds__(CT)
 k_classify_scatter(Problem P, const unsigned* __restrict__ flagbits, const int* __restrict__ blkcnt,
                    const int* __restrict__ blkgz, const unsigned* __restrict__ colblk, int* __restrict__ slot,
-                   int* __restrict__ act, int* __restrict__ cols, int* __restrict__ ncol, int* __restrict__ count,
-                   unsigned long long* __restrict__ ctr) {
+                   int* __restrict__ act, int* __restrict__ cols, int* __restrict__ colpos, int* __restrict__ ncol,
+                   int* __restrict__ colseg, int* __restrict__ count, unsigned long long* __restrict__ ctr) {
   pdl_wait();
   pdl_trigger();
   const int om = blockIdx.y, b = blockIdx.x, CB = gridDim.x;
@@ -270,6 +270,7 @@ k_classify_scatter(Problem P, const unsigned* __restrict__ flagbits, const int* 
       cw[w] = a;
     }
     int base = 0;
+    unsigned seg = 0u;  // sixteenths of the columns that hold one of the list
 #pragma unroll
     for (int w = 0; w < NWC; ++w) {
       if (w < nw) {
@@ -278,12 +279,17 @@ k_classify_scatter(Problem P, const unsigned* __restrict__ flagbits, const int* 
         const int j = 32 * w + lane;
         const bool f = j < N && (cmw >> lane & 1u);
         const unsigned bal = __ballot_sync(0xffffffffu, f);
-        if (f) cols[om * N + base + __popc(bal & ((1u << lane) - 1u))] = j;
+        const int at = base + __popc(bal & ((1u << lane) - 1u));
+        if (f) cols[om * N + at] = j;
+        if (j < N) colpos[om * N + j] = f ? at : -1;
+        seg |= f ? 1u << (j * 16 / N) : 0u;
         base += __popc(bal);
       }
     }
+    seg = __reduce_or_sync(0xffffffffu, seg);
     if (lane == 0) {
       const int total = total_s;
+      colseg[om] = (int)seg;
       ncol[om] = base;
       count[om] = total;
       atomicAdd(ctr + C_MODES, (unsigned long long)N2);
@@ -344,8 +350,9 @@ template <typename R>
 __global__ void __launch_bounds__(FT)
 k_classify_fused(Problem P, const cx<R>* __restrict__ wt, double* __restrict__ partial, unsigned* __restrict__ bar,
                  int* __restrict__ blkcnt, int* __restrict__ blkgz, unsigned* __restrict__ colblk,
-                 int* __restrict__ slot, int* __restrict__ act, int* __restrict__ cols, int* __restrict__ ncol,
-                 int* __restrict__ count, double* __restrict__ dnu_out, unsigned long long* __restrict__ ctr) {
+                 int* __restrict__ slot, int* __restrict__ act, int* __restrict__ cols, int* __restrict__ colpos,
+                 int* __restrict__ ncol, int* __restrict__ colseg, int* __restrict__ count,
+                 double* __restrict__ dnu_out, unsigned long long* __restrict__ ctr) {
   pdl_wait();
   pdl_trigger();
   const int om = blockIdx.y, b = blockIdx.x, CB = gridDim.x;
@@ -495,6 +502,7 @@ k_classify_fused(Problem P, const cx<R>* __restrict__ wt, double* __restrict__ p
     for (int i = lane; i < CB; i += 32) gz += __ldcg(blkgz + om * CB + i);
     for (int o = 16; o > 0; o >>= 1) gz += __shfl_xor_sync(0xffffffffu, gz, o);
     int cbase = 0;
+    unsigned seg = 0u;  // as k_classify_scatter
     for (int j0 = 0; j0 < N; j0 += 32) {
       unsigned cmw = 0u;
       for (int i = lane; i < CB; i += 32) cmw |= __ldcg(colblk + ((long long)om * CB + i) * NWC + (j0 >> 5));
@@ -503,11 +511,16 @@ k_classify_fused(Problem P, const cx<R>* __restrict__ wt, double* __restrict__ p
       const int j = j0 + lane;
       const bool f = j < N && (cmw >> lane & 1u);
       const unsigned bal = __ballot_sync(0xffffffffu, f);
-      if (f) cols[om * N + cbase + __popc(bal & ((1u << lane) - 1u))] = j;
+      const int at = cbase + __popc(bal & ((1u << lane) - 1u));
+      if (f) cols[om * N + at] = j;
+      if (j < N) colpos[om * N + j] = f ? at : -1;
+      seg |= f ? 1u << (j * 16 / N) : 0u;
       cbase += __popc(bal);
     }
+    seg = __reduce_or_sync(0xffffffffu, seg);
     if (lane == 0) {
       const int total = total_s;
+      colseg[om] = (int)seg;
       ncol[om] = cbase;
       count[om] = total;
       atomicAdd(ctr + C_MODES, (unsigned long long)N2);
@@ -1382,7 +1395,8 @@ cudaError_t launch_classify(const Problem& P, const Work<R>& w, cudaStream_t s) 
                              w.n_partial, w.flagbits, w.blkcnt, w.blkgz, w.colblk, w.dnu);
   if (e != cudaSuccess) return e;
   return launch_pdl(k_classify_scatter, g, dim3(CT), 0, s, P, (const unsigned*)w.flagbits, (const int*)w.blkcnt,
-                    (const int*)w.blkgz, (const unsigned*)w.colblk, w.slot, w.act, w.cols, w.ncol, w.count, w.ctr);
+                    (const int*)w.blkgz, (const unsigned*)w.colblk, w.slot, w.act, w.cols, w.colpos, w.ncol, w.colseg,
+                    w.count, w.ctr);
 }
 template cudaError_t launch_classify<double>(const Problem&, const Work<double>&, cudaStream_t);
 template cudaError_t launch_classify<float>(const Problem&, const Work<float>&, cudaStream_t);
@@ -1419,8 +1433,8 @@ cudaError_t launch_classify_fused(const Problem& P, const Work<R>& w, cudaStream
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, k_classify_fused<R>, P, (const cx<R>*)w.wt, w.partial, w.bar,
-                                           w.blkcnt, w.blkgz, w.colblk, w.slot, w.act, w.cols, w.ncol, w.count,
-                                           w.dnu, w.ctr);
+                                           w.blkcnt, w.blkgz, w.colblk, w.slot, w.act, w.cols, w.colpos, w.ncol,
+                                           w.colseg, w.count, w.dnu, w.ctr);
   if (e != cudaSuccess && known) refused[dev].store(1, std::memory_order_relaxed);
   return e;
 }
