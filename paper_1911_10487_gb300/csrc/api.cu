@@ -315,6 +315,9 @@ cudaError_t launch_pipeline(const Problem& P, const Work<R>& w, const void* W, v
     e = launch_classify<R>(P, w, s);
   }
   if (e != cudaSuccess) return e;
+  if constexpr (sizeof(R) == 4) {
+    if (!w.wt64 && norm_groups(P, false) > 0 && (e = launch_fft2_active(P, w, s)) != cudaSuccess) return e;
+  }
   if (ev) cudaEventRecord(ev[3], s);
   *stage = "solve";
   if (P.solve_form == 1) e = launch_solve_rank1<R>(P, w, s);

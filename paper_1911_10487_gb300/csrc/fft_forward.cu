@@ -233,11 +233,34 @@ cudaError_t fwd_tiled(const cx<R>* W, const Problem& P, const Work<R>& w, cudaSt
   cudaError_t e = rows_launch<R, N, false, cx<R>, T, false>(W, w.wt, planes * N, (const cx<R>*)w.tw, R(1), s);
   if (e != cudaSuccess) return e;
   if (mid) cudaEventRecord(mid, s);
+  if constexpr (sizeof(R) == 4) {
+    if (const int G = norms ? norm_groups(P, false) : 0) {
+      // columns and norms in one pass (the group sums in the profiles' place, still unused)
+      using DP = DensePass<R, N, T>;
+      const int ppg = (P.m1 + G - 1) / G;
+      const dim3 g((N + DP::COLS - 1) / DP::COLS, (P.m1 + ppg - 1) / ppg, P.n_omega);
+      R* gn = reinterpret_cast<R*>(w.prof);
+      e = launch_pdl(k_fft_cols_norms<R, N, T>, g, dim3(DP::CT), 0, s, (const cx<R>*)w.wt, gn, P.m1, ppg,
+                     (const cx<R>*)w.tw);
+      if (e != cudaSuccess) return e;
+      return launch_pdl(k_group_norms<R>, dim3((N * N + NORM_T - 1) / NORM_T, P.n_omega), dim3(NORM_T), 0, s,
+                        (const R*)gn, w.norms, w.partial, (int)g.y, N * N, w.ctr);
+    }
+  }
   e = cols_launch<R, N, false, T, false>(w.wt, w.wt, planes, (const cx<R>*)w.tw, norms ? (unsigned*)nullptr : w.bar,
                                          P.n_omega, s);
   if (e != cudaSuccess) return e;
   if (!norms) return cudaGetLastError();
   return launch_mode_norms<R>(P, w, s);
+}
+
+template <int N>
+cudaError_t active_impl(const Problem& P, const Work<float>& w, cudaStream_t s) {
+  using AP = ActivePass<float, N>;
+  constexpr int NCH = (N + AP::GC - 1) / AP::GC;
+  const dim3 g((P.m1 + AP::GL - 1) / AP::GL, P.n_omega, NCH < 8 ? NCH : 8);
+  return launch_pdl(k_fft_cols_active<float, N>, g, dim3(AP::NT), 0, s, w.wt, P.m1, (const int*)w.cols,
+                    (const int*)w.ncol, w.tw);
 }
 
 template <typename R, int N>
@@ -314,6 +337,28 @@ cudaError_t launch_mode_norms(const Problem& P, const Work<R>& w, cudaStream_t s
 }
 template cudaError_t launch_mode_norms<double>(const Problem&, const Work<double>&, cudaStream_t);
 template cudaError_t launch_mode_norms<float>(const Problem&, const Work<float>&, cudaStream_t);
+
+// FP32 from 8 MB of data planes up, where the traffic saved is worth an extra launch, in the
+// two-pass transform under the discrepancy rule (a given alpha makes every column active).
+// About six blocks per SM, each a run of planes.
+int norm_groups(const Problem& P, bool fp64) {
+  const bool two_passes = P.n > 128 || !P.forward_single;
+  if (fp64 || !two_passes || P.alpha_mode != 0 || P.classify_single || wide_route(P, fp64)) return 0;
+  if (8.0 * P.n_omega * P.m1 * P.n * P.n < 8e6) return 0;
+  const int tiles = (P.n + 15) / 16 * P.n_omega;
+  int G = (6 * sm_count() + tiles - 1) / tiles;
+  G = G < P.m1 ? G : P.m1;
+  return G < 4 * P.m ? G : 4 * P.m;  // the group sums fit in the profiles' place
+}
+
+cudaError_t launch_fft2_active(const Problem& P, const Work<float>& w, cudaStream_t s) {
+  switch (P.n) {
+#define FL_CASE(K) case K: return active_impl<K>(P, w, s);
+    FL_SIZES(FL_CASE)
+#undef FL_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
 
 template <typename R>
 cudaError_t launch_fft2_forward(const cx<R>* W, const Problem& P, const Work<R>& w, cudaStream_t s,

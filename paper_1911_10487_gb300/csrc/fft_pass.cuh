@@ -114,6 +114,108 @@ k_fft_cols(const cx<R>* in, cx<R>* out, const cx<R>* __restrict__ tw, unsigned* 
       });
 }
 
+// ---- columns of the data planes and their norms in one pass ----------------------
+// grid (ceil(N/TC), G, n_omega): block (tile, g, om) transforms its columns of the planes
+// g ppg .. g ppg + ppg - 1 one after another and keeps sum |W~_k(nu)|^2 of its modes in
+// registers (a thread's last-stage outputs are the same modes in every plane); gnorm [om][G][N^2]
+// takes the sums, k_group_norms adds the groups.
+// W~ is not written: it is needed only on the few columns that hold an active mode, and
+// k_fft_cols_active transforms those again once they are known.  256 planes of 256^2 (FP32, bound
+// by memory): columns 42 us + norms 32 us -> 30 us + 11 us (groups) + 14 us (active columns).
+// In FP64 the column pass is bound by the FP64 pipe and the norms run behind its tail: fused,
+// with W~ written, 128^2 x 71 planes x 3 frequencies took 820 us for the whole call, 765 us with the
+// two passes, so FP64 keeps those.
+template <typename R, int N, int T>
+__global__ void __launch_bounds__((DensePass<R, N, T>::CT))
+k_fft_cols_norms(const cx<R>* __restrict__ wt, R* __restrict__ gnorm, int m1, int ppg, const cx<R>* __restrict__ tw) {
+  using DP = DensePass<R, N, T>;
+  using PL = IoPlan<N, DP::MAXR, false>;
+  constexpr int TC = DP::COLS, CT = DP::CT, S = PL::stages - 1, RAD = PL::radix(S), NB = N / RAD;
+  constexpr int PER = (TC * NB + CT - 1) / CT;
+  __shared__ cx<R> buf[PL::stages > 1 ? N * TC : 1];
+  __shared__ cx<R> tws[PL::tw_elems];
+  load_stage_twiddles<R, PL, N, CT>(tws, tw);  // a constant table: read while the predecessor drains
+  pdl_wait();
+  pdl_trigger();
+  const int c0 = blockIdx.x * TC, om = blockIdx.z;
+  const int k0 = blockIdx.y * ppg, k1 = min(m1, k0 + ppg);
+  R acc[PER][RAD];
+#pragma unroll
+  for (int p = 0; p < PER; ++p)
+#pragma unroll
+    for (int r = 0; r < RAD; ++r) acc[p][r] = R(0);
+  for (int k = k0; k < k1; ++k) {
+    const cx<R>* pl = wt + ((long long)om * m1 + k) * N * N + c0;
+    auto ld = [&](int b, int i) { return N % TC == 0 || c0 + b < N ? pl[i * N + b] : czero<R>(); };
+    if constexpr (S > 0) {
+      if (k > k0) __syncthreads();  // the last plane's tile has been read
+      io_first<R, PL, N, false, TC, CT, Lay::COL, 0>(buf, tws, ld);
+    }
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      const int t = threadIdx.x + p * CT, b = t % TC, j = t / TC;  // as LayIdx<COL>::map
+      if (TC * NB % CT == 0 || t < TC * NB) {
+        cx<R> v[RAD];
+        if constexpr (S > 0) {
+          io_butterfly<R, PL, N, false, TC, Lay::COL, 0, S>(buf, tws, b, j, v);
+        } else {
+#pragma unroll
+          for (int r = 0; r < RAD; ++r) v[r] = ld(b, r);
+          Dft<R, false>::template run<RAD>(v);
+        }
+#pragma unroll
+        for (int r = 0; r < RAD; ++r) acc[p][r] += v[r].x * v[r].x + v[r].y * v[r].y;
+      }
+    }
+  }
+  R* g = gnorm + ((long long)om * gridDim.y + blockIdx.y) * N * N + c0;
+#pragma unroll
+  for (int p = 0; p < PER; ++p) {
+    const int t = threadIdx.x + p * CT, b = t % TC, j = t / TC;
+    if ((TC * NB % CT == 0 || t < TC * NB) && (N % TC == 0 || c0 + b < N))
+#pragma unroll
+      for (int r = 0; r < RAD; ++r) g[(j + r * NB) * N + b] = acc[p][r];
+  }
+}
+
+// the columns of the compact list of frequency om (those that hold an active mode), in place on
+// the row-transformed planes: 4 columns by 4 planes per tile, as k_ifft_cols_gather
+template <typename R, int N> struct ActivePass {
+  static constexpr int GC = 4, GL = 4, LINES = GC * GL;
+  using PL = IoPlan<N, 16, false>;
+  static constexpr int NT = round32(LINES * N / (N % 3 == 0 ? 12 : 16)) < 256 ? round32(LINES * N / (N % 3 == 0 ? 12 : 16)) : 256;
+};
+template <typename R, int N>
+__global__ void __launch_bounds__((ActivePass<R, N>::NT))
+k_fft_cols_active(cx<R>* wt, int m1, const int* __restrict__ cols, const int* __restrict__ ncol,
+                  const cx<R>* __restrict__ tw) {
+  using AP = ActivePass<R, N>;
+  using PL = typename AP::PL;
+  constexpr int GC = AP::GC, GL = AP::GL;
+  __shared__ cx<R> buf[PL::stages > 1 ? N * AP::LINES : 1];
+  __shared__ cx<R> tws[PL::tw_elems];
+  load_stage_twiddles<R, PL, N, AP::NT>(tws, tw);
+  pdl_wait();
+  pdl_trigger();
+  const int om = blockIdx.y, k0 = blockIdx.x * GL, nc = ncol[om];
+  const int nk = min(GL, m1 - k0);
+  cx<R>* pl = wt + ((long long)om * m1 + k0) * N * N;
+  for (int cb = blockIdx.z * GC; cb < nc; cb += gridDim.z * GC) {
+    if (cb != (int)blockIdx.z * GC) __syncthreads();  // the previous tile has been read
+    const int ncb = min(GC, nc - cb);
+    const int* cl = cols + om * N + cb;
+    // line b: column b % GC, plane b / GC (neighbouring columns are mostly neighbours in a row)
+    fft_lines_io<R, PL, N, false, AP::LINES, AP::NT, Lay::COL, 0>(
+        buf, tws,
+        [&](int b, int i) {
+          return b % GC < ncb && b / GC < nk ? pl[((long long)(b / GC) * N + i) * N + cl[b % GC]] : czero<R>();
+        },
+        [&](int b, int i, cx<R> v) {
+          if (b % GC < ncb && b / GC < nk) pl[((long long)(b / GC) * N + i) * N + cl[b % GC]] = v;
+        });
+  }
+}
+
 // ---- per-mode norms ||W~_nu||^2 = sum_k |W~_k(nu)|^2 ----------------------------
 // grid (n_partial, n_omega), NORM_MB modes per block and NORM_Q threads per mode: warp
 // w sums the planes of quarter q = w / 2 (a contiguous quarter of the planes, its loads
@@ -168,6 +270,44 @@ k_mode_norms(const cx<R>* __restrict__ wt, double* __restrict__ norms, double* _
     __syncthreads();
   }
   if (threadIdx.x == 0) partial[(long long)om * gridDim.x + blockIdx.x] = red[0];
+}
+
+// the norms from the groups of k_fft_cols_norms, and their block sums: as k_mode_norms, the G
+// groups in place of the planes
+template <typename R>
+__global__ void __launch_bounds__(NORM_T)
+k_group_norms(const R* __restrict__ gnorm, double* __restrict__ norms, double* __restrict__ partial, int G, int N2,
+              unsigned long long* __restrict__ ctr) {
+  pdl_wait();
+  pdl_trigger();
+  __shared__ double red[NORM_T / 32];
+  const int om = blockIdx.y;
+  double sum = 0.0;
+  int bad = 0;
+  const int nu = blockIdx.x * NORM_T + threadIdx.x;
+  if (nu < N2) {
+    const R* p = gnorm + (long long)om * G * N2 + nu;
+    R acc = R(0);
+    int g = 0;
+    for (; g + 4 <= G; g += 4) {
+      R v[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) v[t] = p[(long long)(g + t) * N2];
+      acc += (v[0] + v[1]) + (v[2] + v[3]);
+    }
+    for (; g < G; ++g) acc += p[(long long)g * N2];
+    norms[(long long)om * N2 + nu] = (double)acc;
+    sum = (double)acc;
+    bad = !isfinite(acc);
+  }
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
+  const int n_bad = __syncthreads_count(bad);
+  if (n_bad && threadIdx.x == 0) atomicAdd(ctr + C_NONFINITE, (unsigned long long)n_bad);
+  if (threadIdx.x < NORM_T / NORM_MB) {  // block sums of NORM_MB modes each, as k_mode_norms writes them
+    const int np = (N2 + NORM_MB - 1) / NORM_MB, at = blockIdx.x * (NORM_T / NORM_MB) + threadIdx.x;
+    if (at < np) partial[(long long)om * np + at] = red[2 * threadIdx.x] + red[2 * threadIdx.x + 1];
+  }
 }
 
 }  // namespace

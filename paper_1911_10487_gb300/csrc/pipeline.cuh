@@ -222,6 +222,11 @@ cudaError_t opt_in_smem(SmemOptIn& flag, const void* kernel, size_t bytes, bool 
 template <typename R>
 cudaError_t launch_fft2_forward(const cx<R>* W, const Problem& P, const Work<R>& w, cudaStream_t s,
                                 cudaEvent_t mid = nullptr, bool norms = true);
+// groups of planes of the pass that transforms the columns and sums the norms at once (0: the
+// columns, then k_mode_norms); that pass leaves W~ to launch_fft2_active, which transforms the
+// columns holding active modes once the classification has listed them
+int norm_groups(const Problem& P, bool fp64);
+cudaError_t launch_fft2_active(const Problem& P, const Work<float>& w, cudaStream_t s);
 template <typename R>
 cudaError_t launch_mode_norms(const Problem& P, const Work<R>& w, cudaStream_t s);
 // classification from the norms: two kernels (flags, scatter)
