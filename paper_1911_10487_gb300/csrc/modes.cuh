@@ -84,10 +84,10 @@ __device__ __forceinline__ double rcp32(double x) {
 // exp(i kz d) inlined: for small kernels that evaluate several independent
 // exponentials per thread, so that their FP64 chains can overlap
 __device__ __forceinline__ double2 exp_ikz_inline(double2 kz, double d) {
-  const double mag = exp(-kz.y * d);
+  if (kz.x == 0.0) return make_double2(exp(-kz.y * d), 0.0);  // as exp_ikz
   double s, c;
   sincos(kz.x * d, &s, &c);
-  return make_double2(mag * c, mag * s);
+  return make_double2(c, s);
 }
 
 template <typename T> __device__ __forceinline__ T rcp(T x);
@@ -121,11 +121,13 @@ __device__ __forceinline__ float warp_sum(float v) {
 // A real call, not inlined: the FP64 exp and sincos are long, and the per-mode
 // kernels call this from several places executed by different warps, so one
 // shared copy keeps the instruction footprint (and its fetch stalls) down.
+// An evanescent mode takes no sine and cosine, a propagating one no exponential (each 50
+// to 100 FP64 instructions).
 static __device__ __noinline__ double2 exp_ikz(double2 kz, double d) {
-  const double mag = exp(-kz.y * d);
+  if (kz.x == 0.0) return make_double2(exp(-kz.y * d), 0.0);
   double s, c;
   sincos(kz.x * d, &s, &c);
-  return make_double2(mag * c, mag * s);
+  return make_double2(c, s);
 }
 
 // exp(i kz d) for the mixed route: the phase is reduced to [-pi, pi] in FP64

@@ -547,11 +547,13 @@ template <typename B> struct Bulk {
   cx<B> V[DENSE_M1][DENSE_M1 + 1];  // Lanczos basis, column j = q_j (FP64 route)
   cx<B> t[DENSE_M];               // A^H q_j of the Lanczos step
   cx<B> w[DENSE_M1];              // G q_j of the Lanczos step
+  cx<B> h[DENSE_M1];              // its components along the basis
 };
 struct BulkF {
   float2 Q[DENSE_M1][DENSE_M1 + 1];  // Lanczos basis, column j = q_j
   float2 t[DENSE_M];               // A^H q_j of the Lanczos step
   float2 w[DENSE_M1];              // G q_j of the Lanczos step
+  float2 h[DENSE_M1];              // its components along the basis
   float2 p[DENSE_M1];              // model solve (T + a I)^-1 Q^H r
   union {
     float2 A[DENSE_M1][DENSE_M + 1];  // A_nu / sqrt(tr G) in FP32, for the Lanczos products
@@ -581,76 +583,100 @@ struct Shared {
 static_assert(sizeof(Shared) <= 75 * 1024, "three solve blocks per SM");
 
 
+// Sum over groups of `parts` (a power of two) neighbouring lanes.
+template <typename T> __device__ __forceinline__ cx<T> part_sum(cx<T> v, int parts) {
+#pragma unroll 1
+  for (int o = 1; o < parts; o <<= 1) {
+    v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+    v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+  }
+  return v;
+}
+
+// 1/sqrt(x) of the squared norm of a Lanczos vector
+__device__ __forceinline__ float inv_norm(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double inv_norm(double x) { return rsqrt64(x); }
+
 // Lanczos tridiagonalisation of the Hermitian G = A A^H (n x n; A is n x m in
 // shared memory) from the unit vector in column 0 of Q, with full
-// reorthogonalisation (classical Gram-Schmidt, twice): Q^H G Q = T, real symmetric
+// orthogonalisation (classical Gram-Schmidt, twice): Q^H G Q = T, real symmetric
 // tridiagonal with diagonal d and off-diagonal e >= 0.  G is never formed: each
 // step applies it as A (A^H q_j), 2 n m complex products instead of the n^2 m of
-// the normal matrix, spread over the whole block (two threads per column of A for
-// t = A^H q_j, four per row for A t); warp 0 then orthogonalises (lane r owning
-// row r).  Stops when the next off-diagonal is not above tol (the Krylov space of
+// the normal matrix.  Every product of a step is spread over the whole block, the
+// threads of a sum neighbouring lanes of one warp: a warp issues one FP64 instruction
+// per 64 cycles, so the sums are cut over the four warps' schedulers rather than
+// chained in one (orthogonalising in warp 0, one basis vector after another, took 2 (j +
+// 1) 18 of them per step j, 180k cycles of a full-rank FP64 mode with n = 12; now ~7k a
+// step in all).  Stops when the next off-diagonal is not above tol (the Krylov space of
 // q_0 is then invariant to that level) or at n columns, and returns the number k
 // of columns (the same in every thread).  Called by all ST threads; t (m entries),
-// w (n entries) and *go are scratch.
+// w, hs (n entries) and *go are scratch.
 // The (1,1) entries of (T + a I)^-1 and (T + a I)^-2, from which the discrepancy
 // is computed, depend on e only through the squares e_j^2, so stopping at
 // e_k <= tol changes phi^2 by O(tol^2 / a^2) relative.
 template <typename T>
-__device__ int lanczos_block(const cx<T> (*A)[DENSE_M + 1], int n, int m, cx<T>* t, cx<T>* wv,
+__device__ int lanczos_block(const cx<T> (*A)[DENSE_M + 1], int n, int m, cx<T>* t, cx<T>* wv, cx<T>* hs,
                              cx<T> (*Q)[DENSE_M1 + 1], T* d, T* e, T tol, int* go) {
   const int lane = threadIdx.x & 31;
+  // threads per column of A, per row of A and per basis vector
+  const int pc = m <= ST / 4 ? 4 : 2, pr = n <= ST / 8 ? 8 : 4;
+  const int l = threadIdx.x / pc, hl = threadIdx.x % pc;
+  const int r = threadIdx.x / pr, hr = threadIdx.x % pr;
   int k = n;
 #pragma unroll 1
   for (int j = 0; j < n; ++j) {
-    {  // t = A^H q_j: two threads per column l
-      const int l = threadIdx.x >> 1, h = threadIdx.x & 1;
+    {  // t = A^H q_j
       cx<T> acc = czero<T>();
       if (l < m)
 #pragma unroll 1
-        for (int r = h; r < n; r += 2) acc = acc + cmul_conj_a(A[r][l], Q[r][j]);
-      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 1);
-      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 1);
-      if (l < m && h == 0) t[l] = acc;
+        for (int i = hl; i < n; i += pc) acc = acc + cmul_conj_a(A[i][l], Q[i][j]);
+      acc = part_sum<T>(acc, pc);
+      if (l < m && hl == 0) t[l] = acc;
     }
     __syncthreads();
-    {  // w = A t = G q_j: four threads per row r
-      const int r = threadIdx.x >> 2, h = threadIdx.x & 3;
+    {  // w = A t = G q_j
       cx<T> acc = czero<T>();
       if (r < n)
 #pragma unroll 1
-        for (int l = h; l < m; l += 4) acc = acc + A[r][l] * t[l];
-      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 1);
-      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 1);
-      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 2);
-      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 2);
-      if (r < n && h == 0) wv[r] = acc;
+        for (int i = hr; i < m; i += pr) acc = acc + A[r][i] * t[i];
+      acc = part_sum<T>(acc, pr);
+      if (r < n && hr == 0) wv[r] = acc;
     }
     __syncthreads();
-    if (threadIdx.x < 32) {
-      cx<T> w = lane < n ? wv[lane] : czero<T>();
-      const cx<T> qj = lane < n ? Q[lane][j] : czero<T>();
-      const T aj = warp_sum(qj.x * w.x + qj.y * w.y);  // q_j^H G q_j (real)
-      w = w - aj * qj;
-      if (j > 0 && lane < n) w = w - e[j - 1] * Q[lane][j - 1];
+    T aj = T(0);
 #pragma unroll 1
-      for (int pass = 0; pass < 2; ++pass) {  // w -= Q (Q^H w) over q_0 .. q_j
-        cx<T> corr = czero<T>();
+    for (int pass = 0; pass < 2; ++pass) {  // w -= Q (Q^H w) over q_0 .. q_j
+      {  // h_i = q_i^H w, thread group i = r; h_j adds up to q_j^H G q_j (real)
+        cx<T> acc = czero<T>();
+        if (r <= j)
 #pragma unroll 1
-        for (int i = 0; i <= j; ++i) {
-          const cx<T> qi = lane < n ? Q[lane][i] : czero<T>();
-          const cx<T> hh = warp_sum(cmul_conj_a(qi, w));  // q_i^H w
-          corr = corr + qi * hh;
-        }
-        w = w - corr;
+          for (int i = hr; i < n; i += pr) acc = acc + cmul_conj_a(Q[i][r], wv[i]);
+        acc = part_sum<T>(acc, pr);
+        if (r <= j && hr == 0) hs[r] = acc;
       }
-      const T beta = sqrt(warp_sum(abs2(w)));
+      __syncthreads();
+      aj += hs[j].x;
+      {
+        cx<T> acc = czero<T>();
+        if (r < n)
+#pragma unroll 1
+          for (int i = hr; i <= j; i += pr) acc = acc + Q[r][i] * hs[i];
+        acc = part_sum<T>(acc, pr);
+        if (r < n && hr == 0) wv[r] = wv[r] - acc;
+      }
+      __syncthreads();
+    }
+    if (threadIdx.x < 32) {
+      const cx<T> w = lane < n ? wv[lane] : czero<T>();
+      const T nn = warp_sum(abs2(w));
+      const T inv = nn > T(0) ? inv_norm(nn) : T(0), beta = nn * inv;
       const bool stop = j + 1 == n || !(beta > tol);
       if (lane == 0) {
         d[j] = aj;
         if (!stop) e[j] = beta;
         *go = stop ? 0 : 1;
       }
-      if (!stop && lane < n) Q[lane][j + 1] = rcp<T>(beta) * w;
+      if (!stop && lane < n) Q[lane][j + 1] = inv * w;
     }
     __syncthreads();
     if (!*go) {
@@ -741,7 +767,69 @@ __device__ double phi2(const T* d, const T* e, const cx<T>* c, int n, double a, 
   return a * a * (double)zz;
 }
 
-// block-wide sums of one double per thread (all threads get them)
+// (T + a I) z = e_1 and, with S2, (T + a I) s = z for one factorisation; zz = ||z||^2, zs = z.s;
+// single thread, real.  False on a pivot that is not positive.
+template <bool S2>
+__device__ bool tri_solve_e1(const double* d, const double* e, int n, double a, double* z, double& zz, double& zs) {
+  double mu[DENSE_M1], il[DENSE_M1], s[S2 ? DENSE_M1 : 1];
+  double lp = d[0] + a;
+  if (!(lp > 0.0)) return false;
+  il[0] = rcp64(lp);
+  z[0] = 1.0;
+#pragma unroll 1
+  for (int i = 1; i < n; ++i) {
+    const double ei = e[i - 1], m = ei * il[i - 1];
+    lp = fma(-m, ei, d[i] + a);
+    if (!(lp > 0.0)) return false;
+    mu[i] = m;
+    il[i] = rcp64(lp);
+    z[i] = -m * z[i - 1];
+  }
+  z[n - 1] *= il[n - 1];
+  zz = z[n - 1] * z[n - 1];
+#pragma unroll 1
+  for (int i = n - 2; i >= 0; --i) {
+    z[i] = fma(-mu[i + 1], z[i + 1], il[i] * z[i]);
+    zz = fma(z[i], z[i], zz);
+  }
+  if constexpr (S2) {
+    s[0] = z[0];
+#pragma unroll 1
+    for (int i = 1; i < n; ++i) s[i] = fma(-mu[i], s[i - 1], z[i]);
+    s[n - 1] *= il[n - 1];
+    zs = z[n - 1] * s[n - 1];
+#pragma unroll 1
+    for (int i = n - 2; i >= 0; --i) {
+      s[i] = fma(-mu[i + 1], s[i + 1], il[i] * s[i]);
+      zs = fma(z[i], s[i], zs);
+    }
+  }
+  return true;
+}
+
+// Newton in log(a) on log(a^2 ||(T + a I)^-1 e_1||^2 / target) from the FP32 root, to FP64
+// accuracy: the logarithm and the exponential are of 1 + x with |x| <= 1e-2 and taken by their
+// series (an FP64 log or exp costs ~50 instructions of 64 cycles in this one thread), z and its
+// derivative share a factorisation, and the step from |x| < 1e-8 is the last (quadratic: the
+// next x is below rounding).  False when it does not get there: the caller then takes the
+// bracketed search.
+__device__ bool polish_root(const double* d, const double* e, int n, double inv_target, double& a, int max_iter) {
+  double z[DENSE_M1], zz, zs;
+#pragma unroll 1
+  for (int it = 0; it < max_iter && it < 5; ++it) {
+    if (!tri_solve_e1<true>(d, e, n, a, z, zz, zs)) return false;
+    const double x = fma(a * a * inv_target, zz, -1.0);
+    if (!(fabs(x) <= 1e-2)) return false;
+    const double g = x * fma(x, fma(x, fma(x, fma(x, 0.2, -0.25), 0.33333333333333333), -0.5), 1.0);  // log(1 + x)
+    const double gp = 2.0 - 2.0 * a * zs * rcp64(zz);
+    if (!(gp > 0.0)) return false;
+    const double y = -g * rcp64(gp);
+    if (!(fabs(y) <= 1e-1)) return false;
+    a *= fma(y, fma(y, fma(y, fma(y, 0.041666666666666667, 0.16666666666666667), 0.5), 1.0), 1.0);  // exp(y)
+    if (fabs(x) < 1e-8) return true;
+  }
+  return false;
+}
 
 // FP64 route: FP64 Lanczos model of the normal matrix, FP32-seeded root on the
 // scaled tridiagonal, FP64 Newton to full accuracy, y = (||b||/tr) Q (T/tr + a I)^-1 e_1.
@@ -751,7 +839,7 @@ __device__ void solve_fp64(Shared& S, int n, int m, const Problem& P, int om, un
   const double inv_sb = rcp64(S.sb), inv_tr = rcp64(S.tr);
   if (threadIdx.x < n) K.V[threadIdx.x][0] = inv_sb * S.b[threadIdx.x];
   __syncthreads();
-  const int kd = lanczos_block<double>(S.A, n, m, K.t, K.w, K.V, S.d, S.e, LANCZOS_TOL64 * S.tr, &S.go);
+  const int kd = lanczos_block<double>(S.A, n, m, K.t, K.w, K.h, K.V, S.d, S.e, LANCZOS_TOL64 * S.tr, &S.go);
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
     if (lane < kd) {  // scaled model T / tr, c = e_1, and FP32 copies for the seed
@@ -772,26 +860,42 @@ __device__ void solve_fp64(Shared& S, int n, int m, const Problem& P, int om, un
     const double target = (S.dnu * inv_sb) * (S.dnu * inv_sb);
     const double lo = P.alpha_rel, hi = S.hi * inv_tr;
     bool ok = true;
-    double a;
+    double a, z[DENSE_M1], zz, zs;
     if (P.alpha_mode == 1) {
       a = P.alpha_given[om] * inv_tr;
-    } else if (phi2<double>(S.d, S.e, S.c, kd, lo, ok) >= target) {
-      a = lo;
-      atomicAdd(ctr + C_ALPHA_FLOOR, 1ull);
     } else {
+      // the FP32 root, then FP64.  phi grows with a, so a root above lo means phi(lo) below the
+      // target: the floor needs a look only when none was found there
       double gp;
       bool ok32;
       int it32, it64;
-      const double t_mid = 0.5 * (log(lo) + log(hi));
-      double t = newton_log_alpha<float>(S.d32, S.e32, S.c32, kd, lo, hi, target, t_mid, 1e-5, P.max_iter, gp,
-                                         ok32, it32);
-      if (!ok32 || !(t > log(lo) && t < log(hi))) t = t_mid;
-      t = newton_log_alpha<double>(S.d, S.e, S.c, kd, lo, hi, target, t, 1e-14, P.max_iter, gp, ok, it64);
-      if (it64 >= P.max_iter) atomicAdd(ctr + C_ROOT_CAPPED, 1ull);
-      a = exp(t);
+      const float lol = logf((float)lo), hil = logf(fminf((float)hi, 1e38f));
+      const float t32 = (float)newton_log_alpha<float>(S.d32, S.e32, S.c32, kd, lo, hi, target,
+                                                       0.5 * (double)(lol + hil), 1e-5, P.max_iter, gp, ok32, it32);
+      a = (double)expf(t32);
+      const bool inside = ok32 && t32 > lol + 1e-3f && t32 < hil;
+      if (!inside || !polish_root(S.d, S.e, kd, rcp64(target), a, P.max_iter) || !(a > lo)) {
+        if (phi2<double>(S.d, S.e, S.c, kd, lo, ok) >= target) {
+          a = lo;
+          atomicAdd(ctr + C_ALPHA_FLOOR, 1ull);
+        } else {
+          const double ll = log(lo), lh = log(hi), t_mid = 0.5 * (ll + lh);
+          double t = ok32 && (double)t32 > ll && (double)t32 < lh ? (double)t32 : t_mid;
+          t = newton_log_alpha<double>(S.d, S.e, S.c, kd, lo, hi, target, t, 1e-14, P.max_iter, gp, ok, it64);
+          if (it64 >= P.max_iter) atomicAdd(ctr + C_ROOT_CAPPED, 1ull);
+          a = exp(t);
+        }
+      } else if (a > hi) {
+        a = hi;
+      }
     }
     S.a_s = a;
-    tri_solve<double>(S.d, S.e, kd, a, S.c, S.z);
+    if (tri_solve_e1<false>(S.d, S.e, kd, a, z, zz, zs)) {
+#pragma unroll 1
+      for (int i = 0; i < kd; ++i) S.z[i] = make_double2(z[i], 0.0);
+    } else {
+      tri_solve<double>(S.d, S.e, kd, a, S.c, S.z);
+    }
   }
   __syncthreads();
   FL_MARK_S(15);
@@ -1173,7 +1277,7 @@ k_solve(Problem P, const cx<B>* __restrict__ wt, const int* __restrict__ act,
         if (lane < n) K.Q[lane][0] = inq * q0;
       }
       __syncthreads();
-      const int kd = lanczos_block<float>(K.m.A, n, m, K.t, K.w, K.Q, S.d32, S.e32, LANCZOS_TOL32, &S.go);
+      const int kd = lanczos_block<float>(K.m.A, n, m, K.t, K.w, K.h, K.Q, S.d32, S.e32, LANCZOS_TOL32, &S.go);
       if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
         if (lane == 0) S.kd = kd;
