@@ -44,19 +44,22 @@ STAGES = ("fft_x_forward", "fft_y_forward_norms", "classify", "solve", "ifft_y_g
 # changed); to be measured again whenever a kernel changes
 SOLVE_DRAM_BYTES = 237056  # k_solve<float> (dense form, mixed): 237 KB read, nothing written
 STAGE_DRAM_BYTES = {"ifft_x_recover": 4249600}  # k_ifft_rows_recover<float>: 4.25 MB read, writes stay in L2
-STAGE_KERNELS = {"fft_x_forward": "k_fft2_plane<float>", "fft_y_forward_norms": "k_mode_norms<float>",
-                 "classify": "k_classify_flags + k_classify_scatter", "ifft_y_gather": "k_ifft_cols_gather<float>",
+STAGE_KERNELS = {"fft_x_forward": "k_fft2_plane<float>", "fft_y_forward_norms": "k_fft2_plane<float>",
+                 "classify": "k_classify_early", "ifft_y_gather": "k_ifft_cols_gather<float>",
                  "ifft_x_recover": "k_ifft_rows_recover<float>"}
 HEAD_FORM = 1  # the headline's per-mode solver: the rank-one closed form
-# kernels of one mixed step: 2D FFT (one pass at N <= 128, two beyond), mode norms,
-# classify (flags, scatter), solve, gather + y-IFFT, x-IFFT + recover; the plain FP64
-# path transforms in two passes
-KERNELS_PER_STEP_MIXED = 7
+# kernels of one mixed step: 2D FFT (one pass at N <= 128, rows and columns beyond), norms and
+# classification, solve, gather + y-IFFT, x-IFFT + recover; beyond 8 MB of data planes the
+# two-pass transform adds one for the active columns.  The plain FP64 path: rows, columns, norms,
+# flags, scatter, solve, gather, recover
+KERNELS_PER_STEP_MIXED = 5
 KERNELS_PER_STEP = 8
 
 
-def mixed_kernels(n):
-    return KERNELS_PER_STEP_MIXED + (1 if n > 128 else 0)
+def mixed_kernels(wl):
+    if wl.n <= 128:
+        return KERNELS_PER_STEP_MIXED
+    return KERNELS_PER_STEP_MIXED + (2 if 8 * len(wl.omegas) * wl.m1 * wl.n * wl.n >= 8e6 else 1)
 
 
 def peaks():
@@ -169,7 +172,7 @@ def make_inputs(rc, wl, geom):
 def algorithmic_bytes(stage, wl, rep, sc, single=False):
     """Bytes a stage must move at minimum (one launch), sc = bytes per complex; single:
     the forward 2D transform in one pass (the mixed path), so that its first stage is the
-    whole transform and the second the mode norms alone."""
+    whole transform, the second empty, and the norms part of the classification."""
     F, N2, M, M1 = len(wl.omegas), wl.n * wl.n, wl.m, wl.m1
     sr = sc // 2
     act, cols = rep["n_active"], rep["n_columns"]
@@ -177,8 +180,10 @@ def algorithmic_bytes(stage, wl, rep, sc, single=False):
     if stage == "fft_x_forward":
         return 2 * data
     if stage == "fft_y_forward_norms":
-        return (0 if single else 2 * data) + data + 8 * F * N2
+        return 0 if single else 3 * data + 8 * F * N2
     if stage == "classify":
+        if single:
+            return data + 4 * F * N2 + 4 * act
         return 8 * F * N2 + 4 * F * N2 + 4 * act
     if stage == "solve":
         return act * (M1 + 2 * M) * sc
@@ -549,7 +554,7 @@ def run_batch(args, local, flush, world):
            "voxel_freqs": vox, "steps": K, "cuda_graph": True, "unit": UNIT,
            "l2": "flushed (256 MiB write) before every timed step",
            "mixed": res["mixed"], "fp64": res["fp64"],
-           "gpu_launches_per_step": sum(mixed_kernels(wl.n) for wl in wls)}
+           "gpu_launches_per_step": sum(mixed_kernels(wl) for wl in wls)}
     # smallest problem of the batch against the oracle (a parity spot check at full batch)
     j = min(range(len(wls)), key=lambda i: wls[i].voxel_freqs * wls[i].m1)
     out["spot_problem"] = wls[j].name

@@ -138,9 +138,10 @@ Layout layout(int n, int m, int m1, int n_omega, bool fp64) {
   L.colpos = off; off = align_up(off + 4 * (size_t)n_omega * n);
   L.ncol = off; off = align_up(off + 4 * (size_t)n_omega);
   L.colseg = off; off = align_up(off + 4 * (size_t)n_omega);
-  L.count = off; off = align_up(off + 4 * (size_t)n_omega);
   L.dnu = off; off = align_up(off + 8 * (size_t)n_omega);
-  L.bar = off; off = align_up(off + 4 * (size_t)n_omega);
+  L.bar = off; L.count = off + 4 * (size_t)n_omega; L.colmask = off + 8 * (size_t)n_omega;
+  off = align_up(off + 40 * (size_t)n_omega);
+  L.wsum = off; off = align_up(off + 8 * (size_t)n_omega * wsum_max(n, m1));
   L.total = off;
   return L;
 }
@@ -278,6 +279,8 @@ Work<R> carve_work(void* base, const Layout& L, unsigned long long* ctr, const c
   w.count = (int*)(b + L.count);
   w.dnu = (double*)(b + L.dnu);
   w.bar = (unsigned*)(b + L.bar);
+  w.colmask = (unsigned*)(b + L.colmask);
+  w.wsum = (float2*)(b + L.wsum);
   w.ctr = ctr;
   w.tw = tw;
   w.alpha_out = alpha_out;
@@ -296,15 +299,23 @@ template <typename R>
 cudaError_t launch_pipeline(const Problem& P, const Work<R>& w, const void* W, void* xi, void* c, cudaStream_t s,
                             cudaEvent_t* ev, const char** stage) {
   cudaError_t e;
-  // the single-pass classification computes the norms itself; the mixed truncated-SVD
-  // route (W~ in FP64) keeps the separate norms kernel
+  // the single-pass classification computes the norms itself, as the early one does; the mixed
+  // truncated-SVD route (W~ in FP64) keeps the separate norms kernel
   const bool fused = w.wt64 == nullptr && classify_fused_ok(P);
   if (ev) cudaEventRecord(ev[0], s);
   *stage = "fft2_forward";
-  if ((e = launch_fft2_forward<R>((const cx<R>*)W, P, w, s, ev ? ev[1] : nullptr, !fused)) != cudaSuccess) return e;
+  const bool early = w.wt64 == nullptr && classify_early(P, sizeof(R) == 8);
+  int n_wsum = 0, G = 0;
+  if ((e = launch_fft2_forward<R>((const cx<R>*)W, P, w, s, ev ? ev[1] : nullptr, !fused, &n_wsum, &G)) != cudaSuccess)
+    return e;
   if (ev) cudaEventRecord(ev[2], s);
   *stage = "classify";
-  if (fused) {
+  if (early) {
+    if constexpr (sizeof(R) == 4) {
+      if ((e = launch_classify_early(P, w, n_wsum, G, s)) != cudaSuccess) return e;
+      if (G > 0) e = launch_fft2_active(P, w, s);
+    }
+  } else if (fused) {
     e = launch_classify_fused<R>(P, w, s);
     if (e != cudaSuccess) {  // not co-resident on this device: norms, then the two-kernel classification
       cudaGetLastError();
@@ -315,9 +326,6 @@ cudaError_t launch_pipeline(const Problem& P, const Work<R>& w, const void* W, v
     e = launch_classify<R>(P, w, s);
   }
   if (e != cudaSuccess) return e;
-  if constexpr (sizeof(R) == 4) {
-    if (!w.wt64 && norm_groups(P, false) > 0 && (e = launch_fft2_active(P, w, s)) != cudaSuccess) return e;
-  }
   if (ev) cudaEventRecord(ev[3], s);
   *stage = "solve";
   if (P.solve_form == 1) e = launch_solve_rank1<R>(P, w, s);

@@ -34,16 +34,17 @@ __global__ void k_twiddles(cx<R>* tw, int n) {
 // columns r RB .. r RB + RB - 1 of all N rows from the CTAs that hold them
 // (distributed shared memory), transforms them along y and writes them to W~.  The
 // plane crosses global memory once each way, in one launch.
-// clear (may be null): nclear counters zeroed by CTA (0, 0), as in k_fft_cols.
+// clear (may be null): nclear words zeroed by CTA (0, 0), as in k_fft_rows.
 template <typename R, int N> __host__ __device__ constexpr size_t plane_fwd_smem() {
   constexpr int RB = N / fwd_cluster<N>();
   return sizeof(cx<R>) * ((size_t)LayIdx<Lay::ROW, N, RB, 16>::ELEMS + (size_t)RB * N + N);
 }
 
+// wsum (may be null): the CTA's sum of |in|^2, [plane][C].
 template <typename R, int N>
 __global__ void __launch_bounds__(THREADS)
 k_fft2_plane(const cx<R>* __restrict__ in, cx<R>* __restrict__ out, const cx<R>* __restrict__ tw,
-             unsigned* __restrict__ clear, int nclear) {
+             unsigned* __restrict__ clear, int nclear, float2* __restrict__ wsum) {
   constexpr int C = fwd_cluster<N>(), RB = N / C;
   using IA = LayIdx<Lay::ROW, N, RB, 16>;  // this CTA's rows
   constexpr int E = RB * N;                // elements of the row tile and of the column tile
@@ -66,6 +67,10 @@ k_fft2_plane(const cx<R>* __restrict__ in, cx<R>* __restrict__ out, const cx<R>*
     const int e = threadIdx.x + p * THREADS;
     if (E % THREADS == 0 || e < E) v[p] = src[e];
   }
+  float ws = 0.f;
+#pragma unroll
+  for (int p = 0; p < PER; ++p)
+    if (E % THREADS == 0 || threadIdx.x + p * THREADS < E) ws += v[p].x * v[p].x + v[p].y * v[p].y;
 #pragma unroll
   for (int p = 0; p < PER; ++p) {
     const int e = threadIdx.x + p * THREADS;
@@ -98,22 +103,28 @@ k_fft2_plane(const cx<R>* __restrict__ in, cx<R>* __restrict__ out, const cx<R>*
     const int e = threadIdx.x + p * THREADS;
     if (E % THREADS == 0 || e < E) dst[(long long)(e / RB) * N + e % RB] = colt[e];
   }
+  if (wsum) {
+    __shared__ ff red[THREADS / 32];
+    block_sum_ff<THREADS>(ws, red, wsum + (long long)blockIdx.y * C + r);
+  }
   cluster_wait();  // no CTA leaves while another may still read its rows
 }
 
 template <typename R, int N>
 cudaError_t fwd_plane(const cx<R>* W, const Problem& P, const Work<R>& w, cudaStream_t s, cudaEvent_t mid,
-                      bool norms) {
+                      bool norms, int* n_wsum) {
   constexpr size_t smem = plane_fwd_smem<R, N>();
   static SmemOptIn attr;
   cudaError_t e = opt_in_smem(attr, (const void*)k_fft2_plane<R, N>, smem, true);
   if (e != cudaSuccess) return e;
   constexpr int C = fwd_cluster<N>();
+  const bool early = norms && classify_early(P, sizeof(R) == 8);
+  if (early) *n_wsum = C * P.m1;
   e = launch_pdl_cluster(k_fft2_plane<R, N>, dim3(C, (unsigned)(P.n_omega * P.m1)), dim3(THREADS), C, smem, s, W,
-                         w.wt, (const cx<R>*)w.tw, norms ? (unsigned*)nullptr : w.bar, P.n_omega);
+                         w.wt, (const cx<R>*)w.tw, w.bar, clear_words(P), early ? w.wsum : (float2*)nullptr);
   if (e != cudaSuccess) return e;
   if (mid) cudaEventRecord(mid, s);
-  if (!norms) return cudaGetLastError();
+  if (early || !norms) return cudaGetLastError();
   return launch_mode_norms<R>(P, w, s);
 }
 
@@ -191,20 +202,36 @@ template <typename R, int N, bool INV, typename TI, int T, bool D32>
 cudaError_t rows_launch(const TI* in, cx<R>* out, long long nrows, const cx<R>* tw, R scale, cudaStream_t s) {
   using DP = DensePass<R, N, T>;
   return launch_pdl(k_fft_rows<R, N, INV, TI, T, D32>, dim3((unsigned)((nrows + DP::LINES - 1) / DP::LINES)),
-                    dim3(DP::RT), 0, s, in, out, nrows, tw, scale);
+                    dim3(DP::RT), 0, s, in, out, nrows, tw, scale, (unsigned*)nullptr, 0, (float2*)nullptr);
+}
+
+// the rows of the data planes; *n_wsum (not null): the block sums of |W|^2 per frequency too
+template <typename R, int N, typename TI, int T>
+cudaError_t data_rows_launch(const TI* in, cx<R>* out, const Problem& P, const cx<R>* tw, unsigned* clear,
+                             float2* wsum, int* n_wsum, cudaStream_t s) {
+  using DP = DensePass<R, N, T>;
+  const long long nrows = (long long)P.m1 * N;
+  const dim3 g((unsigned)((nrows + DP::LINES - 1) / DP::LINES), P.n_omega);
+  if constexpr (sizeof(R) == 4) {
+    if (n_wsum) {
+      *n_wsum = (int)g.x;
+      return launch_pdl(k_fft_rows<R, N, false, TI, T, false, true>, g, dim3(DP::RT), 0, s, in, out, nrows, tw, R(1),
+                        clear, clear_words(P), wsum);
+    }
+  }
+  return launch_pdl(k_fft_rows<R, N, false, TI, T, false>, g, dim3(DP::RT), 0, s, in, out, nrows, tw, R(1), clear,
+                    clear_words(P), (float2*)nullptr);
 }
 
 template <typename R, int N, bool INV, int T, bool D32>
-cudaError_t cols_launch(const cx<R>* in, cx<R>* out, long long planes, const cx<R>* tw, unsigned* clear, int nclear,
-                        cudaStream_t s) {
+cudaError_t cols_launch(const cx<R>* in, cx<R>* out, long long planes, const cx<R>* tw, cudaStream_t s) {
   using DP = DensePass<R, N, T>;
   constexpr long long MAX_Y = 32768;  // planes per launch (grid y <= 65535)
   for (long long p0 = 0; p0 < planes; p0 += MAX_Y) {
     const long long np = planes - p0 < MAX_Y ? planes - p0 : MAX_Y;
     const cudaError_t e = launch_pdl(k_fft_cols<R, N, INV, T, D32>, dim3((N + DP::COLS - 1) / DP::COLS, (unsigned)np),
-                                     dim3(DP::CT), 0, s, in + p0 * N * N, out + p0 * N * N, tw, clear, nclear);
+                                     dim3(DP::CT), 0, s, in + p0 * N * N, out + p0 * N * N, tw);
     if (e != cudaSuccess) return e;
-    clear = nullptr;
   }
   return cudaSuccess;
 }
@@ -214,10 +241,10 @@ cudaError_t cols_launch(const cx<R>* in, cx<R>* out, long long planes, const cx<
 template <int N>
 cudaError_t fwd_wide_impl(const float2* W, const Problem& P, const Work<float>& w, cudaStream_t s, cudaEvent_t mid) {
   const long long planes = (long long)P.n_omega * P.m1;
-  cudaError_t e = rows_launch<double, N, false, float2, 0, false>(W, w.wt64, planes * N, w.tw64, 1.0, s);
+  cudaError_t e = data_rows_launch<double, N, float2, 0>(W, w.wt64, P, w.tw64, w.bar, nullptr, nullptr, s);
   if (e != cudaSuccess) return e;
   if (mid) cudaEventRecord(mid, s);
-  e = cols_launch<double, N, false, 0, false>(w.wt64, w.wt64, planes, w.tw64, nullptr, 0, s);
+  e = cols_launch<double, N, false, 0, false>(w.wt64, w.wt64, planes, w.tw64, s);
   if (e != cudaSuccess) return e;
   const dim3 gn((unsigned)w.n_partial, (unsigned)P.n_omega);
   e = launch_pdl(k_mode_norms<double>, gn, dim3(NORM_T), 0, s, (const double2*)w.wt64, w.norms, w.partial, P.m1,
@@ -228,29 +255,26 @@ cudaError_t fwd_wide_impl(const float2* W, const Problem& P, const Work<float>& 
 
 template <typename R, int N, int T>
 cudaError_t fwd_tiled(const cx<R>* W, const Problem& P, const Work<R>& w, cudaStream_t s, cudaEvent_t mid,
-                      bool norms) {
-  const long long planes = (long long)P.n_omega * P.m1;
-  cudaError_t e = rows_launch<R, N, false, cx<R>, T, false>(W, w.wt, planes * N, (const cx<R>*)w.tw, R(1), s);
+                      bool norms, int* n_wsum, int* groups) {
+  const bool early = norms && classify_early(P, sizeof(R) == 8);
+  const cx<R>* tw = (const cx<R>*)w.tw;
+  cudaError_t e = data_rows_launch<R, N, cx<R>, T>(W, w.wt, P, tw, w.bar, w.wsum, early ? n_wsum : nullptr, s);
   if (e != cudaSuccess) return e;
   if (mid) cudaEventRecord(mid, s);
   if constexpr (sizeof(R) == 4) {
-    if (const int G = norms ? norm_groups(P, false) : 0) {
+    if (const int G = early ? norm_groups(P, false) : 0) {
       // columns and norms in one pass (the group sums in the profiles' place, still unused)
       using DP = DensePass<R, N, T>;
       const int ppg = (P.m1 + G - 1) / G;
       const dim3 g((N + DP::COLS - 1) / DP::COLS, (P.m1 + ppg - 1) / ppg, P.n_omega);
-      R* gn = reinterpret_cast<R*>(w.prof);
-      e = launch_pdl(k_fft_cols_norms<R, N, T>, g, dim3(DP::CT), 0, s, (const cx<R>*)w.wt, gn, P.m1, ppg,
-                     (const cx<R>*)w.tw);
-      if (e != cudaSuccess) return e;
-      return launch_pdl(k_group_norms<R>, dim3((N * N + NORM_T - 1) / NORM_T, P.n_omega), dim3(NORM_T), 0, s,
-                        (const R*)gn, w.norms, w.partial, (int)g.y, N * N, w.ctr);
+      *groups = (int)g.y;
+      return launch_pdl(k_fft_cols_norms<R, N, T>, g, dim3(DP::CT), 0, s, (const cx<R>*)w.wt,
+                        reinterpret_cast<R*>(w.prof), P.m1, ppg, tw);
     }
   }
-  e = cols_launch<R, N, false, T, false>(w.wt, w.wt, planes, (const cx<R>*)w.tw, norms ? (unsigned*)nullptr : w.bar,
-                                         P.n_omega, s);
+  e = cols_launch<R, N, false, T, false>(w.wt, w.wt, (long long)P.n_omega * P.m1, tw, s);
   if (e != cudaSuccess) return e;
-  if (!norms) return cudaGetLastError();
+  if (early || !norms) return cudaGetLastError();
   return launch_mode_norms<R>(P, w, s);
 }
 
@@ -259,23 +283,23 @@ cudaError_t active_impl(const Problem& P, const Work<float>& w, cudaStream_t s) 
   using AP = ActivePass<float, N>;
   constexpr int NCH = (N + AP::GC - 1) / AP::GC;
   const dim3 g((P.m1 + AP::GL - 1) / AP::GL, P.n_omega, NCH < 8 ? NCH : 8);
-  return launch_pdl(k_fft_cols_active<float, N>, g, dim3(AP::NT), 0, s, w.wt, P.m1, (const int*)w.cols,
-                    (const int*)w.ncol, w.tw);
+  return launch_pdl(k_fft_cols_active<float, N>, g, dim3(AP::NT), 0, s, w.wt, P.m1, (const unsigned*)w.colmask, w.tw);
 }
 
 template <typename R, int N>
 cudaError_t fwd_impl(const cx<R>* W, const Problem& P, const Work<R>& w, cudaStream_t s, cudaEvent_t mid,
-                     bool norms) {
+                     bool norms, int* n_wsum, int* groups) {
   if constexpr (std::is_same<R, float>::value) {
     if (w.wt64) return fwd_wide_impl<N>(W, P, w, s, mid);
     // N = 192 and 256: the cluster's row tiles (77 / 134 KB per CTA) leave one or two
     // CTAs per SM, and the two passes are faster (measured at 256^2 x 64, 29 planes, 6
     // frequencies: 0.139 ms vs 0.122 ms)
     if constexpr (N <= 128) {
-      if (P.forward_single) return fwd_plane<R, N>(W, P, w, s, mid, norms);
+      if (P.forward_single) return fwd_plane<R, N>(W, P, w, s, mid, norms, n_wsum);
     }
   }
-  return P.fft_tile == 1 ? fwd_tiled<R, N, 1>(W, P, w, s, mid, norms) : fwd_tiled<R, N, 0>(W, P, w, s, mid, norms);
+  return P.fft_tile == 1 ? fwd_tiled<R, N, 1>(W, P, w, s, mid, norms, n_wsum, groups)
+                         : fwd_tiled<R, N, 0>(W, P, w, s, mid, norms, n_wsum, groups);
 }
 
 template <typename R, int N>
@@ -284,9 +308,9 @@ cudaError_t dense_impl(const cx<R>* in, cx<R>* out, long long planes, bool inver
   cudaError_t e;
   if (!inverse) {
     if ((e = rows_launch<R, N, false, cx<R>, 0, D32>(in, out, planes * N, tw, R(1), s)) != cudaSuccess) return e;
-    return cols_launch<R, N, false, 0, D32>(out, out, planes, tw, nullptr, 0, s);
+    return cols_launch<R, N, false, 0, D32>(out, out, planes, tw, s);
   }
-  if ((e = cols_launch<R, N, true, 0, D32>(in, out, planes, tw, nullptr, 0, s)) != cudaSuccess) return e;
+  if ((e = cols_launch<R, N, true, 0, D32>(in, out, planes, tw, s)) != cudaSuccess) return e;
   return rows_launch<R, N, true, cx<R>, 0, D32>(out, out, planes * N, tw, R(1.0 / ((double)N * N)), s);
 }
 
@@ -295,7 +319,7 @@ template <typename R, int N>
 cudaError_t xi_impl(const cx<R>* ut, cx<R>* out, const R* xi, long long planes, const cx<R>* tw, cudaStream_t s) {
   using DP = DensePass<R, N, 0>;
   constexpr bool D32 = sizeof(R) == 4;
-  cudaError_t e = cols_launch<R, N, true, 0, D32>(ut, out, planes, tw, nullptr, 0, s);
+  cudaError_t e = cols_launch<R, N, true, 0, D32>(ut, out, planes, tw, s);
   if (e != cudaSuccess) return e;
   const long long nrows = planes * N;
   constexpr size_t smem = 2 * sizeof(cx<R>) * LayIdx<Lay::ROW, N, DP::LINES, DP::SKEW>::ELEMS;
@@ -304,7 +328,7 @@ cudaError_t xi_impl(const cx<R>* ut, cx<R>* out, const R* xi, long long planes, 
   e = launch_pdl(k_rows_xi<R, N>, dim3((unsigned)((nrows + DP::LINES - 1) / DP::LINES)), dim3(DP::RT), smem, s, out,
                  xi, nrows, tw, R(1.0 / ((double)N * N)));
   if (e != cudaSuccess) return e;
-  return cols_launch<R, N, false, 0, D32>(out, out, planes, tw, nullptr, 0, s);
+  return cols_launch<R, N, false, 0, D32>(out, out, planes, tw, s);
 }
 
 template <typename R, int N>
@@ -315,7 +339,7 @@ cudaError_t pairs_impl(const R* xi, cx<R>* out, int m, const cx<R>* tw, cudaStre
   cudaError_t e = launch_pdl(k_fft_rows_pairs<R, N>, dim3((unsigned)((nrows + DP::LINES - 1) / DP::LINES)),
                              dim3(DP::RT), 0, s, xi, out, nrows, m & 1, tw);
   if (e != cudaSuccess) return e;
-  return cols_launch<R, N, false, 0, false>(out, out, np, tw, nullptr, 0, s);
+  return cols_launch<R, N, false, 0, false>(out, out, np, tw, s);
 }
 
 }  // namespace
@@ -362,9 +386,9 @@ cudaError_t launch_fft2_active(const Problem& P, const Work<float>& w, cudaStrea
 
 template <typename R>
 cudaError_t launch_fft2_forward(const cx<R>* W, const Problem& P, const Work<R>& w, cudaStream_t s,
-                                cudaEvent_t mid, bool norms) {
+                                cudaEvent_t mid, bool norms, int* n_wsum, int* groups) {
   switch (P.n) {
-#define FL_CASE(K) case K: return fwd_impl<R, K>(W, P, w, s, mid, norms);
+#define FL_CASE(K) case K: return fwd_impl<R, K>(W, P, w, s, mid, norms, n_wsum, groups);
     FL_SIZES(FL_CASE)
 #undef FL_CASE
     default: return cudaErrorInvalidValue;
@@ -418,9 +442,9 @@ cudaError_t launch_twiddles(cx<R>* tw, int n, cudaStream_t s) {
 }
 
 template cudaError_t launch_fft2_forward<double>(const double2*, const Problem&, const Work<double>&, cudaStream_t,
-                                                 cudaEvent_t, bool);
+                                                 cudaEvent_t, bool, int*, int*);
 template cudaError_t launch_fft2_forward<float>(const float2*, const Problem&, const Work<float>&, cudaStream_t,
-                                                cudaEvent_t, bool);
+                                                cudaEvent_t, bool, int*, int*);
 template cudaError_t launch_twiddles<double>(double2*, int, cudaStream_t);
 template cudaError_t launch_twiddles<float>(float2*, int, cudaStream_t);
 

@@ -11,6 +11,7 @@
 #include "fft.cuh"
 #include "modes.cuh"
 #include "pipeline.cuh"
+#include "twofloat.cuh"
 
 namespace fl {
 
@@ -57,12 +58,29 @@ __device__ __forceinline__ void load_twiddles(cx<R>* tw_s, const cx<R>* __restri
   for (int j = threadIdx.x; j < N; j += THREADS) tw_s[j] = tw[j];
 }
 
+// Sum of one float per thread over the NT threads of a block in two-float (the FP32 pipe): *out
+// on thread 0.  red: NT / 32 values.
+template <int NT> __device__ __forceinline__ void block_sum_ff(float x, ff* red, float2* out) {
+  const ff s = ff_warp_sum(ff{x, 0.f});
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ff t = red[0];
+    for (int w = 1; w < NT / 32; ++w) t = ff_add(t, red[w]);
+    *out = make_float2(t.hi, t.lo);
+  }
+}
+
 // ---- dense pass along x (rows): forward, or inverse with 1/N^2 scaling --------
+// grid (blocks, fields): field blockIdx.y has nrows rows.
 // TI: element type of `in` (cx<R>, or float2 read into an FP64 transform); D32: FftPlan's
-// factors in FP32 (IoPlan)
-template <typename R, int N, bool INV, typename TI = cx<R>, int T = 0, bool D32 = false>
+// factors in FP32 (IoPlan); WS (the data planes in FP32): also the block's sum of |in|^2 to wsum
+// [field][block].  clear (may be null): nclear words zeroed by block (0, 0), the counters of the
+// classification that follows.
+template <typename R, int N, bool INV, typename TI = cx<R>, int T = 0, bool D32 = false, bool WS = false>
 __global__ void __launch_bounds__((DensePass<R, N, T>::RT))
-k_fft_rows(const TI* __restrict__ in, cx<R>* out, long long nrows, const cx<R>* __restrict__ tw, R scale) {
+k_fft_rows(const TI* __restrict__ in, cx<R>* out, long long nrows, const cx<R>* __restrict__ tw, R scale,
+           unsigned* __restrict__ clear, int nclear, float2* __restrict__ wsum) {
   using DP = DensePass<R, N, T>;
   using PL = IoPlan<N, DP::MAXR, D32>;
   constexpr int LINES = DP::LINES;
@@ -71,28 +89,40 @@ k_fft_rows(const TI* __restrict__ in, cx<R>* out, long long nrows, const cx<R>* 
   load_stage_twiddles<R, PL, N, DP::RT>(tws, tw);  // a constant table: read while the predecessor drains
   pdl_wait();
   pdl_trigger();
+  if (clear && blockIdx.x == 0 && blockIdx.y == 0)
+    for (int i = threadIdx.x; i < nclear; i += DP::RT) clear[i] = 0u;
   const long long row0 = (long long)blockIdx.x * LINES;
   const int rows = (int)(nrows - row0 < LINES ? nrows - row0 : LINES);
-  const TI* src = in + row0 * N;
-  cx<R>* dst = out + row0 * N;
+  const TI* src = in + (blockIdx.y * nrows + row0) * N;
+  cx<R>* dst = out + (blockIdx.y * nrows + row0) * N;
+  float ws = 0.f;
   fft_lines_io<R, PL, N, INV, LINES, DP::RT, Lay::ROW, DP::SKEW>(
       buf, tws,
       [&](int b, int i) {
         if (b >= rows) return czero<R>();
-        if constexpr (std::is_same<TI, cx<R>>::value) return src[b * N + i];
-        else return from_d<R>(to_d(src[b * N + i]));
+        if constexpr (WS) {
+          const cx<R> v = src[b * N + i];
+          ws += v.x * v.x + v.y * v.y;
+          return v;
+        } else if constexpr (std::is_same<TI, cx<R>>::value) {
+          return src[b * N + i];
+        } else {
+          return from_d<R>(to_d(src[b * N + i]));
+        }
       },
       [&](int b, int i, cx<R> v) {
         if (b < rows) dst[b * N + i] = INV ? scale * v : v;
       });
+  if constexpr (WS) {
+    __shared__ ff red[DP::RT / 32];
+    block_sum_ff<DP::RT>(ws, red, wsum + (long long)blockIdx.y * gridDim.x + blockIdx.x);
+  }
 }
 
 // ---- dense pass along y (columns); grid (ceil(N/TC), planes); in == out is allowed ---
-// clear (may be null): nclear counters zeroed by block (0, 0) -- the barrier counters
-// of the classification kernel that follows
 template <typename R, int N, bool INV, int T = 0, bool D32 = false>
 __global__ void __launch_bounds__((DensePass<R, N, T>::CT))
-k_fft_cols(const cx<R>* in, cx<R>* out, const cx<R>* __restrict__ tw, unsigned* __restrict__ clear, int nclear) {
+k_fft_cols(const cx<R>* in, cx<R>* out, const cx<R>* __restrict__ tw) {
   using DP = DensePass<R, N, T>;
   using PL = IoPlan<N, DP::MAXR, D32>;
   constexpr int TC = DP::COLS;
@@ -101,8 +131,6 @@ k_fft_cols(const cx<R>* in, cx<R>* out, const cx<R>* __restrict__ tw, unsigned* 
   load_stage_twiddles<R, PL, N, DP::CT>(tws, tw);  // a constant table: read while the predecessor drains
   pdl_wait();
   pdl_trigger();
-  if (clear && blockIdx.x == 0 && blockIdx.y == 0)
-    for (int i = threadIdx.x; i < nclear; i += DP::CT) clear[i] = 0u;
   const int c0 = blockIdx.x * TC;
   const long long o = (long long)blockIdx.y * N * N + c0;
   const cx<R>* src = in + o;
@@ -118,10 +146,10 @@ k_fft_cols(const cx<R>* in, cx<R>* out, const cx<R>* __restrict__ tw, unsigned* 
 // grid (ceil(N/TC), G, n_omega): block (tile, g, om) transforms its columns of the planes
 // g ppg .. g ppg + ppg - 1 one after another and keeps sum |W~_k(nu)|^2 of its modes in
 // registers (a thread's last-stage outputs are the same modes in every plane); gnorm [om][G][N^2]
-// takes the sums, k_group_norms adds the groups.
+// takes the sums, k_classify_early adds the groups.
 // W~ is not written: it is needed only on the few columns that hold an active mode, and
 // k_fft_cols_active transforms those again once they are known.  256 planes of 256^2 (FP32, bound
-// by memory): columns 42 us + norms 32 us -> 30 us + 11 us (groups) + 14 us (active columns).
+// by memory): columns 42 us + norms 32 us -> 30 us, and 14 us for the active columns.
 // In FP64 the column pass is bound by the FP64 pipe and the norms run behind its tail: fused,
 // with W~ written, 128^2 x 71 planes x 3 frequencies took 820 us for the whole call, 765 us with the
 // two passes, so FP64 keeps those.
@@ -187,23 +215,36 @@ template <typename R, int N> struct ActivePass {
 };
 template <typename R, int N>
 __global__ void __launch_bounds__((ActivePass<R, N>::NT))
-k_fft_cols_active(cx<R>* wt, int m1, const int* __restrict__ cols, const int* __restrict__ ncol,
-                  const cx<R>* __restrict__ tw) {
+k_fft_cols_active(cx<R>* wt, int m1, const unsigned* __restrict__ colmask, const cx<R>* __restrict__ tw) {
   using AP = ActivePass<R, N>;
   using PL = typename AP::PL;
   constexpr int GC = AP::GC, GL = AP::GL;
   __shared__ cx<R> buf[PL::stages > 1 ? N * AP::LINES : 1];
   __shared__ cx<R> tws[PL::tw_elems];
+  __shared__ short cols[N];
   load_stage_twiddles<R, PL, N, AP::NT>(tws, tw);
   pdl_wait();
   pdl_trigger();
-  const int om = blockIdx.y, k0 = blockIdx.x * GL, nc = ncol[om];
+  // the list of the columns, from their mask
+  int nc = 0;
+  {
+    const unsigned* cm = colmask + 8 * blockIdx.y;
+    for (int i = threadIdx.x; i < N; i += AP::NT) {
+      int at = 0;
+      for (int w = 0; w < i / 32; ++w) at += __popc(cm[w]);
+      const unsigned m = cm[i / 32];
+      if (m >> (i & 31) & 1u) cols[at + __popc(m & ((1u << (i & 31)) - 1u))] = (short)i;
+    }
+    for (int w = 0; w < (N + 31) / 32; ++w) nc += __popc(cm[w]);
+    __syncthreads();
+  }
+  const int om = blockIdx.y, k0 = blockIdx.x * GL;
   const int nk = min(GL, m1 - k0);
   cx<R>* pl = wt + ((long long)om * m1 + k0) * N * N;
   for (int cb = blockIdx.z * GC; cb < nc; cb += gridDim.z * GC) {
     if (cb != (int)blockIdx.z * GC) __syncthreads();  // the previous tile has been read
     const int ncb = min(GC, nc - cb);
-    const int* cl = cols + om * N + cb;
+    const short* cl = cols + cb;
     // line b: column b % GC, plane b / GC (neighbouring columns are mostly neighbours in a row)
     fft_lines_io<R, PL, N, false, AP::LINES, AP::NT, Lay::COL, 0>(
         buf, tws,
@@ -270,44 +311,6 @@ k_mode_norms(const cx<R>* __restrict__ wt, double* __restrict__ norms, double* _
     __syncthreads();
   }
   if (threadIdx.x == 0) partial[(long long)om * gridDim.x + blockIdx.x] = red[0];
-}
-
-// the norms from the groups of k_fft_cols_norms, and their block sums: as k_mode_norms, the G
-// groups in place of the planes
-template <typename R>
-__global__ void __launch_bounds__(NORM_T)
-k_group_norms(const R* __restrict__ gnorm, double* __restrict__ norms, double* __restrict__ partial, int G, int N2,
-              unsigned long long* __restrict__ ctr) {
-  pdl_wait();
-  pdl_trigger();
-  __shared__ double red[NORM_T / 32];
-  const int om = blockIdx.y;
-  double sum = 0.0;
-  int bad = 0;
-  const int nu = blockIdx.x * NORM_T + threadIdx.x;
-  if (nu < N2) {
-    const R* p = gnorm + (long long)om * G * N2 + nu;
-    R acc = R(0);
-    int g = 0;
-    for (; g + 4 <= G; g += 4) {
-      R v[4];
-#pragma unroll
-      for (int t = 0; t < 4; ++t) v[t] = p[(long long)(g + t) * N2];
-      acc += (v[0] + v[1]) + (v[2] + v[3]);
-    }
-    for (; g < G; ++g) acc += p[(long long)g * N2];
-    norms[(long long)om * N2 + nu] = (double)acc;
-    sum = (double)acc;
-    bad = !isfinite(acc);
-  }
-  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
-  const int n_bad = __syncthreads_count(bad);
-  if (n_bad && threadIdx.x == 0) atomicAdd(ctr + C_NONFINITE, (unsigned long long)n_bad);
-  if (threadIdx.x < NORM_T / NORM_MB) {  // block sums of NORM_MB modes each, as k_mode_norms writes them
-    const int np = (N2 + NORM_MB - 1) / NORM_MB, at = blockIdx.x * (NORM_T / NORM_MB) + threadIdx.x;
-    if (at < np) partial[(long long)om * np + at] = red[2 * threadIdx.x] + red[2 * threadIdx.x + 1];
-  }
 }
 
 }  // namespace

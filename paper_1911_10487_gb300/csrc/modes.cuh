@@ -6,7 +6,7 @@
 
 #include <math.h>
 
-#include "common.cuh"
+#include "pipeline.cuh"
 
 namespace fl {
 
@@ -201,6 +201,33 @@ __device__ __forceinline__ void affine_scan_lanes(const double2* s, int len, dou
   for (int j = 0; j < EPL; ++j) {
     prev = q * prev + v[j];
     if (l0 + j < len) out[l0 + j] = prev;
+  }
+}
+
+// The column lists of the early classification (ColOut) from the masks: one warp per frequency,
+// on the last blocks of the grid, which have the fewest modes.  Called by every thread.
+__device__ __forceinline__ void column_list(const Problem& P, const ColOut& C) {
+  const int N = P.n, lane = threadIdx.x & 31;
+  if (threadIdx.x >= 32) return;
+  for (int om = gridDim.x - 1 - blockIdx.x; om < P.n_omega; om += gridDim.x) {
+    int base = 0;
+    unsigned seg = 0u;
+    for (int j0 = 0; j0 < N; j0 += 32) {
+      const unsigned m = C.mask[om * 8 + (j0 >> 5)];
+      const int j = j0 + lane;
+      const bool f = j < N && (m >> lane & 1u);
+      const int at = base + __popc(m & ((1u << lane) - 1u));
+      if (f) C.cols[om * N + at] = j;
+      if (j < N) C.colpos[om * N + j] = f ? at : -1;
+      seg |= f ? 1u << (j * 16 / N) : 0u;
+      base += __popc(m);
+    }
+    seg = __reduce_or_sync(0xffffffffu, seg);
+    if (lane == 0) {
+      C.colseg[om] = (int)seg;
+      C.ncol[om] = base;
+      atomicAdd(C.ctr + C_COLUMNS, (unsigned long long)base);
+    }
   }
 }
 

@@ -65,6 +65,7 @@ struct Problem {
   // its per-mode set-up runs on the FP32 pipe: k0, k0^2, g0 per frequency, kn^2, h_z,
   // z1, alpha_rel, zy[k] - zy_min and zy_min - z_top (z_top = z1 + (M - 1/2) h_z)
   float2 k0_f[MAX_OMEGA], k0sq_f[MAX_OMEGA], g0_f[MAX_OMEGA];
+  float2 dscale_f;
   float2 knsq_f, hz_f, z1_f, alpha_rel_f, d0_f;
   float2 zyd_f[MAX_M1];
 };
@@ -103,6 +104,7 @@ inline void derive_constants(Problem& P) {
     P.k0sq_f[j] = two_float(P.k0[j] * P.k0[j]);
     P.g0_f[j] = two_float(P.g0[j]);
   }
+  P.dscale_f = two_float(P.dscale);
   P.knsq_f = two_float(P.kn * P.kn);
   P.hz_f = two_float(P.hz);
   P.z1_f = two_float(P.z1);
@@ -129,9 +131,13 @@ template <typename R> struct Work {
   int* colpos;      // [n_omega][N] position of column nu1 in cols, or -1
   int* ncol;        // [n_omega]
   int* colseg;      // [n_omega] bit s: a column of the list in sixteenth s of the N
-  int* count;       // [n_omega] active modes
+  int* count;       // [n_omega] active modes (behind bar: see there)
   double* dnu;      // [n_omega] delta_nu
+  // bar, count and colmask are one region, zeroed by the first kernel of a reconstruction
+  // (clear_words(P) words from bar)
   unsigned* bar;    // [n_omega] barrier counters of the single-pass classification
+  unsigned* colmask;  // [n_omega][8] columns holding an active mode (atomic)
+  float2* wsum;     // [n_omega][WSUM_MAX(n, m1)] block sums of |W|^2 as two floats
   unsigned long long* ctr;  // [C_COUNT]
   const cx<R>* tw;  // [N] twiddles exp(-2 pi i j/N)
   double* alpha_out;  // [n_omega][N*N] or null
@@ -154,6 +160,24 @@ template <typename R> struct Work {
   const cx<R>* u0;
 };
 
+// words of the region from Work::bar that the first kernel zeroes
+inline int clear_words(const Problem& P) { return 10 * P.n_omega; }
+// block sums of |W|^2 per frequency (the first kernel has at least 4 rows per block, or 4 CTAs
+// per plane)
+inline size_t wsum_max(int n, int m1) { return (size_t)m1 * (n / 4 > 4 ? n / 4 : 4); }
+
+// FP32 data classified against delta_nu = dscale ||W|| with ||W|| summed over W itself as the
+// first kernel reads it (norms and flags in one kernel, slots by atomics); otherwise ||W|| comes
+// from the norms (Parseval) and the flags and slots in two more kernels
+inline bool classify_early(const Problem& P, bool fp64) { return !fp64 && !P.classify_single && P.regularizer != 1; }
+
+// What the solve writes of the column list on the early route (mask null: another kernel has)
+struct ColOut {
+  const unsigned* mask;
+  int *cols, *colpos, *ncol, *colseg;
+  unsigned long long* ctr;
+};
+
 // blocks of 1024 consecutive modes in the classification of an N x N grid
 inline int classify_blocks(int n) { return (n * n + 1023) / 1024; }
 
@@ -161,7 +185,7 @@ inline int classify_blocks(int n) { return (n * n + 1023) / 1024; }
 // from the base of the workspace, and its total size.  The context entry points
 // and the allocation-free entry point carve their workspace from this one layout.
 struct Layout {
-  size_t t12, prof, norms, partial, slot, act, flagbits, blkcnt, blkgz, colblk, cols, colpos, ncol, colseg, count, dnu, bar, total;
+  size_t t12, prof, norms, partial, slot, act, flagbits, blkcnt, blkgz, colblk, cols, colpos, ncol, colseg, count, dnu, bar, colmask, wsum, total;
   int n_partial;
 };
 // (the W~ part of the t12 region is sized for complex128 in both precisions, so
@@ -184,6 +208,11 @@ cudaError_t launch_pipeline(const Problem& P, const Work<R>& w, const void* W, v
 // pseudo-inverse damps nothing, so FP32 rounding of W~ would reach V~ amplified by
 // the inverse of each mode's singular value.
 inline bool wide_route(const Problem& P, bool fp64) { return !fp64 && P.regularizer == 1; }
+
+template <typename R> inline ColOut col_out(const Problem& P, const Work<R>& w) {
+  return ColOut{w.wt64 == nullptr && classify_early(P, sizeof(R) == 8) ? w.colmask : nullptr, w.cols, w.colpos, w.ncol,
+                w.colseg, w.ctr};
+}
 
 // Argument checks shared by the entry points (the rules of include/flatlayer.h).
 // ctx may be null: the status is returned without a message.  dense_solve: the call
@@ -219,9 +248,11 @@ cudaError_t opt_in_smem(SmemOptIn& flag, const void* kernel, size_t bytes, bool 
 // `mid` (may be null) is recorded on `s` between the two kernels of the stage
 // norms: also the per-mode norms and their block sums (k_mode_norms); without them the
 // column pass zeroes the barrier counters of the single-pass classification instead
+// (FP32 with classify_early: *n_wsum block sums of |W|^2 per frequency and *G groups of norms, 0
+// for W~ itself, are left for launch_classify_early instead)
 template <typename R>
 cudaError_t launch_fft2_forward(const cx<R>* W, const Problem& P, const Work<R>& w, cudaStream_t s,
-                                cudaEvent_t mid = nullptr, bool norms = true);
+                                cudaEvent_t mid, bool norms, int* n_wsum, int* G);
 // groups of planes of the pass that transforms the columns and sums the norms at once (0: the
 // columns, then k_mode_norms); that pass leaves W~ to launch_fft2_active, which transforms the
 // columns holding active modes once the classification has listed them
@@ -229,6 +260,9 @@ int norm_groups(const Problem& P, bool fp64);
 cudaError_t launch_fft2_active(const Problem& P, const Work<float>& w, cudaStream_t s);
 template <typename R>
 cudaError_t launch_mode_norms(const Problem& P, const Work<R>& w, cudaStream_t s);
+// classification from W's block sums (Work::wsum, n_wsum per frequency) and W~, or with G > 0
+// the group sums of k_fft_cols_norms in Work::prof: one kernel (classify_early)
+cudaError_t launch_classify_early(const Problem& P, const Work<float>& w, int n_wsum, int G, cudaStream_t s);
 // classification from the norms: two kernels (flags, scatter)
 template <typename R>
 cudaError_t launch_classify(const Problem& P, const Work<R>& w, cudaStream_t s);

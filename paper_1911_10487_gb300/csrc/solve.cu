@@ -302,6 +302,142 @@ k_classify_scatter(Problem P, const unsigned* __restrict__ flagbits, const int* 
 }
 
 // ------------------------------------------------------------------------------
+// early classification (FP32 data): delta_nu from ||W|| itself, whose block sums the forward
+// transform's first kernel takes as it reads W, so that no block waits for the norms of all
+// modes: one kernel sums the norms of its modes, tests them and lists the active ones.  Slots
+// come from an atomic counter per frequency and warp; which slot a mode takes differs from run
+// to run, and nothing a caller sees depends on it (each mode is solved alone, every sum over
+// modes follows the columns).  The columns' mask is OR-ed per frequency; the solve turns it into
+// the column list (column_list).  It replaces k_mode_norms, k_classify_flags and
+// k_classify_scatter: three dependent launches of latency each (128^2 x 64, one frequency: 5 + 5 +
+// 4 us of a 52 us call).
+// G = 0: norms of W~, EMB = 64 modes per block, four threads per mode, a quarter of the planes
+// each; G > 0: the G group sums of k_fft_cols_norms, 256 modes per block.
+// ------------------------------------------------------------------------------
+constexpr int ET = 256;
+template <bool GROUPS>
+__global__ void __launch_bounds__(ET)
+k_classify_early(Problem P, const float2* __restrict__ wt, const float* __restrict__ gnorm, int G,
+                 const float2* __restrict__ wsum, int n_wsum, unsigned* __restrict__ colmask, int* __restrict__ slot,
+                 int* __restrict__ act, int* __restrict__ count, double* __restrict__ dnu_out,
+                 unsigned long long* __restrict__ ctr) {
+  constexpr int EMB = GROUPS ? ET : ET / 4;  // modes per block
+  pdl_wait();
+  pdl_trigger();
+  __shared__ float part[4][ET / 4];
+  __shared__ ff red[ET / 32];
+  __shared__ unsigned cm[NWC];
+  __shared__ ff thr_s;
+  __shared__ int tot[3];  // active, grazing, not finite
+  const int om = blockIdx.y;
+  const int N = P.n, N2 = N * N, M1 = P.m1;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int q = GROUPS ? 0 : threadIdx.x / EMB, j = threadIdx.x % EMB;
+  const int nu = blockIdx.x * EMB + j;
+  if (threadIdx.x < NWC) cm[threadIdx.x] = 0u;
+  if (threadIdx.x < 3) tot[threadIdx.x] = 0;
+  // ||W||^2 in two-float: every block adds the block sums in the same order
+  ff s = ff{0.f, 0.f};
+  for (int i = threadIdx.x; i < n_wsum; i += ET) {
+    const float2 v = wsum[(long long)om * n_wsum + i];
+    s = ff_add(s, ff{v.x, v.y});
+  }
+  // the norms, in FP32 (planes in order within a quarter)
+  float acc = 0.f;
+  if (nu < N2) {
+    if constexpr (GROUPS) {
+      const float* p = gnorm + (long long)om * G * N2 + nu;
+      int g = 0;
+      for (; g + 4 <= G; g += 4) {
+        float v[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) v[t] = p[(long long)(g + t) * N2];
+        acc += (v[0] + v[1]) + (v[2] + v[3]);
+      }
+      for (; g < G; ++g) acc += p[(long long)g * N2];
+    } else {
+      const int k0 = q * M1 / 4, k1 = (q + 1) * M1 / 4;
+      const float2* p = wt + (long long)om * M1 * N2 + nu;
+      int k = k0;
+      for (; k + 8 <= k1; k += 8) {  // eight loads in flight
+        float2 v[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) v[t] = p[(long long)(k + t) * N2];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) acc += v[t].x * v[t].x + v[t].y * v[t].y;
+      }
+      for (; k < k1; ++k) {
+        const float2 v = p[(long long)k * N2];
+        acc += v.x * v.x + v.y * v.y;
+      }
+    }
+  }
+  s = ff_warp_sum(s);
+  if (lane == 0) red[wid] = s;
+  if (!GROUPS) part[q][j] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ff t = red[0];
+    for (int w = 1; w < ET / 32; ++w) t = ff_add(t, red[w]);
+    const ff ds = ff{P.dscale_f.x, P.dscale_f.y};
+    const bool fin = isfinite(t.hi);
+    const ff dnu = fin ? ff_mul(ds, ff_sqrt(t)) : t;
+    // a non-finite ||W|| (W holds a NaN or Inf) leaves delta_nu undefined: no mode passes
+    thr_s = fin ? ff_mul(dnu, dnu) : ff{INFINITY, 0.f};
+    if (blockIdx.x == 0) dnu_out[om] = ff_to(dnu);
+  }
+  __syncthreads();
+  if (threadIdx.x < EMB) {  // whole warps
+    const float nrm = GROUPS ? acc : (part[0][j] + part[1][j]) + (part[2][j] + part[3][j]);
+    const ff thr = thr_s;
+    bool on = false, graz = false, bad = false;
+    int i1 = 0;
+    if (nu < N2) {
+      const int i2 = nu / N;
+      i1 = nu - i2 * N;
+      const int m1 = i1 < N / 2 ? i1 : i1 - N, m2 = i2 < N / 2 ? i2 : i2 - N;
+      const int msq = m1 * m1 + m2 * m2;
+      graz = msq >= P.graz_lo[om] && msq <= P.graz_hi[om];
+      bad = !isfinite(nrm);
+      on = !graz && (P.alpha_mode == 1 || ff_gt(ff{nrm, 0.f}, thr));
+      if (on) atomicOr(&cm[i1 >> 5], 1u << (i1 & 31));
+    }
+    const unsigned bal = __ballot_sync(0xffffffffu, on);
+    const int na = __popc(bal);
+    const int ng = __popc(__ballot_sync(0xffffffffu, graz)), nb = __popc(__ballot_sync(0xffffffffu, bad));
+    int base = 0;
+    if (lane == 0) {
+      if (na) {
+        base = atomicAdd(count + om, na);
+        atomicAdd(&tot[0], na);
+      }
+      if (ng) atomicAdd(&tot[1], ng);
+      if (nb) atomicAdd(&tot[2], nb);
+    }
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (nu < N2) {
+      const int at = base + __popc(bal & ((1u << lane) - 1u));
+      slot[(long long)om * N2 + nu] = on ? at : -1;
+      if (on) act[(long long)om * N2 + at] = nu;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < NWC) {
+    // (the incident plane wave lives at nu = 0)
+    const unsigned m = cm[threadIdx.x] | (blockIdx.x == 0 && threadIdx.x == 0 ? 1u : 0u);
+    if (m) atomicOr(colmask + om * 8 + threadIdx.x, m);
+  } else if (threadIdx.x == 32) {
+    const int modes = min(EMB, N2 - (int)blockIdx.x * EMB);
+    atomicAdd(ctr + C_MODES, (unsigned long long)modes);
+    if (tot[0]) atomicAdd(ctr + C_ACTIVE, (unsigned long long)tot[0]);
+    if (tot[1]) atomicAdd(ctr + C_GRAZING, (unsigned long long)tot[1]);
+    if (tot[2]) atomicAdd(ctr + C_NONFINITE, (unsigned long long)tot[2]);
+    if (modes - tot[0] - tot[1]) atomicAdd(ctr + C_ZEROED, (unsigned long long)(modes - tot[0] - tot[1]));
+  }
+}
+static_assert(NWC <= 8, "column mask words per frequency");
+
+// ------------------------------------------------------------------------------
 // single-pass classification: one cooperative launch, grid (CB, n_omega), blocks of
 // CMB modes as above, in three phases separated by barriers over the blocks of a
 // frequency:
@@ -1094,9 +1230,10 @@ __global__ void __launch_bounds__(ST)
 k_solve(Problem P, const cx<B>* __restrict__ wt, const int* __restrict__ act,
         const int* __restrict__ count, const double* __restrict__ dnu_arr,
         cx<B>* __restrict__ prof, double* __restrict__ alpha_out, unsigned long long* __restrict__ ctr,
-        const void* __restrict__ ktab, const double* __restrict__ ktr) {
+        const void* __restrict__ ktab, const double* __restrict__ ktr, ColOut cols) {
   pdl_wait();
   pdl_trigger();
+  if (MIXED && cols.mask) column_list(P, cols);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Shared& S = *reinterpret_cast<Shared*>(smem_raw);
   const int N = P.n, n = P.m1, m = P.m;
@@ -1478,7 +1615,7 @@ cudaError_t solve_variant(const Problem& P, const Work<B>& w, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   return launch_pdl(k_solve<B, MIXED, SAMPLED>, dim3(solve_grid(P.solve_bps)), dim3(ST), smem, s, P,
                     (const cx<B>*)w.wt, (const int*)w.act, (const int*)w.count, (const double*)w.dnu, w.prof,
-                    w.alpha_out, w.ctr, w.ktab, w.ktr);
+                    w.alpha_out, w.ctr, w.ktab, w.ktr, col_out(P, w));
 }
 
 template <typename B, bool MIXED>
@@ -1491,6 +1628,14 @@ cudaError_t solve_impl(const Problem& P, const Work<B>& w, cudaStream_t s) {
 }
 
 }  // namespace
+
+cudaError_t launch_classify_early(const Problem& P, const Work<float>& w, int n_wsum, int G, cudaStream_t s) {
+  const int N2 = P.n * P.n, emb = G > 0 ? ET : ET / 4;
+  const dim3 g((N2 + emb - 1) / emb, P.n_omega);
+  return launch_pdl(G > 0 ? k_classify_early<true> : k_classify_early<false>, g, dim3(ET), 0, s, P,
+                    (const float2*)w.wt, (const float*)w.prof, G, (const float2*)w.wsum, n_wsum, w.colmask, w.slot,
+                    w.act, w.count, w.dnu, w.ctr);
+}
 
 template <typename R>
 cudaError_t launch_classify(const Problem& P, const Work<R>& w, cudaStream_t s) {

@@ -240,9 +240,11 @@ template <int RKE, int RK>
 __global__ void __launch_bounds__(RW * 32)
 k_solve_rank1_mixed(Problem P, const float2* __restrict__ wt, const double2* __restrict__ wt64,
                     const int* __restrict__ act, const int* __restrict__ count, const double* __restrict__ dnu_arr,
-                    float2* __restrict__ prof, double* __restrict__ alpha_out, unsigned long long* __restrict__ ctr) {
+                    float2* __restrict__ prof, double* __restrict__ alpha_out, unsigned long long* __restrict__ ctr,
+                    ColOut cols) {
   pdl_wait();
   pdl_trigger();
+  if (cols.mask) column_list(P, cols);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int N = P.n, n = P.m1, m = P.m;
   const long long N2 = (long long)N * N;
@@ -448,10 +450,10 @@ cudaError_t launch_solve_rank1(const Problem& P, const Work<R>& w, cudaStream_t 
     if (P.m <= 64 && P.m1 <= 32)
       return launch_pdl(k_solve_rank1_mixed<1, 2>, dim3(grid), dim3(RW * 32), 0, s, P, (const float2*)w.wt,
                         (const double2*)w.wt64, (const int*)w.act, (const int*)w.count, (const double*)w.dnu,
-                        (float2*)w.prof, w.alpha_out, w.ctr);
+                        (float2*)w.prof, w.alpha_out, w.ctr, col_out(P, w));
     return launch_pdl(k_solve_rank1_mixed<4, 4>, dim3(grid), dim3(RW * 32), 0, s, P, (const float2*)w.wt,
                       (const double2*)w.wt64, (const int*)w.act, (const int*)w.count, (const double*)w.dnu,
-                      (float2*)w.prof, w.alpha_out, w.ctr);
+                      (float2*)w.prof, w.alpha_out, w.ctr, col_out(P, w));
   } else {
     if (P.m <= 64 && P.m1 <= 32)
       return launch_pdl(k_solve_rank1<1, 2>, dim3(grid), dim3(RW * 32), 0, s, P, (const double2*)w.wt,
