@@ -997,7 +997,7 @@ ScratchLayout scratch_layout(const fs_diff_plan* p, int n_dir) {
   size_t off = 0;
   S.min = off; off = align_up(off + cxs * nd * F * P.m1 * N2);
   S.mout = off; off = align_up(off + cxs * 2 * nd * F * P.m * N2);
-  S.xsp = off; off = align_up(off + cxs * 2 * nd * F * P.m * N2);
+  S.xsp = off; off = align_up(off + cxs * 2 * F * P.m * N2);  // the VJP's V-bar, u-bar
   S.partial = off; off = align_up(off + 8 * nd * F * (size_t)p->gb);
   S.total = off;
   return S;
@@ -1091,19 +1091,16 @@ fs_status diff_jvp(fs_diff_plan* p, const char* tape, char* scr, int n_dir, cons
     cx<R>* dwt = (cx<R>*)(scr + S.min);
     cx<R>* dvt = (cx<R>*)(scr + S.mout);
     cx<R>* dut = dvt + (long long)nd * F * MN2;
-    cx<R>* dVx = (cx<R>*)(scr + S.xsp);
-    cx<R>* dux = dVx + (long long)nd * F * MN2;
     if ((e = launch_fft2_dense<R>((cx<R>*)dWc, dwt, P.n, (long long)nd * F * P.m1, false, tw, s)) != cudaSuccess)
       return cuda_fail(ctx, e, "fft2 dW");
     if ((e = launch_diff_jvp<R>(P, p->tables<R>(), nd, (const double2*)(tape + T.c), tape + T.g, dwt, la + F,
                                 dla ? dla + (long long)d0 * F : nullptr, dvt, dut, part, s)) != cudaSuccess)
       return cuda_fail(ctx, e, "diff jvp");
-    if ((e = launch_fft2_dense<R>(dvt, dVx, P.n, 2LL * nd * F * P.m, true, tw, s)) != cudaSuccess)
-      return cuda_fail(ctx, e, "ifft2 dV, du");
-    if ((e = launch_diff_jvp_point<R>(P, nd, (const cx<R>*)(tape + T.Vx), (const cx<R>*)(tape + T.ux),
-                                      (const R*)(tape + T.xi), dVx, dux, (R*)dxi + (long long)d0 * MN2, s)) !=
-        cudaSuccess)
-      return cuda_fail(ctx, e, "jvp pointwise");
+    if ((e = launch_ifft_cols<R>(dvt, dvt, P.n, 2LL * nd * F * P.m, tw, s)) != cudaSuccess)
+      return cuda_fail(ctx, e, "ifft dV, du");
+    if ((e = launch_diff_jvp_rows<R>(P, nd, dvt, dut, (const cx<R>*)(tape + T.Vx), (const cx<R>*)(tape + T.ux),
+                                     (const R*)(tape + T.xi), (R*)dxi + (long long)d0 * MN2, tw, s)) != cudaSuccess)
+      return cuda_fail(ctx, e, "jvp rows");
     if (dphi && (e = launch_reduce_rows(part, nd * (int)F, p->gb, dphi + (long long)d0 * F, s)) != cudaSuccess)
       return cuda_fail(ctx, e, "phi-dot");
   }

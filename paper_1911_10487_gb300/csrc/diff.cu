@@ -31,8 +31,9 @@
 // all N^2 modes are solved at a fixed alpha; the closed form is O(M1 + M) per mode, and the
 // kernels stream their fields (128^2 x 64, 32 data planes, 4 frequencies, mixed precision;
 // Cholesky factors before, this form now): forward 16.6 ms -> 58 us for 150 MB, VJP 8.6 ms ->
-// 95 us for 170 MB, 16 JVP directions 107.8 ms -> 557 us for 1.4 GB.  A block holds 32 consecutive modes (lanes: every
-// access to a plane is one 256-byte row) and splits the data planes and blocks of PB X planes
+// 95 us for 170 MB, 16 JVP directions 107.8 ms -> 480-495 us for 1.4 GB (565 us with four directions per pass over
+// the planes instead of eight).  A block holds 32 consecutive modes (lanes: every access to a plane
+// is one 256-byte row) and splits the data planes and blocks of PB X planes
 // over its DG warps, so that a small grid still fills the SMs.  The geometry (e, q, gamma, and
 // P and T at one plane of each block of PB) is tabulated once per plan in FP64; inside a block
 // of planes P and T follow by at most PB - 1 products, whose rounding is that of the
@@ -56,7 +57,7 @@ constexpr int PB = DIFF_PB;       // X planes per block of planes
 constexpr int DG = 8;             // warps per block
 constexpr int DT = 32 * DG;       // threads per block of the per-mode kernels
 constexpr int KC = DENSE_M1 / DG; // data planes per warp
-constexpr int JG = 4;             // JVP directions per pass over the planes
+constexpr int JG = 8;             // JVP directions per pass over the planes
 constexpr double AP_MAX = 1e290;  // alpha / tr above this: V~ = 0 in FP64
 static_assert(DENSE_M <= PB * DG, "one block of planes per warp");
 static_assert(DENSE_M1 == KC * DG, "data planes dealt over the warps");
@@ -80,6 +81,10 @@ template <> struct Wide<double> {
   __device__ __forceinline__ static T fma(T a, T b, T c) { return a * b + c; }
   __device__ __forceinline__ static T fmar(T a, double x, T c) { return a * x + c; }
   __device__ __forceinline__ static T wsum(T a) { return warp_sum(a); }
+  using Acc = double;  // a running sum of products
+  __device__ __forceinline__ static void mac(Acc& s, T a, double x) { s = a * x + s; }
+  __device__ __forceinline__ static T sum(Acc s) { return s; }
+  __device__ __forceinline__ static double mulround(T a, T b) { return a * b; }
   __device__ __forceinline__ static SC pack(T re, T im) { return make_double2(re, im); }
   __device__ __forceinline__ static void unpack(SC v, T& re, T& im) { re = v.x; im = v.y; }
 };
@@ -100,24 +105,31 @@ template <> struct Wide<float> {
   __device__ __forceinline__ static T fma(T a, T b, T c) { return ff_add(ff_mul(a, b), c); }
   __device__ __forceinline__ static T fmar(T a, float x, T c) { return ff_add(ff_mul_f(a, x), c); }
   __device__ __forceinline__ static T wsum(T a) { return ff_warp_sum(a); }
+  // compensated sums (Dot2, twofloat.cuh): two thirds of the operations of two-float sums
+  using Acc = dot2;
+  __device__ __forceinline__ static void mac(Acc& s, T a, float x) {
+    const float p = a.hi * x;
+    dot2_add(s, p, fmaf(a.lo, x, fmaf(a.hi, x, -p)));
+  }
+  __device__ __forceinline__ static T sum(Acc s) { return fast_two_sum(s.s, s.e); }
+  // the product rounded to FP32
+  __device__ __forceinline__ static float mulround(T a, T b) {
+    const float p = a.hi * b.hi;
+    return p + fmaf(a.lo, b.hi, fmaf(a.hi, b.lo, fmaf(a.hi, b.hi, -p)));
+  }
   __device__ __forceinline__ static SC pack(T re, T im) { return make_float4(re.hi, re.lo, im.hi, im.lo); }
   __device__ __forceinline__ static void unpack(SC v, T& re, T& im) { re = ff{v.x, v.y}; im = ff{v.z, v.w}; }
 };
 
 template <typename T> struct WC { T re, im; };  // complex value
 
-// 2^e for -252 <= e <= 252 as a product of two floats (both finite and normal)
-__device__ __forceinline__ float2 pow2_pair(int e) {
-  e = e < -252 ? -252 : (e > 252 ? 252 : e);
-  const int a = e / 2, b = e - a;
-  return make_float2(__int_as_float((a + 127) << 23), __int_as_float((b + 127) << 23));
-}
 __device__ __forceinline__ int exponent_of(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff) - 1023; }
 __device__ __forceinline__ int exponent_of(float x) { return (int)((__float_as_int(x) >> 23) & 0xff) - 127; }
 
 // A complex factor that multiplies wide values into outputs.  Two-float holds it as a
 // mantissa and a power of two: FP64 reaches factors (eta c, 2 Phi-bar N^2) outside the FP32
-// range whose products with the fields are inside it.
+// range whose products with the fields are inside it.  (The power goes to 2^+-126; a mantissa
+// takes the rest, to 2^252.)
 template <typename R> struct Factor;
 template <> struct Factor<double> {
   double re, im;
@@ -126,20 +138,21 @@ template <> struct Factor<double> {
 };
 template <> struct Factor<float> {
   ff re, im;
-  float2 s;
+  float s;
   __device__ __forceinline__ static Factor make(double2 v) {
     const double a = fmax(fabs(v.x), fabs(v.y));
     int e = 0;
     if (a > 0.0 && isfinite(a)) e = exponent_of(a);
-    e = e < -252 ? -252 : (e > 252 ? 252 : e);
+    e = e < -126 ? -126 : (e > 126 ? 126 : e);
     const double sc = __longlong_as_double((long long)(1023 - e) << 52);
     Factor f;
     f.re = ff_from(v.x * sc);
     f.im = ff_from(v.y * sc);
-    f.s = pow2_pair(e);
+    f.s = __int_as_float((e + 127) << 23);
     return f;
   }
-  __device__ __forceinline__ float out(ff x) const { return ((x.hi + x.lo) * s.x) * s.y; }
+  __device__ __forceinline__ float out(ff x) const { return (x.hi + x.lo) * s; }
+  __device__ __forceinline__ float out(float x) const { return x * s; }
 };
 
 // exponent of the largest of the warp's values (uniform; 0 for all zero): sums of squares
@@ -396,7 +409,7 @@ k_diff_forward(Problem P, DiffTables<R> tab, const cx<R>* __restrict__ wt, const
   const T zero = W::from(0.0);
   cx<R> b[KC];
   WC<T> e[KC];
-  WC<T> c = WC<T>{zero, zero};
+  typename W::Acc ca{}, cb{};
   R big = R(0);
 #pragma unroll
   for (int i = 0; i < KC; ++i) {
@@ -410,13 +423,14 @@ k_diff_forward(Problem P, DiffTables<R> tab, const cx<R>* __restrict__ wt, const
   }
 #pragma unroll
   for (int i = 0; i < KC; ++i) {  // c = e^H b
-    c.re = W::fmar(e[i].re, b[i].x, c.re);
-    c.im = W::fmar(e[i].re, b[i].y, c.im);
+    W::mac(ca, e[i].re, b[i].x);
+    W::mac(cb, e[i].re, b[i].y);
     if (cplx) {
-      c.re = W::fmar(e[i].im, b[i].y, c.re);
-      c.im = W::fmar(W::neg(e[i].im), b[i].x, c.im);
+      W::mac(ca, e[i].im, b[i].y);
+      W::mac(cb, W::neg(e[i].im), b[i].x);
     }
   }
+  WC<T> c = WC<T>{W::sum(ca), W::sum(cb)};
   sc[w][lane] = c;
   __syncthreads();
   double phi = 0.0;
@@ -601,7 +615,7 @@ k_diff_vjp(Problem P, DiffTables<R> tab, const double2* __restrict__ cs, const t
 // dwt: [nd][n_omega][M1][N2]; dvt, dut: [nd][n_omega][M][N2]
 // ---------------------------------------------------------------------------
 template <typename R>
-__global__ void __launch_bounds__(DT)
+__global__ void __launch_bounds__(DT, 2)
 k_diff_jvp(Problem P, DiffTables<R> tab, int nd, const double2* __restrict__ cs,
            const typename Wide<R>::SC* __restrict__ gs, const cx<R>* __restrict__ dwt,
            const double* __restrict__ alpha_arr, const double* __restrict__ dlog_alpha, cx<R>* __restrict__ dvt,
@@ -610,7 +624,10 @@ k_diff_jvp(Problem P, DiffTables<R> tab, int nd, const double2* __restrict__ cs,
   using T = typename W::T;
   __shared__ WC<T> sc[JG][DG][32];
   __shared__ Factor<R> cv_s[JG][32];
-  __shared__ double ps[JG][DG], pe[JG];  // Phi-dot: the warps' sums and the scalar part
+  // Phi-dot: the warps' sums (times 2^pexp; joined in FP64 by one thread) and the scalar part
+  __shared__ T ps[JG][DG];
+  __shared__ int pexp[JG][DG];
+  __shared__ double pe[JG];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int om = blockIdx.y, n = P.m1, m = P.m, F = P.n_omega;
   const long long N2 = (long long)P.n * P.n;
@@ -661,22 +678,24 @@ k_diff_jvp(Problem P, DiffTables<R> tab, int nd, const double2* __restrict__ cs,
         bb = fmax(bb, fmax(fabs(db[i].x), fabs(db[i].y)));
       }
       const int eb = warp_exponent(bb);
-      WC<T> c = WC<T>{zero, zero};
-      T dp = zero;
+      typename W::Acc cr{}, ci{}, da{};
 #pragma unroll
       for (int i = 0; i < KC; ++i) {
-        c.re = W::fmar(e[i].re, db[i].x, c.re);
-        c.im = W::fmar(e[i].re, db[i].y, c.im);
+        W::mac(cr, e[i].re, db[i].x);
+        W::mac(ci, e[i].re, db[i].y);
         if (cplx) {
-          c.re = W::fmar(e[i].im, db[i].y, c.re);
-          c.im = W::fmar(W::neg(e[i].im), db[i].x, c.im);
+          W::mac(cr, e[i].im, db[i].y);
+          W::mac(ci, W::neg(e[i].im), db[i].x);
         }
-        dp = W::fmar(g[i].re, scale_by(db[i].x, -eb), dp);
-        dp = W::fmar(g[i].im, scale_by(db[i].y, -eb), dp);
+        W::mac(da, g[i].re, scale_by(db[i].x, -eb));
+        W::mac(da, g[i].im, scale_by(db[i].y, -eb));
       }
-      sc[jd][w][lane] = c;
-      dp = W::wsum(dp);
-      if (lane == 0) ps[jd][w] = 2.0 * W::d(dp) * (pow2d(eb) * pow2d(eg));
+      sc[jd][w][lane] = WC<T>{W::sum(cr), W::sum(ci)};
+      const T dp = W::wsum(W::sum(da));
+      if (lane == 0) {
+        ps[jd][w] = dp;
+        pexp[jd][w] = eb + eg;
+      }
     }
     __syncthreads();
     if (w < JG && d0 + w < nd) {  // warp w: the scalars of direction d0 + w
@@ -697,7 +716,7 @@ k_diff_jvp(Problem P, DiffTables<R> tab, int nd, const double2* __restrict__ cs,
     __syncthreads();
     if (threadIdx.x < JG && d0 + threadIdx.x < nd) {
       double t = pe[threadIdx.x];
-      for (int i = 0; i < DG; ++i) t += ps[threadIdx.x][i];
+      for (int i = 0; i < DG; ++i) t += 2.0 * W::d(ps[threadIdx.x][i]) * pow2d(pexp[threadIdx.x][i]);
       partial[((long long)(d0 + threadIdx.x) * F + om) * gridDim.x + blockIdx.x] = t;
     }
     if (valid) {
@@ -712,8 +731,8 @@ k_diff_jvp(Problem P, DiffTables<R> tab, int nd, const double2* __restrict__ cs,
               if (jd < jn) {
                 const Factor<R>& cv = cv_s[jd][lane];
                 const long long o = (((long long)(d0 + jd) * F + om) * m + l) * N2 + nu;
-                dvt[o] = mk<R>(cv.out(W::mul(p, cv.re)), cv.out(W::mul(p, cv.im)));
-                dut[o] = mk<R>(cv.out(W::mul(pt, cv.re)), cv.out(W::mul(pt, cv.im)));
+                dvt[o] = mk<R>(cv.out(W::mulround(p, cv.re)), cv.out(W::mulround(p, cv.im)));
+                dut[o] = mk<R>(cv.out(W::mulround(pt, cv.re)), cv.out(W::mulround(pt, cv.im)));
               }
             }
           });
@@ -776,31 +795,6 @@ __global__ void k_diff_vjp_point(Problem P, const R* __restrict__ gxi, const cx<
       const cx<R> u = ux[om * MN2 + p], V = Vx[om * MN2 + p];
       Vb[om * MN2 + p] = gx * u;
       ub[om * MN2 + p] = gx * (V - x2 * u);
-    }
-  }
-}
-
-// dVx, dux: [nd][n_omega][M N^2];  dxi: [nd][M N^2]
-template <typename R>
-__global__ void k_diff_jvp_point(Problem P, int nd, const cx<R>* __restrict__ Vx, const cx<R>* __restrict__ ux,
-                                 const R* __restrict__ xis, const cx<R>* __restrict__ dVx,
-                                 const cx<R>* __restrict__ dux, R* __restrict__ dxi) {
-  const long long MN2 = (long long)P.m * P.n * P.n;
-  const int F = P.n_omega;
-  const R guard2 = (R)(P.eps_u * P.eps_u * F);
-  for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < MN2; p += (long long)gridDim.x * blockDim.x) {
-    R D = 0;
-    for (int om = 0; om < F; ++om) D += abs2(ux[om * MN2 + p]);
-    const R x = xis[p];
-    for (int d = 0; d < nd; ++d) {
-      R num = 0, dD = 0;
-      for (int om = 0; om < F; ++om) {
-        const cx<R> u = ux[om * MN2 + p], V = Vx[om * MN2 + p];
-        const cx<R> du = dux[((long long)d * F + om) * MN2 + p], dV = dVx[((long long)d * F + om) * MN2 + p];
-        num += du.x * V.x + du.y * V.y + u.x * dV.x + u.y * dV.y;
-        dD += R(2) * (u.x * du.x + u.y * du.y);
-      }
-      dxi[(long long)d * MN2 + p] = D < guard2 ? R(0) : (num - x * dD) / D;
     }
   }
 }
@@ -909,13 +903,6 @@ cudaError_t launch_diff_vjp_point(const Problem& P, const R* gxi, const cx<R>* V
   return cudaGetLastError();
 }
 
-template <typename R>
-cudaError_t launch_diff_jvp_point(const Problem& P, int nd, const cx<R>* Vx, const cx<R>* ux, const R* xis,
-                                  const cx<R>* dVx, const cx<R>* dux, R* dxi, cudaStream_t s) {
-  k_diff_jvp_point<R><<<point_grid((long long)P.m * P.n * P.n), 256, 0, s>>>(P, nd, Vx, ux, xis, dVx, dux, dxi);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_reduce_rows(const double* partial, int rows, int cols, double* out, cudaStream_t s) {
   k_reduce_rows<<<(rows + 3) / 4, 128, 0, s>>>(partial, rows, cols, out);
   return cudaGetLastError();
@@ -937,9 +924,7 @@ cudaError_t launch_reduce_rows(const double* partial, int rows, int cols, double
   template cudaError_t launch_diff_combine<R>(const Problem&, const cx<R>*, const cx<R>*, R*, R*, R*,               \
                                               cudaStream_t);                                                       \
   template cudaError_t launch_diff_vjp_point<R>(const Problem&, const R*, const cx<R>*, const cx<R>*, const R*,     \
-                                                cx<R>*, cx<R>*, cudaStream_t);                                     \
-  template cudaError_t launch_diff_jvp_point<R>(const Problem&, int, const cx<R>*, const cx<R>*, const R*,          \
-                                                const cx<R>*, const cx<R>*, R*, cudaStream_t);
+                                                cx<R>*, cx<R>*, cudaStream_t);
 FL_DIFF_INST(double)
 FL_DIFF_INST(float)
 #undef FL_DIFF_INST

@@ -66,9 +66,11 @@ cudaError_t launch_diff_combine(const Problem& P, const cx<R>* Vx, const cx<R>* 
 template <typename R>
 cudaError_t launch_diff_vjp_point(const Problem& P, const R* gxi, const cx<R>* Vx, const cx<R>* ux, const R* xis,
                                   cx<R>* Vb, cx<R>* ub, cudaStream_t s);
+// dxi of step 3 for nd directions: the inverse transform along x of dV~, dU~ ([nd][n_omega][M][N][N],
+// already transformed along y) with the pointwise derivative (fft_forward.cu)
 template <typename R>
-cudaError_t launch_diff_jvp_point(const Problem& P, int nd, const cx<R>* Vx, const cx<R>* ux, const R* xis,
-                                  const cx<R>* dVx, const cx<R>* dux, R* dxi, cudaStream_t s);
+cudaError_t launch_diff_jvp_rows(const Problem& P, int nd, const cx<R>* dv, const cx<R>* du, const cx<R>* Vx,
+                                 const cx<R>* ux, const R* xis, R* dxi, const cx<R>* tw, cudaStream_t s);
 cudaError_t launch_reduce_rows(const double* partial, int rows, int cols, double* out, cudaStream_t s);
 
 }  // namespace fl

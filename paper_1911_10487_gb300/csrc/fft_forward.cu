@@ -11,6 +11,7 @@
 //                   gathers the solved profiles of the active modes only and
 //                   transforms only the columns nu1 that hold a nonzero mode; the
 //                   row pass scatters those columns and transforms full rows.
+#include "diff.cuh"
 #include "fft_pass.cuh"
 
 namespace fl {
@@ -198,6 +199,87 @@ k_rows_xi(cx<R>* __restrict__ data, const R* __restrict__ xi, long long nrows, c
       });
 }
 
+// ---- inverse rows of a direction's fields with the derivative of step 3 ----------
+// Block (d, b): LINES rows of X of direction d; for every frequency the rows of dV~ and dU~ are
+// transformed along x in the tile and each thread adds its voxels' terms
+//   num = Re(conj(du) V + conj(u) dV),  dD = 2 Re(conj(u) du),  D = |u|^2
+// with V and u of the tape (the directions of a row block run side by side and share them in
+// L2): dxi = (num - xi dD) / D.  Writing dV and du and reading them back for a pointwise kernel took
+// 2.1 of 6.5 GB of a 16-direction call at 128^2 x 64, 4 frequencies (FP32): rows 307 us + point
+// 212 us before, 417 us now.  In FP32 V and u are loaded before the rows are transformed, and
+// 256 threads share a tile from N = 96 on, so that more loads are in flight (420 us without the
+// first at 128 threads, 436 us with it).
+template <typename R, int N> struct JvpPass {
+  static constexpr bool F32 = sizeof(R) == 4;
+  using PL = IoPlan<N, F32 || N != 256 ? 16 : 8, F32>;
+  static constexpr int NT = F32 ? (N >= 96 ? 256 : 128) : (N >= 192 ? 128 : 64);
+  static constexpr int LINES = F32 ? (N <= 16 ? 16 : 8) : (N <= 16 ? 8 : 4);
+  static constexpr int E = LINES * N, PER = (E + NT - 1) / NT;
+  using IX = LayIdx<Lay::ROW, N, 2 * LINES, 16>;
+};
+template <typename R, int N>
+__global__ void __launch_bounds__((JvpPass<R, N>::NT))
+k_jvp_rows(Problem P, const cx<R>* __restrict__ dv, const cx<R>* __restrict__ du, const cx<R>* __restrict__ Vx,
+           const cx<R>* __restrict__ ux, const R* __restrict__ xis, R* __restrict__ dxi, const cx<R>* __restrict__ tw) {
+  using JP = JvpPass<R, N>;
+  using PL = typename JP::PL;
+  using IX = typename JP::IX;
+  constexpr int LINES = JP::LINES, NT = JP::NT, E = JP::E, PER = JP::PER;
+  constexpr int PRE = JP::F32 ? PER : 0;  // FP64: no registers to spare
+  __shared__ cx<R> buf[IX::ELEMS];
+  __shared__ cx<R> tws[PL::tw_elems];
+  load_stage_twiddles<R, PL, N, NT>(tws, tw);
+  pdl_wait();
+  pdl_trigger();
+  const long long nrows = (long long)P.m * N, MN2 = nrows * N;
+  const long long row0 = (long long)blockIdx.y * LINES;
+  const int rows = (int)(nrows - row0 < LINES ? nrows - row0 : LINES);
+  const R scale = R(P.inv_n2), guard2 = R(P.u_guard);
+  R num[PER], dD[PER], D[PER];
+#pragma unroll
+  for (int p = 0; p < PER; ++p) num[p] = dD[p] = D[p] = R(0);
+  for (int om = 0; om < P.n_omega; ++om) {
+    const long long at = ((long long)blockIdx.x * P.n_omega + om) * MN2 + row0 * N;
+    const cx<R>*a = dv + at, *b = du + at;
+    const cx<R>*V = Vx + om * MN2 + row0 * N, *u = ux + om * MN2 + row0 * N;
+    cx<R> pv[PRE + 1], pu[PRE + 1];  // on their way while the rows are transformed
+#pragma unroll
+    for (int p = 0; p < PRE; ++p) {
+      const int e = threadIdx.x + p * NT;
+      pv[p] = e < rows * N ? V[e] : czero<R>();
+      pu[p] = e < rows * N ? u[e] : czero<R>();
+    }
+    if (om > 0) __syncthreads();  // the tile has been read
+    fft_lines_io<R, PL, N, true, 2 * LINES, NT, Lay::ROW, 16>(
+        buf, tws,
+        [&](int line, int i) {
+          const int bl = line >= LINES ? line - LINES : line;
+          return bl < rows ? (line >= LINES ? b : a)[bl * N + i] : czero<R>();
+        },
+        [&](int line, int i, cx<R> v) { buf[IX::at(line, i)] = v; });
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      const int e = threadIdx.x + p * NT;
+      if (e < rows * N) {
+        const cx<R> x = scale * buf[IX::at(e / N, e % N)], y = scale * buf[IX::at(LINES + e / N, e % N)];
+        const cx<R> v = p < PRE ? pv[p] : V[e], w = p < PRE ? pu[p] : u[e];
+        num[p] += y.x * v.x + y.y * v.y + w.x * x.x + w.y * x.y;
+        dD[p] += R(2) * (w.x * y.x + w.y * y.y);
+        D[p] += abs2(w);
+      }
+    }
+  }
+#pragma unroll
+  for (int p = 0; p < PER; ++p) {
+    const int e = threadIdx.x + p * NT;
+    if (e < rows * N) {
+      const long long o = row0 * N + e;
+      dxi[blockIdx.x * MN2 + o] = D[p] < guard2 ? R(0) : (num[p] - xis[o] * dD[p]) / D[p];
+    }
+  }
+}
+
 template <typename R, int N, bool INV, typename TI, int T, bool D32>
 cudaError_t rows_launch(const TI* in, cx<R>* out, long long nrows, const cx<R>* tw, R scale, cudaStream_t s) {
   using DP = DensePass<R, N, T>;
@@ -314,6 +396,15 @@ cudaError_t dense_impl(const cx<R>* in, cx<R>* out, long long planes, bool inver
   return rows_launch<R, N, true, cx<R>, 0, D32>(out, out, planes * N, tw, R(1.0 / ((double)N * N)), s);
 }
 
+template <typename R, int N>
+cudaError_t jvp_rows_impl(const Problem& P, int nd, const cx<R>* dv, const cx<R>* du, const cx<R>* Vx, const cx<R>* ux,
+                          const R* xis, R* dxi, const cx<R>* tw, cudaStream_t s) {
+  using JP = JvpPass<R, N>;
+  const long long nrows = (long long)P.m * N;
+  return launch_pdl(k_jvp_rows<R, N>, dim3((unsigned)nd, (unsigned)((nrows + JP::LINES - 1) / JP::LINES)), dim3(JP::NT),
+                    0, s, P, dv, du, Vx, ux, xis, dxi, tw);
+}
+
 // F[xi F^-1 ut] -> out, M planes
 template <typename R, int N>
 cudaError_t xi_impl(const cx<R>* ut, cx<R>* out, const R* xi, long long planes, const cx<R>* tw, cudaStream_t s) {
@@ -407,6 +498,34 @@ cudaError_t launch_fft2_dense(const cx<R>* in, cx<R>* out, int n, long long plan
 }
 template cudaError_t launch_fft2_dense<double>(const double2*, double2*, int, long long, bool, const double2*, cudaStream_t);
 template cudaError_t launch_fft2_dense<float>(const float2*, float2*, int, long long, bool, const float2*, cudaStream_t);
+
+template <typename R>
+cudaError_t launch_ifft_cols(const cx<R>* in, cx<R>* out, int n, long long planes, const cx<R>* tw, cudaStream_t s) {
+  switch (n) {
+#define FL_CASE(K) case K: return cols_launch<R, K, true, 0, sizeof(R) == 4>(in, out, planes, tw, s);
+    FL_SIZES(FL_CASE)
+#undef FL_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+template cudaError_t launch_ifft_cols<double>(const double2*, double2*, int, long long, const double2*, cudaStream_t);
+template cudaError_t launch_ifft_cols<float>(const float2*, float2*, int, long long, const float2*, cudaStream_t);
+
+template <typename R>
+cudaError_t launch_diff_jvp_rows(const Problem& P, int nd, const cx<R>* dv, const cx<R>* du, const cx<R>* Vx,
+                                 const cx<R>* ux, const R* xis, R* dxi, const cx<R>* tw, cudaStream_t s) {
+  switch (P.n) {
+#define FL_CASE(K) case K: return jvp_rows_impl<R, K>(P, nd, dv, du, Vx, ux, xis, dxi, tw, s);
+    FL_SIZES(FL_CASE)
+#undef FL_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+template cudaError_t launch_diff_jvp_rows<double>(const Problem&, int, const double2*, const double2*, const double2*,
+                                                  const double2*, const double*, double*, const double2*,
+                                                  cudaStream_t);
+template cudaError_t launch_diff_jvp_rows<float>(const Problem&, int, const float2*, const float2*, const float2*,
+                                                 const float2*, const float*, float*, const float2*, cudaStream_t);
 
 template <typename R>
 cudaError_t launch_xi_transform(const cx<R>* ut, cx<R>* out, const R* xi, int n, long long planes, const cx<R>* tw,

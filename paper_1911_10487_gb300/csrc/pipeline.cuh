@@ -286,6 +286,9 @@ cudaError_t launch_twiddles(cx<R>* tw, int n, cudaStream_t s);
 template <typename R>
 cudaError_t launch_fft2_dense(const cx<R>* in, cx<R>* out, int n, long long planes, bool inverse, const cx<R>* tw,
                               cudaStream_t s);
+// the column pass of the inverse transform alone (unscaled)
+template <typename R>
+cudaError_t launch_ifft_cols(const cx<R>* in, cx<R>* out, int n, long long planes, const cx<R>* tw, cudaStream_t s);
 // F[xi F^-1 ut] -> out for `planes` planes (xi [planes][N][N]; out must not be ut)
 template <typename R>
 cudaError_t launch_xi_transform(const cx<R>* ut, cx<R>* out, const R* xi, int n, long long planes, const cx<R>* tw,
