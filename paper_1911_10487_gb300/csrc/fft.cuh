@@ -354,7 +354,9 @@ __device__ __forceinline__ void io_middle(cx<R>* buf, const cx<R>* tws) {
 // First stage: ld(b, i) gives element i of line b; its outputs go to the tile (then a
 // barrier and the middle stages), ready for the last stage.  Only for plans of two stages
 // or more.  PRE: an index load first: the thread's ld.pre(b, i) (ints), then its ld(b, i, index).
-template <typename R, class PL, int N, bool INV, int LINES, int THREADS, Lay L, int SKEW, bool PRE = false, class Ld>
+// TILE: ld reads the same tile (a barrier between the loads and the results).
+template <typename R, class PL, int N, bool INV, int LINES, int THREADS, Lay L, int SKEW, bool PRE = false,
+          bool TILE = false, class Ld>
 __device__ __forceinline__ void io_first(cx<R>* buf, const cx<R>* tws, Ld ld) {
   using IX = LayIdx<L, N, LINES, SKEW>;
   constexpr int RAD = PL::radix(0), NB = N / RAD, TOTAL = LINES * NB;
@@ -388,6 +390,7 @@ __device__ __forceinline__ void io_first(cx<R>* buf, const cx<R>* tws, Ld ld) {
       }
     }
   }
+  if constexpr (TILE) __syncthreads();
 #pragma unroll
   for (int p = 0; p < PER; ++p) {
     const int t = threadIdx.x + p * THREADS;

@@ -162,41 +162,98 @@ k_fft_rows_pairs(const R* __restrict__ xi, cx<R>* __restrict__ out, long long nr
 
 // ---- rows: inverse along x, times xi, forward along x --------------------------------
 // The middle of F[xi F^-1 U~]: between the two column passes everything happens within a
-// row, so one kernel reads and writes the planes once (three kernels before: inverse rows,
-// the product, forward rows; 128^2 x 64 FP64 per iteration 116 us -> 113 us, bound by the FP64
-// pipe; FP32 by memory, where the passes saved count).
+// row, so one kernel reads and writes the planes once.  The product happens between the two
+// transforms' registers: outputs j + r N/R1 of the last inverse stage (radix R1) for j = k, k + N/R0, ..
+// are the inputs k + r N/R0 of butterfly k of the first forward stage (radix R0) when R1 divides R0, and
+// a thread that runs those R0/R1 inverse butterflies goes on with the forward one.  Other plans write
+// the product to the tile in place, from registers.  Either way the kernel needs one tile: a second
+// one for the product left five 64-thread blocks per SM at N = 128 in FP64 (86 registers), and one more
+// crossing.  Bound by the FP64 pipe: 128^2 x 64 FP64 110 us -> 96 us (85% of that pipe's rate).
+template <typename R, int N> struct RowsXi {
+  using DP = DensePass<R, N, 0>;
+  using PL = IoPlan<N, DP::MAXR, sizeof(R) == 4>;
+  using IX = LayIdx<Lay::ROW, N, DP::LINES, DP::SKEW>;
+  static constexpr int S = PL::stages - 1, R0 = PL::radix(0), R1 = PL::radix(S);
+  static constexpr bool REG = S == 1 && R0 % R1 == 0;
+};
 template <typename R, int N>
 __global__ void __launch_bounds__((DensePass<R, N, 0>::RT))
 k_rows_xi(cx<R>* __restrict__ data, const R* __restrict__ xi, long long nrows, const cx<R>* __restrict__ tw,
           R scale) {
-  using DP = DensePass<R, N, 0>;
-  using PL = IoPlan<N, DP::MAXR, sizeof(R) == 4>;
-  constexpr int LINES = DP::LINES;
-  using IX = LayIdx<Lay::ROW, N, LINES, DP::SKEW>;
-  extern __shared__ __align__(16) unsigned char rows_xi_smem[];  // 2 IX::ELEMS elements
+  using RX = RowsXi<R, N>;
+  using DP = typename RX::DP;
+  using PL = typename RX::PL;
+  using IX = typename RX::IX;
+  constexpr int LINES = DP::LINES, NT = DP::RT, SK = DP::SKEW, S = RX::S, R0 = RX::R0, R1 = RX::R1;
+  extern __shared__ __align__(16) unsigned char rows_xi_smem[];  // IX::ELEMS elements
   cx<R>* buf = reinterpret_cast<cx<R>*>(rows_xi_smem);
-  cx<R>* mid = buf + IX::ELEMS;
   __shared__ cx<R> tws[PL::tw_elems];
-  load_stage_twiddles<R, PL, N, DP::RT>(tws, tw);
+  load_stage_twiddles<R, PL, N, NT>(tws, tw);
   pdl_wait();
   pdl_trigger();
   const long long row0 = (long long)blockIdx.x * LINES;
   const int rows = (int)(nrows - row0 < LINES ? nrows - row0 : LINES);
   cx<R>* d = data + row0 * N;
   const R* x = xi + row0 * N;
-  fft_lines_io<R, PL, N, true, LINES, DP::RT, Lay::ROW, DP::SKEW>(
-      buf, tws, [&](int b, int i) { return b < rows ? d[b * N + i] : czero<R>(); },
-      [&](int b, int i, cx<R> v) {
-        const R f = b < rows ? x[b * N + i] : R(0);
-        v = scale * v;
-        mid[IX::at(b, i)] = mk<R>(f * v.x, f * v.y);
-      });
-  __syncthreads();
-  fft_lines_io<R, PL, N, false, LINES, DP::RT, Lay::ROW, DP::SKEW>(
-      buf, tws, [&](int b, int i) { return mid[IX::at(b, i)]; },
-      [&](int b, int i, cx<R> v) {
-        if (b < rows) d[b * N + i] = v;
-      });
+  auto ld = [&](int b, int i) { return b < rows ? d[b * N + i] : czero<R>(); };
+  auto st = [&](int b, int i, cx<R> v) {
+    if (b < rows) d[b * N + i] = v;
+  };
+  auto ldx = [&](int b, int i) { return b < rows ? scale * x[b * N + i] : R(0); };
+  if constexpr (S == 0) {  // a thread owns whole lines
+    for (int b = threadIdx.x; b < rows; b += NT) {
+      cx<R> v[R0];
+#pragma unroll
+      for (int r = 0; r < R0; ++r) v[r] = ld(b, r);
+      Dft<R, true>::template run<R0>(v);
+#pragma unroll
+      for (int r = 0; r < R0; ++r) v[r] = ldx(b, r) * v[r];
+      Dft<R, false>::template run<R0>(v);
+#pragma unroll
+      for (int r = 0; r < R0; ++r) st(b, r, v[r]);
+    }
+  } else {
+    io_first<R, PL, N, true, LINES, NT, Lay::ROW, SK>(buf, tws, ld);
+    // the last inverse stage and the product; in place once every thread has read its inputs
+    constexpr int RAD = RX::REG ? R0 : R1, NB = N / RAD, TOTAL = LINES * NB, PER = (TOTAL + NT - 1) / NT;
+    cx<R> v[PER][RAD];
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      const int t = threadIdx.x + p * NT;
+      if (TOTAL % NT == 0 || t < TOTAL) {
+        int b, k;
+        IX::map(t, NB, b, k);
+        R f[RAD];
+#pragma unroll
+        for (int r = 0; r < RAD; ++r) f[r] = ldx(b, k + r * NB);
+        constexpr int Q = RAD / R1;  // inverse butterflies k, k + NB, ..
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+          cx<R> y[R1];
+          io_butterfly<R, PL, N, true, LINES, Lay::ROW, SK, S>(buf, tws, b, k + q * NB, y);
+#pragma unroll
+          for (int r = 0; r < R1; ++r) v[p][q + r * Q] = f[q + r * Q] * y[r];
+        }
+        if constexpr (RX::REG) Dft<R, false>::template run<R0>(v[p]);
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      const int t = threadIdx.x + p * NT;
+      if (TOTAL % NT == 0 || t < TOTAL) {
+        int b, k;
+        IX::map(t, NB, b, k);
+#pragma unroll
+        for (int r = 0; r < RAD; ++r) buf[IX::at(b, RX::REG ? k * R0 + r : k + r * NB)] = v[p][r];
+      }
+    }
+    __syncthreads();
+    if constexpr (!RX::REG)
+      io_first<R, PL, N, false, LINES, NT, Lay::ROW, SK, false, true>(
+          buf, tws, [&](int b, int i) { return buf[IX::at(b, i)]; });
+    io_last<R, PL, N, false, LINES, NT, Lay::ROW, SK>(buf, tws, st);
+  }
 }
 
 // ---- inverse rows of a direction's fields with the derivative of step 3 ----------
@@ -413,7 +470,7 @@ cudaError_t xi_impl(const cx<R>* ut, cx<R>* out, const R* xi, long long planes, 
   cudaError_t e = cols_launch<R, N, true, 0, D32>(ut, out, planes, tw, s);
   if (e != cudaSuccess) return e;
   const long long nrows = planes * N;
-  constexpr size_t smem = 2 * sizeof(cx<R>) * LayIdx<Lay::ROW, N, DP::LINES, DP::SKEW>::ELEMS;
+  constexpr size_t smem = sizeof(cx<R>) * LayIdx<Lay::ROW, N, DP::LINES, DP::SKEW>::ELEMS;
   static SmemOptIn attr;
   if ((e = opt_in_smem(attr, (const void*)k_rows_xi<R, N>, smem)) != cudaSuccess) return e;
   e = launch_pdl(k_rows_xi<R, N>, dim3((unsigned)((nrows + DP::LINES - 1) / DP::LINES)), dim3(DP::RT), smem, s, out,
