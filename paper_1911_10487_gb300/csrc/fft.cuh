@@ -18,7 +18,10 @@
 // inverse = unnormalised exp(+i...) DFT (the caller applies 1/N^2).
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
+#include "pair.cuh"
 
 namespace fl {
 
@@ -73,15 +76,19 @@ template <Lay L, int N, int LINES, int SKEW> struct LayIdx {
 
 template <typename R, bool INV> struct Dft {
   using C = cx<R>;
+  // a + rot90<I>(b)
+  template <bool I> __device__ __forceinline__ static C add_rot(C a, C b) {
+    return I ? mk<R>(a.x - b.y, a.y + b.x) : mk<R>(a.x + b.y, a.y - b.x);
+  }
   __device__ __forceinline__ static void d2(C* v) {
     C a = v[0], b = v[1];
     v[0] = a + b; v[1] = a - b;
   }
   __device__ __forceinline__ static void d4(C* v) {
     C s02 = v[0] + v[2], d02 = v[0] - v[2];
-    C s13 = v[1] + v[3], d13 = rot90<INV>(v[1] - v[3]);
+    C s13 = v[1] + v[3], e = v[1] - v[3];
     v[0] = s02 + s13; v[2] = s02 - s13;
-    v[1] = d02 + d13; v[3] = d02 - d13;
+    v[1] = add_rot<INV>(d02, e); v[3] = add_rot<!INV>(d02, e);
   }
   // x w16^e, w16 = exp(-2 pi i/16) (conjugated for the inverse); e is a constant (w16^0
   // and w16^4 = -i cost no arithmetic: 10 of 170 FP64 operations of a 16-point DFT, on a
@@ -89,6 +96,12 @@ template <typename R, bool INV> struct Dft {
   __device__ __forceinline__ static C tw16(C x, int e) {
     if (e == 0) return x;
     if (e == 4) return rot90<INV>(x);
+    if constexpr (std::is_same<R, f2>::value) {  // packed products are not contracted
+      if (e == 8) return mk<R>(-x.x, -x.y);
+      if (e == 12) return rot90<!INV>(x);
+      const double cd = cos16(e), sd = INV ? sin16(e) : -sin16(e);
+      return mk<R>(fma(x.y, R(-sd), x.x * R(cd)), fma(x.x, R(sd), x.y * R(cd)));
+    }
     const R c = R(cos16(e)), sn = INV ? R(sin16(e)) : -R(sin16(e));
     return mk<R>(x.x * c - x.y * sn, x.x * sn + x.y * c);
   }
@@ -135,18 +148,19 @@ template <typename R, bool INV> struct Dft {
     C p0 = b0, p1 = b1;  // w4^(3 k1) b
 #pragma unroll
     for (int k1 = 0; k1 < 4; ++k1) {
-      const C t1 = tw16(a1, k1), t2 = tw16(p0, 2 * k1), t3 = tw16(p1, 3 * k1);
+      constexpr bool PK = std::is_same<R, f2>::value;  // packed: w4^(3 k1) and the twiddle in one product
+      const C t1 = tw16(a1, k1), t2 = tw16(PK ? b0 : p0, PK ? 14 * k1 % 16 : 2 * k1),
+              t3 = tw16(PK ? b1 : p1, PK ? 15 * k1 % 16 : 3 * k1);
       if constexpr (E > 1) {
         C z[4] = {a0, t1, t2, t3};
         d4(z);
 #pragma unroll
         for (int k2 = 0; k2 < 4; ++k2) v[k1 + 4 * k2] = z[k2];
       } else {
-        const C d = rot90<INV>(mk<R>(-t3.x, -t3.y));
         v[k1] = a0 + t3;
         v[k1 + 8] = a0 - t3;
-        v[k1 + 4] = a0 + d;
-        v[k1 + 12] = a0 - d;
+        v[k1 + 4] = add_rot<!INV>(a0, t3);
+        v[k1 + 12] = add_rot<INV>(a0, t3);
       }
       p0 = rot90<!INV>(p0);  // w4^3 = conj(w4)
       p1 = rot90<!INV>(p1);
@@ -160,13 +174,13 @@ template <typename R, bool INV> struct Dft {
       const C t = mk<R>(fma(R(-0.5), s.x, v[0].x), fma(R(-0.5), s.y, v[0].y));
       v[0] = v[0] + s;
       v[1] = mk<R>(fma(h, e.x, t.x), fma(h, e.y, t.y));
-      v[2] = mk<R>(fma(-h, e.x, t.x), fma(-h, e.y, t.y));
-      return;
+      v[2] = mk<R>(fma(R(-0.86602540378443864676), e.x, t.x), fma(R(-0.86602540378443864676), e.y, t.y));
+    } else {
+      C s = v[1] + v[2];
+      C t = v[0] - R(0.5) * s;
+      C d = h * rot90<INV>(v[1] - v[2]);
+      v[0] = v[0] + s; v[1] = t + d; v[2] = t - d;
     }
-    C s = v[1] + v[2];
-    C t = v[0] - R(0.5) * s;
-    C d = h * rot90<INV>(v[1] - v[2]);
-    v[0] = v[0] + s; v[1] = t + d; v[2] = t - d;
   }
   // 12 points as 3 x 4 without twiddles (Good-Thomas): n = 4 n1 + 3 n2, k = 4 k1 + 9 k2
   // (mod 12) gives n k = 4 n1 k1 + 3 n2 k2 (mod 12)
@@ -298,6 +312,19 @@ __device__ __forceinline__ void load_stage_twiddles(cx<R>* tws, const cx<R>* __r
   }
 }
 
+// the same table, each entry for both values of a pair
+template <class PL, int N, int THREADS, int S = 1>
+__device__ __forceinline__ void load_stage_twiddles_pairs(cf2* tws, const float2* __restrict__ tw) {
+  if constexpr (S < PL::stages) {
+    constexpr int NS = PL::ns(S), RAD = PL::radix(S), ST = N / (NS * RAD);
+    for (int e = threadIdx.x; e < NS * RAD; e += THREADS) {
+      const float2 w = tw[(e / NS) * (e % NS) * ST];
+      tws[PL::off(S) + e] = pair_of(w, w);
+    }
+    load_stage_twiddles_pairs<PL, N, THREADS, S + 1>(tws, tw);
+  }
+}
+
 // the RAD inputs of butterfly j of line b at stage S >= 1 from the tile, twiddled and transformed
 template <typename R, class PL, int N, bool INV, int LINES, Lay L, int SKEW, int S>
 __device__ __forceinline__ void io_butterfly(const cx<R>* buf, const cx<R>* tws, int b, int j, cx<R>* v) {
@@ -309,8 +336,12 @@ __device__ __forceinline__ void io_butterfly(const cx<R>* buf, const cx<R>* tws,
     cx<R> x = buf[IX::at(b, j + r * NB)];
     if (r > 0) {
       cx<R> w = tws[PL::off(S) + r * NS + k];
-      if (INV) w.y = -w.y;
-      x = x * w;
+      if constexpr (std::is_same<R, f2>::value) {
+        x = INV ? mk<R>(fma(x.y, w.y, x.x * w.x), x.y * w.x - x.x * w.y) : x * w;
+      } else {
+        if (INV) w.y = -w.y;
+        x = x * w;
+      }
     }
     v[r] = x;
   }

@@ -168,7 +168,7 @@ __device__ __forceinline__ void recover_epilogue(const Problem& P, const R* num,
 // What bounds it: shared memory and latency in FP32, the FP64 pipe in FP64.  Clearing the tile,
 // scattering the columns and every stage in place took six crossings of shared memory and five
 // barriers per frequency: 256^2 x 64, 8 frequencies (FP32) 171 us; this split without staging
-// and band 146 us, with both 117 us; 128^2 x 71, 3 frequencies, incident field (FP64) 435 us ->
+// and band 146 us, with both 117 us (100 us as pairs, RecPair); 128^2 x 71, 3 frequencies, incident field (FP64) 435 us ->
 // 322 us, 256 us of it FP64 instructions.  (A V and a u butterfly held in registers beside the
 // sums, one crossing fewer, left half the resident blocks: 131 us.)
 // The sums are taken of the unscaled transforms (raw: N^2 V and N^2 u, a given incident field
@@ -181,7 +181,7 @@ template <typename R, int N, int T> struct RecPass {
   using PL = IoPlan<N, MAXR, false>;
   static constexpr int NT = F32 ? (N >= 192 ? 256 : 128) : (N >= 192 ? 128 : 64);
   static constexpr int ROWS0 = F32 ? (N <= 16 ? 16 : 8) : (N <= 16 ? 8 : 4);
-  static constexpr int LINES = T == 0 ? ROWS0 : ROWS0 / 2;
+  static constexpr int LINES = T == 0 ? (F32 && N == 256 ? 4 : ROWS0) : ROWS0 / 2;
   static constexpr int SKEW = 16;
   // resident blocks the registers are held to: at 128^2 x 64 the pass's 1024 blocks at once
   static constexpr int MINB = !F32 || T == 1 ? 1 : N >= 192 ? 3 : (N == 128 || N == 64) ? 7 : 1;
@@ -189,6 +189,11 @@ template <typename R, int N, int T> struct RecPass {
   static constexpr int E = LINES * N, PER = (E + NT - 1) / NT;  // voxels of the block, of a thread
   using IX = LayIdx<Lay::ROW, N, 2 * LINES, SKEW>;
 };
+
+// Lengths from which V and u run as packed pairs (RecPair): a thread holds twice the registers, so half
+// the warps; below, the pass is one wave of short blocks bound by latency (128^2 x 64: 11 us, 14 us
+// as pairs; the whole dense step 60 -> 64 us).
+constexpr int PAIR_N = 192;
 
 template <typename R> __host__ __device__ constexpr bool raw_sums() { return sizeof(R) == 8; }
 
@@ -217,6 +222,111 @@ __device__ __forceinline__ void recover_first(cx<R>* buf, Ld ld) {
 #pragma unroll
     for (int r = 0; r < 16; ++r) buf[RP::IX::at(b, j * 16 + r)] = v[r];
   }
+}
+
+// FP32, two stages, T = 0: V and u of a voxel as one packed pair (pair.cuh).  Both fields take the
+// same butterflies with the same twiddles, so every operation is one packed instruction, a twiddle is
+// read once for both, and the sums come straight from the last stage's registers (recover_pass takes
+// them through the tile, one more write and read).  256^2 x 64, 8 frequencies: 117 us -> 100 us, the
+// batch of 32 smaller problems 1.37 -> 1.32 ms; bound by issue slots and latency at 16 warps per SM
+// (54% of the slots; a tile of 4 rows at N = 256: static shared memory holds no 8).
+template <typename R, int N, int T> struct RecPair {
+  using RP = RecPass<R, N, T>;
+  using PL = typename RP::PL;
+  static constexpr bool use = sizeof(R) == 4 && T == 0 && PL::stages == 2 && N >= PAIR_N;
+  static constexpr int LINES = RP::LINES, R0 = PL::radix(0), R1 = PL::radix(1), NB = N / R1;
+  static constexpr int NT = LINES * NB < 128 ? LINES * NB : 128;  // one last-stage butterfly per thread
+  static constexpr int PERB = (LINES * NB + NT - 1) / NT, PER = PERB * R1;
+  using IX = LayIdx<Lay::ROW, N, LINES, RP::SKEW>;
+};
+
+// recover_pass on packed pairs: the voxel of sum p is (line, element) = RecPair's last-stage outputs
+template <int N, typename A, bool INC>
+__device__ __forceinline__ void recover_pass_pairs(const Problem& P, const float2* __restrict__ t2,
+                                                   const int* __restrict__ colpos, const int* __restrict__ ncol,
+                                                   const int* __restrict__ colseg, const float2* __restrict__ u0,
+                                                   cf2* buf, const cf2* tws, RecStage<float, N, 0>& stg, A* num,
+                                                   A* den) {
+  using RP = RecPass<float, N, 0>;
+  using PR = RecPair<float, N, 0>;
+  using IX = typename PR::IX;
+  constexpr int LINES = PR::LINES, NT = PR::NT, SC = RP::SC, R0 = PR::R0, R1 = PR::R1, NB0 = N / R0, NB = PR::NB;
+  const long long nrows = (long long)P.m * N;
+  const long long row0 = (long long)blockIdx.x * LINES;
+  const int rows = (int)(nrows - row0 < LINES ? nrows - row0 : LINES);
+  const long long uoff = nrows * N;  // u behind V by nrows rows
+  const f2 scale = f2(P.inv_n2_f);
+#pragma unroll
+  for (int p = 0; p < PR::PER; ++p) { num[p] = A(0); den[p] = A(0); }
+  auto stage = [&](int om, int nc) {
+    const float2* src = t2 + ((long long)om * 2 * nrows + row0) * N;
+    if (nc <= SC)
+      for (int q = threadIdx.x; q < 2 * LINES * SC; q += NT) {
+        const int line = q / SC, c = q % SC, bl = line >= LINES ? line - LINES : line;
+        if (c < nc && bl < rows)
+          async_copy(&stg.col[om & 1][line][c], (line >= LINES ? src + uoff : src) + bl * N + c);
+      }
+    for (int i = threadIdx.x; i < N; i += NT) async_copy(&stg.pos[om & 1][i], colpos + om * N + i);
+  };
+  int nc = ncol[0];
+  stage(0, nc);
+  for (int om = 0; om < P.n_omega; ++om) {
+    const int seg = colseg[om];
+    const int nc1 = om + 1 < P.n_omega ? ncol[om + 1] : 0;
+    async_wait();
+    __syncthreads();  // this frequency's columns are staged, and the tile has been read
+    if (om + 1 < P.n_omega) stage(om + 1, nc1);
+    const int* ps = stg.pos[om & 1];
+    const float2* src = t2 + ((long long)om * 2 * nrows + row0) * N;
+    const bool staged = nc <= SC;
+    auto ld = [&](int b, int i) {
+      const int c = ps[i];
+      if (c < 0 || b >= rows) return cf2{f2(0.f), f2(0.f)};
+      return staged ? pair_of(stg.col[om & 1][b][c], stg.col[om & 1][LINES + b][c])
+                    : pair_of(src[b * N + c], src[uoff + b * N + c]);
+    };
+    auto first = [&](auto edge) {
+      constexpr int E = decltype(edge)::value;
+      for (int t = threadIdx.x; t < LINES * NB0; t += NT) {
+        const int b = t / NB0, j = t % NB0;
+        cf2 v[R0];
+#pragma unroll
+        for (int r = 0; r < R0; ++r)
+          if (E == 0 || r < E || r >= R0 - E) v[r] = ld(b, j + r * NB0);
+        if constexpr (E == 0) Dft<f2, true>::template run<R0>(v);
+        else Dft<f2, true>::template d16_edge<E>(v);
+#pragma unroll
+        for (int r = 0; r < R0; ++r) buf[IX::at(b, j * R0 + r)] = v[r];
+      }
+    };
+    if constexpr (R0 == 16) {
+      if ((seg & ~0x8001) == 0) first(std::integral_constant<int, 1>());
+      else if ((seg & ~0xC003) == 0) first(std::integral_constant<int, 2>());
+      else first(std::integral_constant<int, 0>());
+    } else {
+      first(std::integral_constant<int, 0>());
+    }
+    __syncthreads();
+#pragma unroll
+    for (int pb = 0; pb < PR::PERB; ++pb) {
+      const int t = threadIdx.x + pb * NT;
+      if ((LINES * NB) % NT == 0 || t < LINES * NB) {
+        const int b = t / NB, j = t % NB;
+        cf2 v[R1];
+        io_butterfly<f2, typename RP::PL, N, true, LINES, Lay::ROW, RP::SKEW, 1>(buf, tws, b, j, v);
+#pragma unroll
+        for (int r = 0; r < R1; ++r) {
+          const float2 re = (scale * v[r].x).split(), im = (scale * v[r].y).split();  // (V, u)
+          float2 u = make_float2(re.y, im.y);
+          if (INC && b < rows) u = u + u0[((long long)om * nrows + row0 + b) * N + j + r * NB];  // U~ - U~0
+          num[pb * R1 + r] += (A)u.x * (A)re.x + (A)u.y * (A)im.x;  // Re(conj(u) V)
+          den[pb * R1 + r] += (A)u.x * (A)u.x + (A)u.y * (A)u.y;    // |u|^2
+        }
+      }
+    }
+    nc = nc1;
+  }
+  __syncthreads();  // (a second pass reuses the tile and the staged columns)
 }
 
 // the sums of the thread's voxels e = threadIdx.x + p NT over the frequencies, in the
@@ -299,37 +409,72 @@ __device__ __forceinline__ void recover_pass(const Problem& P, const cx<R>* __re
   __syncthreads();  // (a second pass reuses the tile and the staged columns)
 }
 
+// Shape of the recovery kernel: threads, sums per thread, tile
+template <typename R, int N, int T, bool P = RecPair<R, N, T>::use> struct RecForm {
+  using RP = RecPass<R, N, T>;
+  using V = R;
+  using IX = typename RP::IX;
+  static constexpr bool PAIRS = false;
+  static constexpr int NT = RP::NT, PER = RP::PER, MINB = RP::MINB;
+};
+template <typename R, int N, int T> struct RecForm<R, N, T, true> {
+  using PR = RecPair<R, N, T>;
+  using V = f2;
+  using IX = typename PR::IX;
+  static constexpr bool PAIRS = true;
+  static constexpr int NT = PR::NT, PER = PR::PER, MINB = 512 / PR::NT;
+};
+
 // INC: u0 (the incident field on X) is given and added to u; otherwise the transform
 // already holds the plane wave
 template <typename R, int N, bool INC, int T>
-__global__ void __launch_bounds__((RecPass<R, N, T>::NT), (RecPass<R, N, T>::MINB))
+__global__ void __launch_bounds__((RecForm<R, N, T>::NT), (RecForm<R, N, T>::MINB))
 k_ifft_rows_recover(Problem P, const cx<R>* __restrict__ t2, const int* __restrict__ colpos,
                     const int* __restrict__ ncol, const int* __restrict__ colseg, const cx<R>* __restrict__ u0, R* __restrict__ xi, R* __restrict__ cout,
                     unsigned long long* __restrict__ ctr, const cx<R>* __restrict__ tw) {
   using RP = RecPass<R, N, T>;
   using PL = typename RP::PL;
-  constexpr int NT = RP::NT, E = RP::E, PER = RP::PER;
-  __shared__ cx<R> buf[RP::IX::ELEMS];
-  __shared__ cx<R> tws[PL::tw_elems];
+  using RF = RecForm<R, N, T>;
+  using C = cx<typename RF::V>;
+  constexpr int NT = RF::NT, PER = RF::PER;
+  __shared__ C buf[RF::IX::ELEMS];
+  __shared__ C tws[PL::tw_elems];
   __shared__ RecStage<R, N, T> stg;
   __shared__ unsigned red[NT / 32];
-  load_stage_twiddles<R, PL, N, NT>(tws, tw);  // a constant table: read while the predecessor drains
+  if constexpr (RF::PAIRS) load_stage_twiddles_pairs<PL, N, NT>(tws, tw);
+  else load_stage_twiddles<R, PL, N, NT>(tws, tw);  // a constant table: read while the predecessor drains
   pdl_wait();
   pdl_trigger();
   const long long nrows = (long long)P.m * N;
   const long long row0 = (long long)blockIdx.x * RP::LINES;
   const int el = (int)(nrows - row0 < RP::LINES ? nrows - row0 : RP::LINES) * N;  // voxels of this block
+  auto at = [&](int p) {  // the block's voxel of the thread's sum p (el or more: none)
+    if constexpr (RF::PAIRS) {
+      using PR = RecPair<R, N, T>;
+      const int t = threadIdx.x + p / PR::R1 * NT;
+      return t / PR::NB * N + t % PR::NB + p % PR::R1 * PR::NB;
+    } else {
+      return (int)threadIdx.x + p * NT;
+    }
+  };
+  auto pass = [&](auto* n, auto* d) {
+    using A = std::remove_pointer_t<decltype(n)>;
+    if constexpr (RF::PAIRS)
+      recover_pass_pairs<N, A, INC>(P, t2, colpos, ncol, colseg, u0, buf, tws, stg, n, d);
+    else
+      recover_pass<R, N, A, INC, T>(P, t2, colpos, ncol, colseg, u0, buf, tws, stg, n, d);
+  };
   R num[PER], den[PER];
   const double gd = raw_sums<R>() ? P.u_guard_raw : P.u_guard;
   R guard = sizeof(R) == 4 ? R(P.u_guard_f) : R(gd);
   bool redo = sizeof(R) == 4 && P.sums64;
   if (!redo) {
-    recover_pass<R, N, R, INC, T>(P, t2, colpos, ncol, colseg, u0, buf, tws, stg, num, den);
+    pass(num, den);
     if constexpr (sizeof(R) == 4) {
       bool bad = false;
 #pragma unroll
       for (int p = 0; p < PER; ++p)
-        bad |= threadIdx.x + p * NT < el && !(isfinite(num[p]) && isfinite(den[p]));
+        bad |= at(p) < el && !(isfinite(num[p]) && isfinite(den[p]));
       redo = __syncthreads_or(bad) != 0;
     }
   }
@@ -338,7 +483,7 @@ k_ifft_rows_recover(Problem P, const cx<R>* __restrict__ t2, const int* __restri
       // the sums left the range of R (|u| |V| beyond FP32 for huge evanescent profiles), or
       // were asked for in FP64: FP64 sums; xi itself is in range
       double nd[PER], dd[PER];
-      recover_pass<R, N, double, INC, T>(P, t2, colpos, ncol, colseg, u0, buf, tws, stg, nd, dd);
+      pass(nd, dd);
 #pragma unroll
       for (int p = 0; p < PER; ++p) {
         const bool g = !(dd[p] >= gd);
@@ -351,7 +496,7 @@ k_ifft_rows_recover(Problem P, const cx<R>* __restrict__ t2, const int* __restri
   recover_epilogue<R, PER, NT>(
       P, num, den, guard,
       [&](int p) {
-        const int e = threadIdx.x + p * NT;
+        const int e = at(p);
         return e < el ? row0 * N + e : -1LL;
       },
       xi, cout, ctr, red);
@@ -563,9 +708,9 @@ cudaError_t rec_tiled(const Problem& P, const Work<R>& w, R* xi, R* c, cudaStrea
   if (mid) cudaEventRecord(mid, s);
   const long long nrows = (long long)P.m * N;
   const dim3 gr((unsigned)((nrows + RP::LINES - 1) / RP::LINES));
-  e = w.u0 ? launch_pdl(k_ifft_rows_recover<R, N, true, T>, gr, dim3(RP::NT), 0, s, P, (const cx<R>*)w.t2,
+  e = w.u0 ? launch_pdl(k_ifft_rows_recover<R, N, true, T>, gr, dim3(RecForm<R, N, T>::NT), 0, s, P, (const cx<R>*)w.t2,
                         (const int*)w.colpos, (const int*)w.ncol, (const int*)w.colseg, w.u0, xi, c, w.ctr, (const cx<R>*)w.tw)
-           : launch_pdl(k_ifft_rows_recover<R, N, false, T>, gr, dim3(RP::NT), 0, s, P, (const cx<R>*)w.t2,
+           : launch_pdl(k_ifft_rows_recover<R, N, false, T>, gr, dim3(RecForm<R, N, T>::NT), 0, s, P, (const cx<R>*)w.t2,
                         (const int*)w.colpos, (const int*)w.ncol, (const int*)w.colseg, w.u0, xi, c, w.ctr, (const cx<R>*)w.tw);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
