@@ -2,10 +2,11 @@
 //
 // The horizontal transform F_r of Sec. 2 (and its inverse, Algorithm 2 step 2)
 // is a 2D DFT on the periodic N x N grid, done as two passes of 1D transforms:
-// along x (contiguous rows) and along y (strided columns).  Each pass stages a
-// tile of lines in shared memory and runs a Stockham autosort FFT on it: every
-// stage reads all butterfly inputs into registers, synchronises, and writes the
-// outputs back in place, so one buffer per tile suffices.
+// along x (contiguous rows) and along y (strided columns).  Two forms of a Stockham
+// autosort FFT: fft_lines_io holds a line in registers at both ends (first stage from
+// global memory, last stage to it) and crosses shared memory between stages only; fft_lines
+// (the cluster kernels) works in place on a tile in shared memory: every stage reads all
+// butterfly inputs into registers, synchronises, and writes the outputs back.
 //
 // Radices: 3 (once per factor 3), then the cap MAXR (16, 8 or 4) for as many powers of
 // two as it covers, then one stage of 8, 4 or 2 for the rest: few stages, so few

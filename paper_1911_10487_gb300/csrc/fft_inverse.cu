@@ -1,15 +1,13 @@
 // Inverse 2D FFT passes of Algorithm 2 (step 2) with the pointwise recovery of step
 // 3 fused into the last, for N = 2^a 3^b <= 256, in FP64 (double2) or FP32 (float2).
 //
-//   fft2_forward  : W -> W~ on every data plane (Sec. 4, Algorithm 2 step 1 needs
-//                   W~ = F_r[W]), then ||W~_nu||^2 summed over the planes of a
-//                   frequency, which the discrepancy test needs.
 //   recover       : V~, U~ -> V = F^-1[V~], u = F^-1[U~] (Algorithm 2 step 2) and
 //                   xi = Re(sum conj(u) V)/sum |u|^2, c = (c0^-2 - xi)^-1/2
 //                   (step 3, Sec. 5.2; Sec. 1 for c).  The inverse column pass
 //                   gathers the solved profiles of the active modes only and
 //                   transforms only the columns nu1 that hold a nonzero mode; the
-//                   row pass scatters those columns and transforms full rows.
+//                   row pass reads those columns by their positions and transforms
+//                   full rows.
 #include "fft_pass.cuh"
 
 namespace fl {
