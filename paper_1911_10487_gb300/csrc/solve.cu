@@ -943,12 +943,15 @@ __device__ bool tri_solve_e1(const double* d, const double* e, int n, double a, 
   return true;
 }
 
-// Newton in log(a) on log(a^2 ||(T + a I)^-1 e_1||^2 / target) from the FP32 root, to FP64
+// Newton in log(a) on g = log(a^2 ||(T + a I)^-1 e_1||^2 / target) from the FP32 root, to FP64
 // accuracy: the logarithm and the exponential are of 1 + x with |x| <= 1e-2 and taken by their
-// series (an FP64 log or exp costs ~50 instructions of 64 cycles in this one thread), z and its
-// derivative share a factorisation, and the step from |x| < 1e-8 is the last (quadratic: the
-// next x is below rounding).  False when it does not get there: the caller then takes the
-// bracketed search.
+// series (an FP64 log or exp costs ~50 instructions of 64 cycles in this one thread), and z and its
+// derivative share a factorisation.  The last step y = -g / g' is one below 1e-8: with r = l / (l + a)
+// over the eigenvalues l of T, weighted by their shares of ||z||^2, g' = 2 <r> and g'' = 3 <r^2> - <r> -
+// 2 <r>^2, so |g''| <= 2 g' at any a and the error behind it is at most y^2.  (The residual x says that
+// only where g' is of order one; g' ~ e for a mode with ||b||^2 = delta_nu^2 / (1 - e).)  A residual at
+// rounding also ends it: such a mode's y stays at rounding / g'.  False when it does not get there: the
+// caller then takes the bracketed search.
 __device__ bool polish_root(const double* d, const double* e, int n, double inv_target, double& a, int max_iter) {
   double z[DENSE_M1], zz, zs;
 #pragma unroll 1
@@ -962,7 +965,7 @@ __device__ bool polish_root(const double* d, const double* e, int n, double inv_
     const double y = -g * rcp64(gp);
     if (!(fabs(y) <= 1e-1)) return false;
     a *= fma(y, fma(y, fma(y, fma(y, 0.041666666666666667, 0.16666666666666667), 0.5), 1.0), 1.0);  // exp(y)
-    if (fabs(x) < 1e-8) return true;
+    if (fabs(y) < 1e-8 || fabs(x) < 1e-14) return true;
   }
   return false;
 }
