@@ -133,16 +133,25 @@ Layout layout(int n, int m, int m1, int n_omega, bool fp64) {
   L.flagbits = off; off = align_up(off + 4 * cb * 32);
   L.blkcnt = off; off = align_up(off + 4 * cb);
   L.blkgz = off; off = align_up(off + 4 * cb);
-  L.colblk = off; off = align_up(off + 4 * cb * 8);
   L.cols = off; off = align_up(off + 4 * (size_t)n_omega * n);
-  L.colpos = off; off = align_up(off + 4 * (size_t)n_omega * n);
   L.ncol = off; off = align_up(off + 4 * (size_t)n_omega);
-  L.colseg = off; off = align_up(off + 4 * (size_t)n_omega);
   L.dnu = off; off = align_up(off + 8 * (size_t)n_omega);
-  L.bar = off; L.count = off + 4 * (size_t)n_omega; L.colmask = off + 8 * (size_t)n_omega;
-  off = align_up(off + 40 * (size_t)n_omega);
-  L.wsum = off; off = align_up(off + 8 * (size_t)n_omega * wsum_max(n, m1));
+  // (these three adjoin: clear_words)
+  L.bar = off; off = align_up(off + 4 * (size_t)n_omega);
+  L.count = off; off = align_up(off + 4 * (size_t)n_omega);
+  L.colblk = off; off = align_up(off + 4 * cb * 8);
   L.total = off;
+  // Arrays in the place of others that their route does not use, or no longer, so that the total, which
+  // decides what fits the fixed scratch of fs_reconstruct_static, is that of the arrays above.
+  // The columns' positions and segments: the norms' (read by k_classify_flags before k_classify_scatter
+  // writes these; the single-pass and the early classification have no norms).
+  L.colpos = L.norms;
+  L.colseg = L.norms + 4 * (size_t)n_omega * n;
+  // The early classification's: the column masks in the per-block ones (one block of a frequency holds
+  // 8 words), and the block sums of |W|^2 in the second half of the W~ region (FP32 data fill the
+  // first; N^2 >= 64 sums per plane, wsum_max has at most N^2 / 16 per plane).
+  L.colmask = L.colblk;
+  L.wsum = L.t12 + a / 2;
   return L;
 }
 

@@ -133,11 +133,11 @@ template <typename R> struct Work {
   int* colseg;      // [n_omega] bit s: a column of the list in sixteenth s of the N
   int* count;       // [n_omega] active modes (behind bar: see there)
   double* dnu;      // [n_omega] delta_nu
-  // bar, count and colmask are one region, zeroed by the first kernel of a reconstruction
-  // (clear_words(P) words from bar)
+  // bar, count and colmask adjoin (each on its boundary) and are zeroed by the first kernel of a
+  // reconstruction (clear_words(P) words from bar)
   unsigned* bar;    // [n_omega] barrier counters of the single-pass classification
   unsigned* colmask;  // [n_omega][8] columns holding an active mode (atomic)
-  float2* wsum;     // [n_omega][WSUM_MAX(n, m1)] block sums of |W|^2 as two floats
+  float2* wsum;     // [n_omega][wsum_max(n, m1)] block sums of |W|^2 as two floats
   unsigned long long* ctr;  // [C_COUNT]
   const cx<R>* tw;  // [N] twiddles exp(-2 pi i j/N)
   double* alpha_out;  // [n_omega][N*N] or null
@@ -160,8 +160,9 @@ template <typename R> struct Work {
   const cx<R>* u0;
 };
 
-// words of the region from Work::bar that the first kernel zeroes
-inline int clear_words(const Problem& P) { return 10 * P.n_omega; }
+// words of the region from Work::bar that the first kernel zeroes: bar and count (on 256-byte
+// boundaries, layout()) and the column masks
+inline int clear_words(const Problem& P) { return 2 * ((P.n_omega + 63) / 64 * 64) + 8 * P.n_omega; }
 // block sums of |W|^2 per frequency (the first kernel has at least 4 rows per block, or 4 CTAs
 // per plane)
 inline size_t wsum_max(int n, int m1) { return (size_t)m1 * (n / 4 > 4 ? n / 4 : 4); }
