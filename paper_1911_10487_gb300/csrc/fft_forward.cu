@@ -41,7 +41,7 @@ template <typename R, int N> __host__ __device__ constexpr size_t plane_fwd_smem
   return sizeof(cx<R>) * ((size_t)LayIdx<Lay::ROW, N, RB, 16>::ELEMS + (size_t)RB * N + N);
 }
 
-// wsum (may be null): the CTA's sum of |in|^2, [plane][C].
+// wsum (may be null): the CTA's sum of |in|^2, [plane][C] (block_sum_squares).
 template <typename R, int N>
 __global__ void __launch_bounds__(THREADS)
 k_fft2_plane(const cx<R>* __restrict__ in, cx<R>* __restrict__ out, const cx<R>* __restrict__ tw,
@@ -106,7 +106,7 @@ k_fft2_plane(const cx<R>* __restrict__ in, cx<R>* __restrict__ out, const cx<R>*
   }
   if (wsum) {
     __shared__ ff red[THREADS / 32];
-    block_sum_ff<THREADS>(ws, red, wsum + (long long)blockIdx.y * C + r);
+    block_sum_squares<THREADS>(ws, src, E, red, wsum + (long long)blockIdx.y * C + r);
   }
   cluster_wait();  // no CTA leaves while another may still read its rows
 }

@@ -58,16 +58,29 @@ __device__ __forceinline__ void load_twiddles(cx<R>* tw_s, const cx<R>* __restri
   for (int j = threadIdx.x; j < N; j += THREADS) tw_s[j] = tw[j];
 }
 
-// Sum of one float per thread over the NT threads of a block in two-float (the FP32 pipe): *out
-// on thread 0.  red: NT / 32 values.
-template <int NT> __device__ __forceinline__ void block_sum_ff(float x, ff* red, float2* out) {
-  const ff s = ff_warp_sum(ff{x, 0.f});
+// Sum of |W|^2 over the n values of a block at src, from the NT threads' own sums q of squares, in
+// two-float (the FP32 pipe): *out on thread 0.  Squares of values below 2^-63 leave the normal numbers of
+// FP32, where those of W~, N to N^2 times larger, do not; a block whose threads' sums are all below
+// 2^-64 reads its values again and takes them times SMALL_UNIT (its sum is below 2^-56 before, 2^112
+// then).  Such a sum carries the minus sign, which squares have not; the classification joins the two
+// kinds.  red: NT / 32 values.
+template <int NT> __device__ __forceinline__ void block_sum_squares(float q, const float2* src, int n, ff* red,
+                                                                    float2* out) {
+  const bool unit = __syncthreads_or(!(q < 0x1p-64f)) != 0;  // (a NaN counts as one)
+  if (!unit) {
+    q = 0.f;
+    for (int e = threadIdx.x; e < n; e += NT) {
+      const float x = src[e].x * SMALL_UNIT, y = src[e].y * SMALL_UNIT;
+      q += x * x + y * y;
+    }
+  }
+  const ff s = ff_warp_sum(ff{q, 0.f});
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
   if (threadIdx.x == 0) {
     ff t = red[0];
     for (int w = 1; w < NT / 32; ++w) t = ff_add(t, red[w]);
-    *out = make_float2(t.hi, t.lo);
+    *out = unit ? make_float2(t.hi, t.lo) : make_float2(-t.hi, -t.lo);
   }
 }
 
@@ -75,7 +88,7 @@ template <int NT> __device__ __forceinline__ void block_sum_ff(float x, ff* red,
 // grid (blocks, fields): field blockIdx.y has nrows rows.
 // TI: element type of `in` (cx<R>, or float2 read into an FP64 transform); D32: FftPlan's
 // factors in FP32 (IoPlan); WS (the data planes in FP32): also the block's sum of |in|^2 to wsum
-// [field][block].  clear (may be null): nclear words zeroed by block (0, 0), the counters of the
+// [field][block] (block_sum_squares).  clear (may be null): nclear words zeroed by block (0, 0), the counters of the
 // classification that follows.
 template <typename R, int N, bool INV, typename TI = cx<R>, int T = 0, bool D32 = false, bool WS = false>
 __global__ void __launch_bounds__((DensePass<R, N, T>::RT))
@@ -115,7 +128,7 @@ k_fft_rows(const TI* __restrict__ in, cx<R>* out, long long nrows, const cx<R>* 
       });
   if constexpr (WS) {
     __shared__ ff red[DP::RT / 32];
-    block_sum_ff<DP::RT>(ws, red, wsum + (long long)blockIdx.y * gridDim.x + blockIdx.x);
+    block_sum_squares<DP::RT>(ws, src, rows * N, red, wsum + (long long)blockIdx.y * gridDim.x + blockIdx.x);
   }
 }
 

@@ -65,7 +65,7 @@ struct Problem {
   // its per-mode set-up runs on the FP32 pipe: k0, k0^2, g0 per frequency, kn^2, h_z,
   // z1, alpha_rel, zy[k] - zy_min and zy_min - z_top (z_top = z1 + (M - 1/2) h_z)
   float2 k0_f[MAX_OMEGA], k0sq_f[MAX_OMEGA], g0_f[MAX_OMEGA];
-  float2 dscale_f;
+  float2 dscale2_f;  // dscale^2
   float2 knsq_f, hz_f, z1_f, alpha_rel_f, d0_f;
   float2 zyd_f[MAX_M1];
 };
@@ -104,7 +104,7 @@ inline void derive_constants(Problem& P) {
     P.k0sq_f[j] = two_float(P.k0[j] * P.k0[j]);
     P.g0_f[j] = two_float(P.g0[j]);
   }
-  P.dscale_f = two_float(P.dscale);
+  P.dscale2_f = two_float(P.dscale * P.dscale);
   P.knsq_f = two_float(P.kn * P.kn);
   P.hz_f = two_float(P.hz);
   P.z1_f = two_float(P.z1);
@@ -167,6 +167,8 @@ inline int clear_words(const Problem& P) { return 2 * ((P.n_omega + 63) / 64 * 6
 // per plane)
 inline size_t wsum_max(int n, int m1) { return (size_t)m1 * (n / 4 > 4 ? n / 4 : 4); }
 
+// values times this where their squares leave the FP32 range (block_sum_squares)
+constexpr float SMALL_UNIT = 0x1p84f;
 // FP32 data classified against delta_nu = dscale ||W|| with ||W|| summed over W itself as the
 // first kernel reads it (norms and flags in one kernel, slots by atomics); otherwise ||W|| comes
 // from the norms (Parseval) and the flags and slots in two more kernels

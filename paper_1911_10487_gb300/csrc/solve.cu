@@ -327,7 +327,7 @@ k_classify_early(Problem P, const float2* __restrict__ wt, const float* __restri
   __shared__ float part[4][ET / 4];
   __shared__ ff red[ET / 32];
   __shared__ unsigned cm[NWC];
-  __shared__ ff thr_s;
+  __shared__ ff thr_s, w2_s;  // delta_nu^2 and ||W||^2, in the unit of the sums
   __shared__ int tot[3];  // active, grazing, not finite
   const int om = blockIdx.y;
   const int N = P.n, N2 = N * N, M1 = P.m1;
@@ -336,11 +336,17 @@ k_classify_early(Problem P, const float2* __restrict__ wt, const float* __restri
   const int nu = blockIdx.x * EMB + j;
   if (threadIdx.x < NWC) cm[threadIdx.x] = 0u;
   if (threadIdx.x < 3) tot[threadIdx.x] = 0;
-  // ||W||^2 in two-float: every block adds the block sums in the same order
+  // ||W||^2 in two-float: every block adds the block sums in the same order, those of small values
+  // (block_sum_squares: negative, times SMALL_UNIT^2) brought to the others' unit
+  constexpr float U = 1.f / SMALL_UNIT;
   ff s = ff{0.f, 0.f};
+  bool ordinary = false;
   for (int i = threadIdx.x; i < n_wsum; i += ET) {
     const float2 v = wsum[(long long)om * n_wsum + i];
-    s = ff_add(s, ff{v.x, v.y});
+    const bool small = signbit(v.x);
+    const float f = small ? -U : 1.f, g = small ? U : 1.f;
+    s = ff_add(s, ff{v.x * f * g, v.y * f * g});
+    ordinary |= !small;
   }
   // the norms, in FP32 (planes in order within a quarter)
   float acc = 0.f;
@@ -375,18 +381,29 @@ k_classify_early(Problem P, const float2* __restrict__ wt, const float* __restri
   s = ff_warp_sum(s);
   if (lane == 0) red[wid] = s;
   if (!GROUPS) part[q][j] = acc;
-  __syncthreads();
+  const bool unit = __syncthreads_or(ordinary) != 0;
+  if (!unit) {  // every sum is one of small values: their own unit
+    s = ff{0.f, 0.f};
+    for (int i = threadIdx.x; i < n_wsum; i += ET) {
+      const float2 v = wsum[(long long)om * n_wsum + i];
+      s = ff_add(s, ff{-v.x, -v.y});
+    }
+    s = ff_warp_sum(s);
+    if (lane == 0) red[wid] = s;
+    __syncthreads();
+  }
   if (threadIdx.x == 0) {
     ff t = red[0];
     for (int w = 1; w < ET / 32; ++w) t = ff_add(t, red[w]);
-    const ff ds = ff{P.dscale_f.x, P.dscale_f.y};
-    const bool fin = isfinite(t.hi);
-    const ff dnu = fin ? ff_mul(ds, ff_sqrt(t)) : t;
     // a non-finite ||W|| (W holds a NaN or Inf) leaves delta_nu undefined: no mode passes
-    thr_s = fin ? ff_mul(dnu, dnu) : ff{INFINITY, 0.f};
-    if (blockIdx.x == 0) dnu_out[om] = ff_to(dnu);
+    thr_s = isfinite(t.hi) ? ff_mul(ff{P.dscale2_f.x, P.dscale2_f.y}, t) : ff{INFINITY, 0.f};
+    w2_s = t;
   }
   __syncthreads();
+  if (blockIdx.x == 0 && threadIdx.x == ET - 32) {  // (FP64 in one block of a frequency only)
+    const double w2 = isfinite(w2_s.hi) ? ff_to(w2_s) * (unit ? 1.0 : (double)U * U) : INFINITY;
+    dnu_out[om] = P.dscale * (w2 > 0.0 && isfinite(w2) ? w2 * rsqrt64(w2) : w2);
+  }
   if (threadIdx.x < EMB) {  // whole warps
     const float nrm = GROUPS ? acc : (part[0][j] + part[1][j]) + (part[2][j] + part[3][j]);
     const ff thr = thr_s;
@@ -399,7 +416,7 @@ k_classify_early(Problem P, const float2* __restrict__ wt, const float* __restri
       const int msq = m1 * m1 + m2 * m2;
       graz = msq >= P.graz_lo[om] && msq <= P.graz_hi[om];
       bad = !isfinite(nrm);
-      on = !graz && (P.alpha_mode == 1 || ff_gt(ff{nrm, 0.f}, thr));
+      on = !graz && (P.alpha_mode == 1 || ff_gt(ff{unit ? nrm : nrm * SMALL_UNIT * SMALL_UNIT, 0.f}, thr));
       if (on) atomicOr(&cm[i1 >> 5], 1u << (i1 & 31));
     }
     const unsigned bal = __ballot_sync(0xffffffffu, on);
