@@ -129,34 +129,65 @@ cudaError_t fwd_plane(const cx<R>* W, const Problem& P, const Work<R>& w, cudaSt
   return launch_mode_norms<R>(P, w, s);
 }
 
-// ---- rows of pairs of real planes ------------------------------------------------
-// The forward transform along x of M real planes, two to a complex plane: pair p holds
-// planes 2p - off and 2p + 1 - off (off = M mod 2; plane -1 is zero) in its real and
-// imaginary part; the reader separates them by their symmetry (k_apply_data).
+// ---- real planes -------------------------------------------------------------------
+// Rows: the forward transform along x of real rows, two neighbours (2y, 2y + 1) of one plane to a
+// complex line: with Z their joint transform, twice the two are Z_k + conj(Z_{N-k}) and
+// -i (Z_k - conj(Z_{N-k})), taken apart behind the last stage.  Two PLANES to a line would cost the
+// same, but then the weaker plane's transform carries the stronger one's rounding.  out [plane][N][N/2 + 2]
+// holds the columns k <= N/2 (the rest are their mirror images) and one more, for whole 32-byte
+// sectors.
 template <typename R, int N>
 __global__ void __launch_bounds__((DensePass<R, N, 0>::RT))
-k_fft_rows_pairs(const R* __restrict__ xi, cx<R>* __restrict__ out, long long nrows, int off,
-                 const cx<R>* __restrict__ tw) {
+k_fft_rows_real(const R* __restrict__ xi, cx<R>* __restrict__ out, long long npairs, const cx<R>* __restrict__ tw) {
   using DP = DensePass<R, N, 0>;
   using PL = IoPlan<N, DP::MAXR, false>;
-  constexpr int LINES = DP::LINES;
-  __shared__ cx<R> buf[PL::stages > 1 ? LayIdx<Lay::ROW, N, LINES, DP::SKEW>::ELEMS : 1];
+  constexpr int LINES = DP::LINES, HS = real_stride(N);
+  using IX = LayIdx<Lay::ROW, N, LINES, DP::SKEW>;
+  static_assert(N % 2 == 0, "a pair of rows lies in one plane");
+  __shared__ cx<R> buf[IX::ELEMS];
   __shared__ cx<R> tws[PL::tw_elems];
   load_stage_twiddles<R, PL, N, DP::RT>(tws, tw);
   pdl_wait();
   pdl_trigger();
-  const long long row0 = (long long)blockIdx.x * LINES;
+  const long long p0 = (long long)blockIdx.x * LINES;
+  const int np = (int)(npairs - p0 < LINES ? npairs - p0 : LINES);
+  const R* src = xi + 2 * p0 * N;
+  cx<R>* dst = out + 2 * p0 * HS;
   fft_lines_io<R, PL, N, false, LINES, DP::RT, Lay::ROW, DP::SKEW>(
       buf, tws,
-      [&](int b, int i) {
-        const long long row = row0 + b;
-        if (row >= nrows) return czero<R>();
-        const long long p = row / N, y = row - p * N, l = 2 * p - off;
-        const R re = l >= 0 ? xi[(l * N + y) * N + i] : R(0);
-        return mk<R>(re, xi[((l + 1) * N + y) * N + i]);
-      },
-      [&](int b, int i, cx<R> v) {
-        if (row0 + b < nrows) out[(row0 + b) * N + i] = v;
+      [&](int b, int i) { return b < np ? mk<R>(src[2 * b * N + i], src[(2 * b + 1) * N + i]) : czero<R>(); },
+      [&](int b, int i, cx<R> v) { buf[IX::at(b, i)] = v; });
+  __syncthreads();
+  for (int e = threadIdx.x; e < np * HS; e += DP::RT) {
+    const int b = e / HS, k = e % HS;
+    const cx<R> z = buf[IX::at(b, k)], c = buf[IX::at(b, k == 0 ? 0 : N - k)];
+    dst[2 * b * HS + k] = mk<R>(z.x + c.x, z.y - c.y);
+    dst[(2 * b + 1) * HS + k] = mk<R>(z.y + c.y, c.x - z.x);
+  }
+}
+
+// Columns: the columns k <= N/2 of every plane in place, a tile any COLS consecutive ones of the
+// M (N/2 + 1), so that the odd one of a plane fills no tile of its own (FP64, 37 planes of 192^2: 481
+// tiles plane by plane, a fourth one on some of the SMs, and 449 these)
+template <typename R, int N>
+__global__ void __launch_bounds__((DensePass<R, N, 0>::CT))
+k_fft_cols_real(cx<R>* data, int ncols, const cx<R>* __restrict__ tw) {
+  using DP = DensePass<R, N, 0>;
+  using PL = IoPlan<N, DP::MAXR, false>;
+  constexpr int TC = DP::COLS, H = N / 2 + 1, HS = real_stride(N);
+  static_assert(DP::CT % TC == 0, "a thread stays in its column");
+  __shared__ cx<R> buf[PL::stages > 1 ? N * TC : 1];
+  __shared__ cx<R> tws[PL::tw_elems];
+  load_stage_twiddles<R, PL, N, DP::CT>(tws, tw);
+  pdl_wait();
+  pdl_trigger();
+  const int q = blockIdx.x * TC + threadIdx.x % TC;
+  const bool on = q < ncols;
+  cx<R>* col = data + (on ? (long long)(q / H) * N * HS + q % H : 0);
+  fft_lines_io<R, PL, N, false, TC, DP::CT, Lay::COL, 0>(
+      buf, tws, [&](int, int i) { return on ? col[i * HS] : czero<R>(); },
+      [&](int, int i, cx<R> v) {
+        if (on) col[i * HS] = v;
       });
 }
 
@@ -480,14 +511,17 @@ cudaError_t xi_impl(const cx<R>* ut, cx<R>* out, const R* xi, long long planes, 
 }
 
 template <typename R, int N>
-cudaError_t pairs_impl(const R* xi, cx<R>* out, int m, const cx<R>* tw, cudaStream_t s) {
+cudaError_t real_impl(const R* xi, cx<R>* out, int m, const cx<R>* tw, cudaStream_t s) {
   using DP = DensePass<R, N, 0>;
-  const int np = (m + 1) / 2;
-  const long long nrows = (long long)np * N;
-  cudaError_t e = launch_pdl(k_fft_rows_pairs<R, N>, dim3((unsigned)((nrows + DP::LINES - 1) / DP::LINES)),
-                             dim3(DP::RT), 0, s, xi, out, nrows, m & 1, tw);
+  const long long npairs = (long long)m * N / 2;
+  // A plain launch: about three blocks per SM, bound by the FP64 pipe, and those started while the
+  // predecessor drains crowd on the SMs it has left (FP64, 37 planes of 192^2 in a row of calls: the
+  // rows 77 us and the columns that start behind them 58 us; 35 and 31 us so)
+  k_fft_rows_real<R, N><<<(unsigned)((npairs + DP::LINES - 1) / DP::LINES), DP::RT, 0, s>>>(xi, out, npairs, tw);
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return cols_launch<R, N, false, 0, false>(out, out, np, tw, s);
+  const int ncols = m * (N / 2 + 1);
+  return launch_pdl(k_fft_cols_real<R, N>, dim3((ncols + DP::COLS - 1) / DP::COLS), dim3(DP::CT), 0, s, out, ncols, tw);
 }
 
 }  // namespace
@@ -600,16 +634,16 @@ template cudaError_t launch_xi_transform<float>(const float2*, float2*, const fl
                                                 cudaStream_t);
 
 template <typename R>
-cudaError_t launch_fft2_pairs(const R* xi, cx<R>* out, int n, int m, const cx<R>* tw, cudaStream_t s) {
+cudaError_t launch_fft2_real(const R* xi, cx<R>* out, int n, int m, const cx<R>* tw, cudaStream_t s) {
   switch (n) {
-#define FL_CASE(K) case K: return pairs_impl<R, K>(xi, out, m, tw, s);
+#define FL_CASE(K) case K: return real_impl<R, K>(xi, out, m, tw, s);
     FL_SIZES(FL_CASE)
 #undef FL_CASE
     default: return cudaErrorInvalidValue;
   }
 }
-template cudaError_t launch_fft2_pairs<double>(const double*, double2*, int, int, const double2*, cudaStream_t);
-template cudaError_t launch_fft2_pairs<float>(const float*, float2*, int, int, const float2*, cudaStream_t);
+template cudaError_t launch_fft2_real<double>(const double*, double2*, int, int, const double2*, cudaStream_t);
+template cudaError_t launch_fft2_real<float>(const float*, float2*, int, int, const float2*, cudaStream_t);
 
 template <typename R>
 cudaError_t launch_twiddles(cx<R>* tw, int n, cudaStream_t s) {

@@ -102,15 +102,15 @@ __global__ void k_point_sources(Problem P, const double* __restrict__ spec, int 
 // q and every E_k.  A block takes 32 quadrant modes (m1, m2 >= 0), one warp per sign pair; the
 // four warps deal the exponentials among themselves through shared memory, then each sums its
 // own modes.  An evanescent mode (q, E real) takes real products.  Before, one thread per
-// mode took an exp and a sincos per plane: 192^2, 37 + 19 planes, 5 frequencies (FP64, packed)
+// mode took an exp and a sincos per plane: 192^2, 37 + 19 planes, 5 frequencies (FP64, REAL)
 // 1067 us -> 205 us, 128^2, 64 + 32 planes 363 us -> 44 us.
 //
-// PACKED (the plane incident wave): V~_l = e^{-i k0 z'_l} F[xi_l], and the transform of the
-// real planes xi_l, taken in pairs, serves every frequency (FG of them per block, so that the
-// pairs are separated once).  The phase joins q: rho = q e^{i k0 h_z}.  Otherwise vt holds
-// V~ per frequency.
+// REAL (the plane incident wave): V~_l = e^{-i k0 z'_l} F[xi_l], and the transform of the real planes
+// xi_l, half of its columns (launch_fft2_real), serves every frequency (FG of them per block, so that it
+// is read once for them).  The phase joins q: rho = q e^{i k0 h_z}.  Otherwise vt holds V~ per
+// frequency.
 constexpr int HB = 8;   // planes per block
-constexpr int FG = 2;   // frequencies per thread block (PACKED; 4 left the SMs unevenly loaded)
+constexpr int FG = 2;   // frequencies per thread block (REAL; 4 left the SMs unevenly loaded)
 constexpr int EK = 32;  // data planes per pass over the exponentials (planes not uniform)
 
 struct DataPlanes {  // uniform spacing (0: not uniform) and the offsets from it
@@ -150,22 +150,20 @@ __device__ __forceinline__ void put_data(const Problem& P, const DataPlanes& D, 
   }
 }
 
-template <bool PACKED> constexpr int apply_nf() { return PACKED ? FG : 1; }
-__host__ __device__ inline int apply_blocks(int m) { return (m + (m & 1) + HB - 1) / HB; }
+template <bool REAL> constexpr int apply_nf() { return REAL ? FG : 1; }
+__host__ __device__ inline int apply_blocks(int m) { return (m + HB - 1) / HB; }
 // shared memory: heads [NF][nbk], q [NF], phases [NF][nbk] and the data exponentials
-template <bool PACKED> size_t apply_smem(int m) {
-  return sizeof(double2) * ((size_t)apply_nf<PACKED>() * ((apply_blocks(m) + 1) * 32 + apply_blocks(m)) + EK * 32);
+template <bool REAL> size_t apply_smem(int m) {
+  return sizeof(double2) * ((size_t)apply_nf<REAL>() * ((apply_blocks(m) + 1) * 32 + apply_blocks(m)) + EK * 32);
 }
 
-template <typename R, bool PACKED, bool UNI>
+template <typename R, bool REAL, bool UNI>
 __global__ void __launch_bounds__(128)
 k_apply_data(Problem P, DataPlanes D, const cx<R>* __restrict__ vt, cx<R>* __restrict__ wt) {
-  constexpr int NF = apply_nf<PACKED>();
+  constexpr int NF = apply_nf<REAL>();
   extern __shared__ __align__(16) unsigned char apply_raw[];
   const int N = P.n, M = P.m, H = N / 2 + 1;
-  // M + off planes (off = 1: a zero plane below, so that pairs do not straddle blocks); block b
-  // ends at plane M - 1 - HB (nbk - 1 - b)
-  const int nbk = PACKED ? apply_blocks(M) : (M + HB - 1) / HB;
+  const int nbk = apply_blocks(M);  // block b ends at plane M - 1 - HB (nbk - 1 - b)
   double2 (*ex)[32] = reinterpret_cast<double2 (*)[32]>(apply_raw);
   double2 (*hd)[32] = ex + EK;              // [NF][nbk]
   double2 (*rs)[32] = hd + NF * nbk;        // [NF]
@@ -180,12 +178,11 @@ k_apply_data(Problem P, DataPlanes D, const cx<R>* __restrict__ vt, cx<R>* __res
   const bool valid = in && !(neg1 && (m1 == 0 || m1 == N / 2)) && !(neg2 && (m2 == 0 || m2 == N / 2));
   const int i1 = neg1 ? (N - m1) % N : m1, i2 = neg2 ? (N - m2) % N : m2;
   const long long nu = (long long)i2 * N + i1;
-  const long long mu = (long long)((N - i2) % N) * N + (N - i1) % N;  // -nu
   const int msq = m1 * m1 + m2 * m2;
   const double ztop = P.z1 + (M - 0.5) * P.hz;
-  const int om0 = PACKED ? blockIdx.y * FG : blockIdx.y;
-  const int nf = PACKED ? min(FG, P.n_omega - om0) : 1;
-  if (PACKED) {  // e^{-i k0 z'} of the block tops and e^{i k0 h_z}
+  const int om0 = REAL ? blockIdx.y * FG : blockIdx.y;
+  const int nf = REAL ? min(FG, P.n_omega - om0) : 1;
+  if (REAL) {  // e^{-i k0 z'} of the block tops and e^{i k0 h_z}
     for (int t = threadIdx.x; t < nf * (nbk + 1); t += 128) {
       const int f = t / (nbk + 1), b = t - f * (nbk + 1);
       double s, c;
@@ -206,7 +203,7 @@ k_apply_data(Problem P, DataPlanes D, const cx<R>* __restrict__ vt, cx<R>* __res
     const double qq = P.k0[om] * P.k0[om] - P.kn * P.kn * (double)msq;
     const double r = grazing ? 1.0 : rsqrt64(fabs(qq));
     kz[f] = grazing ? 1.0 : sqrt_from_rsqrt(fabs(qq), r);
-    gam[f] = grazing ? 0.0 : (PACKED ? -0.5 : -1.0) * P.g0[om] * r;  // PACKED: the pairs hold twice the transforms
+    gam[f] = grazing ? 0.0 : (REAL ? -0.5 : -1.0) * P.g0[om] * r;  // REAL: vt is twice the transform
     propm |= (qq >= 0.0 ? 1u : 0u) << f;
   }
   {
@@ -218,7 +215,7 @@ k_apply_data(Problem P, DataPlanes D, const cx<R>* __restrict__ vt, cx<R>* __res
       for (int b = 0; b <= nbk; ++b, ++it) {
         if ((it & 3) != w) continue;
         double2 x = exp_kz(k, b < nbk ? HB * (nbk - 1 - b) * P.hz : P.hz);
-        if (PACKED) x = x * (b < nbk ? phs[f * nbk + b] : ex[f][0]);
+        if (REAL) x = x * (b < nbk ? phs[f * nbk + b] : ex[f][0]);
         if (b < nbk) hd[f * nbk + b][lane] = x;
         else rs[f][lane] = x;
       }
@@ -228,7 +225,7 @@ k_apply_data(Problem P, DataPlanes D, const cx<R>* __restrict__ vt, cx<R>* __res
   double2 acc[NF];
 #pragma unroll
   for (int f = 0; f < NF; ++f) acc[f] = make_double2(0.0, 0.0);
-  if constexpr (PACKED) {
+  if constexpr (REAL) {
     double2 rho[NF], blk[NF];
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
@@ -236,28 +233,27 @@ k_apply_data(Problem P, DataPlanes D, const cx<R>* __restrict__ vt, cx<R>* __res
       blk[f] = make_double2(0.0, 0.0);
     }
     if (valid) {
-      const int np = (M + 1) / 2;  // pairs; planes 2p - off, 2p + 1 - off
-      int left = np - (nbk - 1) * (HB / 2), b = 0;  // pairs left in this block
-#pragma unroll 4
-      for (int p = 0; p < np; ++p) {
-        const double2 z = to_d(vt[p * N2 + nu]), c = to_d(vt[p * N2 + mu]);
-        // twice the transforms of the two planes: z + conj(c) and -i (z - conj(c))
-        const double2 x = make_double2(z.x + c.x, z.y - c.y), y = make_double2(z.y + c.y, c.x - z.x);
+      // a mode with m1 < 0 from its mirror image, which is its conjugate
+      const int HS = real_stride(N);
+      const long long NH = (long long)N * HS;
+      const cx<R>* src = vt + (long long)(neg1 ? (N - i2) % N : i2) * HS + m1;
+      for (int b = 0, l0 = M - HB * nbk; b < nbk; ++b, l0 += HB) {  // (the first block may be short)
+        cx<R> v[HB];
+#pragma unroll
+        for (int j = 0; j < HB; ++j) v[j] = l0 + j >= 0 ? src[(l0 + j) * NH] : czero<R>();
+#pragma unroll
+        for (int j = 0; j < HB; ++j) {
+          if (l0 + j < 0) continue;
+          double2 x = to_d(v[j]);
+          if (neg1) x.y = -x.y;
+#pragma unroll
+          for (int f = 0; f < NF; ++f)
+            if (f < nf) blk[f] = rho[f] * blk[f] + x;
+        }
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
-          if (f < nf) {
-            blk[f] = rho[f] * blk[f] + x;
-            blk[f] = rho[f] * blk[f] + y;
-          }
-        }
-        if (--left == 0) {
-          left = HB / 2;
-#pragma unroll
-          for (int f = 0; f < NF; ++f) {
-            if (f < nf) acc[f] = acc[f] + hd[f * nbk + b][lane] * blk[f];
-            blk[f] = make_double2(0.0, 0.0);
-          }
-          ++b;
+          if (f < nf) acc[f] = acc[f] + hd[f * nbk + b][lane] * blk[f];
+          blk[f] = make_double2(0.0, 0.0);
         }
       }
     }
@@ -326,25 +322,25 @@ inline bool uniform_planes(const Problem& P, DataPlanes* D) {
   return true;
 }
 
-template <typename R, bool PACKED, bool UNI>
+template <typename R, bool REAL, bool UNI>
 cudaError_t apply_variant(const Problem& P, const DataPlanes& D, const cx<R>* vt, cx<R>* wt, cudaStream_t s) {
-  const size_t smem = apply_smem<PACKED>(P.m);
+  const size_t smem = apply_smem<REAL>(P.m);
   static SmemOptIn attr;
-  const cudaError_t e = opt_in_smem(attr, (const void*)k_apply_data<R, PACKED, UNI>, apply_smem<PACKED>(MAX_M));
+  const cudaError_t e = opt_in_smem(attr, (const void*)k_apply_data<R, REAL, UNI>, apply_smem<REAL>(MAX_M));
   if (e != cudaSuccess) return e;
   const int H = P.n / 2 + 1;
-  const dim3 g((unsigned)((H * H + 31) / 32), (P.n_omega + apply_nf<PACKED>() - 1) / apply_nf<PACKED>());
-  k_apply_data<R, PACKED, UNI><<<g, 128, smem, s>>>(P, D, vt, wt);
+  const dim3 g((unsigned)((H * H + 31) / 32), (P.n_omega + apply_nf<REAL>() - 1) / apply_nf<REAL>());
+  k_apply_data<R, REAL, UNI><<<g, 128, smem, s>>>(P, D, vt, wt);
   return cudaGetLastError();
 }
 
 template <typename R>
-cudaError_t launch_apply_data(const Problem& P, const cx<R>* vt, bool packed, cx<R>* wt, cudaStream_t s) {
+cudaError_t launch_apply_data(const Problem& P, const cx<R>* vt, bool real, cx<R>* wt, cudaStream_t s) {
   DataPlanes D;
   memset(&D, 0, sizeof(D));
   if (uniform_planes(P, &D))
-    return packed ? apply_variant<R, true, true>(P, D, vt, wt, s) : apply_variant<R, false, true>(P, D, vt, wt, s);
-  return packed ? apply_variant<R, true, false>(P, D, vt, wt, s) : apply_variant<R, false, false>(P, D, vt, wt, s);
+    return real ? apply_variant<R, true, true>(P, D, vt, wt, s) : apply_variant<R, false, true>(P, D, vt, wt, s);
+  return real ? apply_variant<R, true, false>(P, D, vt, wt, s) : apply_variant<R, false, false>(P, D, vt, wt, s);
 }
 
 }  // namespace
@@ -371,9 +367,9 @@ cudaError_t launch_forward_born(const Problem& P, const R* xi, const cx<R>* u0, 
     k_source<R><<<1024, 256, 0, s>>>(P, xi, u0, src);
     e = launch_fft2_dense<R>(src, src, P.n, (long long)P.n_omega * P.m, false, tw, s);
   } else {
-    // the plane wave is constant on a plane: one transform of the real planes xi_l, two to a
-    // complex plane, instead of one of xi_l e^{-i k0 z'_l} per plane and frequency
-    e = launch_fft2_pairs<R>(xi, src, P.n, P.m, tw, s);
+    // the plane wave is constant on a plane: one transform of the real planes xi_l instead of one of
+    // xi_l e^{-i k0 z'_l} per plane and frequency
+    e = launch_fft2_real<R>(xi, src, P.n, P.m, tw, s);
   }
   if (e != cudaSuccess) return e;
   if ((e = launch_apply_data<R>(P, src, u0 == nullptr, W, s)) != cudaSuccess) return e;

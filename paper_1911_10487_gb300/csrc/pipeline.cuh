@@ -296,10 +296,11 @@ cudaError_t launch_ifft_cols(const cx<R>* in, cx<R>* out, int n, long long plane
 template <typename R>
 cudaError_t launch_xi_transform(const cx<R>* ut, cx<R>* out, const R* xi, int n, long long planes, const cx<R>* tw,
                                 cudaStream_t s);
-// forward 2D FFT of m real planes, two to a complex plane: (m + 1) / 2 planes out, pair p
-// the planes 2p - m % 2 (real part; zero for plane -1) and 2p + 1 - m % 2 (imaginary part)
+// forward 2D FFT of m real planes, times two: out [m][N][real_stride(N)], the columns k <= N/2;
+// F(-nu) = conj(F(nu)) gives the others
+__host__ __device__ constexpr int real_stride(int n) { return n / 2 + 2; }
 template <typename R>
-cudaError_t launch_fft2_pairs(const R* xi, cx<R>* out, int n, int m, const cx<R>* tw, cudaStream_t s);
+cudaError_t launch_fft2_real(const R* xi, cx<R>* out, int n, int m, const cx<R>* tw, cudaStream_t s);
 // the sampled-G kernel tables of one frequency (kernel_plan.cu): G sampled on the grid
 // offsets, its 2D FFT, packed mode-major with omega^2 h_z applied and the traces;
 // gs and ft are scratch of D N^2 complex128 each, tw64 the FP64 twiddles of N
