@@ -351,9 +351,9 @@ typedef enum {
    Returns FS_ENOCONV, with W and u of the remaining frequencies unwritten, when a
    frequency has not converged within max_iter or its iterate grows past 1e30 times the
    incident field (Algorithm 1 with a scatterer too strong for the fixed point:
-   omega^2 ||T xi|| >= 1).  Uses the context workspace; synchronises the context's
-   stream at each stopping test and GMRES inner product, so it cannot be captured in a
-   graph. */
+   omega^2 ||T xi|| >= 1); nothing of the call is left running then.  Uses the context
+   workspace; the host waits at each stopping test and GMRES inner product, so it cannot
+   be captured in a graph. */
 fs_status fs_forward(fs_ctx* ctx, const fs_geometry* geom, fs_precision prec, const void* xi,
                      const void* incident, const double* omega, int n_omega, double c0, fs_forward_method method,
                      int max_iter, double rtol, void* W, void* u, int* iterations);

@@ -692,7 +692,8 @@ cudaError_t norm2_host(const cx<R>* a, long long count, double2* partial, cudaSt
 // V~ = F_r[xi F^-1 U~] of it in *vt.  The stopping test is taken on the host each iteration,
 // but the transform of the next V~, which only reads U~, is enqueued before the host waits for
 // the test's value (mapped page-locked `host`, event `ev`): the wait hides behind it, and at
-// convergence it is the V~ that eq. (7) needs.
+// convergence it is the V~ that eq. (7) needs.  Not so in the last iteration allowed, which mostly ends
+// a solve that fails.  Without convergence nothing is left running on return: xi is the caller's again.
 template <typename R>
 cudaError_t fixed_point_one(const Problem& Q, const R* xi, const cx<R>* u0, const FwdLayout<R>& L, const cx<R>* tw,
                             double rtol, int max_iter, cudaStream_t s, volatile double* host, cudaEvent_t ev,
@@ -724,11 +725,13 @@ cudaError_t fixed_point_one(const Problem& Q, const R* xi, const cx<R>* u0, cons
     if ((e = launch_interior<R, true>(Q, sc, ut, partial, u0t, inc, s)) != cudaSuccess) return e;
     k_sum_partials<<<1, 256, 0, s>>>(partial, nblk, const_cast<double*>(host));
     if ((e = cudaEventRecord(ev, s)) != cudaSuccess) return e;
-    if ((e = launch_xi_transform<R>(ut, sc, xi, Q.n, Q.m, tw, s)) != cudaSuccess) return e;
+    const bool ahead = it < max_iter;
+    if (ahead && (e = launch_xi_transform<R>(ut, sc, xi, Q.n, Q.m, tw, s)) != cudaSuccess) return e;
     if ((e = cudaEventSynchronize(ev)) != cudaSuccess) return e;
     const double diff = sqrt(*host);
     if (diff <= rtol * nrm0) {
       ok = true;
+      if (!ahead && (e = launch_xi_transform<R>(ut, sc, xi, Q.n, Q.m, tw, s)) != cudaSuccess) return e;
       break;
     }
     if (!(diff <= 1e30 * nrm0)) break;  // diverged (or not finite)
@@ -736,7 +739,7 @@ cudaError_t fixed_point_one(const Problem& Q, const R* xi, const cx<R>* u0, cons
   *iters = it;
   *conv = ok;
   *vt = sc;
-  return cudaSuccess;
+  return ok ? cudaSuccess : cudaStreamSynchronize(s);
 }
 
 template <typename R> struct Krylov {
