@@ -64,9 +64,11 @@ fs_status run_static(const Problem& P, const Layout& L, unsigned char* base, con
   unsigned long long* ctr = (unsigned long long*)(base + ctr_off);
   cx<R>* tw = (cx<R>*)(base + tw_off);
   Work<R> w = carve_work<R>(base, L, ctr, tw, nullptr);
-  // the scratch keeps the previous call's contents: the counters start at zero,
-  // the twiddles are rewritten for this N and precision
-  if (cudaMemsetAsync(ctr, 0, sizeof(unsigned long long) * C_COUNT, s) != cudaSuccess) return FS_ECUDA;
+  // the scratch keeps the previous call's contents: the twiddles are rewritten for this N and precision,
+  // the counters start at zero.  The transforms read the table before their programmatic-launch wait,
+  // that is, ordered behind the predecessor's completion but not behind its writes becoming visible:
+  // the table is made first, and the memset between it and the first transform, a full dependency on
+  // both sides, makes it visible.
   if (launch_twiddles<R>(tw, P.n, s) != cudaSuccess) return FS_ECUDA;
   if (wide_route(P, sizeof(R) == 8)) {
     double2* tw64 = (double2*)(base + tw64_off);
@@ -74,6 +76,7 @@ fs_status run_static(const Problem& P, const Layout& L, unsigned char* base, con
     w.wt64 = (double2*)(base + L.t12);
     w.tw64 = tw64;
   }
+  if (cudaMemsetAsync(ctr, 0, sizeof(unsigned long long) * C_COUNT, s) != cudaSuccess) return FS_ECUDA;
   const char* stage = "";
   return launch_pipeline<R>(P, w, W, xi, c, s, nullptr, &stage) == cudaSuccess ? FS_OK : FS_ECUDA;
 }
