@@ -132,15 +132,15 @@ typedef struct {
                           it (solve_form 1 gives FS_EUNSUPPORTED); eq. (9) is applied as the
                           Toeplitz matrix T_nu; no mode is excluded as grazing.  Only
                           fs_reconstruct and fs_reconstruct_host accept it.             */
-  int classify_single_pass; /* 0 (default): the norms of the modes, the discrepancy test and the
-                          active list in three kernels.  1: in one cooperative launch whose
-                          blocks meet at two bounded device-side barriers (a wait that runs
-                          out is reported by fs_sync_status as FS_ETIMEOUT); taken when the
-                          device holds the grid co-resident, else the three-kernel form.
-                          Fewer launches (batches); on one 128^2 problem the three kernels,
-                          overlapped by programmatic dependent launch, are faster (measured).
-                          Results are identical up to the rounding of the sum ||W||^2 (its
-                          terms are grouped differently).                                  */
+  int classify_single_pass; /* 0 (default): FS_MIXED: the norms of the modes, the discrepancy
+                          test and the active list in one kernel, ||W|| being summed by the
+                          forward transform as it reads W; FS_FP64 and the truncated SVD: in
+                          three kernels.  1: in one cooperative launch whose blocks meet at
+                          two bounded device-side barriers (a wait that runs out is reported
+                          by fs_sync_status as FS_ETIMEOUT); taken when the device holds the
+                          grid co-resident, else three kernels.  Results are identical up to
+                          the rounding of the sum ||W||^2 (its terms are grouped
+                          differently).                                                    */
   int fft_tile;        /* tile shape of the transform passes, a tuning knob: 0 (default)
                           up to 16 (FP32) / 8 (FP64) rows or columns per tile, radix cap
                           16; 1: half as many, radix cap 8 (twice the blocks, half the

@@ -35,13 +35,6 @@ __host__ __device__ __forceinline__ double2 operator*(double s, double2 a) { ret
 
 __host__ __device__ __forceinline__ float2 conjx(float2 a) { return make_float2(a.x, -a.y); }
 __host__ __device__ __forceinline__ double2 conjx(double2 a) { return make_double2(a.x, -a.y); }
-// a * conj(b)
-__host__ __device__ __forceinline__ float2 mulc(float2 a, float2 b) {
-  return make_float2(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
-}
-__host__ __device__ __forceinline__ double2 mulc(double2 a, double2 b) {
-  return make_double2(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
-}
 // conj(a) * b
 __host__ __device__ __forceinline__ double2 cmul_conj_a(double2 a, double2 b) {
   return make_double2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
@@ -72,10 +65,10 @@ template <typename R> __host__ __device__ __forceinline__ cx<R> czero() { return
 // Programmatic dependent launch.  The kernels of one reconstruction are launched
 // with programmatic stream serialisation: a kernel may become resident while its
 // predecessor is still running, and waits at pdl_wait() -- before its first
-// global-memory access other than reads of the constant twiddle tables (made and
-// synchronised once, before any reconstruction) -- until the predecessor grid has
-// completed and its writes are visible.  pdl_trigger() lets the successor launch as soon as every block of
-// this grid has started.  Launched without the attribute, both are no-ops.
+// global-memory access other than reads of the constant twiddle tables (synchronised when
+// made, or with a plain launch or a memset between their kernel and the first reader) --
+// until the predecessor grid has completed and its writes are visible.  pdl_trigger() lets
+// the successor launch as soon as every block of this grid has started.  Launched without the attribute, both are no-ops.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

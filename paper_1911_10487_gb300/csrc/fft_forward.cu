@@ -4,13 +4,12 @@
 //
 //   fft2_forward  : W -> W~ on every data plane (Sec. 4, Algorithm 2 step 1 needs
 //                   W~ = F_r[W]), then ||W~_nu||^2 summed over the planes of a
-//                   frequency, which the discrepancy test needs.
-//   recover       : V~, U~ -> V = F^-1[V~], u = F^-1[U~] (Algorithm 2 step 2) and
-//                   xi = Re(sum conj(u) V)/sum |u|^2, c = (c0^-2 - xi)^-1/2
-//                   (step 3, Sec. 5.2; Sec. 1 for c).  The inverse column pass
-//                   gathers the solved profiles of the active modes only and
-//                   transforms only the columns nu1 that hold a nonzero mode; the
-//                   row pass scatters those columns and transforms full rows.
+//                   frequency, which the discrepancy test needs (FP32: in the
+//                   classification, from ||W||^2 summed here over W itself).
+//   real planes   : F_r[xi] of the plane-wave generator; rows around the product
+//                   with xi of Algorithm 1's iteration; the inverse rows of the
+//                   derivatives' directions joined with step 3.
+// The inverse passes of a reconstruction are in fft_inverse.cu.
 #include "diff.cuh"
 #include "fft_pass.cuh"
 
@@ -296,7 +295,9 @@ k_rows_xi(cx<R>* __restrict__ data, const R* __restrict__ xi, long long nrows, c
 // 2.1 of 6.5 GB of a 16-direction call at 128^2 x 64, 4 frequencies (FP32): rows 307 us + point
 // 212 us before, 417 us now.  In FP32 V and u are loaded before the rows are transformed, and
 // 256 threads share a tile from N = 96 on, so that more loads are in flight (420 us without the
-// first at 128 threads, 436 us with it).
+// first at 128 threads, 436 us with it).  16 directions, 32 planes, 2 frequencies, with 128 threads beside:
+// N = 128 133 us (147), but 96 120 (111) and 192 640 (510), whose 12-point last stage leaves 256 threads
+// idle in part; below, 128 against 256: 32 12.0 (14.2), 48 19.6 (23.2), 64 32.9 (33.2).
 template <typename R, int N> struct JvpPass {
   static constexpr bool F32 = sizeof(R) == 4;
   using PL = IoPlan<N, F32 || N != 256 ? 16 : 8, F32>;

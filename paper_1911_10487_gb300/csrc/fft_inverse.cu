@@ -174,14 +174,19 @@ __device__ __forceinline__ void recover_epilogue(const Problem& P, const R* num,
 // instead (Problem::u_guard_raw), which saves FP64 products per voxel and frequency.
 template <typename R, int N, int T> struct RecPass {
   static constexpr bool F32 = sizeof(R) == 4;
-  // radices that give each stage of a small FP64 tile whole warps
+  // Radices that give each stage of a small FP64 tile whole warps, against 16 throughout: one
+  // frequency, 16 planes: N = 16 16.3 us (20.1), 32 19.3 (23.2), 64 45.1 (45.1); 4 frequencies, 64 planes:
+  // 32 95 (103), but 16 68 (55) and 64 194 (157), where the tiles fill the chip and fewer stages win
   static constexpr int MAXR = T == 1 ? 8 : F32 ? 16 : (N == 16 ? 4 : N <= 64 ? 8 : 16);
   using PL = IoPlan<N, MAXR, false>;
   static constexpr int NT = F32 ? (N >= 192 ? 256 : 128) : (N >= 192 ? 128 : 64);
   static constexpr int ROWS0 = F32 ? (N <= 16 ? 16 : 8) : (N <= 16 ? 8 : 4);
   static constexpr int LINES = T == 0 ? (F32 && N == 256 ? 4 : ROWS0) : ROWS0 / 2;
   static constexpr int SKEW = 16;
-  // resident blocks the registers are held to: at 128^2 x 64 the pass's 1024 blocks at once
+  // resident blocks the registers are held to: at 128^2 x 64 the pass's 1024 blocks at once (72
+  // registers, 52-64 bytes of them spilled at N = 128).  128^2 x 64, 4 frequencies: 24.3 us, 27.4
+  // without; 128^2 x 16, one frequency: 7.5 and 7.0.  N = 64: the same registers either way; the other
+  // lengths lose by it (96^2 x 64, 4 frequencies: 20.9 us as here, 25.1 held to 7)
   static constexpr int MINB = !F32 || T == 1 ? 1 : N >= 192 ? 3 : (N == 128 || N == 64) ? 7 : 1;
   static constexpr int SC = !F32 && N == 256 ? 16 : 32;  // staged columns per row (RecStage)
   static constexpr int E = LINES * N, PER = (E + NT - 1) / NT;  // voxels of the block, of a thread
@@ -227,7 +232,9 @@ __device__ __forceinline__ void recover_first(cx<R>* buf, Ld ld) {
 // read once for both, and the sums come straight from the last stage's registers (recover_pass takes
 // them through the tile, one more write and read).  256^2 x 64, 8 frequencies: 117 us -> 100 us, the
 // batch of 32 smaller problems 1.37 -> 1.32 ms; bound by issue slots and latency at 16 warps per SM
-// (54% of the slots; a tile of 4 rows at N = 256: static shared memory holds no 8).
+// (54% of the slots; 128 registers, of which the FP64 redo and the sums spill 192 bytes at N = 256, 360
+// with a given incident field, and 16-48 at 192; a tile of 4 rows at N = 256: static shared memory holds
+// no 8).
 template <typename R, int N, int T> struct RecPair {
   using RP = RecPass<R, N, T>;
   using PL = typename RP::PL;

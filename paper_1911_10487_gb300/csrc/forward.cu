@@ -28,14 +28,6 @@ namespace fl {
 
 namespace {
 
-// e^{i k_z d}, no sine and cosine for an evanescent mode
-__device__ __forceinline__ double2 exp_kz(double2 kz, double d) {
-  if (kz.x == 0.0) return make_double2(exp(-kz.y * d), 0.0);
-  double s, c;
-  sincos(kz.x * d, &s, &c);
-  return make_double2(c, s);
-}
-
 // V = xi u0 on X (omega^2 sits in the kernel factor), u0 the given incident field
 // [n_omega][M][N][N]
 template <typename R>
@@ -77,7 +69,7 @@ __global__ void k_point_sources(Problem P, const double* __restrict__ spec, int 
       const double nu1 = P.kn * m1, nu2 = P.kn * m2;
       for (int j = 0; j < n_src; ++j) {
         const double* sp = spec + 4 * j;
-        const double2 ez = exp_kz(kz, sp[2] - zl);  // sources above X: |dz| = z_s - z'_l
+        const double2 ez = exp_ikz_inline(kz, sp[2] - zl);  // sources above X: |dz| = z_s - z'_l
         double sn, cs;
         sincos(-(nu1 * (sp[0] - x0) + nu2 * (sp[1] - x0)), &sn, &cs);
         acc = acc + sp[3] * (ez * make_double2(cs, sn));
@@ -214,7 +206,7 @@ k_apply_data(Problem P, DataPlanes D, const cx<R>* __restrict__ vt, cx<R>* __res
       const double2 k = kz_vec(propm >> f & 1u, kz[f]);
       for (int b = 0; b <= nbk; ++b, ++it) {
         if ((it & 3) != w) continue;
-        double2 x = exp_kz(k, b < nbk ? HB * (nbk - 1 - b) * P.hz : P.hz);
+        double2 x = exp_ikz_inline(k, b < nbk ? HB * (nbk - 1 - b) * P.hz : P.hz);
         if (REAL) x = x * (b < nbk ? phs[f * nbk + b] : ex[f][0]);
         if (b < nbk) hd[f * nbk + b][lane] = x;
         else rs[f][lane] = x;
@@ -296,7 +288,7 @@ k_apply_data(Problem P, DataPlanes D, const cx<R>* __restrict__ vt, cx<R>* __res
       const int items = UNI ? 1 + (P.m1 + HB - 1) / HB : kn;  // UNI: the step, then the block heads
       __syncthreads();
       for (int j = w; j < items; j += 4)
-        ex[j][lane] = exp_kz(k, UNI ? (j == 0 ? D.dz : P.zy[HB * (j - 1)] - ztop) : P.zy[k0 + j] - ztop);
+        ex[j][lane] = exp_ikz_inline(k, UNI ? (j == 0 ? D.dz : P.zy[HB * (j - 1)] - ztop) : P.zy[k0 + j] - ztop);
       __syncthreads();
       if (valid) {
         if (cplx) put_data<R, UNI, true>(P, D, ex, lane, k0, kn, k, a, out, N2);
@@ -526,7 +518,7 @@ k_interior(Problem P, const cx<R>* __restrict__ vt, cx<R>* __restrict__ ut, doub
   for (int j = 0; j < CP; ++j) v[j] = valid && l0 + j < l1 ? vt[(l0 + j) * N2 + nu] : czero<R>();
   if (w < 2) {
     const double r = off ? 0.0 : rsqrt64(fabs(qq)), kz = sqrt_from_rsqrt(fabs(qq), r);
-    qs[w][lane] = off ? czero<R>() : from_d<R>(exp_kz(kz_vec(prop, kz), w ? CP * P.hz : P.hz));
+    qs[w][lane] = off ? czero<R>() : from_d<R>(exp_ikz_inline(kz_vec(prop, kz), w ? CP * P.hz : P.hz));
     if (w == 0) gs[lane] = (R)(-P.g0[0] * r);
   }
   __syncthreads();

@@ -122,7 +122,9 @@ template <typename R> struct Work {
   double* partial;  // [n_omega][n_partial] block sums of norms (fixed order)
   int n_partial;
   int* slot;        // [n_omega][N*N] slot of an active mode or -1
-  int* act;         // [n_omega][N*N] active mode list (mode index, ascending)
+  // [n_omega][N*N] active modes: ascending, but in any order on the early route (classify_early), so
+  // nothing may depend on it
+  int* act;
   unsigned* flagbits;  // [n_omega][classify_blocks][32] active-mode bitmask (classification)
   int* blkcnt;      // [n_omega][classify_blocks] active modes per classification block
   int* blkgz;       // [n_omega][classify_blocks] grazing modes per classification block

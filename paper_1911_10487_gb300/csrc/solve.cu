@@ -86,7 +86,7 @@ constexpr int ST = 128;
 // tr(G): a few units of round-off of the normal matrix in each precision
 constexpr float LANCZOS_TOL32 = 1e-6f;
 constexpr double LANCZOS_TOL64 = 1e-14;
-static_assert(ST == 2 * DENSE_M && ST == 4 * DENSE_M1, "thread maps of the solve assume 2 threads per plane l and 4 per data plane k");
+static_assert(ST == 2 * DENSE_M && ST == 4 * DENSE_M1, "two threads per plane l and four per data plane k at the largest sizes");
 
 // ------------------------------------------------------------------------------
 // classification (integer arithmetic only), in two passes over blocks of CMB

@@ -4,9 +4,9 @@ For a batch signature (the sorted multiset of (N, M, M1, n_omega) and the
 precision) it times the candidate launch configurations -- the number of
 concurrent streams the batch is dealt over (1 to 64), the resident blocks per SM of
 the dense per-mode solve, the tile shape of the transform passes (fs_options.fft_tile:
-2048-element tiles with radix cap 16, or 1024-element tiles with radix cap 8) and
-the form of the classification (fs_options.classify_single_pass: three kernels, or
-one cooperative launch) --
+radix cap 16, or half the lines per tile and radix cap 8) and
+the form of the classification (fs_options.classify_single_pass: one kernel after
+the forward transform in FP32 and three in FP64, or one cooperative launch) --
 with CUDA events on the library's stream, and keeps the fastest.  The signature
 ignores the plane heights and the noise level: they change neither the launch
 shapes nor the work per mode of the transforms.  Results are cached in memory and,
