@@ -95,7 +95,7 @@ __global__ void k_point_sources(Problem P, const double* __restrict__ spec, int 
 // four warps deal the exponentials among themselves through shared memory, then each sums its
 // own modes.  An evanescent mode (q, E real) takes real products.  Before, one thread per
 // mode took an exp and a sincos per plane: 192^2, 37 + 19 planes, 5 frequencies (FP64, REAL)
-// 1067 us -> 205 us, 128^2, 64 + 32 planes 363 us -> 44 us.
+// 1067 us -> 194 us (85% of the FP64 rate), 128^2, 64 + 32 planes 363 us -> 44 us.
 //
 // REAL (the plane incident wave): V~_l = e^{-i k0 z'_l} F[xi_l], and the transform of the real planes
 // xi_l, half of its columns (launch_fft2_real), serves every frequency (FG of them per block, so that it
