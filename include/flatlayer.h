@@ -77,7 +77,8 @@ typedef enum {
    above that.  Below it (the paper's noise levels 0 and 1e-7 of Sec. 5 with a small
    delta_floor) fs_reconstruct returns FS_EUNSUPPORTED: FS_FP64 is the path for such
    data.  Given alpha (alpha_mode 1) and the truncated SVD (whose route transforms W
-   in FP64) are not limited. */
+   in FP64) are not limited.  The norms ||W~_nu||^2 of the modes are FP32 numbers: W~,
+   N to N^2 times W, has to lie between about 1e-19 and 1e19. */
 #define FS_MIXED_MIN_NOISE 1e-6
 
 /* Limits of this build: N in {8,12,16,24,32,48,64,96,128,192,256}; 1 <= M <= 128;
